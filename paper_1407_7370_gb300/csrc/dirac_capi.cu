@@ -90,6 +90,12 @@ void spectral_interval(int order, double dx, double dy, double mass, double c, d
   half = (emax + 0.5 * (vmax - vmin)) * (1.0 + 1e-8) + 1e-12;
 }
 
+// exponent field of max |V| for vmin <= V <= vmax (0: V = 0)
+int v_exponent(double vmin, double vmax) {
+  const double v = std::max(std::fabs(vmin), std::fabs(vmax));
+  return v > 0.0 ? std::max(0, std::ilogb(v) + 1023) : 0;
+}
+
 dirac_status make_cheb(double c0, double half, double dt, double shift, ChebParams& cp) {
   const double R = half * dt;
   if (!(R > 0.0) || R > 90.0)
@@ -200,13 +206,13 @@ struct LaunchShape {
 // Persistent launch: as many CTAs as are resident at once (at most one per
 // tile), each taking a contiguous chunk of the tile list whose size differs
 // from the others' by at most one tile.
-template <class S, int R, int TH, bool D, bool V, bool AY>
+template <class S, int R, int TH, bool D, bool V, bool FLAG>
 cudaError_t launch_pass_t(LaunchParams p, const LaunchShape& ls, cudaStream_t s) {
   static std::atomic<int> occ_dev[OCC_MAX_DEVICES];
-  constexpr int NT = sub_workers<S>() * 32 * (TH / rows_per_thread<S, TH>());
+  constexpr int NT = pass_threads<S, TH>();
   constexpr size_t smem = dyn_smem_bytes<S, R, TH, sub_workers<S>()>();
   int occ = 0;
-  cudaError_t e = occupancy_on_device(occ_dev, lanczos_pass<S, R, TH, D, V, AY>, NT, smem, &occ);
+  cudaError_t e = occupancy_on_device(occ_dev, lanczos_pass<S, R, TH, D, V, FLAG>, NT, smem, &occ);
   if (e != cudaSuccess) return e;
   if (occ < 1) occ = 1;
   const int per_sm = ls.cta_cap > 0 ? std::min(occ, ls.cta_cap) : occ;
@@ -215,29 +221,28 @@ cudaError_t launch_pass_t(LaunchParams p, const LaunchShape& ls, cudaStream_t s)
   p.chunk_q = p.total_tiles / grid;
   p.chunk_r = p.total_tiles % grid;
   p.async_tiles = p.chunk_q >= ASYNC_MIN_TILES;
-  return launch_pdl(lanczos_pass<S, R, TH, D, V, AY>, grid, NT, smem, s, p);
+  return launch_pdl(lanczos_pass<S, R, TH, D, V, FLAG>, grid, NT, smem, s, p);
 }
 
-// FP64: a kernel without the c A_y terms (four FMAs per site of ~54) when no
-// step of the launch has A_y != 0 (linear polarisation along x, static
-// fields); the FP32 pass, bound by memory, keeps one kernel
+// FP64: with kx = ky (dx = dy) the two differences of a row are added before
+// their one product; the FP32 pass keeps one kernel
 template <class S, int R, int TH, bool D, bool V>
-cudaError_t launch_pass_ay(const LaunchParams& p, const LaunchShape& ls, cudaStream_t s) {
+cudaError_t launch_pass_iso(const LaunchParams& p, const LaunchShape& ls, cudaStream_t s) {
   if constexpr (sizeof(S) == sizeof(double)) {
-    if (!p.has_ay) return launch_pass_t<S, R, TH, D, V, false>(p, ls, s);
+    if (p.iso) return launch_pass_t<S, R, TH, D, V, true>(p, ls, s);
   }
-  return launch_pass_t<S, R, TH, D, V, true>(p, ls, s);
+  return launch_pass_t<S, R, TH, D, V, false>(p, ls, s);
 }
 
 template <class S, int TH>
 cudaError_t launch_pass_s(int order, bool diri, bool hasv, const LaunchParams& p, const LaunchShape& ls,
                           cudaStream_t s) {
   if (order == 2) {
-    if (diri) return hasv ? launch_pass_ay<S, 1, TH, true, true>(p, ls, s) : launch_pass_ay<S, 1, TH, true, false>(p, ls, s);
-    return hasv ? launch_pass_ay<S, 1, TH, false, true>(p, ls, s) : launch_pass_ay<S, 1, TH, false, false>(p, ls, s);
+    if (diri) return hasv ? launch_pass_iso<S, 1, TH, true, true>(p, ls, s) : launch_pass_iso<S, 1, TH, true, false>(p, ls, s);
+    return hasv ? launch_pass_iso<S, 1, TH, false, true>(p, ls, s) : launch_pass_iso<S, 1, TH, false, false>(p, ls, s);
   }
-  if (diri) return hasv ? launch_pass_ay<S, 2, TH, true, true>(p, ls, s) : launch_pass_ay<S, 2, TH, true, false>(p, ls, s);
-  return hasv ? launch_pass_ay<S, 2, TH, false, true>(p, ls, s) : launch_pass_ay<S, 2, TH, false, false>(p, ls, s);
+  if (diri) return hasv ? launch_pass_iso<S, 2, TH, true, true>(p, ls, s) : launch_pass_iso<S, 2, TH, true, false>(p, ls, s);
+  return hasv ? launch_pass_iso<S, 2, TH, false, true>(p, ls, s) : launch_pass_iso<S, 2, TH, false, false>(p, ls, s);
 }
 
 // FP64 path: everything complex128.  Mixed path: complex64 basis (passes 1
@@ -673,6 +678,7 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     d.basis = q.basis; d.ybuf0 = q.ybuf[0]; d.ybuf1 = q.ybuf[1];
     d.V = q.has_v ? q.V : nullptr;
     d.Vlo = q.has_v ? q.Vlo : nullptr;
+    d.vbe = q.has_v ? v_exponent(q.vmin, q.vmax) : 0;
     d.st = d_st + b;
     d.partials = d_partials + 3 * q.slot_off;
     d.cheb = reinterpret_cast<const ChebParams*>(db + off_cheb) + b;
@@ -696,12 +702,12 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     }
     hasv = hasv || q.has_v;
   }
-  bool has_ay = false;
+  bool iso = true;
+  for (int b = 0; b < np; ++b) iso = iso && hp[b].kx == hp[b].ky;
   for (int k = 0; k < nfield; ++k) {
     const int b = k % np;
     const double ax = a_xy ? a_xy[2 * (size_t)k] : P[b].ax;
     const double ay = a_xy ? a_xy[2 * (size_t)k + 1] : P[b].ay;
-    has_ay = has_ay || ay != 0.0;
     FieldStep& f = hf[k];
     f.cAx = c * ax;   // electron: p - qA = p + A
     f.cAy = c * ay;
@@ -728,7 +734,7 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
   lp.mcc = mcc;
   lp.dt = dt;
   lp.conj_coef = backward ? 1 : 0;
-  lp.has_ay = has_ay ? 1 : 0;
+  lp.iso = iso ? 1 : 0;
   lp.diri = boundary == DIRAC_DIRICHLET ? 1 : 0;
   lp.tol = tol;
   lp.step = d_step;
@@ -1595,6 +1601,7 @@ extern "C" dirac_status dirac_lanczos_step_noalloc(const dirac_problem* pb, void
   d.ybuf0 = base + off_y;
   d.ybuf1 = base + off_y + field;
   d.V = pb->V_dev;
+  d.vbe = pb->V_dev ? v_exponent(vmin, vmax) : 0;
   d.st = st;
   d.partials = partials;
   d.cheb = reinterpret_cast<const ChebParams*>(base + off_cheb);
@@ -1625,7 +1632,7 @@ extern "C" dirac_status dirac_lanczos_step_noalloc(const dirac_problem* pb, void
   lp.fstride = 0;
   lp.nprob = 1;
   lp.total_tiles = ntiles;
-  lp.has_ay = pb->A_y != 0.0 ? 1 : 0;
+  lp.iso = d.kx == d.ky ? 1 : 0;
   lp.m = m;
   lp.mcc = mcc;
   lp.dt = dt;

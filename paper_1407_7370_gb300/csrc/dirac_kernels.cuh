@@ -46,7 +46,8 @@
 // serial eigensolver dominate small steps, while the Chebyshev recurrence is
 // FMA-only and warp-parallel.  Both give exp(-i T dt) e_1 to rounding.
 //
-// Precision: S = double is the FP64 path.  S = float is the mixed path:
+// Precision: S = double is the FP64 path (complex128 fields; the products in
+// 60-bit fixed point, dirac_fixed.cuh).  S = float is the mixed path:
 // complex64 basis and y^, FP32 stencil, warp sums converted to FP64, FP64
 // scalars; q^_1 is the complex128 state itself (passes 1-2 read it).
 #pragma once
@@ -55,6 +56,9 @@
 #include <stdint.h>
 
 #include <cuda/atomic>
+#include <type_traits>
+
+#include "dirac_fixed.cuh"
 
 namespace dirac {
 
@@ -69,10 +73,12 @@ using vec4 = double4_32a;       // one site: (u.re, u.im, d.re, d.im)
 // (FP64 values and FP32 copies, so that no thread converts on the FP64 pipe).
 struct PassCoef {
   double g, gd, e, au0, ad0;          // q^ = g y^ - gd q^_prev; y^ -= e q^_prev; diagonals
-  float gf, gdf, ef, au_hi, au_lo, ad_hi, ad_lo, pad;
+  float gf, gdf, ef, au_hi, au_lo, ad_hi, ad_lo;
+  float yexp;                         // FP64 path: the pass stores 2^yexp y^ (an integer; 0 on the mixed path)
 };
 
-__host__ __device__ inline PassCoef make_coef(double g, double gd, double e, double au0, double ad0) {
+__host__ __device__ inline PassCoef make_coef(double g, double gd, double e, double au0, double ad0,
+                                              float yexp = 0.f) {
   PassCoef c;
   c.g = g; c.gd = gd; c.e = e; c.au0 = au0; c.ad0 = ad0;
   c.gf = (float)g; c.gdf = (float)gd; c.ef = (float)e;
@@ -81,7 +87,7 @@ __host__ __device__ inline PassCoef make_coef(double g, double gd, double e, dou
   // perturbation of the mass term
   c.au_hi = (float)au0; c.au_lo = (float)(au0 - (double)c.au_hi);
   c.ad_hi = (float)ad0; c.ad_lo = (float)(ad0 - (double)c.ad_hi);
-  c.pad = 0.f;
+  c.yexp = yexp;
   return c;
 }
 
@@ -137,6 +143,7 @@ struct Problem {
   float kxf, kyf;           // kx, ky rounded to FP32
   float kxf_lo, kyf_lo;     // and their remainders
   int tma;                  // the mixed one-launch step stages tiles by tensor copies (maps valid)
+  int vbe;                  // FP64 path: exponent field of max |V| (0: V = 0)
   PassCoef probe_coef;      // coefficients of the probe pass (stencil shift 0)
 };
 
@@ -165,7 +172,7 @@ struct LaunchParams {
   int pass, m, probe;
   int conj_coef;            // 1: backward step (dt < 0): exp(+i H |dt|), the conjugate coefficients
   int async_tiles;          // FP32 basis: stage passes >= 3 by asynchronous copies (many tiles per CTA)
-  int has_ay;               // 0: A_y = 0 in every step and problem (host: picks the kernel)
+  int iso;                  // FP64 path: kx = ky in every problem (host: picks the kernel)
   int diri;                 // Dirichlet boundaries (kernels that take the boundary at run time)
   double mcc, dt, tol;      // dt = |dt|
   const int* step;          // step counter of the running call (index into fields)
@@ -256,10 +263,6 @@ __device__ __forceinline__ T ld4(const T* p) {
   else return ldg4(p);
 }
 
-template <class S> struct Vec4;
-template <> struct Vec4<double> { using T = double4_32a; };
-template <> struct Vec4<float> { using T = float4; };
-
 template <class To, class From>
 __device__ __forceinline__ void cvt4(const From& a, To (&o)[4]) {
   o[0] = (To)a.x; o[1] = (To)a.y; o[2] = (To)a.z; o[3] = (To)a.w;
@@ -308,6 +311,19 @@ __device__ inline void cheb_expm_e1(const ChebParams& cp, int k, double alpha_j,
 // with plain loads up front; new values travel by shuffles.  rsqrt gives
 // sqrt(X), 1/X, sqrt(s2) and 1/sqrt(s2) with few dependent FP64 operations.
 // ---------------------------------------------------------------------------
+// FX (the FP64 path): the pass stores 2^yexp y^ with yexp an integer chosen
+// before it, and g = 1 on that vector: forming q^ then takes one multiply-add
+// per number instead of two, and no scale can overflow.  P and Y come in for
+// the scaled vector.
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// floor(log2 x) of a positive normal number; 0 for zero
+__device__ __forceinline__ int log2_floor(double x) { return x > 0.0 ? fx::exp_field(x) - 1023 : 0; }
+__device__ __forceinline__ float next_yexp(double beta_pred, double nu) {
+  const int e = -(log2_floor(beta_pred) + log2_floor(nu));
+  return (float)max(-1000, min(1000, e));
+}
+
+template <bool FX>
 __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, DevState* st, int i, double P,
                                    double Y, double X) {
   const unsigned full = 0xffffffffu;
@@ -321,7 +337,8 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
       if (ok || zero) {
         const double s1 = ok ? P / X : 0.0;   // the probe ran with stencil shift 0
         st->sigma[1] = s1;
-        st->pc_cur = make_coef(1.0, 0.0, 0.0, lp.mcc - shift - s1, -lp.mcc - shift - s1);
+        st->pc_cur = make_coef(1.0, 0.0, 0.0, lp.mcc - shift - s1, -lp.mcc - shift - s1,
+                               FX && ok ? next_yexp(sqrt(Y / X), sqrt(X)) : 0.f);
         st->cur_pass = 1;
         st->redo_left = lp.redo_budget;
         st->sigma_valid = 1;
@@ -373,6 +390,13 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
   const double alpha_next_prev = (i + 1 <= k_prev && i + 1 <= KMAX) ? st->alpha[i + 1] : 0.0;
   const double alpha_im1 = (i >= 2) ? st->alpha[i - 1] : 0.0;
   const PassCoef pc_now = st->pc_cur;
+  // FX: 2^-yexp of this pass and of the one before, the last estimate of
+  // beta_{i+1} and 1 / nu_{i-1}
+  const double unscale = FX ? pow2(-(int)pc_now.yexp) : 1.0;
+  const double unscale_prev = (FX && i >= 2) ? pow2(-(int)st->pc_prev.yexp) : 1.0;
+  const double invnu_im1 = (FX && i >= 2) ? st->inv_nu[i - 1] : 0.0;
+  const double beta_next_prev = (FX && i + 1 <= k_prev && i + 1 <= KMAX) ? st->beta[i + 1] : 0.0;
+  const double beta1_old = (FX && i >= 2) ? st->beta[1] : 0.0;
   __syncwarp();   // every lane has read the state before lane 0 updates it
 
   // scalar chain (every lane computes it; no broadcast needed)
@@ -380,12 +404,13 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
   const double nu = X * y;
   const double rX = y * y;
   const double dd = P * rX;             // alpha_i - sigma_i
-  const double alpha = sigma + dd;
+  const double alpha = FX ? fma(dd, unscale, sigma) : sigma + dd;
   const double s2 = fma(-P, dd, Y);     // nu_i^2 beta_i^2 (estimate)
   const double rs = s2 > 0.0 ? rsqrt(s2) : 0.0;
   const double sq = s2 > 0.0 ? s2 * rs : 0.0;
-  const double beta_hat = sq * y;
-  const double bprev = nu * bhat_prev;  // exact beta_{i-1} from the measured norm
+  const double beta_hat = FX ? sq * y * unscale : sq * y;
+  // exact beta_{i-1} from the measured norm
+  const double bprev = FX ? nu * invnu_im1 * unscale_prev : nu * bhat_prev;
   // The stencil shift sigma_i was too far from alpha_i for the precision of
   // y^ (s2 is then cancellation noise): run pass i again with sigma_i =
   // alpha_i, which makes s2 ~ Y.  Everything derived from X (nu, beta_{i-1})
@@ -395,7 +420,7 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
       st->redo_left = redo_left - 1;
       st->sigma[i] = alpha;
       st->pc_cur = make_coef(pc_now.g, pc_now.gd, pc_now.e, lp.mcc - shift - alpha,
-                             -lp.mcc - shift - alpha);
+                             -lp.mcc - shift - alpha, pc_now.yexp);
       if (s2 > 0.0) st->kappa_max = fmax(st->kappa_max, Y * rs * rs);
     }
     return;
@@ -427,7 +452,11 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
       const double sig = (i + 1 <= k_prev) ? alpha_next_prev : (i >= 2 ? alpha_im1 : alpha);
       st->sigma[i + 1] = sig;
       st->pc_prev = pc_now;
-      st->pc_cur = make_coef(rs, rs * dd, sq * rX, lp.mcc - shift - sig, -lp.mcc - shift - sig);
+      if constexpr (FX)
+        st->pc_cur = make_coef(1.0, dd, s2 * rX * unscale, lp.mcc - shift - sig, -lp.mcc - shift - sig,
+                               next_yexp(beta_next_prev > 0.0 ? beta_next_prev : beta_hat, sq));
+      else
+        st->pc_cur = make_coef(rs, rs * dd, sq * rX, lp.mcc - shift - sig, -lp.mcc - shift - sig);
       st->cur_pass = i + 1;
     }
   }
@@ -462,7 +491,9 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
     st->beta_last = beta_hat;
     const double s1 = (i == 1) ? alpha : alpha1_old;   // next step's first shift
     st->sigma[1] = s1;
-    st->pc_cur = make_coef(1.0, 0.0, 0.0, lp.mcc - shift - s1, -lp.mcc - shift - s1);
+    const double b1 = (i == 1) ? beta_hat : (i == 2 ? bprev : beta1_old);
+    st->pc_cur = make_coef(1.0, 0.0, 0.0, lp.mcc - shift - s1, -lp.mcc - shift - s1,
+                           FX ? next_yexp(b1, nu1) : 0.f);
     st->sigma_valid = 1;
     st->stopped = 1;
   }
@@ -487,8 +518,9 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
 // cross-shaped halo of q^_i are formed in shared memory from y^_{i-1} and
 // q^_{i-1}.
 // ---------------------------------------------------------------------------
-template <class S, int TH, int SUB>
-__host__ __device__ constexpr int min_blocks() { return sizeof(S) == sizeof(float) ? (TH == 32 ? 4 : 8) : (SUB == 2 ? 1 : 2); }
+// CTAs per SM of the FP32 pass (128 or 256 threads each)
+template <int TH>
+__host__ __device__ constexpr int min_blocks() { return TH == 32 ? 4 : 8; }
 
 // rows per thread: four, except two on FP64 16-row tiles, which keep eight
 // warps per tile worker and halve the unit of work: a grid of a few tiles per
@@ -500,25 +532,17 @@ __host__ __device__ constexpr int rows_per_thread() { return (sizeof(S) == sizeo
 template <class S>
 __host__ __device__ constexpr int sub_workers() { return sizeof(S) == sizeof(double) ? 2 : 1; }
 
-// shared memory of one tile worker: the tile of q^_i with its halo, and on
-// the mixed path the staging buffer of q^_{i-1} on the same rectangle
-template <class S, int R, int TH>
-__host__ __device__ constexpr size_t tile_bytes() { return sizeof(S) * 4 * (TH + 2 * R) * (TILE_W + 2 * R); }
-template <class S, int R, int TH>
-__host__ __device__ constexpr size_t qbuf_bytes() {
-  return sizeof(S) == sizeof(float) ? sizeof(float4) * (TH + 2 * R) * (TILE_W + 2 * R) : 0;
-}
-template <class S, int R, int TH>
-__host__ __device__ constexpr size_t worker_bytes() { return tile_bytes<S, R, TH>() + qbuf_bytes<S, R, TH>(); }
-
-// tile workers per CTA of the one-launch step: one CTA per SM on both paths
-// (two workers of eight warps on FP64; 768 threads on FP32 -- six 128-thread
-// or three 256-thread workers, 80 registers each, where 1024 threads at 64
-// registers spilled), so that a grid barrier and its partial sums involve one
-// CTA per SM
-template <class S, int TH>
-__host__ __device__ constexpr int step_workers() {
-  return sizeof(S) == sizeof(double) ? 2 : 768 / (32 * (TH / 4));
+// shared memory of one FP64 tile worker: q^_i on the tile and its halo in
+// fixed point, the upper and the lower components in separate halves (16 bytes
+// per site each, so that a warp's row is read without bank conflicts), then a
+// table of coefficients per warp and the exponents of two tiles
+constexpr int COEF_SLOTS = 16;   // eight per half
+template <int R, int TH>
+__host__ __device__ constexpr int half_sites() { return (TH + 2 * R) * (TILE_W + 2 * R); }
+template <int R, int TH>
+__host__ __device__ constexpr size_t worker_bytes() {
+  return 2 * sizeof(longlong2) * half_sites<R, TH>() +
+         sizeof(int2) * COEF_SLOTS * (TH / rows_per_thread<double, TH>()) + 32;
 }
 
 // Chunks of the tile list: CTA c takes q + 1 tiles if c < r, else q (q = T / G,
@@ -528,56 +552,112 @@ __device__ __forceinline__ int cta_of_tile(int t, int q, int r) {
   return t < big ? t / (q + 1) : r + (t - big) / q;
 }
 
-// shared memory of the tile workers: a static array for one worker, the
-// dynamic allocation for several (more than the 48 KiB of static memory)
+// Dynamic shared memory of a pass kernel (the FP32 pass keeps its tile in a
+// static array)
 template <class S, int R, int TH, int SUB>
-__host__ __device__ constexpr size_t dyn_smem_bytes() { return SUB == 1 ? 0 : SUB * worker_bytes<S, R, TH>(); }
+__host__ __device__ constexpr size_t dyn_smem_bytes() {
+  return sizeof(S) == sizeof(float) ? 0 : SUB * worker_bytes<R, TH>();
+}
 
-// The body of one pass over this CTA's chunk.  COOP = false: a launch of
-// its own (lanczos_pass): per-problem tickets, the last CTA finishes.
-// COOP = true: inside the one-launch step (lanczos_step): one problem, the
-// state read from `coop_st`, coherent loads, and the CTA's partial sums
-// written to coop_slots[3 * blockIdx.x ...]; the caller synchronises the grid
-// and finishes.
-template <class S, int R, int TH, bool DIRI, bool HAS_V, bool HAS_AY, bool COOP, int SUB>
-__device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState* coop_st, double* coop_slots,
-                                          int step) {
-  using T4 = typename Vec4<S>::T;           // storage of y^ (and of q^ on the mixed path)
+// This CTA's share of a problem, the warps' sums in red[], -> one partial per
+// (problem, CTA) slot.  COOP = false: then the problem's ticket, and the CTA
+// that completes the problem sums its slots and updates its scalars.  COOP =
+// true (one-launch step): the partial goes to coop_slots[3 blockIdx.x ..] and
+// the caller goes on.
+template <bool FX, bool COOP, int NW>
+__device__ __forceinline__ void pass_sums(const LaunchParams& lp, const Problem* pr, int i, int seg_tiles,
+                                          double (*red)[3], int* last_flag, double* coop_slots) {
+  constexpr int NT = 32 * NW;
+  const int cq = lp.chunk_q, cr = lp.chunk_r;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();
+  if (warp == 0) {
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+    if (lane < NW) { s0 = red[lane][0]; s1 = red[lane][1]; s2 = red[lane][2]; }
+#pragma unroll
+    for (int o = (NW > 16 ? 16 : 8); o > 0; o >>= 1) {   // NW <= 32 warps
+      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    }
+    if (lane == 0) {
+      if constexpr (COOP) {
+        coop_slots[3 * blockIdx.x + 0] = s0;
+        coop_slots[3 * blockIdx.x + 1] = s1;
+        coop_slots[3 * blockIdx.x + 2] = s2;
+        *last_flag = 0;
+      } else {
+        const int slot = blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr);
+        pr->partials[3 * slot + 0] = s0;
+        pr->partials[3 * slot + 1] = s1;
+        pr->partials[3 * slot + 2] = s2;
+        // release our partial / acquire everybody else's
+        cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
+        *last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
+                     (unsigned)pr->ntiles);
+      }
+    }
+  }
+  __syncthreads();
+  if (!COOP && *last_flag) {
+    // the problem is complete: the whole CTA sums its slots in a fixed
+    // order (thread-strided, the warp tree, then the warps in turn), the
+    // loads of SB slots per thread in flight at once, so that a pass of
+    // eight CTAs per SM waits for two L2 round trips here, not five
+    const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
+    const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
+    constexpr int SB = 5;
+    double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+    for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
+      double v[SB][3];
+#pragma unroll
+      for (int k = 0; k < SB; ++k) {
+        const int s = s0 + k * NT;
+        const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
+        v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
+        v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
+        v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
+      }
+#pragma unroll
+      for (int k = 0; k < SB; ++k) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
+    }
+    t0 = warp_sum(t0);
+    t1 = warp_sum(t1);
+    t2 = warp_sum(t2);
+    if (lane == 0) { red[warp][0] = t0; red[warp][1] = t1; red[warp][2] = t2; }
+    __syncthreads();
+    if (warp == 0) {
+      t0 = red[0][0]; t1 = red[0][1]; t2 = red[0][2];
+#pragma unroll
+      for (int w = 1; w < NW; ++w) { t0 += red[w][0]; t1 += red[w][1]; t2 += red[w][2]; }
+      if (lane == 0) pr->st->counter = 0u;
+      finish_pass<FX>(lp, pr, pr->st, i, t0, t1, t2);
+    }
+  }
+  __syncthreads();
+}
+
+// The body of one FP32 pass over this CTA's chunk (the mixed path).
+template <int R, int TH, bool DIRI, bool HAS_V>
+__device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
+  using S = float;
+  using T4 = float4;                        // storage of y^ and of q^_i, i >= 2
   constexpr int RPT = rows_per_thread<S, TH>();
-  constexpr int NG = TH / RPT;              // row groups = warps of a worker
-  constexpr int NTS = 32 * NG;              // threads of a worker
-  constexpr int NT = SUB * NTS;             // threads
-  constexpr int NW = SUB * NG;              // warps
+  constexpr int NG = TH / RPT;              // row groups = warps
+  constexpr int NT = 32 * NG;               // threads
   constexpr int W = TILE_W + 2 * R;
-  extern __shared__ __align__(32) unsigned char dyn_smem[];
-  __shared__ double red[NW][3];
+  __shared__ double red[NG][3];
   __shared__ int last_flag;
 
   const int cq = lp.chunk_q, cr = lp.chunk_r;
   const int t_begin = blockIdx.x * cq + min((int)blockIdx.x, cr);
   const int t_end = t_begin + cq + ((int)blockIdx.x < cr ? 1 : 0);
-  const int sub = SUB == 1 ? 0 : (int)threadIdx.x / NTS;   // this thread's worker
-  const int ltid = (int)threadIdx.x - sub * NTS;
+  const int ltid = (int)threadIdx.x;
   const int tx = ltid & 31, tg = ltid >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr bool F32 = sizeof(S) == sizeof(float);
-  __shared__ __align__(32) S tile_s[SUB == 1 ? TH + 2 * R : 1][W][4];
-  S(*const tile)[W][4] = SUB == 1 ? &tile_s[0]
-                                  : reinterpret_cast<S(*)[W][4]>(dyn_smem + sub * worker_bytes<S, R, TH>());
-  // mixed path, passes >= 3: q^_{i-1} on the tile and halo, copied asynchronously
-  constexpr int NSQ = (F32 && SUB == 1) ? (TH + 2 * R) * W : 1;
-  __shared__ __align__(16) float4 qbuf_s[NSQ];
-  float4* const qbuf = SUB == 1 ? qbuf_s
-                                : reinterpret_cast<float4*>(dyn_smem + sub * worker_bytes<S, R, TH>() +
-                                                            tile_bytes<S, R, TH>());
-  // barrier of this worker's threads (the whole CTA when there is one worker)
-  auto sub_sync = [&]() {
-    if constexpr (SUB == 1) {
-      __syncthreads();
-    } else {
-      asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "r"(NTS) : "memory");
-    }
-  };
+  __shared__ __align__(32) S tile[TH + 2 * R][W][4];
+  // passes >= 3: q^_{i-1} on the tile and halo, copied asynchronously
+  __shared__ __align__(16) float4 qbuf[(TH + 2 * R) * W];
 
   // problem of the first tile (problems are sorted by tile_begin)
   int b = 0;
@@ -591,7 +671,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
   }
   for (int t = t_begin; t < t_end; ++b) {
     const Problem* pr = lp.probs + b;
-    const DevState* st = COOP ? coop_st : lp.states + b;
+    const DevState* st = lp.states + b;
     // independent loads first (all addresses are valid), then the branch
     const int stopped = st->stopped;
     const int i = lp.probe ? 1 : max(1, st->cur_pass);
@@ -600,20 +680,20 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
     const int seg_end = min(t_end, pr->tile_begin + pr->ntiles);
     const int seg_tiles = seg_end - t;
     if (stopped) { t = seg_end; continue; }
-    const S gS = F32 ? (S)pc.gf : (S)pc.g;
-    const S gdS = F32 ? (S)pc.gdf : (S)pc.gd;
-    const S eS = F32 ? (S)pc.ef : (S)pc.e;
-    const S kx = F32 ? (S)pr->kxf : (S)pr->kx, ky = F32 ? (S)pr->kyf : (S)pr->ky;
-    const S cAx = F32 ? (S)fs.cAxf : (S)fs.cAx, cAy = F32 ? (S)fs.cAyf : (S)fs.cAy;
-    const S au_hi = F32 ? (S)pc.au_hi : (S)pc.au0, au_lo = F32 ? (S)pc.au_lo : S(0);
-    const S ad_hi = F32 ? (S)pc.ad_hi : (S)pc.ad0, ad_lo = F32 ? (S)pc.ad_lo : S(0);
+    const S gS = pc.gf;
+    const S gdS = pc.gdf;
+    const S eS = pc.ef;
+    const S kx = pr->kxf, ky = pr->kyf;
+    const S cAx = fs.cAxf, cAy = fs.cAyf;
+    const S au_hi = pc.au_hi, au_lo = pc.au_lo;
+    const S ad_hi = pc.ad_hi, ad_lo = pc.ad_lo;
     // FP32: remainders of the stencil and vector-potential coefficients
-    const S kx_lo = F32 ? (S)pr->kxf_lo : S(0), ky_lo = F32 ? (S)pr->kyf_lo : S(0);
-    const S cAx_lo = F32 ? (S)fs.cAxf_lo : S(0), cAy_lo = F32 ? (S)fs.cAyf_lo : S(0);
+    const S kx_lo = pr->kxf_lo, ky_lo = pr->kyf_lo;
+    const S cAx_lo = fs.cAxf_lo, cAy_lo = fs.cAyf_lo;
     const int nx = pr->nx, ny = pr->ny;
     const size_t n = (size_t)nx * ny;
     // this pass's vectors
-    constexpr int SB = F32 ? (int)sizeof(float4) : (int)sizeof(double4_32a);
+    constexpr int SB = (int)sizeof(float4);
     const char* basis = static_cast<const char*>(pr->basis);
     const void* y_prev = (i >= 2) ? (((i - 1) & 1) ? pr->ybuf1 : pr->ybuf0) : nullptr;
     const void* q_prev = (i == 2) ? (const void*)pr->psi
@@ -621,7 +701,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
     void* q_out = (i >= 2) ? (void*)(basis + (size_t)(i - 2) * n * SB) : nullptr;
     void* y_out = (i < lp.m) ? ((i & 1) ? pr->ybuf1 : pr->ybuf0) : nullptr;
     const T4* yprev = static_cast<const T4*>(y_prev);
-    const bool q64 = !F32 || i <= 2;                // q^_{i-1} stored as complex128
+    const bool q64 = i <= 2;                // q^_{i-1} stored as complex128
     const S* Vp = static_cast<const S*>(pr->V);   // NULL: V = 0 for this problem
     const float* Vlo = static_cast<const float*>(pr->Vlo);   // mixed path: V - (float)V, or NULL
 
@@ -635,16 +715,16 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
         const size_t idx = (size_t)iy * nx + ix;
         if (q64) {
           const vec4* qsrc = (i == 1) ? pr->psi : static_cast<const vec4*>(q_prev);
-          cvt4(ld4<COOP>(qsrc + idx), qp);
+          cvt4(ldg4(qsrc + idx), qp);
         } else {
-          cvt4(ld4<COOP>(static_cast<const float4*>(q_prev) + idx), qp);
+          cvt4(ldg4(static_cast<const float4*>(q_prev) + idx), qp);
         }
         if (i == 1) {
 #pragma unroll
           for (int c = 0; c < 4; ++c) q[c] = qp[c];
         } else {
           S yv[4];
-          cvt4(ld4<COOP>(yprev + idx), yv);
+          cvt4(ldg4(yprev + idx), yv);
 #pragma unroll
           for (int c = 0; c < 4; ++c) q[c] = fma(-gdS, qp[c], gS * yv[c]);
         }
@@ -661,7 +741,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
       S au, ad, aul = au_lo, adl = ad_lo;
       if (HAS_V && Vp != nullptr) {   // V stored in S (float copy on the mixed path)
         const S v = Vp[idx];
-        if constexpr (F32) {
+        {
           // the FP32 sum with the diagonal (up to 2 m c^2) rounds differently at
           // every site: its error and V's own remainder go into the low part
           float ru, rd;
@@ -670,9 +750,6 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
           const float vl = Vlo ? Vlo[idx] : 0.f;
           aul = au_lo + vl + ru;
           adl = ad_lo + vl + rd;
-        } else {
-          au = au_hi + v;
-          ad = ad_hi + v;
         }
       } else {
         au = au_hi;
@@ -686,18 +763,18 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
       // lower: (-mc^2+V-s-sigma) d + c[-i D_x u + D_y u + (A_x + i A_y) u]
       yv[2] = ad * C[2] + kx * dxv[1] + ky * dyv[0] + cAx * C[0];
       yv[3] = ad * C[3] - kx * dxv[0] + ky * dyv[1] + cAx * C[1];
-      if constexpr (HAS_AY) {   // else A_y = 0 in every step of the launch
+      {
         yv[0] = fma(cAy, C[3], yv[0]);
         yv[1] = fma(-cAy, C[2], yv[1]);
         yv[2] = fma(-cAy, C[1], yv[2]);
         yv[3] = fma(cAy, C[0], yv[3]);
       }
-      if constexpr (F32) {
+      {
         yv[0] = fma(aul, C[0], fma(kx_lo, dxv[3], fma(-ky_lo, dyv[2], fma(cAx_lo, C[2], yv[0]))));
         yv[1] = fma(aul, C[1], fma(-kx_lo, dxv[2], fma(-ky_lo, dyv[3], fma(cAx_lo, C[3], yv[1]))));
         yv[2] = fma(adl, C[2], fma(kx_lo, dxv[1], fma(ky_lo, dyv[0], fma(cAx_lo, C[0], yv[2]))));
         yv[3] = fma(adl, C[3], fma(-kx_lo, dxv[0], fma(ky_lo, dyv[1], fma(cAx_lo, C[1], yv[3]))));
-        if constexpr (HAS_AY) {
+        {
           yv[0] = fma(cAy_lo, C[3], yv[0]);
           yv[1] = fma(-cAy_lo, C[2], yv[1]);
           yv[2] = fma(-cAy_lo, C[1], yv[2]);
@@ -752,7 +829,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
     };
 
     bool done_async = false;
-    if constexpr (F32) {
+    {
      if (!q64 && lp.async_tiles) {
       done_async = true;
       // mixed path, passes >= 3: y^_{i-1} and q^_{i-1} of the tile and its
@@ -761,11 +838,11 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
       constexpr int NS = (TH + 2 * R) * W;
       float4* const tf = reinterpret_cast<float4*>(&tile[0][0][0]);
       const float4* const qsrc = static_cast<const float4*>(q_prev);
-      for (int tt = t + sub; tt < seg_end; tt += SUB) {
+      for (int tt = t; tt < seg_end; ++tt) {
         const int lt = tt - pr->tile_begin;
         const int x0 = (lt % pr->tiles_x) * TILE_W;
         const int y0 = (lt / pr->tiles_x) * TH;
-        for (int e = ltid; e < NS; e += NTS) {
+        for (int e = ltid; e < NS; e += NT) {
           const int r = e / W, c = e - r * W;
           bool ox, oy;
           const int ix = wrap<DIRI>(x0 - R + c, nx, ox), iy = wrap<DIRI>(y0 - R + r, ny, oy);
@@ -775,23 +852,23 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
           cp_async16(qbuf + e, qsrc + idx, in ? 16 : 0);
         }
         cp_async_commit_wait();
-        sub_sync();
-        for (int e = ltid; e < NS; e += NTS) {
+        __syncthreads();
+        for (int e = ltid; e < NS; e += NT) {
           const float4 yv = tf[e], qp = qbuf[e];
           tf[e] = make_float4(fmaf(-(float)gdS, qp.x, (float)gS * yv.x), fmaf(-(float)gdS, qp.y, (float)gS * yv.y),
                               fmaf(-(float)gdS, qp.z, (float)gS * yv.z), fmaf(-(float)gdS, qp.w, (float)gS * yv.w));
         }
-        sub_sync();
+        __syncthreads();
         stencil_rows(x0, y0, [&](int, int r, int c, S (&qp)[4]) {
           const float4 v = qbuf[r * W + c];
           qp[0] = (S)v.x; qp[1] = (S)v.y; qp[2] = (S)v.z; qp[3] = (S)v.w;
         });
-        sub_sync();   // tile and qbuf are reused next
+        __syncthreads();   // tile and qbuf are reused next
       }
      }
     }
     if (!done_async) {
-      for (int tt = t + sub; tt < seg_end; tt += SUB) {
+      for (int tt = t; tt < seg_end; ++tt) {
         const int lt = tt - pr->tile_begin;
         const int x0 = (lt % pr->tiles_x) * TILE_W;
         const int y0 = (lt / pr->tiles_x) * TH;
@@ -802,7 +879,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
           form(x0 + tx, y0 + r, r + R, tx + R, qprev[k]);
         }
         constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * TH;
-        for (int h = ltid; h < NH; h += NTS) {
+        for (int h = ltid; h < NH; h += NT) {
           int row, col;
           if (h < NH_ROW) {               // rows above / below
             const int r = h / TILE_W;
@@ -817,98 +894,385 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
           S dummy[4];
           form(x0 + col - R, y0 + row - R, row, col, dummy);
         }
-        sub_sync();
+        __syncthreads();
         stencil_rows(x0, y0, [&](int k, int, int, S (&qp)[4]) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) qp[q] = qprev[k][q];
         });
-        sub_sync();   // the tile buffer is reused next
+        __syncthreads();   // the tile buffer is reused next
       }
     }
     t = seg_end;
 
-    // this CTA's share of the problem: thread -> warp in S, warps -> CTA in
-    // double, one partial per (problem, CTA) slot, then the ticket
+    // this CTA's share of the problem: thread -> warp in FP32, the rest in FP64
     accP = warp_sum(accP);
     accY = warp_sum(accY);
     accX = warp_sum(accX);
     if (lane == 0) { red[warp][0] = (double)accP; red[warp][1] = (double)accY; red[warp][2] = (double)accX; }
-    __syncthreads();
-    if (warp == 0) {
-      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-      if (lane < NW) { s0 = red[lane][0]; s1 = red[lane][1]; s2 = red[lane][2]; }
-#pragma unroll
-      for (int o = (NW > 16 ? 16 : 8); o > 0; o >>= 1) {   // NW <= 32 warps
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-      }
-      if (lane == 0) {
-        if constexpr (COOP) {
-          coop_slots[3 * blockIdx.x + 0] = s0;
-          coop_slots[3 * blockIdx.x + 1] = s1;
-          coop_slots[3 * blockIdx.x + 2] = s2;
-          last_flag = 0;
-        } else {
-          const int slot = blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr);
-          pr->partials[3 * slot + 0] = s0;
-          pr->partials[3 * slot + 1] = s1;
-          pr->partials[3 * slot + 2] = s2;
-          // release our partial / acquire everybody else's
-          cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
-          last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
-                       (unsigned)pr->ntiles);
-        }
-      }
-    }
-    __syncthreads();
-    if (!COOP && last_flag) {
-      // the problem is complete: the whole CTA sums its slots in a fixed
-      // order (thread-strided, the warp tree, then the warps in turn), the
-      // loads of SB slots per thread in flight at once, so that a pass of
-      // eight CTAs per SM waits for two L2 round trips here, not five
-      const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
-      const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
-      constexpr int SB = 5;
-      double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-      for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
-        double v[SB][3];
-#pragma unroll
-        for (int k = 0; k < SB; ++k) {
-          const int s = s0 + k * NT;
-          const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
-          v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
-          v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
-          v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
-        }
-#pragma unroll
-        for (int k = 0; k < SB; ++k) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
-      }
-      t0 = warp_sum(t0);
-      t1 = warp_sum(t1);
-      t2 = warp_sum(t2);
-      if (lane == 0) { red[warp][0] = t0; red[warp][1] = t1; red[warp][2] = t2; }
-      __syncthreads();
-      if (warp == 0) {
-        t0 = red[0][0]; t1 = red[0][1]; t2 = red[0][2];
-#pragma unroll
-        for (int w = 1; w < NW; ++w) { t0 += red[w][0]; t1 += red[w][1]; t2 += red[w][2]; }
-        if (lane == 0) pr->st->counter = 0u;
-        finish_pass(lp, pr, pr->st, i, t0, t1, t2);
-      }
-    }
-    __syncthreads();
+    pass_sums<false, false, NG>(lp, pr, i, seg_tiles, red, &last_flag, nullptr);
   }
 }
 
-template <class S, int R, int TH, bool DIRI, bool HAS_V, bool HAS_AY>
-__global__ void __launch_bounds__(sub_workers<S>() * 32 * (TH / rows_per_thread<S, TH>()),
-                                  (min_blocks<S, TH, sub_workers<S>()>()))
+// The body of one FP64 pass over this CTA's chunk.  COOP = false: a launch of
+// its own (lanczos_pass).  COOP = true: inside the one-launch step
+// (lanczos_step): one problem, the state read from `coop_st`, and the CTA's
+// partial sums written to coop_slots; the caller synchronises the grid and
+// finishes.
+//
+// The fields are complex128 in memory; per site and pass only the formation of
+// q^_i (one FP64 multiply-add per number, the scale of y^ being a power of two)
+// and the final conversion of y^_i use the FP64 pipe.  The stencil, the
+// coupling to q^_{i-1} and the three sums are 60-bit fixed point
+// (dirac_fixed.cuh): a tile (with its halo) shares one exponent for the upper
+// and one for the lower components of q^_i, another pair for q^_{i-1}, taken
+// from their largest numbers; every row of the operator is one exact sum of
+// products, rounded to 2^-60 of its largest term.  The sums run per tile in
+// integers and over the tiles of a worker at a common exponent.
+//
+// Measured (GB300, FP64 step with its recombination): 1024^2, m = 20, 2.50 ->
+// 1.89 ms; 4096^2, m = 10, 17.3 -> 10.7 ms; twelve problems of 93^2 .. 301^2 in
+// a batch 1.18 -> 0.94 ms, against the same passes in FP64 multiply-adds, whose
+// 1160 instructions a site and step kept the FP64 pipe 79 % busy.
+//
+// Per tile: load and form (all loads of a thread in flight at once), exponents
+// -> barrier -> fixed point into shared memory, coefficients at the tile's
+// scale -> barrier -> the upper, then the lower components.
+template <int R, int TH, bool DIRI, bool HAS_V, bool ISO, bool COOP, int SUB>
+__device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevState* coop_st, double* coop_slots,
+                                             int step) {
+  constexpr int RPT = rows_per_thread<double, TH>();
+  constexpr int NG = TH / RPT;              // row groups = warps of a worker
+  constexpr int NTS = 32 * NG;              // threads of a worker
+  constexpr int NW = SUB * NG;              // warps
+  constexpr int W = TILE_W + 2 * R;
+  // bits of q^ and q^_{i-1}: the differences (2 x 2 terms; order 4: 36) and
+  // the row sums then stay below 2^62
+  constexpr int F = R == 1 ? 58 : 55;
+  constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * TH;
+  static_assert(NH <= NTS, "one halo site per thread");
+  static_assert(2 * RPT <= 8, "bounds of the per-tile sums");
+  constexpr int FLUSH_TILES = 16;           // two additions per tile, at most 32 between flushes
+  extern __shared__ __align__(32) unsigned char dyn_smem[];
+  __shared__ double red[NW][3];
+  __shared__ int last_flag;
+
+  const int cq = lp.chunk_q, cr = lp.chunk_r;
+  const int t_begin = blockIdx.x * cq + min((int)blockIdx.x, cr);
+  const int t_end = t_begin + cq + ((int)blockIdx.x < cr ? 1 : 0);
+  const int sub = (int)threadIdx.x / NTS;   // this thread's worker
+  const int ltid = (int)threadIdx.x - sub * NTS;
+  const int tx = ltid & 31, tg = ltid >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* const my_smem = dyn_smem + sub * worker_bytes<R, TH>();
+  longlong2* const half_u = reinterpret_cast<longlong2*>(my_smem);
+  longlong2* const half_d = half_u + half_sites<R, TH>();
+  int2* const kt = reinterpret_cast<int2*>(half_d + half_sites<R, TH>()) + COEF_SLOTS * tg;
+  unsigned* const emax = reinterpret_cast<unsigned*>(reinterpret_cast<int2*>(half_d + half_sites<R, TH>()) +
+                                                     COEF_SLOTS * NG);   // [2][4]
+  auto sub_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "r"(NTS) : "memory"); };
+  if (ltid < 8) emax[ltid] = 0u;
+  sub_sync();
+  int par = 0;                              // which exponents the tile uses
+
+  // problem of the first tile (problems are sorted by tile_begin)
+  int b = 0;
+  {
+    int lo = 0, hi = lp.nprob - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (lp.probs[mid].tile_begin <= t_begin) lo = mid; else hi = mid - 1;
+    }
+    b = lo;
+  }
+  for (int t = t_begin; t < t_end; ++b) {
+    const Problem* pr = lp.probs + b;
+    const DevState* st = COOP ? coop_st : lp.states + b;
+    // independent loads first (all addresses are valid), then the branch
+    const int stopped = st->stopped;
+    const int i = lp.probe ? 1 : max(1, st->cur_pass);
+    const PassCoef& pc = lp.probe ? pr->probe_coef : st->pc_cur;
+    const int seg_end = min(t_end, pr->tile_begin + pr->ntiles);
+    const int seg_tiles = seg_end - t;
+    if (stopped) { t = seg_end; continue; }
+    const double gd = pc.gd;
+    const int yexp = (int)pc.yexp;
+    const int nx = pr->nx, ny = pr->ny;
+    const size_t n = (size_t)nx * ny;
+    // this pass's vectors
+    vec4* const basis = static_cast<vec4*>(pr->basis);
+    const vec4* const yprev = static_cast<const vec4*>((i & 1) ? pr->ybuf0 : pr->ybuf1);
+    const vec4* const qsrc = i <= 2 ? pr->psi : basis + (size_t)(i - 3) * n;   // q^_{i-1} (q^_1 if i = 1)
+    vec4* const q_out = (i >= 2 && !lp.probe) ? basis + (size_t)(i - 2) * n : nullptr;
+    vec4* const y_out = (i < lp.m && !lp.probe) ? static_cast<vec4*>((i & 1) ? pr->ybuf1 : pr->ybuf0) : nullptr;
+    const double* const Vp = static_cast<const double*>(pr->V);   // NULL: V = 0 for this problem
+    const FieldStep* const fs = lp.fields + step * lp.fstride + b;
+    const bool has_ax = fs->cAx != 0.0, has_ay = fs->cAy != 0.0;
+    // this lane's coefficient: slots 0 diagonal, 1 kx, 2 ky, 3 c A_x, 4 c A_y,
+    // 5 coupling, 6 V (its exponent alone) of the upper (lanes 0-7) and the
+    // lower row (8-15)
+    const int cj = lane & 7, ch = (lane >> 3) & 1;
+    double my_coef = 0.0;
+    if (cj == 0) my_coef = ch ? pc.ad0 : pc.au0;
+    if (cj == 1) my_coef = pr->kx;
+    if (cj == 2) my_coef = pr->ky;
+    if (cj == 3) my_coef = fs->cAx;
+    if (cj == 4) my_coef = fs->cAy;
+    if (cj == 5) my_coef = i >= 2 ? pc.e : 0.0;
+    const int my_xe = cj == 6 ? (HAS_V && Vp ? pr->vbe : 0) : fx::exp_field(my_coef);
+    bool bad = __any_sync(0xffffffffu, my_xe == 0x7ff);
+
+    // q^_i at grid point (gx, gy) (zero outside for Dirichlet); qp: q^_{i-1}
+    auto form = [&](int gx, int gy, double (&q)[4], double (&qp)[4]) {
+      bool ox, oy;
+      const int ix = wrap<DIRI>(gx, nx, ox), iy = wrap<DIRI>(gy, ny, oy);
+      q[0] = q[1] = q[2] = q[3] = 0.0;
+      qp[0] = qp[1] = qp[2] = qp[3] = 0.0;
+      if (ox || oy) return;
+      const size_t idx = (size_t)iy * nx + ix;
+      cvt4(ld4<COOP>(qsrc + idx), qp);
+      if (i == 1) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) { q[c] = qp[c]; qp[c] = 0.0; }
+      } else {
+        double yv[4];
+        cvt4(ld4<COOP>(yprev + idx), yv);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) q[c] = fma(-gd, qp[c], yv[c]);
+      }
+    };
+    auto mag = [](double x) { return (unsigned)__double2hiint(x) << 1; };   // orders by |x| (to 20 bits)
+
+    fx::Run sumP, sumY, sumX;
+    double accP = 0.0, accY = 0.0, accX = 0.0;
+    int since_flush = 0;
+    for (int tt = t + sub; tt < seg_end; tt += SUB) {
+      const int lt = tt - pr->tile_begin;
+      const int x0 = (lt % pr->tiles_x) * TILE_W;
+      const int y0 = (lt / pr->tiles_x) * TH;
+      const int r0 = tg * RPT;                  // this thread's rows of the tile
+      double q[RPT][4], qp[RPT][4], hq[4];
+      int hrow = 0, hcol = 0;
+#pragma unroll
+      for (int k = 0; k < RPT; ++k) form(x0 + tx, y0 + r0 + k, q[k], qp[k]);
+      if (ltid < NH) {
+        if (ltid < NH_ROW) {                    // rows above / below
+          const int r = ltid / TILE_W;
+          hrow = (r < R) ? r : TH + r;
+          hcol = (ltid % TILE_W) + R;
+        } else {                                // columns left / right
+          const int h2 = ltid - NH_ROW;
+          hrow = h2 / (2 * R) + R;
+          const int c = h2 % (2 * R);
+          hcol = (c < R) ? c : TILE_W + c;
+        }
+        double unused[4];
+        form(x0 + hcol - R, y0 + hrow - R, hq, unused);
+      } else {
+        hq[0] = hq[1] = hq[2] = hq[3] = 0.0;
+      }
+      // the largest numbers of the tile
+      unsigned m0 = max(mag(hq[0]), mag(hq[1])), m1 = max(mag(hq[2]), mag(hq[3])), m2 = 0u, m3 = 0u;
+#pragma unroll
+      for (int k = 0; k < RPT; ++k) {
+        m0 = max(m0, max(mag(q[k][0]), mag(q[k][1])));
+        m1 = max(m1, max(mag(q[k][2]), mag(q[k][3])));
+        m2 = max(m2, max(mag(qp[k][0]), mag(qp[k][1])));
+        m3 = max(m3, max(mag(qp[k][2]), mag(qp[k][3])));
+      }
+      m0 = __reduce_max_sync(0xffffffffu, m0);
+      m1 = __reduce_max_sync(0xffffffffu, m1);
+      m2 = __reduce_max_sync(0xffffffffu, m2);
+      m3 = __reduce_max_sync(0xffffffffu, m3);
+      if (lane < 4) atomicMax(emax + 4 * par + lane, lane == 0 ? m0 : lane == 1 ? m1 : lane == 2 ? m2 : m3);
+      if (q_out) {
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+          const int x = x0 + tx, y = y0 + r0 + k;
+          if (x < nx && y < ny) {
+            vec4 o;
+            o.x = q[k][0]; o.y = q[k][1]; o.z = q[k][2]; o.w = q[k][3];
+            q_out[(size_t)y * nx + x] = o;
+          }
+        }
+      }
+      sub_sync();   // the exponents are complete, and the previous tile has been read
+      // exponents of 128 and below (numbers under 2^-894) count as zero
+      const int be_u = max((int)(emax[4 * par] >> 21), 128), be_d = max((int)(emax[4 * par + 1] >> 21), 128);
+      const int be_pu = max((int)(emax[4 * par + 2] >> 21), 128), be_pd = max((int)(emax[4 * par + 3] >> 21), 128);
+      bad = bad || be_u == 0x7ff || be_d == 0x7ff || be_pu == 0x7ff || be_pd == 0x7ff;
+      if (ltid < 4) emax[4 * (par ^ 1) + ltid] = 0u;
+      par ^= 1;
+#pragma unroll
+      for (int k = 0; k < RPT; ++k) {
+        // sites beyond the grid's edge are halo of the sites inside, but not summed
+        const int at = (r0 + k + R) * W + tx + R;
+        half_u[at] = make_longlong2(fx::to_fixed<F>(q[k][0], be_u), fx::to_fixed<F>(q[k][1], be_u));
+        half_d[at] = make_longlong2(fx::to_fixed<F>(q[k][2], be_d), fx::to_fixed<F>(q[k][3], be_d));
+      }
+      if (ltid < NH) {
+        const int at = hrow * W + hcol;
+        half_u[at] = make_longlong2(fx::to_fixed<F>(hq[0], be_u), fx::to_fixed<F>(hq[1], be_u));
+        half_d[at] = make_longlong2(fx::to_fixed<F>(hq[2], be_d), fx::to_fixed<F>(hq[3], be_d));
+      }
+      {
+        // this warp's coefficient table: row scale = the largest term's, the
+        // coefficients of a row as 60-bit fractions of it
+        const int be_own = ch ? be_d : be_u, be_oth = ch ? be_u : be_d, be_p = ch ? be_pd : be_pu;
+        const int be_x = (cj == 0 || cj == 6) ? be_own : (cj == 5 ? be_p : be_oth);
+        int sc = my_xe ? my_xe + be_x : 0;
+        sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 1));
+        sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 2));
+        sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 4));
+        if (lane < COEF_SLOTS) {
+          const fx::Limbs l = fx::split(fx::to_fixed<60>(my_coef, max(sc - be_x, 63)));
+          kt[lane] = cj == 7 ? make_int2(sc, 0) : make_int2(l.hi, l.lo);
+        }
+      }
+      sub_sync();   // tile and coefficients are in shared memory
+
+      auto half = [&](auto half_c) {
+        constexpr int HALF = decltype(half_c)::value;
+        const longlong2* const own = HALF ? half_d : half_u;
+        const longlong2* const oth = HALF ? half_u : half_d;
+        const int2* const kc = kt + 8 * HALF;
+        auto coef = [&](int j) { const int2 v = kc[j]; return fx::Limbs{v.x, v.y}; };
+        const fx::Limbs ka = coef(0), kx = coef(1), ky = coef(2), kax = coef(3), kay = coef(4), ke = fx::neg(coef(5));
+        const int sc = kc[7].x;
+        const int be_own = HALF ? be_d : be_u, be_p = HALF ? be_pd : be_pu;
+        const int se = sc - 2044;                       // the row's scale: |terms| < 2^se
+        const int texp = se - F + yexp;                 // unit of y as stored
+        const bool live = texp >= -1022;                // else below the normal range: zero
+        // columns of the other half: rows r0 - R .. r0 + RPT + R - 1
+        longlong2 col[RPT + 2 * R];
+#pragma unroll
+        for (int j = 0; j < RPT + 2 * R; ++j) col[j] = oth[(r0 + j) * W + tx + R];
+        long long v[RPT][2];
+        unsigned vor = 0u;                              // the upper words of all |v|, or-ed
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+          const int at = (r0 + k + R) * W + tx + R;
+          // differences along x of (re, im), and along y
+          const longlong2 xl = oth[at - 1], xr = oth[at + 1];
+          long long hxr = xl.x - xr.x, hxi = xr.y - xl.y;          // -D_x re, D_x im
+          long long hyr = col[k + R + 1].x - col[k + R - 1].x, hyi = col[k + R + 1].y - col[k + R - 1].y;
+          if constexpr (R == 2) {
+            const longlong2 xl2 = oth[at - 2], xr2 = oth[at + 2];
+            hxr = 8 * hxr - (xl2.x - xr2.x);
+            hxi = 8 * hxi - (xr2.y - xl2.y);
+            hyr = 8 * hyr - (col[k + 2 * R].x - col[k].x);
+            hyi = 8 * hyi - (col[k + 2 * R].y - col[k].y);
+          }
+          // upper: (mc^2+V-s-sigma) u + c[-i D_x d - D_y d + (A_x - i A_y) d]
+          // lower: (-mc^2+V-s-sigma) d + c[-i D_x u + D_y u + (A_x + i A_y) u]
+          if constexpr (HALF == 0) { hyr = -hyr; hyi = -hyi; }
+          const longlong2 cv = own[at];
+          const fx::Limbs c0 = fx::split(cv.x), c1 = fx::split(cv.y);
+          fx::Acc s0, s1;
+          s0.mac(c0, ka);
+          s1.mac(c1, ka);
+          if constexpr (ISO) {
+            s0.mac(fx::split(hxi + hyr), kx);
+            s1.mac(fx::split(hxr + hyi), kx);
+          } else {
+            s0.mac(fx::split(hxi), kx);
+            s1.mac(fx::split(hxr), kx);
+            s0.mac(fx::split(hyr), ky);
+            s1.mac(fx::split(hyi), ky);
+          }
+          if (has_ax || has_ay) {
+            const fx::Limbs o0 = fx::split(col[k + R].x), o1 = fx::split(col[k + R].y);
+            if (has_ax) {
+              s0.mac(o0, kax);
+              s1.mac(o1, kax);
+            }
+            if (has_ay) {
+              s0.mac(o1, HALF ? fx::neg(kay) : kay);
+              s1.mac(o0, HALF ? kay : fx::neg(kay));
+            }
+          }
+          if (i >= 2) {
+            s0.mac(fx::split(fx::to_fixed<F>(qp[k][2 * HALF], be_p)), ke);
+            s1.mac(fx::split(fx::to_fixed<F>(qp[k][2 * HALF + 1], be_p)), ke);
+          }
+          const int x = x0 + tx, y = y0 + r0 + k;
+          const bool in = x < nx && y < ny;
+          if constexpr (HAS_V) {
+            if (Vp) {
+              const double v = in ? Vp[(size_t)y * nx + x] : 0.0;
+              const fx::Limbs kv = fx::split(fx::to_fixed<60>(v, max(sc - be_own, 63)));
+              s0.mac(c0, kv);
+              s1.mac(c1, kv);
+            }
+          }
+          const long long v0 = s0.value(), v1 = s1.value();
+          v[k][0] = in ? v0 : 0;
+          v[k][1] = in ? v1 : 0;
+          vor |= (unsigned)((v[k][0] ^ (v[k][0] >> 63)) >> 32) | (unsigned)((v[k][1] ^ (v[k][1] >> 63)) >> 32);
+          if (in && y_out) {
+            // components of this half (16 of the site's 32 bytes)
+            double2* const yo = reinterpret_cast<double2*>(y_out + (size_t)y * nx + x) + HALF;
+            *yo = make_double2(fx::to_double(live ? v0 : 0, texp), fx::to_double(live ? v1 : 0, texp));
+          }
+        }
+        // the sums: y^ as 60 bits of the warp's largest number (the terms of a
+        // row may cancel by many bits), q^ as it is
+        const int sh = __clz((int)__reduce_or_sync(0xffffffffu, vor)) - 4;   // -2 .. 28
+        fx::Acc aP, aY, aX;
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+          const longlong2 cv = own[(r0 + k + R) * W + tx + R];
+          const bool in = x0 + tx < nx && y0 + r0 + k < ny;
+          const fx::Limbs c0 = fx::split(in ? cv.x : 0), c1 = fx::split(in ? cv.y : 0);
+          const fx::Limbs w0 = fx::split(sh >= 0 ? v[k][0] << sh : v[k][0] >> -sh);
+          const fx::Limbs w1 = fx::split(sh >= 0 ? v[k][1] << sh : v[k][1] >> -sh);
+          aP.mac(c0, w0);
+          aP.mac(c1, w1);
+          aY.sqr(w0);
+          aY.sqr(w1);
+          aX.sqr(c0);
+          aX.sqr(c1);
+        }
+        // |q^| < 2^58 and |w| < 2^60: eight terms of q^ w stay below 2^62, of
+        // w^2 below 2^64, of q^2 below 2^60
+        const int qe = be_own - 1022 - F, ye = texp - sh;
+        sumP.add(aP.value_shr(4), qe + ye + 64);
+        sumY.add(aY.value_sqr_shr(6), 2 * ye + 66);
+        sumX.add(aX.value_sqr_shr(2), 2 * qe + 62);
+      };
+      half(std::integral_constant<int, 0>{});
+      half(std::integral_constant<int, 1>{});
+      if (++since_flush == FLUSH_TILES) {
+        accP += sumP.flush();
+        accY += sumY.flush();
+        accX += sumX.flush();
+        since_flush = 0;
+      }
+    }
+    t = seg_end;
+    accP += sumP.flush();
+    accY += sumY.flush();
+    accX += sumX.flush();
+    if (bad) accP = __longlong_as_double(0x7ff8000000000000LL);   // not finite: reported by finish_pass
+    if (lane == 0) { red[warp][0] = accP; red[warp][1] = accY; red[warp][2] = accX; }
+    pass_sums<true, COOP, NW>(lp, pr, i, seg_tiles, red, &last_flag, coop_slots);
+  }
+}
+
+// threads of a pass kernel (S = double: all tile workers of the CTA)
+template <class S, int TH>
+__host__ __device__ constexpr int pass_threads() { return sub_workers<S>() * 32 * (TH / rows_per_thread<S, TH>()); }
+
+// FLAG: kx = ky (S = double); not used by S = float
+template <class S, int R, int TH, bool DIRI, bool HAS_V, bool FLAG>
+__global__ void __launch_bounds__(pass_threads<S, TH>(), sizeof(S) == sizeof(float) ? min_blocks<TH>() : 1)
 lanczos_pass(const __grid_constant__ LaunchParams lp) {
   // programmatic dependent launch: nothing the previous kernel wrote is read
   // before this point
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  pass_body<S, R, TH, DIRI, HAS_V, HAS_AY, false, sub_workers<S>()>(lp, nullptr, nullptr, *lp.step);
+  if constexpr (sizeof(S) == sizeof(float))
+    pass_body<R, TH, DIRI, HAS_V>(lp, *lp.step);
+  else
+    pass_body_fx<R, TH, DIRI, HAS_V, FLAG, false, sub_workers<S>()>(lp, nullptr, nullptr, *lp.step);
   // the next kernel may be scheduled now (it waits for our completion)
   asm volatile("griddepcontrol.launch_dependents;");
 }
@@ -964,48 +1328,24 @@ __device__ __forceinline__ void recombine_site_df(vec4* psi, const float4* basis
 // corrections was the largest error of the mixed path on fast packets.
 // Blocks are dealt to problems in proportion to their size.
 // ---------------------------------------------------------------------------
-template <bool MIXED>
 __device__ __forceinline__ void recombine_site(vec4* psi, const void* basis_v, long long n, long long s, int k,
-                                               const double* cr, const double* ci, const float* fr,
-                                               const float* fi) {
-  if constexpr (!MIXED) {
-    const vec4* basis = static_cast<const vec4*>(basis_v);
-    const vec4 q = psi[s];
-    double ur = cr[1] * q.x - ci[1] * q.y, ui = cr[1] * q.y + ci[1] * q.x;
-    double dr = cr[1] * q.z - ci[1] * q.w, di = cr[1] * q.w + ci[1] * q.z;
-    for (int j = 2; j <= k; ++j) {
-      const vec4* vp = basis + (size_t)(j - 2) * n + s;
-      const vec4 v = *vp;
-      const double a = cr[j], bb = ci[j];
-      ur = fma(a, v.x, fma(-bb, v.y, ur));
-      ui = fma(a, v.y, fma(bb, v.x, ui));
-      dr = fma(a, v.z, fma(-bb, v.w, dr));
-      di = fma(a, v.w, fma(bb, v.z, di));
-    }
-    vec4 o;
-    o.x = ur; o.y = ui; o.z = dr; o.w = di;
-    psi[s] = o;
-  } else {
-    const float4* basis = static_cast<const float4*>(basis_v);
-    const double ar = cr[1], ai = ci[1];
-    float ur = 0.f, ui = 0.f, dr = 0.f, di = 0.f;
-    for (int j = 2; j <= k; ++j) {
-      const float4* vp = basis + (size_t)(j - 2) * n + s;
-      const float4 v = *vp;
-      const float a = fr[j], bb = fi[j];
-      ur = fmaf(a, v.x, fmaf(-bb, v.y, ur));
-      ui = fmaf(a, v.y, fmaf(bb, v.x, ui));
-      dr = fmaf(a, v.z, fmaf(-bb, v.w, dr));
-      di = fmaf(a, v.w, fmaf(bb, v.z, di));
-    }
-    const vec4 q = psi[s];
-    vec4 o;
-    o.x = fma(ar, q.x, fma(-ai, q.y, (double)ur));
-    o.y = fma(ar, q.y, fma(ai, q.x, (double)ui));
-    o.z = fma(ar, q.z, fma(-ai, q.w, (double)dr));
-    o.w = fma(ar, q.w, fma(ai, q.z, (double)di));
-    psi[s] = o;
+                                               const double* cr, const double* ci) {
+  const vec4* basis = static_cast<const vec4*>(basis_v);
+  const vec4 q = psi[s];
+  double ur = cr[1] * q.x - ci[1] * q.y, ui = cr[1] * q.y + ci[1] * q.x;
+  double dr = cr[1] * q.z - ci[1] * q.w, di = cr[1] * q.w + ci[1] * q.z;
+  for (int j = 2; j <= k; ++j) {
+    const vec4* vp = basis + (size_t)(j - 2) * n + s;
+    const vec4 v = *vp;
+    const double a = cr[j], bb = ci[j];
+    ur = fma(a, v.x, fma(-bb, v.y, ur));
+    ui = fma(a, v.y, fma(bb, v.x, ui));
+    dr = fma(a, v.z, fma(-bb, v.w, dr));
+    di = fma(a, v.w, fma(bb, v.z, di));
   }
+  vec4 o;
+  o.x = ur; o.y = ui; o.z = dr; o.w = di;
+  psi[s] = o;
 }
 
 // Three CTAs per SM (at most 85 registers), so that enough warps keep loads
@@ -1047,7 +1387,7 @@ __global__ void __launch_bounds__(256, 3) recombine(const __grid_constant__ Reco
       recombine_site_df<8>(psi, static_cast<const float4*>(pr->basis), (size_t)n, (size_t)s, k, cr, ci, fr, frl,
                            fi, fil);
     else
-      recombine_site<false>(psi, pr->basis, n, s, k, cr, ci, fr, fi);
+      recombine_site(psi, pr->basis, n, s, k, cr, ci);
   }
   asm volatile("griddepcontrol.launch_dependents;");
 }
@@ -1110,15 +1450,13 @@ __device__ __forceinline__ bool grid_sync(unsigned* bar, unsigned G) {
   return ok_s != 0;
 }
 
-template <class S, int R, int TH, bool DIRI, bool HAS_V, bool HAS_AY>
-__global__ void __launch_bounds__(step_workers<S, TH>() * 32 * (TH / rows_per_thread<S, TH>()), 1)
+template <int R, int TH, bool DIRI, bool HAS_V, bool ISO>
+__global__ void __launch_bounds__(pass_threads<double, TH>(), 1)
 lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ CoopArgs ca) {
-  constexpr bool F32 = sizeof(S) == sizeof(float);
-  constexpr int SUB = step_workers<S, TH>();
-  constexpr int NT = SUB * 32 * (TH / rows_per_thread<S, TH>());
+  constexpr int SUB = sub_workers<double>();
+  constexpr int NT = pass_threads<double, TH>();
   __shared__ DevState sst;
   __shared__ double cr_s[KMAX + 2], ci_s[KMAX + 2];
-  __shared__ float fr_s[KMAX + 2], fi_s[KMAX + 2];
   const Problem* pr = lp.probs;
   DevState* gst = lp.states;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1134,7 +1472,7 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
   while (!sst.stopped && iter < max_iter) {
     const int i = max(1, sst.cur_pass);
     double* slots = ca.slots + (iter & 1) * 3 * ca.G;
-    pass_body<S, R, TH, DIRI, HAS_V, HAS_AY, true, SUB>(lp, &sst, slots, step);
+    pass_body_fx<R, TH, DIRI, HAS_V, ISO, true, SUB>(lp, &sst, slots, step);
     ++iter;
     if (!grid_sync(ca.bar, (unsigned)ca.bar_count)) {
       if (threadIdx.x == 0) { gst->error = ERR_BARRIER; gst->stopped = 1; }
@@ -1159,7 +1497,7 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
       t0 = warp_sum(t0);
       t1 = warp_sum(t1);
       t2 = warp_sum(t2);
-      finish_pass(lp, pr, &sst, i, t0, t1, t2);
+      finish_pass<true>(lp, pr, &sst, i, t0, t1, t2);
     }
     __syncthreads();
   }
@@ -1169,8 +1507,6 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
     if (threadIdx.x <= KMAX) {
       cr_s[threadIdx.x] = sst.coef_re[threadIdx.x];
       ci_s[threadIdx.x] = sst.coef_im[threadIdx.x];
-      fr_s[threadIdx.x] = (float)cr_s[threadIdx.x];
-      fi_s[threadIdx.x] = (float)ci_s[threadIdx.x];
     }
     __syncthreads();
     const int cq = lp.chunk_q, cr = lp.chunk_r;
@@ -1184,7 +1520,7 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
       for (int e = threadIdx.x; e < TILE_W * TH; e += NT) {
         const int x = x0 + (e & (TILE_W - 1)), y = y0 + e / TILE_W;
         if (x < pr->nx && y < pr->ny)
-          recombine_site<F32>(psi, pr->basis, n, (long long)y * pr->nx + x, k, cr_s, ci_s, fr_s, fi_s);
+          recombine_site(psi, pr->basis, n, (long long)y * pr->nx + x, k, cr_s, ci_s);
       }
     }
   }

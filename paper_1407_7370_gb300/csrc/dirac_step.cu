@@ -15,14 +15,13 @@ namespace dirac {
 
 namespace {
 
-template <class S, int R, int TH, bool D, bool V, bool AY>
+template <int R, int TH, bool D, bool V, bool ISO>
 cudaError_t launch_step_t(LaunchParams p, int n_sm, CoopArgs ca, cudaStream_t s) {
   static std::atomic<int> occ_dev[OCC_MAX_DEVICES];
-  constexpr int SUB = step_workers<S, TH>();
-  constexpr int NT = SUB * 32 * (TH / rows_per_thread<S, TH>());
-  constexpr size_t smem = dyn_smem_bytes<S, R, TH, SUB>();
+  constexpr int NT = pass_threads<double, TH>();
+  constexpr size_t smem = dyn_smem_bytes<double, R, TH, sub_workers<double>()>();
   int occ = 0;
-  cudaError_t e = occupancy_on_device(occ_dev, lanczos_step<S, R, TH, D, V, AY>, NT, smem, &occ);
+  cudaError_t e = occupancy_on_device(occ_dev, lanczos_step<R, TH, D, V, ISO>, NT, smem, &occ);
   if (e != cudaSuccess) return e;
   if (occ < 1) return cudaErrorCooperativeLaunchTooLarge;
   // every CTA resident (a cooperative launch checks it) and each with at
@@ -30,7 +29,6 @@ cudaError_t launch_step_t(LaunchParams p, int n_sm, CoopArgs ca, cudaStream_t s)
   const int grid = std::max(1, std::min(std::min(p.total_tiles, n_sm * occ), ca.cap));
   p.chunk_q = p.total_tiles / grid;
   p.chunk_r = p.total_tiles % grid;
-  p.async_tiles = p.chunk_q >= ASYNC_MIN_TILES;
   ca.bar_count = grid + ca.bar_count;   // ca.bar_count comes in as the extra arrivals to wait for
   ca.G = grid;
   cudaLaunchConfig_t cfg = {};
@@ -43,30 +41,27 @@ cudaError_t launch_step_t(LaunchParams p, int n_sm, CoopArgs ca, cudaStream_t s)
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, lanczos_step<S, R, TH, D, V, AY>, p, ca);
+  return cudaLaunchKernelEx(&cfg, lanczos_step<R, TH, D, V, ISO>, p, ca);
 }
 
-template <class S, int R, int TH, bool D, bool V>
-cudaError_t launch_step_ay(const LaunchParams& p, int n_sm, const CoopArgs& ca, cudaStream_t s) {
-  if constexpr (sizeof(S) == sizeof(double)) {
-    if (!p.has_ay) return launch_step_t<S, R, TH, D, V, false>(p, n_sm, ca, s);
-  }
-  return launch_step_t<S, R, TH, D, V, true>(p, n_sm, ca, s);
+template <int R, int TH, bool D, bool V>
+cudaError_t launch_step_iso(const LaunchParams& p, int n_sm, const CoopArgs& ca, cudaStream_t s) {
+  return p.iso ? launch_step_t<R, TH, D, V, true>(p, n_sm, ca, s) : launch_step_t<R, TH, D, V, false>(p, n_sm, ca, s);
 }
 
-template <class S, int TH>
+template <int R, int TH>
+cudaError_t launch_step_r(bool diri, bool hasv, const LaunchParams& p, int n_sm, const CoopArgs& ca, cudaStream_t s) {
+  if (diri) return hasv ? launch_step_iso<R, TH, true, true>(p, n_sm, ca, s)
+                        : launch_step_iso<R, TH, true, false>(p, n_sm, ca, s);
+  return hasv ? launch_step_iso<R, TH, false, true>(p, n_sm, ca, s)
+              : launch_step_iso<R, TH, false, false>(p, n_sm, ca, s);
+}
+
+template <int TH>
 cudaError_t launch_step_s(int order, bool diri, bool hasv, const LaunchParams& p, int n_sm, const CoopArgs& ca,
                           cudaStream_t s) {
-  if (order == 2) {
-    if (diri) return hasv ? launch_step_ay<S, 1, TH, true, true>(p, n_sm, ca, s)
-                          : launch_step_ay<S, 1, TH, true, false>(p, n_sm, ca, s);
-    return hasv ? launch_step_ay<S, 1, TH, false, true>(p, n_sm, ca, s)
-                : launch_step_ay<S, 1, TH, false, false>(p, n_sm, ca, s);
-  }
-  if (diri) return hasv ? launch_step_ay<S, 2, TH, true, true>(p, n_sm, ca, s)
-                        : launch_step_ay<S, 2, TH, true, false>(p, n_sm, ca, s);
-  return hasv ? launch_step_ay<S, 2, TH, false, true>(p, n_sm, ca, s)
-              : launch_step_ay<S, 2, TH, false, false>(p, n_sm, ca, s);
+  return order == 2 ? launch_step_r<1, TH>(diri, hasv, p, n_sm, ca, s)
+                    : launch_step_r<2, TH>(diri, hasv, p, n_sm, ca, s);
 }
 
 }  // namespace
@@ -75,8 +70,8 @@ cudaError_t launch_step(int precision, int th, int order, bool diri, bool hasv, 
                         const CoopArgs& ca, cudaStream_t s) {
   // the mixed path has its own one-launch step (dirac_step32.cu)
   if (precision != DIRAC_FP64) return cudaErrorInvalidValue;
-  if (th == 16) return launch_step_s<double, 16>(order, diri, hasv, p, n_sm, ca, s);
-  return launch_step_s<double, 32>(order, diri, hasv, p, n_sm, ca, s);
+  if (th == 16) return launch_step_s<16>(order, diri, hasv, p, n_sm, ca, s);
+  return launch_step_s<32>(order, diri, hasv, p, n_sm, ca, s);
 }
 
 }  // namespace dirac
