@@ -16,8 +16,6 @@
 namespace dirac {
 namespace fx {
 
-constexpr int LIMB = 30;
-
 // Exponent field ("be") of a double; |x| < 2^(be - 1022).
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
@@ -40,20 +38,21 @@ __device__ __forceinline__ double to_double(long long v, int e) {
   return v ? __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d)) : 0.0;
 }
 
-// v = hi 2^30 + lo, lo in [-2^29, 2^29): products that drop lo x lo stay unbiased
+// v = hi 2^32 + lo with a signed lo, so that products without lo x lo stay
+// unbiased: two instructions, the words themselves
 struct Limbs {
   int hi, lo;
 };
 __device__ __forceinline__ Limbs split(long long v) {
   Limbs l;
-  l.hi = (int)((v + (1LL << (LIMB - 1))) >> LIMB);
-  l.lo = (int)((unsigned)v - ((unsigned)l.hi << LIMB));
+  l.lo = (int)(unsigned)v;
+  l.hi = (int)(v >> 32) + (int)((unsigned)v >> 31);
   return l;
 }
-__device__ __forceinline__ Limbs neg(const Limbs& a) { return Limbs{-a.hi, -a.lo}; }
+__device__ __forceinline__ Limbs neg(const Limbs& a) { return split(-(((long long)a.hi << 32) + a.lo)); }
 
-// Sum of products in units of 2^60: h exactly, x in units of 2^30.  The sums
-// wrap like unsigned numbers, so a sum of squares may use all 64 bits of h.
+// Sum of products a b, a and b in limbs, without their lo x lo: h in units of
+// 2^64, x of 2^32 (both wrap like unsigned numbers).
 struct Acc {
   unsigned long long h = 0, x = 0;
   __device__ __forceinline__ void mac(const Limbs& a, const Limbs& b) {
@@ -61,19 +60,26 @@ struct Acc {
     x += (unsigned long long)((long long)a.hi * b.lo);
     x += (unsigned long long)((long long)a.lo * b.hi);
   }
-  __device__ __forceinline__ void sqr(const Limbs& a) {   // x holds half of the cross terms
+  // the sum in units of 2^(32 + S), rounded
+  template <int S>
+  __device__ __forceinline__ long long value() const {
+    return (long long)((h << (32 - S)) + (unsigned long long)((long long)(x + (1ULL << (S - 1))) >> S));
+  }
+};
+
+// Sum of squares: x holds half of the cross terms; lo x lo, never negative, is
+// kept too (to 2^-29 of itself): without it the sum had a bias
+struct SqAcc {
+  unsigned long long h = 0, x = 0, l = 0;
+  __device__ __forceinline__ void sqr(const Limbs& a) {
     h += (unsigned long long)((long long)a.hi * a.hi);
     x += (unsigned long long)((long long)a.hi * a.lo);
+    const int b = a.lo >> 2;
+    l += (unsigned long long)((long long)b * b);
   }
-  __device__ __forceinline__ long long value() const {
-    return (long long)h + ((long long)(x + (1ULL << (LIMB - 1))) >> LIMB);
-  }
-  // the sum / 2^s, rounded (s >= 1): signed products
-  __device__ __forceinline__ long long value_shr(int s) const { return (value() + (1LL << (s - 1))) >> s; }
-  // the same for squares (not negative, up to 2^64)
-  __device__ __forceinline__ long long value_sqr_shr(int s) const {
-    const unsigned long long v = h + (unsigned long long)((long long)(x + (1ULL << (LIMB - 2))) >> (LIMB - 1));
-    return (long long)((v >> s) + ((v >> (s - 1)) & 1));
+  // the sum in units of 2^60, rounded (up to 2^63)
+  __device__ __forceinline__ unsigned long long value() const {
+    return (h << 4) + (unsigned long long)((long long)(x + (l >> 29) + (1ULL << 26)) >> 27);
   }
 };
 
@@ -84,33 +90,22 @@ __device__ __forceinline__ long long shr_round(long long v, int s) {
   return (v + (1LL << (s - 1))) >> s;
 }
 
-// Running sum of terms whose scale changes from tile to tile (the same for all
-// threads of a warp): v in units of 2^e.  Terms of magnitude below 2^58 may be
-// added 32 times between two flushes.
-struct Run {
-  long long v = 0;
-  int e = -100000;
-  __device__ __forceinline__ void add(long long t, int te) {
-    if (te > e) {
-      v = shr_round(v, te - e);
-      e = te;
-    } else {
-      t = shr_round(t, e - te);
-    }
-    v += t;
-  }
-  // the sum over a warp, as a double in every lane; starts again from zero.
-  // The 32 terms are added exactly, in three pieces of 21 bits.
-  __device__ __forceinline__ double flush() {
-    const int p2 = __reduce_add_sync(0xffffffffu, (int)(v >> 42));
-    const int p1 = __reduce_add_sync(0xffffffffu, (int)(v >> 21) & 0x1fffff);
-    const int p0 = __reduce_add_sync(0xffffffffu, (int)v & 0x1fffff);
-    const double d = scalbn(fma((double)(((long long)p2 << 21) + p1), 2097152.0, (double)p0), e);
-    v = 0;
-    e = -100000;
-    return d;
-  }
+// Sum over the warp of a number of each lane, exactly, in three pieces of 21
+// and 22 bits (the top piece signed or not, as T is): t2 2^42 + t1 2^21 + t0
+struct WarpSum {
+  int t2, t1, t0;
 };
+template <class T>
+__device__ __forceinline__ WarpSum warp_sum(T v) {
+  WarpSum s;
+  s.t2 = __reduce_add_sync(0xffffffffu, (int)(v >> 42));
+  s.t1 = __reduce_add_sync(0xffffffffu, (int)(v >> 21) & 0x1fffff);
+  s.t0 = __reduce_add_sync(0xffffffffu, (int)v & 0x1fffff);
+  return s;
+}
+__device__ __forceinline__ double to_double(const WarpSum& s) {
+  return fma((double)(((long long)s.t2 << 21) + s.t1), 2097152.0, (double)s.t0);
+}
 
 }  // namespace fx
 }  // namespace dirac

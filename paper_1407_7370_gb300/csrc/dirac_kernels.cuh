@@ -951,7 +951,6 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
   constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * TH;
   static_assert(NH <= NTS, "one halo site per thread");
   static_assert(2 * RPT <= 8, "bounds of the per-tile sums");
-  constexpr int FLUSH_TILES = 16;           // two additions per tile, at most 32 between flushes
   extern __shared__ __align__(32) unsigned char dyn_smem[];
   __shared__ double red[NW][3];
   __shared__ int last_flag;
@@ -1021,14 +1020,8 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
     const int my_xe = cj == 6 ? (HAS_V && Vp ? pr->vbe : 0) : fx::exp_field(my_coef);
     bool bad = __any_sync(0xffffffffu, my_xe == 0x7ff);
 
-    // q^_i at grid point (gx, gy) (zero outside for Dirichlet); qp: q^_{i-1}
-    auto form = [&](int gx, int gy, double (&q)[4], double (&qp)[4]) {
-      bool ox, oy;
-      const int ix = wrap<DIRI>(gx, nx, ox), iy = wrap<DIRI>(gy, ny, oy);
-      q[0] = q[1] = q[2] = q[3] = 0.0;
-      qp[0] = qp[1] = qp[2] = qp[3] = 0.0;
-      if (ox || oy) return;
-      const size_t idx = (size_t)iy * nx + ix;
+    // q^_i at a site, and q^_{i-1} there (zero if i = 1)
+    auto load = [&](size_t idx, double (&q)[4], double (&qp)[4]) {
       cvt4(ld4<COOP>(qsrc + idx), qp);
       if (i == 1) {
 #pragma unroll
@@ -1040,21 +1033,39 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
         for (int c = 0; c < 4; ++c) q[c] = fma(-gd, qp[c], yv[c]);
       }
     };
+    // the same at grid point (gx, gy), wrapped, or zero outside for Dirichlet
+    auto form = [&](int gx, int gy, double (&q)[4], double (&qp)[4]) {
+      bool ox, oy;
+      const int ix = wrap<DIRI>(gx, nx, ox), iy = wrap<DIRI>(gy, ny, oy);
+      q[0] = q[1] = q[2] = q[3] = 0.0;
+      qp[0] = qp[1] = qp[2] = qp[3] = 0.0;
+      if (ox || oy) return;
+      load((size_t)iy * nx + ix, q, qp);
+    };
     auto mag = [](double x) { return (unsigned)__double2hiint(x) << 1; };   // orders by |x| (to 20 bits)
 
-    fx::Run sumP, sumY, sumX;
-    double accP = 0.0, accY = 0.0, accX = 0.0;
-    int since_flush = 0;
+    // lane 0-5 of each warp: P, Y, X of the upper, then of the lower components
+    double acc = 0.0;
     for (int tt = t + sub; tt < seg_end; tt += SUB) {
       const int lt = tt - pr->tile_begin;
       const int x0 = (lt % pr->tiles_x) * TILE_W;
       const int y0 = (lt / pr->tiles_x) * TH;
       const int r0 = tg * RPT;                  // this thread's rows of the tile
+      const bool full = x0 + TILE_W <= nx && y0 + TH <= ny;
+      const bool in_x = x0 + tx < nx;
+      const int rows_in = in_x ? ny - (y0 + r0) : 0;              // row k is in the grid if k < rows_in
+      const size_t idx0 = (size_t)(y0 + r0) * nx + (x0 + tx);     // row 0 (used where in the grid)
       double q[RPT][4], qp[RPT][4], hq[4];
-      int hrow = 0, hcol = 0;
+      int hat = 0;                              // the halo site's place in the tile
+      if (full) {
 #pragma unroll
-      for (int k = 0; k < RPT; ++k) form(x0 + tx, y0 + r0 + k, q[k], qp[k]);
+        for (int k = 0; k < RPT; ++k) load(idx0 + (size_t)k * nx, q[k], qp[k]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) form(x0 + tx, y0 + r0 + k, q[k], qp[k]);
+      }
       if (ltid < NH) {
+        int hrow, hcol;
         if (ltid < NH_ROW) {                    // rows above / below
           const int r = ltid / TILE_W;
           hrow = (r < R) ? r : TH + r;
@@ -1065,6 +1076,7 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
           const int c = h2 % (2 * R);
           hcol = (c < R) ? c : TILE_W + c;
         }
+        hat = hrow * W + hcol;
         double unused[4];
         form(x0 + hcol - R, y0 + hrow - R, hq, unused);
       } else {
@@ -1087,11 +1099,10 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
       if (q_out) {
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
-          const int x = x0 + tx, y = y0 + r0 + k;
-          if (x < nx && y < ny) {
+          if (k < rows_in) {
             vec4 o;
             o.x = q[k][0]; o.y = q[k][1]; o.z = q[k][2]; o.w = q[k][3];
-            q_out[(size_t)y * nx + x] = o;
+            q_out[idx0 + (size_t)k * nx] = o;
           }
         }
       }
@@ -1102,17 +1113,16 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
       bad = bad || be_u == 0x7ff || be_d == 0x7ff || be_pu == 0x7ff || be_pd == 0x7ff;
       if (ltid < 4) emax[4 * (par ^ 1) + ltid] = 0u;
       par ^= 1;
+      const int at0 = (r0 + R) * W + tx + R;    // this thread's first site in the tile
 #pragma unroll
       for (int k = 0; k < RPT; ++k) {
         // sites beyond the grid's edge are halo of the sites inside, but not summed
-        const int at = (r0 + k + R) * W + tx + R;
-        half_u[at] = make_longlong2(fx::to_fixed<F>(q[k][0], be_u), fx::to_fixed<F>(q[k][1], be_u));
-        half_d[at] = make_longlong2(fx::to_fixed<F>(q[k][2], be_d), fx::to_fixed<F>(q[k][3], be_d));
+        half_u[at0 + k * W] = make_longlong2(fx::to_fixed<F>(q[k][0], be_u), fx::to_fixed<F>(q[k][1], be_u));
+        half_d[at0 + k * W] = make_longlong2(fx::to_fixed<F>(q[k][2], be_d), fx::to_fixed<F>(q[k][3], be_d));
       }
       if (ltid < NH) {
-        const int at = hrow * W + hcol;
-        half_u[at] = make_longlong2(fx::to_fixed<F>(hq[0], be_u), fx::to_fixed<F>(hq[1], be_u));
-        half_d[at] = make_longlong2(fx::to_fixed<F>(hq[2], be_d), fx::to_fixed<F>(hq[3], be_d));
+        half_u[hat] = make_longlong2(fx::to_fixed<F>(hq[0], be_u), fx::to_fixed<F>(hq[1], be_u));
+        half_d[hat] = make_longlong2(fx::to_fixed<F>(hq[2], be_d), fx::to_fixed<F>(hq[3], be_d));
       }
       {
         // this warp's coefficient table: row scale = the largest term's, the
@@ -1130,13 +1140,14 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
       }
       sub_sync();   // tile and coefficients are in shared memory
 
+      fx::WarpSum ws[6];
+      int we[6];
       auto half = [&](auto half_c) {
         constexpr int HALF = decltype(half_c)::value;
-        const longlong2* const own = HALF ? half_d : half_u;
-        const longlong2* const oth = HALF ? half_u : half_d;
+        const longlong2* const own = (HALF ? half_d : half_u) + at0;
+        const longlong2* const oth = (HALF ? half_u : half_d) + at0;
         const int2* const kc = kt + 8 * HALF;
         auto coef = [&](int j) { const int2 v = kc[j]; return fx::Limbs{v.x, v.y}; };
-        const fx::Limbs ka = coef(0), kx = coef(1), ky = coef(2), kax = coef(3), kay = coef(4), ke = fx::neg(coef(5));
         const int sc = kc[7].x;
         const int be_own = HALF ? be_d : be_u, be_p = HALF ? be_pd : be_pu;
         const int se = sc - 2044;                       // the row's scale: |terms| < 2^se
@@ -1145,18 +1156,18 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
         // columns of the other half: rows r0 - R .. r0 + RPT + R - 1
         longlong2 col[RPT + 2 * R];
 #pragma unroll
-        for (int j = 0; j < RPT + 2 * R; ++j) col[j] = oth[(r0 + j) * W + tx + R];
+        for (int j = 0; j < RPT + 2 * R; ++j) col[j] = oth[(j - R) * W];
         long long v[RPT][2];
         unsigned vor = 0u;                              // the upper words of all |v|, or-ed
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
-          const int at = (r0 + k + R) * W + tx + R;
+          const longlong2* const row = oth + k * W;
           // differences along x of (re, im), and along y
-          const longlong2 xl = oth[at - 1], xr = oth[at + 1];
+          const longlong2 xl = row[-1], xr = row[1];
           long long hxr = xl.x - xr.x, hxi = xr.y - xl.y;          // -D_x re, D_x im
           long long hyr = col[k + R + 1].x - col[k + R - 1].x, hyi = col[k + R + 1].y - col[k + R - 1].y;
           if constexpr (R == 2) {
-            const longlong2 xl2 = oth[at - 2], xr2 = oth[at + 2];
+            const longlong2 xl2 = row[-2], xr2 = row[2];
             hxr = 8 * hxr - (xl2.x - xr2.x);
             hxi = 8 * hxi - (xr2.y - xl2.y);
             hyr = 8 * hyr - (col[k + 2 * R].x - col[k].x);
@@ -1164,67 +1175,70 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
           }
           // upper: (mc^2+V-s-sigma) u + c[-i D_x d - D_y d + (A_x - i A_y) d]
           // lower: (-mc^2+V-s-sigma) d + c[-i D_x u + D_y u + (A_x + i A_y) u]
-          if constexpr (HALF == 0) { hyr = -hyr; hyi = -hyi; }
-          const longlong2 cv = own[at];
+          const longlong2 cv = own[k * W];
           const fx::Limbs c0 = fx::split(cv.x), c1 = fx::split(cv.y);
           fx::Acc s0, s1;
-          s0.mac(c0, ka);
-          s1.mac(c1, ka);
+          {
+            const fx::Limbs ka = coef(0);
+            s0.mac(c0, ka);
+            s1.mac(c1, ka);
+          }
           if constexpr (ISO) {
-            s0.mac(fx::split(hxi + hyr), kx);
-            s1.mac(fx::split(hxr + hyi), kx);
+            const fx::Limbs kx = coef(1);
+            s0.mac(fx::split(HALF ? hxi + hyr : hxi - hyr), kx);
+            s1.mac(fx::split(HALF ? hxr + hyi : hxr - hyi), kx);
           } else {
+            const fx::Limbs kx = coef(1), ky = coef(2);
             s0.mac(fx::split(hxi), kx);
             s1.mac(fx::split(hxr), kx);
-            s0.mac(fx::split(hyr), ky);
-            s1.mac(fx::split(hyi), ky);
+            s0.mac(fx::split(HALF ? hyr : -hyr), ky);
+            s1.mac(fx::split(HALF ? hyi : -hyi), ky);
           }
-          if (has_ax || has_ay) {
-            const fx::Limbs o0 = fx::split(col[k + R].x), o1 = fx::split(col[k + R].y);
-            if (has_ax) {
-              s0.mac(o0, kax);
-              s1.mac(o1, kax);
-            }
-            if (has_ay) {
-              s0.mac(o1, HALF ? fx::neg(kay) : kay);
-              s1.mac(o0, HALF ? kay : fx::neg(kay));
-            }
+          if (has_ax) {
+            const fx::Limbs kax = coef(3);
+            s0.mac(fx::split(col[k + R].x), kax);
+            s1.mac(fx::split(col[k + R].y), kax);
+          }
+          if (has_ay) {
+            const fx::Limbs kay = coef(4);
+            s0.mac(fx::split(HALF ? -col[k + R].y : col[k + R].y), kay);
+            s1.mac(fx::split(HALF ? col[k + R].x : -col[k + R].x), kay);
           }
           if (i >= 2) {
-            s0.mac(fx::split(fx::to_fixed<F>(qp[k][2 * HALF], be_p)), ke);
-            s1.mac(fx::split(fx::to_fixed<F>(qp[k][2 * HALF + 1], be_p)), ke);
+            const fx::Limbs ke = coef(5);
+            s0.mac(fx::split(-fx::to_fixed<F>(qp[k][2 * HALF], be_p)), ke);
+            s1.mac(fx::split(-fx::to_fixed<F>(qp[k][2 * HALF + 1], be_p)), ke);
           }
-          const int x = x0 + tx, y = y0 + r0 + k;
-          const bool in = x < nx && y < ny;
           if constexpr (HAS_V) {
             if (Vp) {
-              const double v = in ? Vp[(size_t)y * nx + x] : 0.0;
-              const fx::Limbs kv = fx::split(fx::to_fixed<60>(v, max(sc - be_own, 63)));
+              const double pot = k < rows_in ? Vp[idx0 + (size_t)k * nx] : 0.0;
+              const fx::Limbs kv = fx::split(fx::to_fixed<60>(pot, max(sc - be_own, 63)));
               s0.mac(c0, kv);
               s1.mac(c1, kv);
             }
           }
-          const long long v0 = s0.value(), v1 = s1.value();
-          v[k][0] = in ? v0 : 0;
-          v[k][1] = in ? v1 : 0;
+          v[k][0] = s0.template value<28>();
+          v[k][1] = s1.template value<28>();
+          if (!full && k >= rows_in) v[k][0] = v[k][1] = 0;
           vor |= (unsigned)((v[k][0] ^ (v[k][0] >> 63)) >> 32) | (unsigned)((v[k][1] ^ (v[k][1] >> 63)) >> 32);
-          if (in && y_out) {
+          if (y_out && k < rows_in) {
             // components of this half (16 of the site's 32 bytes)
-            double2* const yo = reinterpret_cast<double2*>(y_out + (size_t)y * nx + x) + HALF;
-            *yo = make_double2(fx::to_double(live ? v0 : 0, texp), fx::to_double(live ? v1 : 0, texp));
+            double2* const yo = reinterpret_cast<double2*>(y_out + idx0 + (size_t)k * nx) + HALF;
+            *yo = live ? make_double2(fx::to_double(v[k][0], texp), fx::to_double(v[k][1], texp))
+                       : make_double2(0.0, 0.0);
           }
         }
         // the sums: y^ as 60 bits of the warp's largest number (the terms of a
         // row may cancel by many bits), q^ as it is
-        const int sh = __clz((int)__reduce_or_sync(0xffffffffu, vor)) - 4;   // -2 .. 28
-        fx::Acc aP, aY, aX;
+        const int sl = __clz((int)__reduce_or_sync(0xffffffffu, vor)) - 2;   // 0 .. 30
+        fx::Acc aP;
+        fx::SqAcc aY, aX;
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
-          const longlong2 cv = own[(r0 + k + R) * W + tx + R];
-          const bool in = x0 + tx < nx && y0 + r0 + k < ny;
-          const fx::Limbs c0 = fx::split(in ? cv.x : 0), c1 = fx::split(in ? cv.y : 0);
-          const fx::Limbs w0 = fx::split(sh >= 0 ? v[k][0] << sh : v[k][0] >> -sh);
-          const fx::Limbs w1 = fx::split(sh >= 0 ? v[k][1] << sh : v[k][1] >> -sh);
+          longlong2 cv = own[k * W];
+          if (!full && k >= rows_in) cv.x = cv.y = 0;
+          const fx::Limbs c0 = fx::split(cv.x << (58 - F)), c1 = fx::split(cv.y << (58 - F));
+          const fx::Limbs w0 = fx::split((v[k][0] << sl) >> 2), w1 = fx::split((v[k][1] << sl) >> 2);
           aP.mac(c0, w0);
           aP.mac(c1, w1);
           aY.sqr(w0);
@@ -1232,26 +1246,30 @@ __device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevSt
           aX.sqr(c0);
           aX.sqr(c1);
         }
-        // |q^| < 2^58 and |w| < 2^60: eight terms of q^ w stay below 2^62, of
-        // w^2 below 2^64, of q^2 below 2^60
-        const int qe = be_own - 1022 - F, ye = texp - sh;
-        sumP.add(aP.value_shr(4), qe + ye + 64);
-        sumY.add(aY.value_sqr_shr(6), 2 * ye + 66);
-        sumX.add(aX.value_sqr_shr(2), 2 * qe + 62);
+        // |q^| < 2^58 and |w| < 2^60: eight terms of q^ w stay below 2^61 in
+        // units of 2^60, of w^2 below 2^63, of q^2 below 2^59
+        const int qe = be_own - 1022 - 58, ye = texp + 2 - sl;
+        ws[3 * HALF] = fx::warp_sum(aP.template value<28>());
+        ws[3 * HALF + 1] = fx::warp_sum(aY.value());
+        ws[3 * HALF + 2] = fx::warp_sum(aX.value());
+        we[3 * HALF] = qe + ye + 60;
+        we[3 * HALF + 1] = 2 * ye + 60;
+        we[3 * HALF + 2] = 2 * qe + 60;
       };
       half(std::integral_constant<int, 0>{});
       half(std::integral_constant<int, 1>{});
-      if (++since_flush == FLUSH_TILES) {
-        accP += sumP.flush();
-        accY += sumY.flush();
-        accX += sumX.flush();
-        since_flush = 0;
+      // one conversion for all six sums: each by its lane
+      fx::WarpSum mine = ws[0];
+      int me = we[0];
+#pragma unroll
+      for (int j = 1; j < 6; ++j) {
+        if (lane == j) { mine = ws[j]; me = we[j]; }
       }
+      acc += scalbn(fx::to_double(mine), me);
     }
     t = seg_end;
-    accP += sumP.flush();
-    accY += sumY.flush();
-    accX += sumX.flush();
+    double accP = acc + __shfl_down_sync(0xffffffffu, acc, 3);
+    const double accY = __shfl_sync(0xffffffffu, accP, 1), accX = __shfl_sync(0xffffffffu, accP, 2);
     if (bad) accP = __longlong_as_double(0x7ff8000000000000LL);   // not finite: reported by finish_pass
     if (lane == 0) { red[warp][0] = accP; red[warp][1] = accY; red[warp][2] = accX; }
     pass_sums<true, COOP, NW>(lp, pr, i, seg_tiles, red, &last_flag, coop_slots);
@@ -1321,30 +1339,92 @@ __device__ __forceinline__ void recombine_site_df(vec4* psi, const float4* basis
 
 // ---------------------------------------------------------------------------
 // psi <- sum_j C_j q^_j (Eq. 17), q^_1 = psi, q^_j = basis[j-2] for j >= 2.
-// FP64 path: complex128 throughout.  Mixed path: the basis is complex64;
-// C_1 psi is formed in FP64 so that the FP32 rounding of the basis only
-// enters the (small) Krylov corrections, and those are summed with
-// compensation (recombine_site_df): plain FP32 accumulation of the
-// corrections was the largest error of the mixed path on fast packets.
+// Mixed path: the basis is complex64; C_1 psi is formed in FP64 so that the
+// FP32 rounding of the basis only enters the (small) Krylov corrections, and
+// those are summed with compensation (recombine_site_df): plain FP32
+// accumulation of the corrections was the largest error of the mixed path on
+// fast packets.
+//
+// FP64 path: complex128 fields, the sums in fixed point (dirac_fixed.cuh): in
+// FP64 the 16 multiply-adds per site and vector took 1024 cycles of a
+// sub-partition against the 190 that reading the vector takes; in limbs they
+// take about as long as the read.  Each site has its own scale, that of its
+// largest |C_j q^_j| so far (the sums are shifted when a batch of D vectors
+// raises it), so the relative error of every site is about 2^-54 of its
+// largest term.
 // Blocks are dealt to problems in proportion to their size.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void recombine_site(vec4* psi, const void* basis_v, long long n, long long s, int k,
-                                               const double* cr, const double* ci) {
-  const vec4* basis = static_cast<const vec4*>(basis_v);
-  const vec4 q = psi[s];
-  double ur = cr[1] * q.x - ci[1] * q.y, ui = cr[1] * q.y + ci[1] * q.x;
-  double dr = cr[1] * q.z - ci[1] * q.w, di = cr[1] * q.w + ci[1] * q.z;
-  for (int j = 2; j <= k; ++j) {
-    const vec4* vp = basis + (size_t)(j - 2) * n + s;
-    const vec4 v = *vp;
-    const double a = cr[j], bb = ci[j];
-    ur = fma(a, v.x, fma(-bb, v.y, ur));
-    ui = fma(a, v.y, fma(bb, v.x, ui));
-    dr = fma(a, v.z, fma(-bb, v.w, dr));
-    di = fma(a, v.w, fma(bb, v.z, di));
+struct FxCoef {
+  fx::Limbs re, im, mim;   // C_j and -Im C_j as 59-bit fractions of 2^(be - 1022)
+  int be;
+};
+__device__ __forceinline__ FxCoef fx_coef(double re, double im) {
+  FxCoef c;
+  c.be = max(fx::exp_field(re), fx::exp_field(im));
+  const long long i = fx::to_fixed<59>(im, max(c.be, 63));
+  c.re = fx::split(fx::to_fixed<59>(re, max(c.be, 63)));
+  c.im = fx::split(i);
+  c.mim = fx::split(-i);
+  return c;
+}
+
+template <int D>
+__device__ __forceinline__ void recombine_site_fx(vec4* psi, const vec4* basis, size_t n, size_t s, int k,
+                                                  const FxCoef* coef) {
+  // factors below 2^59: 8 products in x stay below 2^62, all 64 below 2^62 in
+  // units of 2^62
+  static_assert(D % 4 == 0 && 2 * KMAX <= 64, "bounds of the sums");
+  long long sum[4] = {0, 0, 0, 0};
+  int be = 1100;   // exponent sum of the largest term (terms below 2^-938 count as zero)
+  for (int j0 = 1; j0 <= k; j0 += D) {
+    vec4 v[D];
+#pragma unroll
+    for (int u = 0; u < D; ++u) {
+      const int j = j0 + u;
+      if (j <= k) v[u] = j == 1 ? psi[s] : basis[(size_t)(j - 2) * n + s];
+    }
+    int nb = be;
+#pragma unroll
+    for (int u = 0; u < D; ++u) {
+      if (j0 + u <= k) {
+        const unsigned a = max((unsigned)__double2hiint(v[u].x) << 1, (unsigned)__double2hiint(v[u].y) << 1);
+        const unsigned b = max((unsigned)__double2hiint(v[u].z) << 1, (unsigned)__double2hiint(v[u].w) << 1);
+        nb = max(nb, (int)(max(a, b) >> 21) + coef[j0 + u].be);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) sum[c] = fx::shr_round(sum[c], nb - be);
+    be = nb;
+#pragma unroll
+    for (int g = 0; g < D; g += 4) {
+      fx::Acc acc[4];
+#pragma unroll
+      for (int u = g; u < g + 4; ++u) {
+        if (j0 + u <= k) {
+          const FxCoef cf = coef[j0 + u];
+          const int bq = max(be - cf.be, 63);
+          const fx::Limbs x = fx::split(fx::to_fixed<59>(v[u].x, bq)), y = fx::split(fx::to_fixed<59>(v[u].y, bq));
+          const fx::Limbs z = fx::split(fx::to_fixed<59>(v[u].z, bq)), w = fx::split(fx::to_fixed<59>(v[u].w, bq));
+          acc[0].mac(x, cf.re);
+          acc[0].mac(y, cf.mim);
+          acc[1].mac(y, cf.re);
+          acc[1].mac(x, cf.im);
+          acc[2].mac(z, cf.re);
+          acc[2].mac(w, cf.mim);
+          acc[3].mac(w, cf.re);
+          acc[3].mac(z, cf.im);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) sum[c] += acc[c].template value<30>();
+    }
   }
+  const int e = be - 2044 - 56;   // 2^62 of the products' 2^-118
   vec4 o;
-  o.x = ur; o.y = ui; o.z = dr; o.w = di;
+  o.x = fx::to_double(sum[0], e);
+  o.y = fx::to_double(sum[1], e);
+  o.z = fx::to_double(sum[2], e);
+  o.w = fx::to_double(sum[3], e);
   psi[s] = o;
 }
 
@@ -1353,8 +1433,10 @@ __device__ __forceinline__ void recombine_site(vec4* psi, const void* basis_v, l
 template <bool MIXED>
 __global__ void __launch_bounds__(256, 3) recombine(const __grid_constant__ RecombParams rp) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  __shared__ double cr[KMAX + 2], ci[KMAX + 2];
-  __shared__ float fr[KMAX + 2], fi[KMAX + 2], frl[KMAX + 2], fil[KMAX + 2];
+  __shared__ double cr[MIXED ? KMAX + 2 : 1], ci[MIXED ? KMAX + 2 : 1];
+  __shared__ float fr[MIXED ? KMAX + 2 : 1], fi[MIXED ? KMAX + 2 : 1];
+  __shared__ float frl[MIXED ? KMAX + 2 : 1], fil[MIXED ? KMAX + 2 : 1];
+  __shared__ FxCoef fc[MIXED ? 1 : KMAX + 2];
   __shared__ int k_s, err_s;
   const int b = rp.blk_prob[blockIdx.x];
   const Problem* pr = rp.probs + b;
@@ -1362,12 +1444,16 @@ __global__ void __launch_bounds__(256, 3) recombine(const __grid_constant__ Reco
   if (threadIdx.x == 0) { k_s = st->k_used; err_s = st->error; }
   if (threadIdx.x <= KMAX) {
     const double a = st->coef_re[threadIdx.x], c = st->coef_im[threadIdx.x];
-    cr[threadIdx.x] = a;
-    ci[threadIdx.x] = c;
-    fr[threadIdx.x] = (float)a;
-    fi[threadIdx.x] = (float)c;
-    frl[threadIdx.x] = (float)(a - (double)fr[threadIdx.x]);
-    fil[threadIdx.x] = (float)(c - (double)fi[threadIdx.x]);
+    if constexpr (MIXED) {
+      cr[threadIdx.x] = a;
+      ci[threadIdx.x] = c;
+      fr[threadIdx.x] = (float)a;
+      fi[threadIdx.x] = (float)c;
+      frl[threadIdx.x] = (float)(a - (double)fr[threadIdx.x]);
+      fil[threadIdx.x] = (float)(c - (double)fi[threadIdx.x]);
+    } else {
+      fc[threadIdx.x] = fx_coef(a, c);
+    }
   }
   __syncthreads();
   const int lb = blockIdx.x - pr->rblk_begin;
@@ -1387,7 +1473,7 @@ __global__ void __launch_bounds__(256, 3) recombine(const __grid_constant__ Reco
       recombine_site_df<8>(psi, static_cast<const float4*>(pr->basis), (size_t)n, (size_t)s, k, cr, ci, fr, frl,
                            fi, fil);
     else
-      recombine_site(psi, pr->basis, n, s, k, cr, ci);
+      recombine_site_fx<4>(psi, static_cast<const vec4*>(pr->basis), (size_t)n, (size_t)s, k, fc);
   }
   asm volatile("griddepcontrol.launch_dependents;");
 }
@@ -1456,7 +1542,7 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
   constexpr int SUB = sub_workers<double>();
   constexpr int NT = pass_threads<double, TH>();
   __shared__ DevState sst;
-  __shared__ double cr_s[KMAX + 2], ci_s[KMAX + 2];
+  __shared__ FxCoef fc_s[KMAX + 2];
   const Problem* pr = lp.probs;
   DevState* gst = lp.states;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1504,15 +1590,12 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
   const int err = sst.error;
   if (!err) {
     // psi <- sum_j C_j q^_j on this CTA's tiles (no CTA reads psi any more)
-    if (threadIdx.x <= KMAX) {
-      cr_s[threadIdx.x] = sst.coef_re[threadIdx.x];
-      ci_s[threadIdx.x] = sst.coef_im[threadIdx.x];
-    }
+    if (threadIdx.x <= KMAX) fc_s[threadIdx.x] = fx_coef(sst.coef_re[threadIdx.x], sst.coef_im[threadIdx.x]);
     __syncthreads();
     const int cq = lp.chunk_q, cr = lp.chunk_r;
     const int t_begin = blockIdx.x * cq + min((int)blockIdx.x, cr);
     const int t_end = t_begin + cq + ((int)blockIdx.x < cr ? 1 : 0);
-    const long long n = (long long)pr->nx * pr->ny;
+    const size_t n = (size_t)pr->nx * pr->ny;
     const int k = sst.k_used;
     vec4* psi = const_cast<vec4*>(pr->psi);
     for (int tt = t_begin; tt < t_end; ++tt) {
@@ -1520,7 +1603,7 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
       for (int e = threadIdx.x; e < TILE_W * TH; e += NT) {
         const int x = x0 + (e & (TILE_W - 1)), y = y0 + e / TILE_W;
         if (x < pr->nx && y < pr->ny)
-          recombine_site(psi, pr->basis, n, (long long)y * pr->nx + x, k, cr_s, ci_s);
+          recombine_site_fx<8>(psi, static_cast<const vec4*>(pr->basis), n, (size_t)y * pr->nx + x, k, fc_s);
       }
     }
   }
