@@ -7,10 +7,13 @@ import subprocess
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
-SOURCES = [os.path.join(HERE, "csrc", n) for n in ("dirac_capi.cu", "dirac_step.cu", "dirac_step32.cu",
-                                                    "dirac_eigs.cu", "dirac_adjoint.cu")]
+SOURCES = [os.path.join(HERE, "csrc", n) for n in ("dirac_pass64.cu", "dirac_step64.cu", "dirac_step.cu",
+                                                    "dirac_capi.cu", "dirac_step32.cu", "dirac_eigs.cu",
+                                                    "dirac_adjoint.cu")]
 DEPS = SOURCES + [os.path.join(HERE, "csrc", "dirac_kernels.cuh"),
                   os.path.join(HERE, "csrc", "dirac_fixed.cuh"),
+                  os.path.join(HERE, "csrc", "dirac_pass64.cuh"),
+                  os.path.join(HERE, "csrc", "dirac_launch.cuh"),
                   os.path.join(HERE, "csrc", "dirac_internal.h"),
                   os.path.join(ROOT, "include", "dirac.h")]
 OUT_DIR = os.path.join(HERE, "_build")

@@ -327,6 +327,13 @@ struct CtxGuard {
   ~CtxGuard() { if (c) dirac_destroy(c); }
 };
 
+// the caller's context steps in multiply-adds during the call
+struct MuladdGuard {
+  dirac_ctx* c;
+  explicit MuladdGuard(dirac_ctx* ctx) : c(ctx) { ctx_muladd64(c, true); }
+  ~MuladdGuard() { ctx_muladd64(c, false); }
+};
+
 #define ADJ_TRY(call)                                                                   \
   do {                                                                                  \
     cudaError_t e_ = (call);                                                            \
@@ -412,6 +419,9 @@ dirac_status dirac_adjoint_gradient(dirac_ctx* ctx, const void* psi0_dev, int ns
     if (!std::isfinite(A_xy_host[k])) return fail(DIRAC_EINVAL, "non-finite vector potential");
   if (info) std::memset(info, 0, sizeof(*info));
 
+  // gradients with respect to A are sums that cancel to 1e-6 of their terms:
+  // both sweeps keep the multiply-add kernels and their rounding
+  const MuladdGuard muladd(ctx);
   const long long n = (long long)v.nx * v.ny;
   const size_t vb = sizeof(v4) * (size_t)n;
   const int K = std::min(opts->checkpoint_every, nsteps);
@@ -485,6 +495,7 @@ dirac_status dirac_adjoint_gradient(dirac_ctx* ctx, const void* psi0_dev, int ns
   CtxGuard back;
   ADJ_CHECK(dirac_create(&back.c, v.nx, v.ny, v.dx, v.dy, v.mass, v.c, v.order, v.boundary, DIRAC_FP64, m,
                          (void*)s));
+  ctx_muladd64(back.c, true);
   ADJ_CHECK(dirac_set_fields(back.c, v.V, v.ax, v.ay, v.shift));
   CtxView vb_view;
   ADJ_CHECK(ctx_view(back.c, &vb_view));

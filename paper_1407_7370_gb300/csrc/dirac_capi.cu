@@ -3,6 +3,7 @@
 #include "dirac.h"
 #include "dirac_internal.h"
 #include "dirac_kernels.cuh"
+#include "dirac_launch.cuh"
 
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
@@ -169,90 +170,12 @@ bool encode_field_map(CUtensorMap* map, bool fp64, const void* base, int nx, int
 // launches
 // ---------------------------------------------------------------------------
 
-// DIRAC_NO_PDL=1 in the environment turns the launch overlap off (debugging aid).
-bool pdl_enabled() {
-  static const bool on = [] {
-    const char* v = std::getenv("DIRAC_NO_PDL");
-    return !(v && v[0] == '1');
-  }();
-  return on;
-}
-
-// Launch with programmatic stream serialisation: the kernel may be scheduled
-// while the previous kernel in the stream finishes; it waits for it (and sees
-// its writes) at its griddepcontrol.wait.
-template <class... KArgs, class... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
-                       Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl_enabled() ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
-struct LaunchShape {
-  int n_sm;          // SMs of the device
-  int th;            // tile height (32 or 16; FP64 always 32)
-  int cta_cap;       // 0: as many CTAs per SM as fit; else at most this many
-};
-
-// Persistent launch: as many CTAs as are resident at once (at most one per
-// tile), each taking a contiguous chunk of the tile list whose size differs
-// from the others' by at most one tile.
-template <class S, int R, int TH, bool D, bool V, bool FLAG>
-cudaError_t launch_pass_t(LaunchParams p, const LaunchShape& ls, cudaStream_t s) {
-  static std::atomic<int> occ_dev[OCC_MAX_DEVICES];
-  constexpr int NT = pass_threads<S, TH>();
-  constexpr size_t smem = dyn_smem_bytes<S, R, TH, sub_workers<S>()>();
-  int occ = 0;
-  cudaError_t e = occupancy_on_device(occ_dev, lanczos_pass<S, R, TH, D, V, FLAG>, NT, smem, &occ);
-  if (e != cudaSuccess) return e;
-  if (occ < 1) occ = 1;
-  const int per_sm = ls.cta_cap > 0 ? std::min(occ, ls.cta_cap) : occ;
-  const int slots = std::max(1, ls.n_sm * per_sm);
-  const int grid = std::max(1, std::min(p.total_tiles, slots));
-  p.chunk_q = p.total_tiles / grid;
-  p.chunk_r = p.total_tiles % grid;
-  p.async_tiles = p.chunk_q >= ASYNC_MIN_TILES;
-  return launch_pdl(lanczos_pass<S, R, TH, D, V, FLAG>, grid, NT, smem, s, p);
-}
-
-// FP64: with kx = ky (dx = dy) the two differences of a row are added before
-// their one product; the FP32 pass keeps one kernel
-template <class S, int R, int TH, bool D, bool V>
-cudaError_t launch_pass_iso(const LaunchParams& p, const LaunchShape& ls, cudaStream_t s) {
-  if constexpr (sizeof(S) == sizeof(double)) {
-    if (p.iso) return launch_pass_t<S, R, TH, D, V, true>(p, ls, s);
-  }
-  return launch_pass_t<S, R, TH, D, V, false>(p, ls, s);
-}
-
-template <class S, int TH>
-cudaError_t launch_pass_s(int order, bool diri, bool hasv, const LaunchParams& p, const LaunchShape& ls,
-                          cudaStream_t s) {
-  if (order == 2) {
-    if (diri) return hasv ? launch_pass_iso<S, 1, TH, true, true>(p, ls, s) : launch_pass_iso<S, 1, TH, true, false>(p, ls, s);
-    return hasv ? launch_pass_iso<S, 1, TH, false, true>(p, ls, s) : launch_pass_iso<S, 1, TH, false, false>(p, ls, s);
-  }
-  if (diri) return hasv ? launch_pass_iso<S, 2, TH, true, true>(p, ls, s) : launch_pass_iso<S, 2, TH, true, false>(p, ls, s);
-  return hasv ? launch_pass_iso<S, 2, TH, false, true>(p, ls, s) : launch_pass_iso<S, 2, TH, false, false>(p, ls, s);
-}
-
-// FP64 path: everything complex128.  Mixed path: complex64 basis (passes 1
-// and 2 read the complex128 state as q^_1; the kernel picks per problem).
-cudaError_t launch_pass(int precision, int order, bool diri, bool hasv, const LaunchParams& p,
+// One FP32 or FP64 pass.  FP64: in fixed point (dirac_pass64.cu), or, for the
+// adjoint, in FP64 multiply-adds (dirac_step.cu).
+cudaError_t launch_pass(int precision, bool muladd, int order, bool diri, bool hasv, const LaunchParams& p,
                         const LaunchShape& ls, cudaStream_t s) {
-  if (precision == DIRAC_FP64) {
-    if (ls.th == 16) return launch_pass_s<double, 16>(order, diri, hasv, p, ls, s);
-    return launch_pass_s<double, 32>(order, diri, hasv, p, ls, s);
-  }
+  if (precision == DIRAC_FP64)
+    return muladd ? launch_pass_muladd(order, diri, hasv, p, ls, s) : launch_pass64(order, diri, hasv, p, ls, s);
   if (ls.th == 16) return launch_pass_s<float, 16>(order, diri, hasv, p, ls, s);
   return launch_pass_s<float, 32>(order, diri, hasv, p, ls, s);
 }
@@ -268,8 +191,9 @@ cudaError_t launch_pass(int precision, int order, bool diri, bool hasv, const La
 int redo_budget(int precision, int m) { return precision == DIRAC_FP64 ? 2 : 2 + m / 5; }
 double kappa_redo(int precision) { return precision == DIRAC_FP64 ? 1e12 : 1e2; }
 
-cudaError_t launch_recombine(int precision, const RecombParams& rp, int grid, cudaStream_t s) {
-  if (precision == DIRAC_FP64) return launch_pdl(recombine<false>, grid, 256, 0, s, rp);
+cudaError_t launch_recombine(int precision, bool muladd, const RecombParams& rp, int grid, cudaStream_t s) {
+  if (precision == DIRAC_FP64)
+    return muladd ? launch_pdl(recombine<false>, grid, 256, 0, s, rp) : launch_recombine64(rp, grid, s);
   return launch_pdl(recombine<true>, grid, 256, 0, s, rp);
 }
 
@@ -352,8 +276,10 @@ struct Engine {
   double* d_coop_slots = nullptr;
   unsigned* d_coop_bar = nullptr;
   int coop_cap = 0;                // CTAs the slot buffer holds
+  size_t coop_bar_bytes = 0;
   int step_mode = DIRAC_STEP_AUTO;
   int barrier_extra = 0;           // 1 only inside dirac_debug_barrier_timeout
+  bool muladd64 = false;           // FP64 kernels in multiply-adds (set by the adjoint for its call)
   int* d_blk_prob = nullptr;
   int* d_step = nullptr;
   // per-call tables: [Problem x nprob][ChebParams x nprob][FieldStep x nfield]
@@ -433,12 +359,24 @@ dirac_status check_grid(int nx, int ny, double dx, double dy) {
 // tiles of a problem at tile height th
 int tiles_of(int nx, int ny, int th) { return ((nx + TILE_W - 1) / TILE_W) * ((ny + th - 1) / th); }
 
-// FP64 tile height when none is set.  One CTA per SM streams its chunk of
+// Tile height of the fixed-point FP64 kernels, 16 or 8 rows.  `set`: the height
+// asked for by dirac_batch_set_launch_shape (32: the tall tiles, 16: the short
+// ones), 0 for none: short tiles while the tall ones are fewer than two per SM,
+// where a pass takes the time of one tile (m = 20, ms per step, short / tall:
+// 256^2 0.31 / 0.37, 384^2 0.45 / 0.45, 512^2 0.60 / 0.55, 1024^2 1.58 / 1.43).
+int fx_tile_height(int set, const std::vector<HostProblem>& P, int n_sm) {
+  if (set) return set == 32 ? 16 : 8;
+  long long t = 0;
+  for (const HostProblem& q : P) t += tiles_of(q.nx, q.ny, 16);
+  return t >= 2LL * n_sm ? 16 : 8;
+}
+
+// Tile height of the FP64 multiply-add kernels when none is set.  One CTA per SM streams its chunk of
 // tiles, so the SM with the most tiles sets the pass time:
 // ceil(tiles / SMs) x (rows + about a quarter row of per-tile cost: halo,
 // barriers).  16-row tiles win on grids that leave SMs idle or end with a
 // nearly empty last tile per SM; 32-row tiles otherwise.
-int fp64_tile_height(const std::vector<HostProblem>& P, int n_sm) {
+int muladd_tile_height(const std::vector<HostProblem>& P, int n_sm) {
   double best = 1e300;
   int pick = 32;
   for (int th : {32, 16}) {
@@ -469,7 +407,7 @@ dirac_status Engine::init(int n, const int* nx, const int* ny, const double* dx,
     q.n = (long long)q.nx * q.ny;
     q.tiles_x = (q.nx + TILE_W - 1) / TILE_W;
     q.slot_off = slots;
-    slots += (size_t)tiles_of(q.nx, q.ny, 16);   // at least one tile per slot
+    slots += (size_t)tiles_of(q.nx, q.ny, 8);   // at least one tile per slot
     sites += q.n;
   }
   // workspace: (m_max - 1) basis fields + 2 y^ fields per problem, one block
@@ -500,7 +438,11 @@ dirac_status Engine::init(int n, const int* nx, const int* ny, const double* dx,
     coop_cap = shape.n_sm * 8;     // the most resident CTAs of any pass kernel
     CUDA_TRY(cudaMalloc(&d_coop_slots, 2 * 3 * sizeof(double) * coop_cap));
   }
-  CUDA_TRY(cudaMalloc(&d_coop_bar, GRID_SYNC_WORDS * sizeof(unsigned)));
+  // barrier words, then the partials of the fixed-point step by pass parity (one
+  // CTA per SM, and one more that no CTA writes, for the test of the timeout)
+  coop_bar_bytes = GRID_SYNC_WORDS * sizeof(unsigned) +
+                   (n == 1 && precision == DIRAC_FP64 ? 12 * (size_t)(shape.n_sm + 1) * sizeof(unsigned long long) : 0);
+  CUDA_TRY(cudaMalloc(&d_coop_bar, coop_bar_bytes));
   CUDA_TRY(cudaMemsetAsync(d_st, 0, sizeof(DevState) * n, stream));
   CUDA_TRY(cudaEventCreateWithFlags(&tab_ev, cudaEventDisableTiming));
   // recombination blocks in proportion to the problem sizes
@@ -617,8 +559,11 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     for (long long k = 0; k < 2LL * nsteps * np; ++k)
       if (!std::isfinite(a_xy[k])) return fail(DIRAC_EINVAL, "non-finite vector potential in the schedule");
   const bool m32 = use_m32();
-  const int th = m32 ? M32_TILE_H
-                     : (shape.th ? shape.th : (precision == DIRAC_FP64 ? fp64_tile_height(P, shape.n_sm) : 16));
+  const int th = m32                                ? M32_TILE_H
+             : precision == DIRAC_FP64 && !muladd64 ? fx_tile_height(shape.th, P, shape.n_sm)
+             : shape.th                             ? shape.th
+             : precision == DIRAC_FP64              ? muladd_tile_height(P, shape.n_sm)
+                                                    : 16;
   // tile list for this tile height
   int tt = 0;
   for (HostProblem& q : P) {
@@ -702,12 +647,12 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     }
     hasv = hasv || q.has_v;
   }
-  bool iso = true;
-  for (int b = 0; b < np; ++b) iso = iso && hp[b].kx == hp[b].ky;
+  bool has_ay = false;
   for (int k = 0; k < nfield; ++k) {
     const int b = k % np;
     const double ax = a_xy ? a_xy[2 * (size_t)k] : P[b].ax;
     const double ay = a_xy ? a_xy[2 * (size_t)k + 1] : P[b].ay;
+    has_ay = has_ay || ay != 0.0;
     FieldStep& f = hf[k];
     f.cAx = c * ax;   // electron: p - qA = p + A
     f.cAy = c * ay;
@@ -734,7 +679,10 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
   lp.mcc = mcc;
   lp.dt = dt;
   lp.conj_coef = backward ? 1 : 0;
-  lp.iso = iso ? 1 : 0;
+  lp.has_ay = has_ay ? 1 : 0;
+  lp.iso = 1;
+  for (int b = 0; b < np; ++b)
+    if (hp[b].kx != hp[b].ky) lp.iso = 0;
   lp.diri = boundary == DIRAC_DIRICHLET ? 1 : 0;
   lp.tol = tol;
   lp.step = d_step;
@@ -752,7 +700,7 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     lp.pass = 1;
     lp.probe = 1;
     CUDA_TRY(mark(KIND_PASS));
-    CUDA_TRY(launch_pass(precision, order, diri, hasv, lp, ls, stream));
+    CUDA_TRY(launch_pass(precision, muladd64, order, diri, hasv, lp, ls, stream));
     ++launches;
     lp.probe = 0;
     need_probe = false;
@@ -765,10 +713,13 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     ca.G = 0;
     ca.cap = coop_cap;
     ca.bar_count = barrier_extra;
+    ca.packets = reinterpret_cast<unsigned long long*>(d_coop_bar + GRID_SYNC_WORDS);
+    if (!muladd64) ca.cap = shape.n_sm + 1;
     for (int s = 0; s < nsteps; ++s) {
-      CUDA_TRY(cudaMemsetAsync(d_coop_bar, 0, GRID_SYNC_WORDS * sizeof(unsigned), stream));
+      CUDA_TRY(cudaMemsetAsync(d_coop_bar, 0, coop_bar_bytes, stream));
       CUDA_TRY(mark(KIND_STEP));
-      CUDA_TRY(launch_step(precision, th, order, diri, hasv, lp, shape.n_sm, ca, stream));
+      CUDA_TRY(muladd64 ? launch_step_muladd(th, order, diri, hasv, lp, shape.n_sm, ca, stream)
+                        : launch_step64(th, order, diri, hasv, lp, shape.n_sm, ca, stream));
       ++launches;
     }
     CUDA_TRY(mark(KIND_END));
@@ -784,6 +735,7 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
   ca32.G = 0;
   ca32.cap = coop_cap;
   ca32.bar_count = barrier_extra;
+  ca32.packets = nullptr;
   auto enqueue_step = [&](cudaStream_t st, bool count) -> dirac_status {
     if (m32) {   // the whole step in one launch (the barrier words restart at zero)
       CUDA_TRY(cudaMemsetAsync(d_coop_bar, 0, GRID_SYNC_WORDS * sizeof(unsigned), st));
@@ -798,11 +750,11 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     for (int i = 1; i <= m + lp.redo_budget; ++i) {
       lp.pass = i;
       if (count) CUDA_TRY(mark(KIND_PASS));
-      CUDA_TRY(launch_pass(precision, order, diri, hasv, lp, ls, st));
+      CUDA_TRY(launch_pass(precision, muladd64, order, diri, hasv, lp, ls, st));
       if (count) ++launches;
     }
     if (count) CUDA_TRY(mark(KIND_RECOMBINE));
-    CUDA_TRY(launch_recombine(precision, rp, rgrid, st));
+    CUDA_TRY(launch_recombine(precision, muladd64, rp, rgrid, st));
     if (count) {
       ++launches;
       CUDA_TRY(mark(KIND_END));
@@ -818,7 +770,7 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     std::memcpy(kp, &lk, sizeof(lk)); kp += sizeof(lk);
     std::memcpy(kp, &rp, sizeof(rp)); kp += sizeof(rp);
     std::memcpy(kp, &ls, sizeof(ls)); kp += sizeof(ls);
-    const int extra[3] = {precision + 2 * (int)m32, (int)hasv, rgrid};
+    const int extra[3] = {precision + 2 * (int)m32 + 4 * (int)muladd64, (int)hasv, rgrid};
     std::memcpy(kp, extra, sizeof(extra));
     if (!step_graph || key != graph_key) {
       if (!cap_stream) CUDA_TRY(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking));
@@ -937,6 +889,8 @@ dirac_status ctx_view(dirac_ctx* ctx, CtxView* v) {
   v->basis = q.basis;
   return DIRAC_OK;
 }
+
+void ctx_muladd64(dirac_ctx* ctx, bool on) { ctx->e.muladd64 = on; }
 
 dirac_status operator_interval(dirac_ctx* ctx, double ax_max, double ay_max, double* c0, double* half) {
   if (!ctx) return fail(DIRAC_EINVAL, "null context");
@@ -1543,7 +1497,7 @@ extern "C" dirac_status dirac_lanczos_step_noalloc(const dirac_problem* pb, void
   const int nx = pb->nx, ny = pb->ny;
   const long long n = (long long)nx * ny;
   const int tiles_x = (nx + TILE_W - 1) / TILE_W;
-  const int ntiles = tiles_of(nx, ny, 32);
+  const int ntiles = tiles_of(nx, ny, 8);     // short tiles: these are small grids
   constexpr int RB_MAX = 64;                   // recombination blocks
   const size_t field = align256((size_t)n * sizeof(vec4));
   const size_t off_cheb = align256(sizeof(Problem));
@@ -1551,7 +1505,10 @@ extern "C" dirac_status dirac_lanczos_step_noalloc(const dirac_problem* pb, void
   const size_t off_step = off_field + align256(sizeof(FieldStep));
   const size_t off_st = off_step + align256(sizeof(int) * (1 + RB_MAX));
   const size_t off_part = off_st + align256(sizeof(DevState));
-  const size_t off_y = off_part + align256(3 * sizeof(double) * ntiles);
+  // partials: one slot per 32-row tile at least; the launch has no more CTAs than slots
+  const size_t part_bytes = align256(3 * sizeof(double) * tiles_of(nx, ny, 32));
+  const int slots = (int)std::min<size_t>(part_bytes / (3 * sizeof(double)), 1u << 20);
+  const size_t off_y = off_part + part_bytes;
   const size_t off_basis = off_y + 2 * field;
   const size_t need = off_basis + (size_t)std::max(1, m - 1) * field;
   if (need > NOALLOC_SCRATCH_BYTES)
@@ -1632,6 +1589,7 @@ extern "C" dirac_status dirac_lanczos_step_noalloc(const dirac_problem* pb, void
   lp.fstride = 0;
   lp.nprob = 1;
   lp.total_tiles = ntiles;
+  lp.has_ay = pb->A_y != 0.0 ? 1 : 0;
   lp.iso = d.kx == d.ky ? 1 : 0;
   lp.m = m;
   lp.mcc = mcc;
@@ -1641,22 +1599,22 @@ extern "C" dirac_status dirac_lanczos_step_noalloc(const dirac_problem* pb, void
   lp.step = step;
   lp.redo_budget = redo_budget(DIRAC_FP64, m);
   lp.kappa_redo = kappa_redo(DIRAC_FP64);
-  LaunchShape ls{n_sm, 32, 0};
+  LaunchShape ls{std::min(n_sm, slots), 8, 1};
   const bool diri = pb->boundary == DIRAC_DIRICHLET, hasv = pb->V_dev != nullptr;
   lp.pass = 1;
   lp.probe = 1;
-  CUDA_TRY(launch_pass(DIRAC_FP64, pb->stencil_order, diri, hasv, lp, ls, stream));
+  CUDA_TRY(launch_pass(DIRAC_FP64, false, pb->stencil_order, diri, hasv, lp, ls, stream));
   lp.probe = 0;
   for (int i = 1; i <= m + lp.redo_budget; ++i) {
     lp.pass = i;
-    CUDA_TRY(launch_pass(DIRAC_FP64, pb->stencil_order, diri, hasv, lp, ls, stream));
+    CUDA_TRY(launch_pass(DIRAC_FP64, false, pb->stencil_order, diri, hasv, lp, ls, stream));
   }
   RecombParams rp;
   rp.probs = lp.probs;
   rp.blk_prob = blk;
   rp.step = step;
   rp.redo_budget = lp.redo_budget;
-  CUDA_TRY(launch_recombine(DIRAC_FP64, rp, rblocks, stream));
+  CUDA_TRY(launch_recombine(DIRAC_FP64, false, rp, rblocks, stream));
 
   if (info) {
     DevState h;

@@ -107,5 +107,14 @@ __device__ __forceinline__ double to_double(const WarpSum& s) {
   return fma((double)(((long long)s.t2 << 21) + s.t1), 2097152.0, (double)s.t0);
 }
 
+
+// d 2^e by its exponent field; scalbn only where the result leaves the normal range
+__device__ __forceinline__ double scale2(double d, int e) {
+  const int f = exp_field(d) + e;
+  if (d == 0.0) return 0.0;
+  if (f <= 0 || f >= 0x7ff) return scalbn(d, e);
+  return __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
+}
+
 }  // namespace fx
 }  // namespace dirac

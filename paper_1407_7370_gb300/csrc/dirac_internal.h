@@ -9,6 +9,8 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <atomic>
+#include <cstdlib>
+#include <utility>
 
 namespace dirac {
 
@@ -48,6 +50,7 @@ dirac_status ctx_view(dirac_ctx* ctx, CtxView* v);
 struct ChebParams;
 struct LaunchParams;
 struct CoopArgs;
+struct RecombParams;
 
 // Resident CTAs per SM of `kernel` (threads, dynamic shared memory smem) on
 // the current device.  Computed once per device -- after raising the
@@ -76,6 +79,40 @@ cudaError_t occupancy_on_device(std::atomic<int>* cache, Kernel kernel, int thre
   return cudaSuccess;
 }
 
+// DIRAC_NO_PDL=1 in the environment turns the launch overlap off (debugging aid).
+inline bool pdl_enabled() {
+  static const bool on = [] {
+    const char* v = std::getenv("DIRAC_NO_PDL");
+    return !(v && v[0] == '1');
+  }();
+  return on;
+}
+
+// Launch with programmatic stream serialisation: the kernel may be scheduled
+// while the previous kernel in the stream finishes; it waits for it (and sees
+// its writes) at its griddepcontrol.wait.
+template <class... KArgs, class... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                       Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl_enabled() ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+struct LaunchShape {
+  int n_sm;          // SMs of the device
+  int th;            // tile height (32 or 16; fixed-point FP64: 32 or 8)
+  int cta_cap;       // 0: as many CTAs per SM as fit; else at most this many
+};
+
 // FP32 passes stage their tiles by asynchronous copies from this many tiles
 // per CTA on (below that the extra barrier costs more than it hides)
 constexpr int ASYNC_MIN_TILES = 4;
@@ -92,12 +129,26 @@ constexpr int M32_TILE_H = 16;
 cudaError_t launch_step_m32(int order, bool diri, const LaunchParams& p, int n_sm, const CoopArgs& ca,
                             cudaStream_t s);
 
-// One time step of the single problem in `p` as one cooperative launch
-// (lanczos_step); sets the grid, the chunks and ca.G.  ca.bar_count on entry:
-// arrivals the barriers wait for beyond the launch's CTAs (0; 1 only in the
-// test of the barrier timeout).
-cudaError_t launch_step(int precision, int th, int order, bool diri, bool hasv, const LaunchParams& p, int n_sm,
-                        const CoopArgs& ca, cudaStream_t s);
+// One time step of the single problem in `p` as one cooperative launch; sets
+// the grid, the chunks and ca.G.  ca.bar_count on entry: arrivals the barriers
+// wait for beyond the launch's CTAs (0; 1 only in the test of the barrier
+// timeout).  launch_step64: fixed-point FP64 (lanczos_step64); launch_step_muladd:
+// FP64 multiply-adds (lanczos_step).
+cudaError_t launch_step64(int th, int order, bool diri, bool hasv, const LaunchParams& p, int n_sm,
+                          const CoopArgs& ca, cudaStream_t s);
+cudaError_t launch_step_muladd(int th, int order, bool diri, bool hasv, const LaunchParams& p, int n_sm,
+                               const CoopArgs& ca, cudaStream_t s);
+
+// One pass of every problem in `p` in a launch of its own, and the
+// recombination, on the same two FP64 paths
+cudaError_t launch_pass64(int order, bool diri, bool hasv, const LaunchParams& p, const LaunchShape& ls,
+                          cudaStream_t s);
+cudaError_t launch_recombine64(const RecombParams& rp, int grid, cudaStream_t s);
+cudaError_t launch_pass_muladd(int order, bool diri, bool hasv, const LaunchParams& p, const LaunchShape& ls,
+                               cudaStream_t s);
+
+// FP64 kernels of this context in multiply-adds from now on (or not)
+void ctx_muladd64(dirac_ctx* ctx, bool on);
 
 // [c0 - half, c0 + half] contains the spectrum of H - s for any vector
 // potential with |A_x| <= ax_max, |A_y| <= ay_max

@@ -46,8 +46,11 @@
 // serial eigensolver dominate small steps, while the Chebyshev recurrence is
 // FMA-only and warp-parallel.  Both give exp(-i T dt) e_1 to rounding.
 //
-// Precision: S = double is the FP64 path (complex128 fields; the products in
-// 60-bit fixed point, dirac_fixed.cuh).  S = float is the mixed path:
+// Precision: the FP64 path keeps complex128 fields and takes its products in
+// 60-bit fixed point (dirac_pass64.cuh).  The kernels below with S = double are
+// the same pass in FP64 multiply-adds; the adjoint runs on them (its gradients
+// with respect to A are sums that cancel to 1e-6 of their terms, so that
+// another rounding shows in their ninth digit).  S = float is the mixed path:
 // complex64 basis and y^, FP32 stencil, warp sums converted to FP64, FP64
 // scalars; q^_1 is the complex128 state itself (passes 1-2 read it).
 #pragma once
@@ -56,7 +59,6 @@
 #include <stdint.h>
 
 #include <cuda/atomic>
-#include <type_traits>
 
 #include "dirac_fixed.cuh"
 
@@ -74,7 +76,7 @@ using vec4 = double4_32a;       // one site: (u.re, u.im, d.re, d.im)
 struct PassCoef {
   double g, gd, e, au0, ad0;          // q^ = g y^ - gd q^_prev; y^ -= e q^_prev; diagonals
   float gf, gdf, ef, au_hi, au_lo, ad_hi, ad_lo;
-  float yexp;                         // FP64 path: the pass stores 2^yexp y^ (an integer; 0 on the mixed path)
+  float yexp;                         // fixed-point FP64 path: the pass stores 2^yexp y^ (an integer; else 0)
 };
 
 __host__ __device__ inline PassCoef make_coef(double g, double gd, double e, double au0, double ad0,
@@ -143,7 +145,7 @@ struct Problem {
   float kxf, kyf;           // kx, ky rounded to FP32
   float kxf_lo, kyf_lo;     // and their remainders
   int tma;                  // the mixed one-launch step stages tiles by tensor copies (maps valid)
-  int vbe;                  // FP64 path: exponent field of max |V| (0: V = 0)
+  int vbe;                  // fixed-point FP64 path: exponent field of max |V| (0: V = 0)
   PassCoef probe_coef;      // coefficients of the probe pass (stencil shift 0)
 };
 
@@ -172,7 +174,8 @@ struct LaunchParams {
   int pass, m, probe;
   int conj_coef;            // 1: backward step (dt < 0): exp(+i H |dt|), the conjugate coefficients
   int async_tiles;          // FP32 basis: stage passes >= 3 by asynchronous copies (many tiles per CTA)
-  int iso;                  // FP64 path: kx = ky in every problem (host: picks the kernel)
+  int has_ay;               // 0: A_y = 0 in every step and problem (host: picks the kernel)
+  int iso;                  // kx = ky in every problem (fixed-point FP64 path; host: picks the kernel)
   int diri;                 // Dirichlet boundaries (kernels that take the boundary at run time)
   double mcc, dt, tol;      // dt = |dt|
   const int* step;          // step counter of the running call (index into fields)
@@ -262,6 +265,10 @@ __device__ __forceinline__ T ld4(const T* p) {
   if constexpr (COHERENT) return ldw4(p);
   else return ldg4(p);
 }
+
+template <class S> struct Vec4;
+template <> struct Vec4<double> { using T = double4_32a; };
+template <> struct Vec4<float> { using T = float4; };
 
 template <class To, class From>
 __device__ __forceinline__ void cvt4(const From& a, To (&o)[4]) {
@@ -518,9 +525,8 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
 // cross-shaped halo of q^_i are formed in shared memory from y^_{i-1} and
 // q^_{i-1}.
 // ---------------------------------------------------------------------------
-// CTAs per SM of the FP32 pass (128 or 256 threads each)
-template <int TH>
-__host__ __device__ constexpr int min_blocks() { return TH == 32 ? 4 : 8; }
+template <class S, int TH, int SUB>
+__host__ __device__ constexpr int min_blocks() { return sizeof(S) == sizeof(float) ? (TH == 32 ? 4 : 8) : (SUB == 2 ? 1 : 2); }
 
 // rows per thread: four, except two on FP64 16-row tiles, which keep eight
 // warps per tile worker and halve the unit of work: a grid of a few tiles per
@@ -532,17 +538,25 @@ __host__ __device__ constexpr int rows_per_thread() { return (sizeof(S) == sizeo
 template <class S>
 __host__ __device__ constexpr int sub_workers() { return sizeof(S) == sizeof(double) ? 2 : 1; }
 
-// shared memory of one FP64 tile worker: q^_i on the tile and its halo in
-// fixed point, the upper and the lower components in separate halves (16 bytes
-// per site each, so that a warp's row is read without bank conflicts), then a
-// table of coefficients per warp and the exponents of two tiles
-constexpr int COEF_SLOTS = 16;   // eight per half
-template <int R, int TH>
-__host__ __device__ constexpr int half_sites() { return (TH + 2 * R) * (TILE_W + 2 * R); }
-template <int R, int TH>
-__host__ __device__ constexpr size_t worker_bytes() {
-  return 2 * sizeof(longlong2) * half_sites<R, TH>() +
-         sizeof(int2) * COEF_SLOTS * (TH / rows_per_thread<double, TH>()) + 32;
+// shared memory of one tile worker: the tile of q^_i with its halo, and on
+// the mixed path the staging buffer of q^_{i-1} on the same rectangle
+template <class S, int R, int TH>
+__host__ __device__ constexpr size_t tile_bytes() { return sizeof(S) * 4 * (TH + 2 * R) * (TILE_W + 2 * R); }
+template <class S, int R, int TH>
+__host__ __device__ constexpr size_t qbuf_bytes() {
+  return sizeof(S) == sizeof(float) ? sizeof(float4) * (TH + 2 * R) * (TILE_W + 2 * R) : 0;
+}
+template <class S, int R, int TH>
+__host__ __device__ constexpr size_t worker_bytes() { return tile_bytes<S, R, TH>() + qbuf_bytes<S, R, TH>(); }
+
+// tile workers per CTA of the one-launch step: one CTA per SM on both paths
+// (two workers of eight warps on FP64; 768 threads on FP32 -- six 128-thread
+// or three 256-thread workers, 80 registers each, where 1024 threads at 64
+// registers spilled), so that a grid barrier and its partial sums involve one
+// CTA per SM
+template <class S, int TH>
+__host__ __device__ constexpr int step_workers() {
+  return sizeof(S) == sizeof(double) ? 2 : 768 / (32 * (TH / 4));
 }
 
 // Chunks of the tile list: CTA c takes q + 1 tiles if c < r, else q (q = T / G,
@@ -552,112 +566,56 @@ __device__ __forceinline__ int cta_of_tile(int t, int q, int r) {
   return t < big ? t / (q + 1) : r + (t - big) / q;
 }
 
-// Dynamic shared memory of a pass kernel (the FP32 pass keeps its tile in a
-// static array)
+// shared memory of the tile workers: a static array for one worker, the
+// dynamic allocation for several (more than the 48 KiB of static memory)
 template <class S, int R, int TH, int SUB>
-__host__ __device__ constexpr size_t dyn_smem_bytes() {
-  return sizeof(S) == sizeof(float) ? 0 : SUB * worker_bytes<R, TH>();
-}
+__host__ __device__ constexpr size_t dyn_smem_bytes() { return SUB == 1 ? 0 : SUB * worker_bytes<S, R, TH>(); }
 
-// This CTA's share of a problem, the warps' sums in red[], -> one partial per
-// (problem, CTA) slot.  COOP = false: then the problem's ticket, and the CTA
-// that completes the problem sums its slots and updates its scalars.  COOP =
-// true (one-launch step): the partial goes to coop_slots[3 blockIdx.x ..] and
-// the caller goes on.
-template <bool FX, bool COOP, int NW>
-__device__ __forceinline__ void pass_sums(const LaunchParams& lp, const Problem* pr, int i, int seg_tiles,
-                                          double (*red)[3], int* last_flag, double* coop_slots) {
-  constexpr int NT = 32 * NW;
-  const int cq = lp.chunk_q, cr = lp.chunk_r;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (warp == 0) {
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    if (lane < NW) { s0 = red[lane][0]; s1 = red[lane][1]; s2 = red[lane][2]; }
-#pragma unroll
-    for (int o = (NW > 16 ? 16 : 8); o > 0; o >>= 1) {   // NW <= 32 warps
-      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    if (lane == 0) {
-      if constexpr (COOP) {
-        coop_slots[3 * blockIdx.x + 0] = s0;
-        coop_slots[3 * blockIdx.x + 1] = s1;
-        coop_slots[3 * blockIdx.x + 2] = s2;
-        *last_flag = 0;
-      } else {
-        const int slot = blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr);
-        pr->partials[3 * slot + 0] = s0;
-        pr->partials[3 * slot + 1] = s1;
-        pr->partials[3 * slot + 2] = s2;
-        // release our partial / acquire everybody else's
-        cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
-        *last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
-                     (unsigned)pr->ntiles);
-      }
-    }
-  }
-  __syncthreads();
-  if (!COOP && *last_flag) {
-    // the problem is complete: the whole CTA sums its slots in a fixed
-    // order (thread-strided, the warp tree, then the warps in turn), the
-    // loads of SB slots per thread in flight at once, so that a pass of
-    // eight CTAs per SM waits for two L2 round trips here, not five
-    const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
-    const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
-    constexpr int SB = 5;
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-    for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
-      double v[SB][3];
-#pragma unroll
-      for (int k = 0; k < SB; ++k) {
-        const int s = s0 + k * NT;
-        const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
-        v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
-        v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
-        v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
-      }
-#pragma unroll
-      for (int k = 0; k < SB; ++k) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
-    }
-    t0 = warp_sum(t0);
-    t1 = warp_sum(t1);
-    t2 = warp_sum(t2);
-    if (lane == 0) { red[warp][0] = t0; red[warp][1] = t1; red[warp][2] = t2; }
-    __syncthreads();
-    if (warp == 0) {
-      t0 = red[0][0]; t1 = red[0][1]; t2 = red[0][2];
-#pragma unroll
-      for (int w = 1; w < NW; ++w) { t0 += red[w][0]; t1 += red[w][1]; t2 += red[w][2]; }
-      if (lane == 0) pr->st->counter = 0u;
-      finish_pass<FX>(lp, pr, pr->st, i, t0, t1, t2);
-    }
-  }
-  __syncthreads();
-}
-
-// The body of one FP32 pass over this CTA's chunk (the mixed path).
-template <int R, int TH, bool DIRI, bool HAS_V>
-__device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
-  using S = float;
-  using T4 = float4;                        // storage of y^ and of q^_i, i >= 2
+// The body of one pass over this CTA's chunk.  COOP = false: a launch of
+// its own (lanczos_pass): per-problem tickets, the last CTA finishes.
+// COOP = true: inside the one-launch step (lanczos_step): one problem, the
+// state read from `coop_st`, coherent loads, and the CTA's partial sums
+// written to coop_slots[3 * blockIdx.x ...]; the caller synchronises the grid
+// and finishes.
+template <class S, int R, int TH, bool DIRI, bool HAS_V, bool HAS_AY, bool COOP, int SUB>
+__device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState* coop_st, double* coop_slots,
+                                          int step) {
+  using T4 = typename Vec4<S>::T;           // storage of y^ (and of q^ on the mixed path)
   constexpr int RPT = rows_per_thread<S, TH>();
-  constexpr int NG = TH / RPT;              // row groups = warps
-  constexpr int NT = 32 * NG;               // threads
+  constexpr int NG = TH / RPT;              // row groups = warps of a worker
+  constexpr int NTS = 32 * NG;              // threads of a worker
+  constexpr int NT = SUB * NTS;             // threads
+  constexpr int NW = SUB * NG;              // warps
   constexpr int W = TILE_W + 2 * R;
-  __shared__ double red[NG][3];
+  extern __shared__ __align__(32) unsigned char dyn_smem[];
+  __shared__ double red[NW][3];
   __shared__ int last_flag;
 
   const int cq = lp.chunk_q, cr = lp.chunk_r;
   const int t_begin = blockIdx.x * cq + min((int)blockIdx.x, cr);
   const int t_end = t_begin + cq + ((int)blockIdx.x < cr ? 1 : 0);
-  const int ltid = (int)threadIdx.x;
+  const int sub = SUB == 1 ? 0 : (int)threadIdx.x / NTS;   // this thread's worker
+  const int ltid = (int)threadIdx.x - sub * NTS;
   const int tx = ltid & 31, tg = ltid >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ __align__(32) S tile[TH + 2 * R][W][4];
-  // passes >= 3: q^_{i-1} on the tile and halo, copied asynchronously
-  __shared__ __align__(16) float4 qbuf[(TH + 2 * R) * W];
+  constexpr bool F32 = sizeof(S) == sizeof(float);
+  __shared__ __align__(32) S tile_s[SUB == 1 ? TH + 2 * R : 1][W][4];
+  S(*const tile)[W][4] = SUB == 1 ? &tile_s[0]
+                                  : reinterpret_cast<S(*)[W][4]>(dyn_smem + sub * worker_bytes<S, R, TH>());
+  // mixed path, passes >= 3: q^_{i-1} on the tile and halo, copied asynchronously
+  constexpr int NSQ = (F32 && SUB == 1) ? (TH + 2 * R) * W : 1;
+  __shared__ __align__(16) float4 qbuf_s[NSQ];
+  float4* const qbuf = SUB == 1 ? qbuf_s
+                                : reinterpret_cast<float4*>(dyn_smem + sub * worker_bytes<S, R, TH>() +
+                                                            tile_bytes<S, R, TH>());
+  // barrier of this worker's threads (the whole CTA when there is one worker)
+  auto sub_sync = [&]() {
+    if constexpr (SUB == 1) {
+      __syncthreads();
+    } else {
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "r"(NTS) : "memory");
+    }
+  };
 
   // problem of the first tile (problems are sorted by tile_begin)
   int b = 0;
@@ -671,7 +629,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
   }
   for (int t = t_begin; t < t_end; ++b) {
     const Problem* pr = lp.probs + b;
-    const DevState* st = lp.states + b;
+    const DevState* st = COOP ? coop_st : lp.states + b;
     // independent loads first (all addresses are valid), then the branch
     const int stopped = st->stopped;
     const int i = lp.probe ? 1 : max(1, st->cur_pass);
@@ -680,20 +638,20 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
     const int seg_end = min(t_end, pr->tile_begin + pr->ntiles);
     const int seg_tiles = seg_end - t;
     if (stopped) { t = seg_end; continue; }
-    const S gS = pc.gf;
-    const S gdS = pc.gdf;
-    const S eS = pc.ef;
-    const S kx = pr->kxf, ky = pr->kyf;
-    const S cAx = fs.cAxf, cAy = fs.cAyf;
-    const S au_hi = pc.au_hi, au_lo = pc.au_lo;
-    const S ad_hi = pc.ad_hi, ad_lo = pc.ad_lo;
+    const S gS = F32 ? (S)pc.gf : (S)pc.g;
+    const S gdS = F32 ? (S)pc.gdf : (S)pc.gd;
+    const S eS = F32 ? (S)pc.ef : (S)pc.e;
+    const S kx = F32 ? (S)pr->kxf : (S)pr->kx, ky = F32 ? (S)pr->kyf : (S)pr->ky;
+    const S cAx = F32 ? (S)fs.cAxf : (S)fs.cAx, cAy = F32 ? (S)fs.cAyf : (S)fs.cAy;
+    const S au_hi = F32 ? (S)pc.au_hi : (S)pc.au0, au_lo = F32 ? (S)pc.au_lo : S(0);
+    const S ad_hi = F32 ? (S)pc.ad_hi : (S)pc.ad0, ad_lo = F32 ? (S)pc.ad_lo : S(0);
     // FP32: remainders of the stencil and vector-potential coefficients
-    const S kx_lo = pr->kxf_lo, ky_lo = pr->kyf_lo;
-    const S cAx_lo = fs.cAxf_lo, cAy_lo = fs.cAyf_lo;
+    const S kx_lo = F32 ? (S)pr->kxf_lo : S(0), ky_lo = F32 ? (S)pr->kyf_lo : S(0);
+    const S cAx_lo = F32 ? (S)fs.cAxf_lo : S(0), cAy_lo = F32 ? (S)fs.cAyf_lo : S(0);
     const int nx = pr->nx, ny = pr->ny;
     const size_t n = (size_t)nx * ny;
     // this pass's vectors
-    constexpr int SB = (int)sizeof(float4);
+    constexpr int SB = F32 ? (int)sizeof(float4) : (int)sizeof(double4_32a);
     const char* basis = static_cast<const char*>(pr->basis);
     const void* y_prev = (i >= 2) ? (((i - 1) & 1) ? pr->ybuf1 : pr->ybuf0) : nullptr;
     const void* q_prev = (i == 2) ? (const void*)pr->psi
@@ -701,7 +659,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
     void* q_out = (i >= 2) ? (void*)(basis + (size_t)(i - 2) * n * SB) : nullptr;
     void* y_out = (i < lp.m) ? ((i & 1) ? pr->ybuf1 : pr->ybuf0) : nullptr;
     const T4* yprev = static_cast<const T4*>(y_prev);
-    const bool q64 = i <= 2;                // q^_{i-1} stored as complex128
+    const bool q64 = !F32 || i <= 2;                // q^_{i-1} stored as complex128
     const S* Vp = static_cast<const S*>(pr->V);   // NULL: V = 0 for this problem
     const float* Vlo = static_cast<const float*>(pr->Vlo);   // mixed path: V - (float)V, or NULL
 
@@ -715,16 +673,16 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
         const size_t idx = (size_t)iy * nx + ix;
         if (q64) {
           const vec4* qsrc = (i == 1) ? pr->psi : static_cast<const vec4*>(q_prev);
-          cvt4(ldg4(qsrc + idx), qp);
+          cvt4(ld4<COOP>(qsrc + idx), qp);
         } else {
-          cvt4(ldg4(static_cast<const float4*>(q_prev) + idx), qp);
+          cvt4(ld4<COOP>(static_cast<const float4*>(q_prev) + idx), qp);
         }
         if (i == 1) {
 #pragma unroll
           for (int c = 0; c < 4; ++c) q[c] = qp[c];
         } else {
           S yv[4];
-          cvt4(ldg4(yprev + idx), yv);
+          cvt4(ld4<COOP>(yprev + idx), yv);
 #pragma unroll
           for (int c = 0; c < 4; ++c) q[c] = fma(-gdS, qp[c], gS * yv[c]);
         }
@@ -741,7 +699,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
       S au, ad, aul = au_lo, adl = ad_lo;
       if (HAS_V && Vp != nullptr) {   // V stored in S (float copy on the mixed path)
         const S v = Vp[idx];
-        {
+        if constexpr (F32) {
           // the FP32 sum with the diagonal (up to 2 m c^2) rounds differently at
           // every site: its error and V's own remainder go into the low part
           float ru, rd;
@@ -750,6 +708,9 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
           const float vl = Vlo ? Vlo[idx] : 0.f;
           aul = au_lo + vl + ru;
           adl = ad_lo + vl + rd;
+        } else {
+          au = au_hi + v;
+          ad = ad_hi + v;
         }
       } else {
         au = au_hi;
@@ -763,18 +724,18 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
       // lower: (-mc^2+V-s-sigma) d + c[-i D_x u + D_y u + (A_x + i A_y) u]
       yv[2] = ad * C[2] + kx * dxv[1] + ky * dyv[0] + cAx * C[0];
       yv[3] = ad * C[3] - kx * dxv[0] + ky * dyv[1] + cAx * C[1];
-      {
+      if constexpr (HAS_AY) {   // else A_y = 0 in every step of the launch
         yv[0] = fma(cAy, C[3], yv[0]);
         yv[1] = fma(-cAy, C[2], yv[1]);
         yv[2] = fma(-cAy, C[1], yv[2]);
         yv[3] = fma(cAy, C[0], yv[3]);
       }
-      {
+      if constexpr (F32) {
         yv[0] = fma(aul, C[0], fma(kx_lo, dxv[3], fma(-ky_lo, dyv[2], fma(cAx_lo, C[2], yv[0]))));
         yv[1] = fma(aul, C[1], fma(-kx_lo, dxv[2], fma(-ky_lo, dyv[3], fma(cAx_lo, C[3], yv[1]))));
         yv[2] = fma(adl, C[2], fma(kx_lo, dxv[1], fma(ky_lo, dyv[0], fma(cAx_lo, C[0], yv[2]))));
         yv[3] = fma(adl, C[3], fma(-kx_lo, dxv[0], fma(ky_lo, dyv[1], fma(cAx_lo, C[1], yv[3]))));
-        {
+        if constexpr (HAS_AY) {
           yv[0] = fma(cAy_lo, C[3], yv[0]);
           yv[1] = fma(-cAy_lo, C[2], yv[1]);
           yv[2] = fma(-cAy_lo, C[1], yv[2]);
@@ -829,7 +790,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
     };
 
     bool done_async = false;
-    {
+    if constexpr (F32) {
      if (!q64 && lp.async_tiles) {
       done_async = true;
       // mixed path, passes >= 3: y^_{i-1} and q^_{i-1} of the tile and its
@@ -838,11 +799,11 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
       constexpr int NS = (TH + 2 * R) * W;
       float4* const tf = reinterpret_cast<float4*>(&tile[0][0][0]);
       const float4* const qsrc = static_cast<const float4*>(q_prev);
-      for (int tt = t; tt < seg_end; ++tt) {
+      for (int tt = t + sub; tt < seg_end; tt += SUB) {
         const int lt = tt - pr->tile_begin;
         const int x0 = (lt % pr->tiles_x) * TILE_W;
         const int y0 = (lt / pr->tiles_x) * TH;
-        for (int e = ltid; e < NS; e += NT) {
+        for (int e = ltid; e < NS; e += NTS) {
           const int r = e / W, c = e - r * W;
           bool ox, oy;
           const int ix = wrap<DIRI>(x0 - R + c, nx, ox), iy = wrap<DIRI>(y0 - R + r, ny, oy);
@@ -852,23 +813,23 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
           cp_async16(qbuf + e, qsrc + idx, in ? 16 : 0);
         }
         cp_async_commit_wait();
-        __syncthreads();
-        for (int e = ltid; e < NS; e += NT) {
+        sub_sync();
+        for (int e = ltid; e < NS; e += NTS) {
           const float4 yv = tf[e], qp = qbuf[e];
           tf[e] = make_float4(fmaf(-(float)gdS, qp.x, (float)gS * yv.x), fmaf(-(float)gdS, qp.y, (float)gS * yv.y),
                               fmaf(-(float)gdS, qp.z, (float)gS * yv.z), fmaf(-(float)gdS, qp.w, (float)gS * yv.w));
         }
-        __syncthreads();
+        sub_sync();
         stencil_rows(x0, y0, [&](int, int r, int c, S (&qp)[4]) {
           const float4 v = qbuf[r * W + c];
           qp[0] = (S)v.x; qp[1] = (S)v.y; qp[2] = (S)v.z; qp[3] = (S)v.w;
         });
-        __syncthreads();   // tile and qbuf are reused next
+        sub_sync();   // tile and qbuf are reused next
       }
      }
     }
     if (!done_async) {
-      for (int tt = t; tt < seg_end; ++tt) {
+      for (int tt = t + sub; tt < seg_end; tt += SUB) {
         const int lt = tt - pr->tile_begin;
         const int x0 = (lt % pr->tiles_x) * TILE_W;
         const int y0 = (lt / pr->tiles_x) * TH;
@@ -879,7 +840,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
           form(x0 + tx, y0 + r, r + R, tx + R, qprev[k]);
         }
         constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * TH;
-        for (int h = ltid; h < NH; h += NT) {
+        for (int h = ltid; h < NH; h += NTS) {
           int row, col;
           if (h < NH_ROW) {               // rows above / below
             const int r = h / TILE_W;
@@ -894,403 +855,98 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, int step) {
           S dummy[4];
           form(x0 + col - R, y0 + row - R, row, col, dummy);
         }
-        __syncthreads();
+        sub_sync();
         stencil_rows(x0, y0, [&](int k, int, int, S (&qp)[4]) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) qp[q] = qprev[k][q];
         });
-        __syncthreads();   // the tile buffer is reused next
+        sub_sync();   // the tile buffer is reused next
       }
     }
     t = seg_end;
 
-    // this CTA's share of the problem: thread -> warp in FP32, the rest in FP64
+    // this CTA's share of the problem: thread -> warp in S, warps -> CTA in
+    // double, one partial per (problem, CTA) slot, then the ticket
     accP = warp_sum(accP);
     accY = warp_sum(accY);
     accX = warp_sum(accX);
     if (lane == 0) { red[warp][0] = (double)accP; red[warp][1] = (double)accY; red[warp][2] = (double)accX; }
-    pass_sums<false, false, NG>(lp, pr, i, seg_tiles, red, &last_flag, nullptr);
+    __syncthreads();
+    if (warp == 0) {
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+      if (lane < NW) { s0 = red[lane][0]; s1 = red[lane][1]; s2 = red[lane][2]; }
+#pragma unroll
+      for (int o = (NW > 16 ? 16 : 8); o > 0; o >>= 1) {   // NW <= 32 warps
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      }
+      if (lane == 0) {
+        if constexpr (COOP) {
+          coop_slots[3 * blockIdx.x + 0] = s0;
+          coop_slots[3 * blockIdx.x + 1] = s1;
+          coop_slots[3 * blockIdx.x + 2] = s2;
+          last_flag = 0;
+        } else {
+          const int slot = blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr);
+          pr->partials[3 * slot + 0] = s0;
+          pr->partials[3 * slot + 1] = s1;
+          pr->partials[3 * slot + 2] = s2;
+          // release our partial / acquire everybody else's
+          cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
+          last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
+                       (unsigned)pr->ntiles);
+        }
+      }
+    }
+    __syncthreads();
+    if (!COOP && last_flag) {
+      // the problem is complete: the whole CTA sums its slots in a fixed
+      // order (thread-strided, the warp tree, then the warps in turn), the
+      // loads of SB slots per thread in flight at once, so that a pass of
+      // eight CTAs per SM waits for two L2 round trips here, not five
+      const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
+      const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
+      constexpr int SB = 5;
+      double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+      for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
+        double v[SB][3];
+#pragma unroll
+        for (int k = 0; k < SB; ++k) {
+          const int s = s0 + k * NT;
+          const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
+          v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
+          v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
+          v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < SB; ++k) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
+      }
+      t0 = warp_sum(t0);
+      t1 = warp_sum(t1);
+      t2 = warp_sum(t2);
+      if (lane == 0) { red[warp][0] = t0; red[warp][1] = t1; red[warp][2] = t2; }
+      __syncthreads();
+      if (warp == 0) {
+        t0 = red[0][0]; t1 = red[0][1]; t2 = red[0][2];
+#pragma unroll
+        for (int w = 1; w < NW; ++w) { t0 += red[w][0]; t1 += red[w][1]; t2 += red[w][2]; }
+        if (lane == 0) pr->st->counter = 0u;
+        finish_pass<false>(lp, pr, pr->st, i, t0, t1, t2);
+      }
+    }
+    __syncthreads();
   }
 }
 
-// The body of one FP64 pass over this CTA's chunk.  COOP = false: a launch of
-// its own (lanczos_pass).  COOP = true: inside the one-launch step
-// (lanczos_step): one problem, the state read from `coop_st`, and the CTA's
-// partial sums written to coop_slots; the caller synchronises the grid and
-// finishes.
-//
-// The fields are complex128 in memory; per site and pass only the formation of
-// q^_i (one FP64 multiply-add per number, the scale of y^ being a power of two)
-// and the final conversion of y^_i use the FP64 pipe.  The stencil, the
-// coupling to q^_{i-1} and the three sums are 60-bit fixed point
-// (dirac_fixed.cuh): a tile (with its halo) shares one exponent for the upper
-// and one for the lower components of q^_i, another pair for q^_{i-1}, taken
-// from their largest numbers; every row of the operator is one exact sum of
-// products, rounded to 2^-60 of its largest term.  The sums run per tile in
-// integers and over the tiles of a worker at a common exponent.
-//
-// Measured (GB300, FP64 step with its recombination): 1024^2, m = 20, 2.50 ->
-// 1.89 ms; 4096^2, m = 10, 17.3 -> 10.7 ms; twelve problems of 93^2 .. 301^2 in
-// a batch 1.18 -> 0.94 ms, against the same passes in FP64 multiply-adds, whose
-// 1160 instructions a site and step kept the FP64 pipe 79 % busy.
-//
-// Per tile: load and form (all loads of a thread in flight at once), exponents
-// -> barrier -> fixed point into shared memory, coefficients at the tile's
-// scale -> barrier -> the upper, then the lower components.
-template <int R, int TH, bool DIRI, bool HAS_V, bool ISO, bool COOP, int SUB>
-__device__ __forceinline__ void pass_body_fx(const LaunchParams& lp, const DevState* coop_st, double* coop_slots,
-                                             int step) {
-  constexpr int RPT = rows_per_thread<double, TH>();
-  constexpr int NG = TH / RPT;              // row groups = warps of a worker
-  constexpr int NTS = 32 * NG;              // threads of a worker
-  constexpr int NW = SUB * NG;              // warps
-  constexpr int W = TILE_W + 2 * R;
-  // bits of q^ and q^_{i-1}: the differences (2 x 2 terms; order 4: 36) and
-  // the row sums then stay below 2^62
-  constexpr int F = R == 1 ? 58 : 55;
-  constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * TH;
-  static_assert(NH <= NTS, "one halo site per thread");
-  static_assert(2 * RPT <= 8, "bounds of the per-tile sums");
-  extern __shared__ __align__(32) unsigned char dyn_smem[];
-  __shared__ double red[NW][3];
-  __shared__ int last_flag;
-
-  const int cq = lp.chunk_q, cr = lp.chunk_r;
-  const int t_begin = blockIdx.x * cq + min((int)blockIdx.x, cr);
-  const int t_end = t_begin + cq + ((int)blockIdx.x < cr ? 1 : 0);
-  const int sub = (int)threadIdx.x / NTS;   // this thread's worker
-  const int ltid = (int)threadIdx.x - sub * NTS;
-  const int tx = ltid & 31, tg = ltid >> 5;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char* const my_smem = dyn_smem + sub * worker_bytes<R, TH>();
-  longlong2* const half_u = reinterpret_cast<longlong2*>(my_smem);
-  longlong2* const half_d = half_u + half_sites<R, TH>();
-  int2* const kt = reinterpret_cast<int2*>(half_d + half_sites<R, TH>()) + COEF_SLOTS * tg;
-  unsigned* const emax = reinterpret_cast<unsigned*>(reinterpret_cast<int2*>(half_d + half_sites<R, TH>()) +
-                                                     COEF_SLOTS * NG);   // [2][4]
-  auto sub_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "r"(NTS) : "memory"); };
-  if (ltid < 8) emax[ltid] = 0u;
-  sub_sync();
-  int par = 0;                              // which exponents the tile uses
-
-  // problem of the first tile (problems are sorted by tile_begin)
-  int b = 0;
-  {
-    int lo = 0, hi = lp.nprob - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (lp.probs[mid].tile_begin <= t_begin) lo = mid; else hi = mid - 1;
-    }
-    b = lo;
-  }
-  for (int t = t_begin; t < t_end; ++b) {
-    const Problem* pr = lp.probs + b;
-    const DevState* st = COOP ? coop_st : lp.states + b;
-    // independent loads first (all addresses are valid), then the branch
-    const int stopped = st->stopped;
-    const int i = lp.probe ? 1 : max(1, st->cur_pass);
-    const PassCoef& pc = lp.probe ? pr->probe_coef : st->pc_cur;
-    const int seg_end = min(t_end, pr->tile_begin + pr->ntiles);
-    const int seg_tiles = seg_end - t;
-    if (stopped) { t = seg_end; continue; }
-    const double gd = pc.gd;
-    const int yexp = (int)pc.yexp;
-    const int nx = pr->nx, ny = pr->ny;
-    const size_t n = (size_t)nx * ny;
-    // this pass's vectors
-    vec4* const basis = static_cast<vec4*>(pr->basis);
-    const vec4* const yprev = static_cast<const vec4*>((i & 1) ? pr->ybuf0 : pr->ybuf1);
-    const vec4* const qsrc = i <= 2 ? pr->psi : basis + (size_t)(i - 3) * n;   // q^_{i-1} (q^_1 if i = 1)
-    vec4* const q_out = (i >= 2 && !lp.probe) ? basis + (size_t)(i - 2) * n : nullptr;
-    vec4* const y_out = (i < lp.m && !lp.probe) ? static_cast<vec4*>((i & 1) ? pr->ybuf1 : pr->ybuf0) : nullptr;
-    const double* const Vp = static_cast<const double*>(pr->V);   // NULL: V = 0 for this problem
-    const FieldStep* const fs = lp.fields + step * lp.fstride + b;
-    const bool has_ax = fs->cAx != 0.0, has_ay = fs->cAy != 0.0;
-    // this lane's coefficient: slots 0 diagonal, 1 kx, 2 ky, 3 c A_x, 4 c A_y,
-    // 5 coupling, 6 V (its exponent alone) of the upper (lanes 0-7) and the
-    // lower row (8-15)
-    const int cj = lane & 7, ch = (lane >> 3) & 1;
-    double my_coef = 0.0;
-    if (cj == 0) my_coef = ch ? pc.ad0 : pc.au0;
-    if (cj == 1) my_coef = pr->kx;
-    if (cj == 2) my_coef = pr->ky;
-    if (cj == 3) my_coef = fs->cAx;
-    if (cj == 4) my_coef = fs->cAy;
-    if (cj == 5) my_coef = i >= 2 ? pc.e : 0.0;
-    const int my_xe = cj == 6 ? (HAS_V && Vp ? pr->vbe : 0) : fx::exp_field(my_coef);
-    bool bad = __any_sync(0xffffffffu, my_xe == 0x7ff);
-
-    // q^_i at a site, and q^_{i-1} there (zero if i = 1)
-    auto load = [&](size_t idx, double (&q)[4], double (&qp)[4]) {
-      cvt4(ld4<COOP>(qsrc + idx), qp);
-      if (i == 1) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) { q[c] = qp[c]; qp[c] = 0.0; }
-      } else {
-        double yv[4];
-        cvt4(ld4<COOP>(yprev + idx), yv);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) q[c] = fma(-gd, qp[c], yv[c]);
-      }
-    };
-    // the same at grid point (gx, gy), wrapped, or zero outside for Dirichlet
-    auto form = [&](int gx, int gy, double (&q)[4], double (&qp)[4]) {
-      bool ox, oy;
-      const int ix = wrap<DIRI>(gx, nx, ox), iy = wrap<DIRI>(gy, ny, oy);
-      q[0] = q[1] = q[2] = q[3] = 0.0;
-      qp[0] = qp[1] = qp[2] = qp[3] = 0.0;
-      if (ox || oy) return;
-      load((size_t)iy * nx + ix, q, qp);
-    };
-    auto mag = [](double x) { return (unsigned)__double2hiint(x) << 1; };   // orders by |x| (to 20 bits)
-
-    // lane 0-5 of each warp: P, Y, X of the upper, then of the lower components
-    double acc = 0.0;
-    for (int tt = t + sub; tt < seg_end; tt += SUB) {
-      const int lt = tt - pr->tile_begin;
-      const int x0 = (lt % pr->tiles_x) * TILE_W;
-      const int y0 = (lt / pr->tiles_x) * TH;
-      const int r0 = tg * RPT;                  // this thread's rows of the tile
-      const bool full = x0 + TILE_W <= nx && y0 + TH <= ny;
-      const bool in_x = x0 + tx < nx;
-      const int rows_in = in_x ? ny - (y0 + r0) : 0;              // row k is in the grid if k < rows_in
-      const size_t idx0 = (size_t)(y0 + r0) * nx + (x0 + tx);     // row 0 (used where in the grid)
-      double q[RPT][4], qp[RPT][4], hq[4];
-      int hat = 0;                              // the halo site's place in the tile
-      if (full) {
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) load(idx0 + (size_t)k * nx, q[k], qp[k]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) form(x0 + tx, y0 + r0 + k, q[k], qp[k]);
-      }
-      if (ltid < NH) {
-        int hrow, hcol;
-        if (ltid < NH_ROW) {                    // rows above / below
-          const int r = ltid / TILE_W;
-          hrow = (r < R) ? r : TH + r;
-          hcol = (ltid % TILE_W) + R;
-        } else {                                // columns left / right
-          const int h2 = ltid - NH_ROW;
-          hrow = h2 / (2 * R) + R;
-          const int c = h2 % (2 * R);
-          hcol = (c < R) ? c : TILE_W + c;
-        }
-        hat = hrow * W + hcol;
-        double unused[4];
-        form(x0 + hcol - R, y0 + hrow - R, hq, unused);
-      } else {
-        hq[0] = hq[1] = hq[2] = hq[3] = 0.0;
-      }
-      // the largest numbers of the tile
-      unsigned m0 = max(mag(hq[0]), mag(hq[1])), m1 = max(mag(hq[2]), mag(hq[3])), m2 = 0u, m3 = 0u;
-#pragma unroll
-      for (int k = 0; k < RPT; ++k) {
-        m0 = max(m0, max(mag(q[k][0]), mag(q[k][1])));
-        m1 = max(m1, max(mag(q[k][2]), mag(q[k][3])));
-        m2 = max(m2, max(mag(qp[k][0]), mag(qp[k][1])));
-        m3 = max(m3, max(mag(qp[k][2]), mag(qp[k][3])));
-      }
-      m0 = __reduce_max_sync(0xffffffffu, m0);
-      m1 = __reduce_max_sync(0xffffffffu, m1);
-      m2 = __reduce_max_sync(0xffffffffu, m2);
-      m3 = __reduce_max_sync(0xffffffffu, m3);
-      if (lane < 4) atomicMax(emax + 4 * par + lane, lane == 0 ? m0 : lane == 1 ? m1 : lane == 2 ? m2 : m3);
-      if (q_out) {
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-          if (k < rows_in) {
-            vec4 o;
-            o.x = q[k][0]; o.y = q[k][1]; o.z = q[k][2]; o.w = q[k][3];
-            q_out[idx0 + (size_t)k * nx] = o;
-          }
-        }
-      }
-      sub_sync();   // the exponents are complete, and the previous tile has been read
-      // exponents of 128 and below (numbers under 2^-894) count as zero
-      const int be_u = max((int)(emax[4 * par] >> 21), 128), be_d = max((int)(emax[4 * par + 1] >> 21), 128);
-      const int be_pu = max((int)(emax[4 * par + 2] >> 21), 128), be_pd = max((int)(emax[4 * par + 3] >> 21), 128);
-      bad = bad || be_u == 0x7ff || be_d == 0x7ff || be_pu == 0x7ff || be_pd == 0x7ff;
-      if (ltid < 4) emax[4 * (par ^ 1) + ltid] = 0u;
-      par ^= 1;
-      const int at0 = (r0 + R) * W + tx + R;    // this thread's first site in the tile
-#pragma unroll
-      for (int k = 0; k < RPT; ++k) {
-        // sites beyond the grid's edge are halo of the sites inside, but not summed
-        half_u[at0 + k * W] = make_longlong2(fx::to_fixed<F>(q[k][0], be_u), fx::to_fixed<F>(q[k][1], be_u));
-        half_d[at0 + k * W] = make_longlong2(fx::to_fixed<F>(q[k][2], be_d), fx::to_fixed<F>(q[k][3], be_d));
-      }
-      if (ltid < NH) {
-        half_u[hat] = make_longlong2(fx::to_fixed<F>(hq[0], be_u), fx::to_fixed<F>(hq[1], be_u));
-        half_d[hat] = make_longlong2(fx::to_fixed<F>(hq[2], be_d), fx::to_fixed<F>(hq[3], be_d));
-      }
-      {
-        // this warp's coefficient table: row scale = the largest term's, the
-        // coefficients of a row as 60-bit fractions of it
-        const int be_own = ch ? be_d : be_u, be_oth = ch ? be_u : be_d, be_p = ch ? be_pd : be_pu;
-        const int be_x = (cj == 0 || cj == 6) ? be_own : (cj == 5 ? be_p : be_oth);
-        int sc = my_xe ? my_xe + be_x : 0;
-        sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 1));
-        sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 2));
-        sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 4));
-        if (lane < COEF_SLOTS) {
-          const fx::Limbs l = fx::split(fx::to_fixed<60>(my_coef, max(sc - be_x, 63)));
-          kt[lane] = cj == 7 ? make_int2(sc, 0) : make_int2(l.hi, l.lo);
-        }
-      }
-      sub_sync();   // tile and coefficients are in shared memory
-
-      fx::WarpSum ws[6];
-      int we[6];
-      auto half = [&](auto half_c) {
-        constexpr int HALF = decltype(half_c)::value;
-        const longlong2* const own = (HALF ? half_d : half_u) + at0;
-        const longlong2* const oth = (HALF ? half_u : half_d) + at0;
-        const int2* const kc = kt + 8 * HALF;
-        auto coef = [&](int j) { const int2 v = kc[j]; return fx::Limbs{v.x, v.y}; };
-        const int sc = kc[7].x;
-        const int be_own = HALF ? be_d : be_u, be_p = HALF ? be_pd : be_pu;
-        const int se = sc - 2044;                       // the row's scale: |terms| < 2^se
-        const int texp = se - F + yexp;                 // unit of y as stored
-        const bool live = texp >= -1022;                // else below the normal range: zero
-        // columns of the other half: rows r0 - R .. r0 + RPT + R - 1
-        longlong2 col[RPT + 2 * R];
-#pragma unroll
-        for (int j = 0; j < RPT + 2 * R; ++j) col[j] = oth[(j - R) * W];
-        long long v[RPT][2];
-        unsigned vor = 0u;                              // the upper words of all |v|, or-ed
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-          const longlong2* const row = oth + k * W;
-          // differences along x of (re, im), and along y
-          const longlong2 xl = row[-1], xr = row[1];
-          long long hxr = xl.x - xr.x, hxi = xr.y - xl.y;          // -D_x re, D_x im
-          long long hyr = col[k + R + 1].x - col[k + R - 1].x, hyi = col[k + R + 1].y - col[k + R - 1].y;
-          if constexpr (R == 2) {
-            const longlong2 xl2 = row[-2], xr2 = row[2];
-            hxr = 8 * hxr - (xl2.x - xr2.x);
-            hxi = 8 * hxi - (xr2.y - xl2.y);
-            hyr = 8 * hyr - (col[k + 2 * R].x - col[k].x);
-            hyi = 8 * hyi - (col[k + 2 * R].y - col[k].y);
-          }
-          // upper: (mc^2+V-s-sigma) u + c[-i D_x d - D_y d + (A_x - i A_y) d]
-          // lower: (-mc^2+V-s-sigma) d + c[-i D_x u + D_y u + (A_x + i A_y) u]
-          const longlong2 cv = own[k * W];
-          const fx::Limbs c0 = fx::split(cv.x), c1 = fx::split(cv.y);
-          fx::Acc s0, s1;
-          {
-            const fx::Limbs ka = coef(0);
-            s0.mac(c0, ka);
-            s1.mac(c1, ka);
-          }
-          if constexpr (ISO) {
-            const fx::Limbs kx = coef(1);
-            s0.mac(fx::split(HALF ? hxi + hyr : hxi - hyr), kx);
-            s1.mac(fx::split(HALF ? hxr + hyi : hxr - hyi), kx);
-          } else {
-            const fx::Limbs kx = coef(1), ky = coef(2);
-            s0.mac(fx::split(hxi), kx);
-            s1.mac(fx::split(hxr), kx);
-            s0.mac(fx::split(HALF ? hyr : -hyr), ky);
-            s1.mac(fx::split(HALF ? hyi : -hyi), ky);
-          }
-          if (has_ax) {
-            const fx::Limbs kax = coef(3);
-            s0.mac(fx::split(col[k + R].x), kax);
-            s1.mac(fx::split(col[k + R].y), kax);
-          }
-          if (has_ay) {
-            const fx::Limbs kay = coef(4);
-            s0.mac(fx::split(HALF ? -col[k + R].y : col[k + R].y), kay);
-            s1.mac(fx::split(HALF ? col[k + R].x : -col[k + R].x), kay);
-          }
-          if (i >= 2) {
-            const fx::Limbs ke = coef(5);
-            s0.mac(fx::split(-fx::to_fixed<F>(qp[k][2 * HALF], be_p)), ke);
-            s1.mac(fx::split(-fx::to_fixed<F>(qp[k][2 * HALF + 1], be_p)), ke);
-          }
-          if constexpr (HAS_V) {
-            if (Vp) {
-              const double pot = k < rows_in ? Vp[idx0 + (size_t)k * nx] : 0.0;
-              const fx::Limbs kv = fx::split(fx::to_fixed<60>(pot, max(sc - be_own, 63)));
-              s0.mac(c0, kv);
-              s1.mac(c1, kv);
-            }
-          }
-          v[k][0] = s0.template value<28>();
-          v[k][1] = s1.template value<28>();
-          if (!full && k >= rows_in) v[k][0] = v[k][1] = 0;
-          vor |= (unsigned)((v[k][0] ^ (v[k][0] >> 63)) >> 32) | (unsigned)((v[k][1] ^ (v[k][1] >> 63)) >> 32);
-          if (y_out && k < rows_in) {
-            // components of this half (16 of the site's 32 bytes)
-            double2* const yo = reinterpret_cast<double2*>(y_out + idx0 + (size_t)k * nx) + HALF;
-            *yo = live ? make_double2(fx::to_double(v[k][0], texp), fx::to_double(v[k][1], texp))
-                       : make_double2(0.0, 0.0);
-          }
-        }
-        // the sums: y^ as 60 bits of the warp's largest number (the terms of a
-        // row may cancel by many bits), q^ as it is
-        const int sl = __clz((int)__reduce_or_sync(0xffffffffu, vor)) - 2;   // 0 .. 30
-        fx::Acc aP;
-        fx::SqAcc aY, aX;
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-          longlong2 cv = own[k * W];
-          if (!full && k >= rows_in) cv.x = cv.y = 0;
-          const fx::Limbs c0 = fx::split(cv.x << (58 - F)), c1 = fx::split(cv.y << (58 - F));
-          const fx::Limbs w0 = fx::split((v[k][0] << sl) >> 2), w1 = fx::split((v[k][1] << sl) >> 2);
-          aP.mac(c0, w0);
-          aP.mac(c1, w1);
-          aY.sqr(w0);
-          aY.sqr(w1);
-          aX.sqr(c0);
-          aX.sqr(c1);
-        }
-        // |q^| < 2^58 and |w| < 2^60: eight terms of q^ w stay below 2^61 in
-        // units of 2^60, of w^2 below 2^63, of q^2 below 2^59
-        const int qe = be_own - 1022 - 58, ye = texp + 2 - sl;
-        ws[3 * HALF] = fx::warp_sum(aP.template value<28>());
-        ws[3 * HALF + 1] = fx::warp_sum(aY.value());
-        ws[3 * HALF + 2] = fx::warp_sum(aX.value());
-        we[3 * HALF] = qe + ye + 60;
-        we[3 * HALF + 1] = 2 * ye + 60;
-        we[3 * HALF + 2] = 2 * qe + 60;
-      };
-      half(std::integral_constant<int, 0>{});
-      half(std::integral_constant<int, 1>{});
-      // one conversion for all six sums: each by its lane
-      fx::WarpSum mine = ws[0];
-      int me = we[0];
-#pragma unroll
-      for (int j = 1; j < 6; ++j) {
-        if (lane == j) { mine = ws[j]; me = we[j]; }
-      }
-      acc += scalbn(fx::to_double(mine), me);
-    }
-    t = seg_end;
-    double accP = acc + __shfl_down_sync(0xffffffffu, acc, 3);
-    const double accY = __shfl_sync(0xffffffffu, accP, 1), accX = __shfl_sync(0xffffffffu, accP, 2);
-    if (bad) accP = __longlong_as_double(0x7ff8000000000000LL);   // not finite: reported by finish_pass
-    if (lane == 0) { red[warp][0] = accP; red[warp][1] = accY; red[warp][2] = accX; }
-    pass_sums<true, COOP, NW>(lp, pr, i, seg_tiles, red, &last_flag, coop_slots);
-  }
-}
-
-// threads of a pass kernel (S = double: all tile workers of the CTA)
-template <class S, int TH>
-__host__ __device__ constexpr int pass_threads() { return sub_workers<S>() * 32 * (TH / rows_per_thread<S, TH>()); }
-
-// FLAG: kx = ky (S = double); not used by S = float
-template <class S, int R, int TH, bool DIRI, bool HAS_V, bool FLAG>
-__global__ void __launch_bounds__(pass_threads<S, TH>(), sizeof(S) == sizeof(float) ? min_blocks<TH>() : 1)
+template <class S, int R, int TH, bool DIRI, bool HAS_V, bool HAS_AY>
+__global__ void __launch_bounds__(sub_workers<S>() * 32 * (TH / rows_per_thread<S, TH>()),
+                                  (min_blocks<S, TH, sub_workers<S>()>()))
 lanczos_pass(const __grid_constant__ LaunchParams lp) {
   // programmatic dependent launch: nothing the previous kernel wrote is read
   // before this point
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if constexpr (sizeof(S) == sizeof(float))
-    pass_body<R, TH, DIRI, HAS_V>(lp, *lp.step);
-  else
-    pass_body_fx<R, TH, DIRI, HAS_V, FLAG, false, sub_workers<S>()>(lp, nullptr, nullptr, *lp.step);
+  pass_body<S, R, TH, DIRI, HAS_V, HAS_AY, false, sub_workers<S>()>(lp, nullptr, nullptr, *lp.step);
   // the next kernel may be scheduled now (it waits for our completion)
   asm volatile("griddepcontrol.launch_dependents;");
 }
@@ -1339,93 +995,55 @@ __device__ __forceinline__ void recombine_site_df(vec4* psi, const float4* basis
 
 // ---------------------------------------------------------------------------
 // psi <- sum_j C_j q^_j (Eq. 17), q^_1 = psi, q^_j = basis[j-2] for j >= 2.
-// Mixed path: the basis is complex64; C_1 psi is formed in FP64 so that the
-// FP32 rounding of the basis only enters the (small) Krylov corrections, and
-// those are summed with compensation (recombine_site_df): plain FP32
-// accumulation of the corrections was the largest error of the mixed path on
-// fast packets.
-//
-// FP64 path: complex128 fields, the sums in fixed point (dirac_fixed.cuh): in
-// FP64 the 16 multiply-adds per site and vector took 1024 cycles of a
-// sub-partition against the 190 that reading the vector takes; in limbs they
-// take about as long as the read.  Each site has its own scale, that of its
-// largest |C_j q^_j| so far (the sums are shifted when a batch of D vectors
-// raises it), so the relative error of every site is about 2^-54 of its
-// largest term.
+// FP64 path: complex128 throughout.  Mixed path: the basis is complex64;
+// C_1 psi is formed in FP64 so that the FP32 rounding of the basis only
+// enters the (small) Krylov corrections, and those are summed with
+// compensation (recombine_site_df): plain FP32 accumulation of the
+// corrections was the largest error of the mixed path on fast packets.
 // Blocks are dealt to problems in proportion to their size.
 // ---------------------------------------------------------------------------
-struct FxCoef {
-  fx::Limbs re, im, mim;   // C_j and -Im C_j as 59-bit fractions of 2^(be - 1022)
-  int be;
-};
-__device__ __forceinline__ FxCoef fx_coef(double re, double im) {
-  FxCoef c;
-  c.be = max(fx::exp_field(re), fx::exp_field(im));
-  const long long i = fx::to_fixed<59>(im, max(c.be, 63));
-  c.re = fx::split(fx::to_fixed<59>(re, max(c.be, 63)));
-  c.im = fx::split(i);
-  c.mim = fx::split(-i);
-  return c;
-}
-
-template <int D>
-__device__ __forceinline__ void recombine_site_fx(vec4* psi, const vec4* basis, size_t n, size_t s, int k,
-                                                  const FxCoef* coef) {
-  // factors below 2^59: 8 products in x stay below 2^62, all 64 below 2^62 in
-  // units of 2^62
-  static_assert(D % 4 == 0 && 2 * KMAX <= 64, "bounds of the sums");
-  long long sum[4] = {0, 0, 0, 0};
-  int be = 1100;   // exponent sum of the largest term (terms below 2^-938 count as zero)
-  for (int j0 = 1; j0 <= k; j0 += D) {
-    vec4 v[D];
-#pragma unroll
-    for (int u = 0; u < D; ++u) {
-      const int j = j0 + u;
-      if (j <= k) v[u] = j == 1 ? psi[s] : basis[(size_t)(j - 2) * n + s];
+template <bool MIXED>
+__device__ __forceinline__ void recombine_site(vec4* psi, const void* basis_v, long long n, long long s, int k,
+                                               const double* cr, const double* ci, const float* fr,
+                                               const float* fi) {
+  if constexpr (!MIXED) {
+    const vec4* basis = static_cast<const vec4*>(basis_v);
+    const vec4 q = psi[s];
+    double ur = cr[1] * q.x - ci[1] * q.y, ui = cr[1] * q.y + ci[1] * q.x;
+    double dr = cr[1] * q.z - ci[1] * q.w, di = cr[1] * q.w + ci[1] * q.z;
+    for (int j = 2; j <= k; ++j) {
+      const vec4* vp = basis + (size_t)(j - 2) * n + s;
+      const vec4 v = *vp;
+      const double a = cr[j], bb = ci[j];
+      ur = fma(a, v.x, fma(-bb, v.y, ur));
+      ui = fma(a, v.y, fma(bb, v.x, ui));
+      dr = fma(a, v.z, fma(-bb, v.w, dr));
+      di = fma(a, v.w, fma(bb, v.z, di));
     }
-    int nb = be;
-#pragma unroll
-    for (int u = 0; u < D; ++u) {
-      if (j0 + u <= k) {
-        const unsigned a = max((unsigned)__double2hiint(v[u].x) << 1, (unsigned)__double2hiint(v[u].y) << 1);
-        const unsigned b = max((unsigned)__double2hiint(v[u].z) << 1, (unsigned)__double2hiint(v[u].w) << 1);
-        nb = max(nb, (int)(max(a, b) >> 21) + coef[j0 + u].be);
-      }
+    vec4 o;
+    o.x = ur; o.y = ui; o.z = dr; o.w = di;
+    psi[s] = o;
+  } else {
+    const float4* basis = static_cast<const float4*>(basis_v);
+    const double ar = cr[1], ai = ci[1];
+    float ur = 0.f, ui = 0.f, dr = 0.f, di = 0.f;
+    for (int j = 2; j <= k; ++j) {
+      const float4* vp = basis + (size_t)(j - 2) * n + s;
+      const float4 v = *vp;
+      const float a = fr[j], bb = fi[j];
+      ur = fmaf(a, v.x, fmaf(-bb, v.y, ur));
+      ui = fmaf(a, v.y, fmaf(bb, v.x, ui));
+      dr = fmaf(a, v.z, fmaf(-bb, v.w, dr));
+      di = fmaf(a, v.w, fmaf(bb, v.z, di));
     }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) sum[c] = fx::shr_round(sum[c], nb - be);
-    be = nb;
-#pragma unroll
-    for (int g = 0; g < D; g += 4) {
-      fx::Acc acc[4];
-#pragma unroll
-      for (int u = g; u < g + 4; ++u) {
-        if (j0 + u <= k) {
-          const FxCoef cf = coef[j0 + u];
-          const int bq = max(be - cf.be, 63);
-          const fx::Limbs x = fx::split(fx::to_fixed<59>(v[u].x, bq)), y = fx::split(fx::to_fixed<59>(v[u].y, bq));
-          const fx::Limbs z = fx::split(fx::to_fixed<59>(v[u].z, bq)), w = fx::split(fx::to_fixed<59>(v[u].w, bq));
-          acc[0].mac(x, cf.re);
-          acc[0].mac(y, cf.mim);
-          acc[1].mac(y, cf.re);
-          acc[1].mac(x, cf.im);
-          acc[2].mac(z, cf.re);
-          acc[2].mac(w, cf.mim);
-          acc[3].mac(w, cf.re);
-          acc[3].mac(z, cf.im);
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) sum[c] += acc[c].template value<30>();
-    }
+    const vec4 q = psi[s];
+    vec4 o;
+    o.x = fma(ar, q.x, fma(-ai, q.y, (double)ur));
+    o.y = fma(ar, q.y, fma(ai, q.x, (double)ui));
+    o.z = fma(ar, q.z, fma(-ai, q.w, (double)dr));
+    o.w = fma(ar, q.w, fma(ai, q.z, (double)di));
+    psi[s] = o;
   }
-  const int e = be - 2044 - 56;   // 2^62 of the products' 2^-118
-  vec4 o;
-  o.x = fx::to_double(sum[0], e);
-  o.y = fx::to_double(sum[1], e);
-  o.z = fx::to_double(sum[2], e);
-  o.w = fx::to_double(sum[3], e);
-  psi[s] = o;
 }
 
 // Three CTAs per SM (at most 85 registers), so that enough warps keep loads
@@ -1433,10 +1051,8 @@ __device__ __forceinline__ void recombine_site_fx(vec4* psi, const vec4* basis, 
 template <bool MIXED>
 __global__ void __launch_bounds__(256, 3) recombine(const __grid_constant__ RecombParams rp) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  __shared__ double cr[MIXED ? KMAX + 2 : 1], ci[MIXED ? KMAX + 2 : 1];
-  __shared__ float fr[MIXED ? KMAX + 2 : 1], fi[MIXED ? KMAX + 2 : 1];
-  __shared__ float frl[MIXED ? KMAX + 2 : 1], fil[MIXED ? KMAX + 2 : 1];
-  __shared__ FxCoef fc[MIXED ? 1 : KMAX + 2];
+  __shared__ double cr[KMAX + 2], ci[KMAX + 2];
+  __shared__ float fr[KMAX + 2], fi[KMAX + 2], frl[KMAX + 2], fil[KMAX + 2];
   __shared__ int k_s, err_s;
   const int b = rp.blk_prob[blockIdx.x];
   const Problem* pr = rp.probs + b;
@@ -1444,16 +1060,12 @@ __global__ void __launch_bounds__(256, 3) recombine(const __grid_constant__ Reco
   if (threadIdx.x == 0) { k_s = st->k_used; err_s = st->error; }
   if (threadIdx.x <= KMAX) {
     const double a = st->coef_re[threadIdx.x], c = st->coef_im[threadIdx.x];
-    if constexpr (MIXED) {
-      cr[threadIdx.x] = a;
-      ci[threadIdx.x] = c;
-      fr[threadIdx.x] = (float)a;
-      fi[threadIdx.x] = (float)c;
-      frl[threadIdx.x] = (float)(a - (double)fr[threadIdx.x]);
-      fil[threadIdx.x] = (float)(c - (double)fi[threadIdx.x]);
-    } else {
-      fc[threadIdx.x] = fx_coef(a, c);
-    }
+    cr[threadIdx.x] = a;
+    ci[threadIdx.x] = c;
+    fr[threadIdx.x] = (float)a;
+    fi[threadIdx.x] = (float)c;
+    frl[threadIdx.x] = (float)(a - (double)fr[threadIdx.x]);
+    fil[threadIdx.x] = (float)(c - (double)fi[threadIdx.x]);
   }
   __syncthreads();
   const int lb = blockIdx.x - pr->rblk_begin;
@@ -1473,7 +1085,7 @@ __global__ void __launch_bounds__(256, 3) recombine(const __grid_constant__ Reco
       recombine_site_df<8>(psi, static_cast<const float4*>(pr->basis), (size_t)n, (size_t)s, k, cr, ci, fr, frl,
                            fi, fil);
     else
-      recombine_site_fx<4>(psi, static_cast<const vec4*>(pr->basis), (size_t)n, (size_t)s, k, fc);
+      recombine_site<false>(psi, pr->basis, n, s, k, cr, ci, fr, fi);
   }
   asm volatile("griddepcontrol.launch_dependents;");
 }
@@ -1498,6 +1110,7 @@ struct CoopArgs {
   int G;           // CTAs of the launch
   int cap;         // CTAs the slot buffer holds
   int bar_count;   // CTAs each grid barrier waits for: G (G + 1 only in the timeout test)
+  unsigned long long* packets;   // lanczos_step64: 2 x 6 x cap words by pass parity, zeroed before each launch
 };
 
 // Barrier of all CTAs of a cooperative launch.  Thread 0 of each CTA arrives
@@ -1536,13 +1149,15 @@ __device__ __forceinline__ bool grid_sync(unsigned* bar, unsigned G) {
   return ok_s != 0;
 }
 
-template <int R, int TH, bool DIRI, bool HAS_V, bool ISO>
-__global__ void __launch_bounds__(pass_threads<double, TH>(), 1)
+template <class S, int R, int TH, bool DIRI, bool HAS_V, bool HAS_AY>
+__global__ void __launch_bounds__(step_workers<S, TH>() * 32 * (TH / rows_per_thread<S, TH>()), 1)
 lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ CoopArgs ca) {
-  constexpr int SUB = sub_workers<double>();
-  constexpr int NT = pass_threads<double, TH>();
+  constexpr bool F32 = sizeof(S) == sizeof(float);
+  constexpr int SUB = step_workers<S, TH>();
+  constexpr int NT = SUB * 32 * (TH / rows_per_thread<S, TH>());
   __shared__ DevState sst;
-  __shared__ FxCoef fc_s[KMAX + 2];
+  __shared__ double cr_s[KMAX + 2], ci_s[KMAX + 2];
+  __shared__ float fr_s[KMAX + 2], fi_s[KMAX + 2];
   const Problem* pr = lp.probs;
   DevState* gst = lp.states;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1558,7 +1173,7 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
   while (!sst.stopped && iter < max_iter) {
     const int i = max(1, sst.cur_pass);
     double* slots = ca.slots + (iter & 1) * 3 * ca.G;
-    pass_body_fx<R, TH, DIRI, HAS_V, ISO, true, SUB>(lp, &sst, slots, step);
+    pass_body<S, R, TH, DIRI, HAS_V, HAS_AY, true, SUB>(lp, &sst, slots, step);
     ++iter;
     if (!grid_sync(ca.bar, (unsigned)ca.bar_count)) {
       if (threadIdx.x == 0) { gst->error = ERR_BARRIER; gst->stopped = 1; }
@@ -1583,19 +1198,24 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
       t0 = warp_sum(t0);
       t1 = warp_sum(t1);
       t2 = warp_sum(t2);
-      finish_pass<true>(lp, pr, &sst, i, t0, t1, t2);
+      finish_pass<false>(lp, pr, &sst, i, t0, t1, t2);
     }
     __syncthreads();
   }
   const int err = sst.error;
   if (!err) {
     // psi <- sum_j C_j q^_j on this CTA's tiles (no CTA reads psi any more)
-    if (threadIdx.x <= KMAX) fc_s[threadIdx.x] = fx_coef(sst.coef_re[threadIdx.x], sst.coef_im[threadIdx.x]);
+    if (threadIdx.x <= KMAX) {
+      cr_s[threadIdx.x] = sst.coef_re[threadIdx.x];
+      ci_s[threadIdx.x] = sst.coef_im[threadIdx.x];
+      fr_s[threadIdx.x] = (float)cr_s[threadIdx.x];
+      fi_s[threadIdx.x] = (float)ci_s[threadIdx.x];
+    }
     __syncthreads();
     const int cq = lp.chunk_q, cr = lp.chunk_r;
     const int t_begin = blockIdx.x * cq + min((int)blockIdx.x, cr);
     const int t_end = t_begin + cq + ((int)blockIdx.x < cr ? 1 : 0);
-    const size_t n = (size_t)pr->nx * pr->ny;
+    const long long n = (long long)pr->nx * pr->ny;
     const int k = sst.k_used;
     vec4* psi = const_cast<vec4*>(pr->psi);
     for (int tt = t_begin; tt < t_end; ++tt) {
@@ -1603,7 +1223,7 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
       for (int e = threadIdx.x; e < TILE_W * TH; e += NT) {
         const int x = x0 + (e & (TILE_W - 1)), y = y0 + e / TILE_W;
         if (x < pr->nx && y < pr->ny)
-          recombine_site_fx<8>(psi, static_cast<const vec4*>(pr->basis), n, (size_t)y * pr->nx + x, k, fc_s);
+          recombine_site<F32>(psi, pr->basis, n, (long long)y * pr->nx + x, k, cr_s, ci_s, fr_s, fi_s);
       }
     }
   }
