@@ -27,6 +27,7 @@
 // within clusters of close values); T_k is scaled by a power of two so that
 // the characteristic-polynomial recurrence stays in range.
 #include "dirac.h"
+#include "dirac_fixed.cuh"
 #include "dirac_internal.h"
 
 #include <cuda_runtime.h>
@@ -46,7 +47,7 @@ using v4 = double4_32a;   // one site: (u.re, u.im, d.re, d.im)
 
 constexpr int RITZ_CAP = DIRAC_EIG_RITZ_MAX;   // Ritz values examined per check
 constexpr int MAX_ITER = DIRAC_EIG_ITER_MAX;
-constexpr int CH_MAX = 1024;                   // sites per dot-kernel chunk
+constexpr int CH_MAX = 256;                    // sites per dot-kernel chunk
 constexpr double BREAKDOWN_REL = 1e-12;
 
 struct EigDev {
@@ -74,6 +75,24 @@ __device__ __forceinline__ double wsum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+
+// Largest |x| of a vector, by the upper 31 bits of its numbers (their exponent
+// and 20 bits): max over a block, then one atomic
+__device__ __forceinline__ unsigned mag(double x) { return (unsigned)__double2hiint(x) << 1; }
+__device__ __forceinline__ unsigned mag4(const v4& v) { return max(max(mag(v.x), mag(v.y)), max(mag(v.z), mag(v.w))); }
+__device__ void block_max(unsigned m, unsigned* out) {
+  __shared__ unsigned red[32];
+  m = __reduce_max_sync(0xffffffffu, m);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) red[warp] = m;
+  __syncthreads();
+  if (warp == 0) {
+    m = __reduce_max_sync(0xffffffffu, lane < (int)(blockDim.x >> 5) ? red[lane] : 0u);
+    if (lane == 0) atomicMax(out, m);
+  }
+}
+// exponent field of a recorded maximum (192 and below count as zero)
+__device__ __forceinline__ int max_field(unsigned m) { return max((int)(m >> 21), 192); }
 
 __device__ __forceinline__ double wmax(double v) {
 #pragma unroll
@@ -106,6 +125,7 @@ struct ApplyArgs {
   double* s;
   int iter;
   int prologue;         // 1: s_i and beta_{i-1} from norm_part, breakdown test, scale by s_i
+  unsigned* vmax;       // largest number of `out` (or null)
 };
 
 template <bool DIRI, class T>
@@ -166,9 +186,10 @@ __global__ void __launch_bounds__(256) eig_apply(const ApplyArgs a) {
       csub = a.beta[i - 1] * a.s[i - 1];
     }
   }
-  const int x = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
-  if (x >= a.nx || y >= a.ny) return;
+  // threads beyond the grid's edge repeat its last site and store nothing
+  const int xt = blockIdx.x * 32 + (threadIdx.x & 31), yt = blockIdx.y * 8 + (threadIdx.x >> 5);
+  const bool valid = xt < a.nx && yt < a.ny;
+  const int x = min(xt, a.nx - 1), y = min(yt, a.ny - 1);
   const int nx = a.nx, ny = a.ny;
   T C[4], xp[4], xm[4], yp[4], ym[4], dxv[4], dyv[4];
   double C64[4];
@@ -221,62 +242,150 @@ __global__ void __launch_bounds__(256) eig_apply(const ApplyArgs a) {
   } else {
     r.x = s_in * o[0]; r.y = s_in * o[1]; r.z = s_in * o[2]; r.w = s_in * o[3];
   }
-  a.out[idx] = r;
+  if (valid) a.out[idx] = r;
+  if (a.vmax) block_max(valid ? mag4(r) : 0u, a.vmax);
 }
 
 // ---------------------------------------------------------------------------
-// h_j = <q^_j, z> for j = j0..j1: per-CTA partials, z chunk staged in shared
-// memory, one warp per basis vector at a time
+// h_j = <q^_j, z> for j = j0..j1, and ||z||^2 (z is the basis slot after j1):
+// per-CTA partials, the z chunk staged in shared memory, one warp per vector at
+// a time.
+//
+// The products are 58-bit fixed point (dirac_fixed.cuh), each vector relative to
+// its own largest number: in FP64 the eight multiply-adds per site and vector
+// occupied a sub-partition for 512 cycles, against the 190 in which its share of
+// the memory bandwidth delivers the vector; conversion and limb products take
+// 270.  Sums are exact to 2^-56 of the largest product per four sites, then
+// integers over the chunk and FP64 from chunk to chunk.  The FP64 pipe takes
+// every third vector meanwhile, at FP64_SHARE's cost ratio.
 // ---------------------------------------------------------------------------
+constexpr int FP64_SHARE = 3;   // one vector in so many goes to the FP64 pipe
+
 struct DotArgs {
-  const v4* z;
   const v4* basis;
   long long n;
-  int j0, j1;
+  int j0, j1;           // z is slot j1 + 1
   int cs;               // sites per chunk (multiple of 32, <= CH_MAX)
-  double2* part;        // [j - j0][CTA]
+  double2* part;        // [j - j0][CTA], the last row ||z||^2
+  const unsigned* vmax; // largest numbers: [3 slot + stage]
+  int stage;            // of z: 0 after the product, 1 after the first update
   const EigDev* ed;
 };
 
-__global__ void __launch_bounds__(256) eig_dot(const DotArgs a) {
+__global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
   extern __shared__ __align__(32) unsigned char smem[];
-  if (a.ed && (a.ed->breakdown | a.ed->error)) return;
-  v4* zc = reinterpret_cast<v4*>(smem);
-  double2* acc = reinterpret_cast<double2*>(smem + (size_t)a.cs * sizeof(v4));
-  const int count = a.j1 - a.j0 + 1;
+  if (a.ed->breakdown | a.ed->error) return;
+  int4* const zu = reinterpret_cast<int4*>(smem);       // limbs of (x, y), then of (z, w)
+  int4* const zd = zu + a.cs;
+  v4* const zf = reinterpret_cast<v4*>(zd + a.cs);
+  double2* acc = reinterpret_cast<double2*>(zf + a.cs);
+  const int count = a.j1 - a.j0 + 2;
   for (int t = threadIdx.x; t < count; t += blockDim.x) acc[t] = make_double2(0.0, 0.0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int zbe = max_field(a.vmax[3 * (a.j1 + 1) + a.stage]);
   const long long nchunks = (a.n + a.cs - 1) / a.cs;
+  const v4* const z = a.basis + (size_t)(a.j1 + 1) * a.n;
   for (long long ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
     const long long base = ch * a.cs;
     const int len = (int)min((long long)a.cs, a.n - base);
     __syncthreads();
-    for (int t = threadIdx.x; t < len; t += blockDim.x) zc[t] = a.z[base + t];
+    for (int t = threadIdx.x; t < a.cs; t += blockDim.x) {
+      v4 v;
+      v.x = v.y = v.z = v.w = 0.0;
+      if (t < len) v = z[base + t];
+      const fx::Limbs x = fx::split(fx::to_fixed<58>(v.x, zbe)), y = fx::split(fx::to_fixed<58>(v.y, zbe));
+      const fx::Limbs u = fx::split(fx::to_fixed<58>(v.z, zbe)), w = fx::split(fx::to_fixed<58>(v.w, zbe));
+      zu[t] = make_int4(x.hi, x.lo, y.hi, y.lo);
+      zd[t] = make_int4(u.hi, u.lo, w.hi, w.lo);
+      zf[t] = v;
+    }
     __syncthreads();
     for (int jj = warp; jj < count; jj += nw) {
       const v4* __restrict__ q = a.basis + (size_t)(a.j0 + jj) * a.n + base;
-      double re0 = 0.0, im0 = 0.0, re1 = 0.0, im1 = 0.0;
-      int t = lane;
-      for (; t + 32 < len; t += 64) {
-        const v4 qa = q[t], qb = q[t + 32];
-        const v4 za = zc[t], zb = zc[t + 32];
-        re0 = fma(qa.x, za.x, fma(qa.y, za.y, fma(qa.z, za.z, fma(qa.w, za.w, re0))));
-        im0 = fma(qa.x, za.y, fma(-qa.y, za.x, fma(qa.z, za.w, fma(-qa.w, za.z, im0))));
-        re1 = fma(qb.x, zb.x, fma(qb.y, zb.y, fma(qb.z, zb.z, fma(qb.w, zb.w, re1))));
-        im1 = fma(qb.x, zb.y, fma(-qb.y, zb.x, fma(qb.z, zb.w, fma(-qb.w, zb.z, im1))));
+      if ((jj / nw + warp) % FP64_SHARE == FP64_SHARE - 1) {
+        double re = 0.0, im = 0.0;
+        for (int t0 = 0; t0 < len; t0 += 128) {
+          v4 v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int t = t0 + 32 * u + lane;
+            v[u].x = v[u].y = v[u].z = v[u].w = 0.0;
+            if (t < len) v[u] = q[t];
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const v4 zz = zf[min(t0 + 32 * u + lane, a.cs - 1)];
+            re = fma(v[u].x, zz.x, fma(v[u].y, zz.y, fma(v[u].z, zz.z, fma(v[u].w, zz.w, re))));
+            im = fma(v[u].x, zz.y, fma(-v[u].y, zz.x, fma(v[u].z, zz.w, fma(-v[u].w, zz.z, im))));
+          }
+        }
+        // both sums over the warp with one addition per level: even lanes re, odd lanes im
+        double part = (lane & 1 ? im : re) + __shfl_xor_sync(0xffffffffu, lane & 1 ? re : im, 1);
+#pragma unroll
+        for (int o = 16; o > 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += part;
+        continue;
       }
-      if (t < len) {
-        const v4 qa = q[t], za = zc[t];
-        re0 = fma(qa.x, za.x, fma(qa.y, za.y, fma(qa.z, za.z, fma(qa.w, za.w, re0))));
-        im0 = fma(qa.x, za.y, fma(-qa.y, za.x, fma(qa.z, za.w, fma(-qa.w, za.z, im0))));
+      const int be = jj + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + jj) + 2]);
+      long long re = 0, im = 0;   // 64 products below 2^56 in units of 2^60
+      for (int t0 = 0; t0 < len; t0 += 128) {
+        v4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int t = t0 + 32 * u + lane;
+          v[u].x = v[u].y = v[u].z = v[u].w = 0.0;
+          if (t < len) v[u] = q[t];
+        }
+        fx::Acc ar, ai, am;       // at most 16 products each: cross terms below 2^62
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int t = t0 + 32 * u + lane;
+          const fx::Limbs x = fx::split(fx::to_fixed<58>(v[u].x, be)), y = fx::split(fx::to_fixed<58>(v[u].y, be));
+          const fx::Limbs z = fx::split(fx::to_fixed<58>(v[u].z, be)), w = fx::split(fx::to_fixed<58>(v[u].w, be));
+          const int4 s0 = zu[min(t, a.cs - 1)], s1 = zd[min(t, a.cs - 1)];   // (zero times it beyond the end)
+          const fx::Limbs zx{s0.x, s0.y}, zy{s0.z, s0.w}, zz{s1.x, s1.y}, zw{s1.z, s1.w};
+          ar.mac(x, zx);
+          ar.mac(y, zy);
+          ar.mac(z, zz);
+          ar.mac(w, zw);
+          ai.mac(x, zy);
+          ai.mac(z, zw);
+          am.mac(y, zx);
+          am.mac(w, zz);
+        }
+        re += ar.template value<28>();
+        im += ai.template value<28>() - am.template value<28>();
       }
-      const double re = wsum(re0 + re1), im = wsum(im0 + im1);
-      if (lane == 0) { acc[jj].x += re; acc[jj].y += im; }
+      const fx::WarpSum sr = fx::warp_sum(re), si = fx::warp_sum(im);
+      if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += fx::to_double(lane == 0 ? sr : si);
     }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < count; t += blockDim.x)
-    a.part[(size_t)t * gridDim.x + blockIdx.x] = acc[t];
+  for (int t = threadIdx.x; t < count; t += blockDim.x) {
+    // units: (2^(be - 1022 - 58)) (2^(zbe - 1022 - 58)) 2^60
+    const int be = t + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + t) + 2]);
+    const int e = (t / nw + t % nw) % FP64_SHARE == FP64_SHARE - 1 ? 0 : be + zbe - 2100;
+    a.part[(size_t)t * gridDim.x + blockIdx.x] = make_double2(fx::scale2(acc[t].x, e), fx::scale2(acc[t].y, e));
+  }
+}
+
+// <q, z> of one vector in FP64: per-CTA partials (the folded mode's Rayleigh quotients)
+__global__ void __launch_bounds__(256) eig_inner(const v4* q, const v4* z, long long n, double2* part) {
+  double re = 0.0;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += stride) {
+    const v4 a = q[t], b = z[t];
+    re = fma(a.x, b.x, fma(a.y, b.y, fma(a.z, b.z, fma(a.w, b.w, re))));
+  }
+  __shared__ double red[32];
+  re = wsum(re);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) red[warp] = re;
+  __syncthreads();
+  if (warp == 0) {
+    re = wsum(lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0);
+    if (lane == 0) part[blockIdx.x] = make_double2(re, 0.0);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -293,7 +402,15 @@ struct FinishArgs {
   const double* beta;
   EigDev* ed;
   double ashift;        // shift of A for the breakdown scale (s direct, 0 folded)
+  const unsigned* vmax;
+  int4* rec;            // update record of q^_j: see eig_update
 };
+
+// A coefficient of the update below this part of ||z|| (by |h_j|) is applied in
+// FP32: its products' rounding, 2^-24 of it, summed over at most 8192 vectors,
+// stays below 2^-53 ||z||.  After the first orthogonalisation, and for all but
+// the last one or two vectors before it, the coefficients are far smaller.
+constexpr double SMALL_COEF = 0x1p-36;
 
 __global__ void __launch_bounds__(256) eig_dot_finish(const FinishArgs a) {
   if (a.ed->breakdown | a.ed->error) return;
@@ -303,14 +420,26 @@ __global__ void __launch_bounds__(256) eig_dot_finish(const FinishArgs a) {
   double re = 0.0, im = 0.0;
   const double2* p = a.part + (size_t)jj * a.n_cta;
   for (int c = lane; c < a.n_cta; c += 32) { re += p[c].x; im += p[c].y; }
+  double zz = 0.0;   // ||z||^2, from the row after the last vector's
+  const double2* pz = a.part + (size_t)(a.j1 - a.j0 + 1) * a.n_cta;
+  for (int c = lane; c < a.n_cta; c += 32) zz += pz[c].x;
   re = wsum(re);
   im = wsum(im);
+  zz = wsum(zz);
   if (lane != 0) return;
   const int j = a.j0 + jj;
   const double sj = a.s[j];
   const double hr = sj * re;                      // h_j = <q_j, z>
   const double hi = a.reorth ? sj * im : 0.0;     // Fig. 1 removes alpha_i q_i, alpha real
   a.coef[jj] = make_double2(sj * hr, sj * hi);
+  {
+    const unsigned mz = a.vmax[3 * (a.j1 + 1) + a.pass], mq = a.vmax[3 * j + 2];
+    const int big = !(hr * hr + hi * hi <= SMALL_COEF * SMALL_COEF * zz);
+    const int de = max_field(mq) - max_field(mz);
+    a.rec[jj] = make_int4(__float_as_int((float)fx::scale2(sj * hr, de)), __float_as_int((float)fx::scale2(sj * hi, de)),
+                          max_field(mq), big);
+    if ((mz >> 21) == 0x7ffu || (mq >> 21) == 0x7ffu) a.ed->error = 1;   // not finite
+  }
   if (j == a.iter) {
     if (!isfinite(hr) || !isfinite(hi)) a.ed->error = 1;
     const double al = (a.pass == 0 ? 0.0 : a.alpha[j]) + hr;
@@ -324,7 +453,12 @@ __global__ void __launch_bounds__(256) eig_dot_finish(const FinishArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// z -= sum_j coef_j q^_j; with `last`, per-CTA partials of ||z||^2
+// z -= sum_j coef_j q^_j; with `last`, per-CTA partials of ||z||^2.  Vectors with
+// small coefficients (SMALL_COEF) are accumulated in FP32, as fractions of their
+// own largest number and of z's; the rest in FP64.  Eight FP64 multiply-adds per
+// site and vector took 512 cycles of a sub-partition against the 190 of the read.
+// Record of vector j: coefficient (re, im) as FP32 in units of z's largest number
+// over q^_j's, q^_j's exponent field, and 1 for FP64.
 // ---------------------------------------------------------------------------
 struct UpdArgs {
   v4* z;
@@ -332,10 +466,21 @@ struct UpdArgs {
   long long n;
   int j0, j1;
   const double2* coef;
+  const int4* rec;
   int last;
   double* norm_part;
+  const unsigned* zmax; // z's largest number before
+  unsigned* zmax_out;   // and after
   const EigDev* ed;
 };
+
+// x 2^-(be - 1022) as FP32 (below 1), truncated; zero below 2^-126
+__device__ __forceinline__ float to_fp32(double x, int be) {
+  const int hi = __double2hiint(x);
+  const unsigned t = __funnelshift_l((unsigned)__double2loint(x), (unsigned)hi, 3) - ((unsigned)(be - 126) << 23);
+  const bool tiny = (hi & 0x7ff00000) <= ((be - 126) << 20);
+  return __int_as_float(tiny ? 0 : (int)((t & 0x7fffffffu) | (hi & 0x80000000u)));
+}
 
 __device__ __forceinline__ void axpy_c(v4& z, double cr, double ci, const v4& q) {
   z.x = fma(-cr, q.x, fma(ci, q.y, z.x));
@@ -358,43 +503,66 @@ __device__ void block_partial(double v, double* out) {
 }
 
 __global__ void __launch_bounds__(256) eig_update(const UpdArgs a) {
-  if (a.ed && (a.ed->breakdown | a.ed->error)) return;
+  if (a.ed->breakdown | a.ed->error) return;
   const int count = a.j1 - a.j0 + 1;
+  const int zbe = max_field(*a.zmax);
   double nrm = 0.0;
+  unsigned m = 0u;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < a.n; x += stride) {
     v4 zv = a.z[x];
+    float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
     const v4* __restrict__ q = a.basis + (size_t)a.j0 * a.n + x;
+    auto one = [&](int jj, const v4& v, const int4& rc) {
+      if (rc.w) {
+        const double2 c = __ldg(a.coef + jj);
+        axpy_c(zv, c.x, c.y, v);
+      } else {
+        const float cr = __int_as_float(rc.x), ci = __int_as_float(rc.y);
+        const float qx = to_fp32(v.x, rc.z), qy = to_fp32(v.y, rc.z), qz = to_fp32(v.z, rc.z), qw = to_fp32(v.w, rc.z);
+        f0 = fmaf(cr, qx, fmaf(-ci, qy, f0));
+        f1 = fmaf(cr, qy, fmaf(ci, qx, f1));
+        f2 = fmaf(cr, qz, fmaf(-ci, qw, f2));
+        f3 = fmaf(cr, qw, fmaf(ci, qz, f3));
+      }
+    };
     int jj = 0;
     for (; jj + 4 <= count; jj += 4) {
       const v4 q0 = q[(size_t)jj * a.n], q1 = q[(size_t)(jj + 1) * a.n];
       const v4 q2 = q[(size_t)(jj + 2) * a.n], q3 = q[(size_t)(jj + 3) * a.n];
-      const double2 c0 = __ldg(a.coef + jj), c1 = __ldg(a.coef + jj + 1);
-      const double2 c2 = __ldg(a.coef + jj + 2), c3 = __ldg(a.coef + jj + 3);
-      axpy_c(zv, c0.x, c0.y, q0);
-      axpy_c(zv, c1.x, c1.y, q1);
-      axpy_c(zv, c2.x, c2.y, q2);
-      axpy_c(zv, c3.x, c3.y, q3);
+      const int4 r0 = __ldg(a.rec + jj), r1 = __ldg(a.rec + jj + 1), r2 = __ldg(a.rec + jj + 2), r3 = __ldg(a.rec + jj + 3);
+      one(jj, q0, r0);
+      one(jj + 1, q1, r1);
+      one(jj + 2, q2, r2);
+      one(jj + 3, q3, r3);
     }
-    for (; jj < count; ++jj) {
-      const double2 c = __ldg(a.coef + jj);
-      axpy_c(zv, c.x, c.y, q[(size_t)jj * a.n]);
-    }
+    for (; jj < count; ++jj) one(jj, q[(size_t)jj * a.n], __ldg(a.rec + jj));
+    // the FP32 sums in units of 2^(zbe - 1022)
+    zv.x -= fx::scale2((double)f0, zbe - 1022);
+    zv.y -= fx::scale2((double)f1, zbe - 1022);
+    zv.z -= fx::scale2((double)f2, zbe - 1022);
+    zv.w -= fx::scale2((double)f3, zbe - 1022);
     a.z[x] = zv;
-    nrm = fma(zv.x, zv.x, fma(zv.y, zv.y, fma(zv.z, zv.z, fma(zv.w, zv.w, nrm))));
+    m = max(m, mag4(zv));
+    if (a.last) nrm = fma(zv.x, zv.x, fma(zv.y, zv.y, fma(zv.z, zv.z, fma(zv.w, zv.w, nrm))));
   }
+  block_max(m, a.zmax_out);
   if (a.last) block_partial(nrm, a.norm_part + blockIdx.x);
 }
 
 // slot 0 = start, with the ||start||^2 partials
-__global__ void __launch_bounds__(256) eig_start(const v4* in, v4* out, long long n, double* norm_part) {
+__global__ void __launch_bounds__(256) eig_start(const v4* in, v4* out, long long n, double* norm_part,
+                                                 unsigned* vmax) {
   double nrm = 0.0;
+  unsigned m = 0u;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) {
     const v4 v = in[x];
     out[x] = v;
+    m = max(m, mag4(v));
     nrm = fma(v.x, v.x, fma(v.y, v.y, fma(v.z, v.z, fma(v.w, v.w, nrm))));
   }
+  block_max(m, vmax);
   block_partial(nrm, norm_part + blockIdx.x);
 }
 
@@ -898,11 +1066,11 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
   cudaStream_t s = v.stream;
 
   // launch geometry, fixed for the call
-  int cs = (int)std::min<long long>(CH_MAX, std::max<long long>(32, (n + 2LL * sm - 1) / (2LL * sm)));
+  int cs = (int)std::min<long long>(CH_MAX, std::max<long long>(32, (n + 4LL * sm - 1) / (4LL * sm)));
   cs = (cs + 31) / 32 * 32;
-  const int n_dot = (int)std::min<long long>(2LL * sm, (n + cs - 1) / cs);
+  const int n_dot = (int)std::min<long long>(4LL * sm, (n + cs - 1) / cs);
   const int n_upd = (int)std::min<long long>(4LL * sm, std::max<long long>(1, (n + 255) / 256));
-  const size_t dot_smem_max = (size_t)cs * sizeof(v4) + sizeof(double2) * (size_t)(kmax + 1);
+  const size_t dot_smem_max = (size_t)cs * 2 * sizeof(v4) + sizeof(double2) * (size_t)(kmax + 2);
   EIG_TRY(cudaFuncSetAttribute(eig_dot, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dot_smem_max));
 
   // device memory: basis slots 0..max_iter, then (folded) one product buffer
@@ -928,7 +1096,9 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
   const size_t o_beta = take(sizeof(double) * (kmax + 1));
   const size_t o_s = take(sizeof(double) * (kmax + 1));
   const size_t o_coef = take(sizeof(double2) * (kmax + 1));
-  const size_t o_dpart = take(sizeof(double2) * (size_t)n_dot * (kmax + 1));
+  const size_t o_dpart = take(sizeof(double2) * (size_t)n_dot * (kmax + 2));
+  const size_t o_rec = take(sizeof(int4) * (kmax + 1));
+  const size_t o_vmax = take(sizeof(unsigned) * 3 * (kmax + 2));
   const size_t o_npart = take(sizeof(double) * n_upd);
   const size_t o_as = take(sizeof(double) * kmax);
   const size_t o_bs = take(sizeof(double) * kmax);
@@ -949,9 +1119,13 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
   double2* coef = reinterpret_cast<double2*>(sb + o_coef);
   double2* dpart = reinterpret_cast<double2*>(sb + o_dpart);
   double* npart = reinterpret_cast<double*>(sb + o_npart);
+  int4* rec = reinterpret_cast<int4*>(sb + o_rec);
+  unsigned* vmax = reinterpret_cast<unsigned*>(sb + o_vmax);   // largest numbers by slot: after the product, the first
+                                                               // update, and at the end
   int* d_sel = reinterpret_cast<int*>(sb + o_sel);
   double* d_fres = reinterpret_cast<double*>(sb + o_fres);
   EIG_TRY(cudaMemsetAsync(ed, 0, sizeof(EigDev), s));
+  EIG_TRY(cudaMemsetAsync(vmax, 0, sizeof(unsigned) * 3 * (kmax + 2), s));
   EIG_TRY(cudaMemsetAsync(alpha, 0, sizeof(double) * (kmax + 1), s));
   EIG_TRY(cudaMemsetAsync(beta, 0, sizeof(double) * (kmax + 1), s));
 
@@ -990,7 +1164,7 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
   } finish_guard{tm, v, info};
 
   EIG_TRY(tm.mark(K_START));
-  eig_start<<<n_upd, 256, 0, s>>>(static_cast<const v4*>(start_dev), basis, n, npart);
+  eig_start<<<n_upd, 256, 0, s>>>(static_cast<const v4*>(start_dev), basis, n, npart, vmax + 2);
   EIG_TRY(cudaGetLastError());
   EIG_TRY(tm.mark(K_OTHER));
 
@@ -1014,6 +1188,7 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
     if (!fold) {
       a.sub = qim;
       a.out = z;
+      a.vmax = vmax + 3 * (i + 1);
       EIG_TRY(launch_apply(v, a, f32));
       EIG_TRY(tm.mark(K_APPLY));
     } else {
@@ -1025,6 +1200,7 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
       a.in = tmp;
       a.sub = qim;
       a.out = z;
+      a.vmax = vmax + 3 * (i + 1);
       EIG_TRY(launch_apply(v, a, f32));
       EIG_TRY(tm.mark(K_APPLY));
     }
@@ -1032,16 +1208,19 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
     const int j0 = reorth ? 0 : i;
     const int count = i - j0 + 1;
     for (int p = 0; p < passes; ++p) {
-      DotArgs da{z, basis, n, j0, i, cs, dpart, ed};
-      const size_t smem = (size_t)cs * sizeof(v4) + sizeof(double2) * (size_t)count;
+      DotArgs da{basis, n, j0, i, cs, dpart, vmax, p, ed};
+      const size_t smem = (size_t)cs * 2 * sizeof(v4) + sizeof(double2) * (size_t)(count + 1);
       eig_dot<<<n_dot, 256, smem, s>>>(da);
       EIG_TRY(cudaGetLastError());
       EIG_TRY(tm.mark(K_DOT));
-      FinishArgs fa{dpart, n_dot, j0, i, i, p, p == passes - 1, reorth ? 1 : 0, sarr, coef, alpha, beta, ed, ashift};
+      FinishArgs fa{dpart, n_dot, j0, i, i, p, p == passes - 1, reorth ? 1 : 0, sarr, coef, alpha, beta, ed, ashift,
+                    vmax, rec};
       eig_dot_finish<<<(count + 7) / 8, 256, 0, s>>>(fa);
       EIG_TRY(cudaGetLastError());
       EIG_TRY(tm.mark(K_OTHER));
-      UpdArgs ua{z, basis, n, j0, i, coef, p == passes - 1 ? 1 : 0, npart, ed};
+      const bool last = p == passes - 1;
+      UpdArgs ua{z, basis, n, j0, i, coef, rec, last ? 1 : 0, npart, vmax + 3 * (i + 1) + p,
+                 vmax + 3 * (i + 1) + (last ? 2 : 1), ed};
       eig_update<<<n_upd, 256, 0, s>>>(ua);
       EIG_TRY(cudaGetLastError());
       EIG_TRY(tm.mark(K_UPDATE));
@@ -1129,8 +1308,7 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
     a.out = tmp;
     EIG_TRY(launch_apply(v, a));
     EIG_TRY(tm.mark(K_APPLY));
-    DotArgs da{tmp, fold_vecs + (size_t)l * n, n, 0, 0, cs, dpart, nullptr};
-    eig_dot<<<n_dot, 256, (size_t)cs * sizeof(v4) + sizeof(double2), s>>>(da);
+    eig_inner<<<n_dot, 256, 0, s>>>(fold_vecs + (size_t)l * n, tmp, n, dpart);
     EIG_TRY(cudaGetLastError());
     EIG_TRY(tm.mark(K_DOT));
     eig_fold_finish<<<1, 32, 0, s>>>(dpart, n_dot, h.theta[sel[l]], h.bound[sel[l]], sigma, d_fres + 2 * l);
