@@ -38,6 +38,7 @@
 #include <cstdint>
 #include <cstring>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 namespace dirac {
@@ -47,6 +48,7 @@ using v4 = double4_32a;   // one site: (u.re, u.im, d.re, d.im)
 
 constexpr int RITZ_CAP = DIRAC_EIG_RITZ_MAX;   // Ritz values examined per check
 constexpr int MAX_ITER = DIRAC_EIG_ITER_MAX;
+constexpr int TILE_W = 32;                     // tile width of the product (one warp)
 constexpr int CH_MAX = 256;                    // sites per dot-kernel chunk
 constexpr double BREAKDOWN_REL = 1e-12;
 
@@ -126,6 +128,7 @@ struct ApplyArgs {
   int iter;
   int prologue;         // 1: s_i and beta_{i-1} from norm_part, breakdown test, scale by s_i
   unsigned* vmax;       // largest number of `out` (or null)
+  int vbe;              // exponent field of max |V| (0: V = 0)
 };
 
 template <bool DIRI, class T>
@@ -141,55 +144,59 @@ __device__ __forceinline__ void load_site(const v4* __restrict__ in, int gx, int
   o[0] = (T)v.x; o[1] = (T)v.y; o[2] = (T)v.z; o[3] = (T)v.w;
 }
 
-// T = double: the FP64 product.  T = float: the mixed-precision product --
-// the off-diagonal part (differences and vector potential) on FP32 copies of
-// the vector, the diagonal (m c^2 + V - e0 and -m c^2 + V - e0) on the FP64
-// vector itself, so that the -2 m c^2 of the lower components adds no
-// u32 * 2 m c^2 rounding to the product; the Lanczos combination
-// s_i y - c q^_{i-1} in FP64.
-template <int R, bool DIRI, bool HAS_V, class T>
-__global__ void __launch_bounds__(256) eig_apply(const ApplyArgs a) {
+// The scalars of a product inside the Lanczos iteration: s_i (the scale of the
+// input) and the coefficient of q^_{i-1}, from the norm partials of slot i, with
+// the breakdown test; false once the iteration has ended.  A plain product leaves
+// s_in = 1, csub = 0.  Every thread of the block takes the same branch.
+__device__ __forceinline__ bool apply_scalars(const ApplyArgs& a, double& s_in, double& csub) {
   __shared__ double sh_nrm;
   __shared__ int sh_stop;
-  double s_in = 1.0, csub = 0.0;
-  if (a.ed) {
-    // one read of the flags per block (the lead CTA of a prologue launch may
-    // set them meanwhile), so that every thread takes the same branch
-    if (threadIdx.x == 0) sh_stop = a.ed->breakdown | a.ed->error;
-    if (a.prologue && threadIdx.x < 32) {
-      double nrm = 0.0;
-      for (int c = threadIdx.x; c < a.n_part; c += 32) nrm += a.norm_part[c];
-      nrm = wsum(nrm);
-      if (threadIdx.x == 0) sh_nrm = nrm;
-    }
-    __syncthreads();
-    if (sh_stop) return;
-    const int i = a.iter;
-    if (a.prologue) {
-      const double bt = sqrt(sh_nrm);          // ||q^_i||: beta_{i-1}, or ||start|| at i = 0
-      const bool lead = blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0;
-      if (!isfinite(bt) || !(bt > 0.0)) {
-        if (lead) a.ed->error = 1;
-        return;
-      }
-      if (i >= 1 && bt <= BREAKDOWN_REL * a.ed->scale) {
-        if (lead) { a.ed->breakdown = 1; a.ed->k_final = i; a.beta[i - 1] = bt; }
-        return;
-      }
-      s_in = 1.0 / bt;
-      if (i >= 1 && a.sub) csub = bt * a.s[i - 1];
-      if (lead) {
-        a.s[i] = s_in;
-        if (i >= 1) a.beta[i - 1] = bt;
-      }
-    } else if (a.sub && i >= 1) {
-      csub = a.beta[i - 1] * a.s[i - 1];
-    }
+  s_in = 1.0;
+  csub = 0.0;
+  if (!a.ed) return true;
+  // one read of the flags per block (the lead CTA of a prologue launch may set
+  // them meanwhile)
+  if (threadIdx.x == 0) sh_stop = a.ed->breakdown | a.ed->error;
+  if (a.prologue && threadIdx.x < 32) {
+    double nrm = 0.0;
+    for (int c = threadIdx.x; c < a.n_part; c += 32) nrm += a.norm_part[c];
+    nrm = wsum(nrm);
+    if (threadIdx.x == 0) sh_nrm = nrm;
   }
-  // threads beyond the grid's edge repeat its last site and store nothing
-  const int xt = blockIdx.x * 32 + (threadIdx.x & 31), yt = blockIdx.y * 8 + (threadIdx.x >> 5);
-  const bool valid = xt < a.nx && yt < a.ny;
-  const int x = min(xt, a.nx - 1), y = min(yt, a.ny - 1);
+  __syncthreads();
+  if (sh_stop) return false;
+  const int i = a.iter;
+  if (a.prologue) {
+    const double bt = sqrt(sh_nrm);          // ||q^_i||: beta_{i-1}, or ||start|| at i = 0
+    const bool lead = blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0;
+    if (!isfinite(bt) || !(bt > 0.0)) {
+      if (lead) a.ed->error = 1;
+      return false;
+    }
+    if (i >= 1 && bt <= BREAKDOWN_REL * a.ed->scale) {
+      if (lead) { a.ed->breakdown = 1; a.ed->k_final = i; a.beta[i - 1] = bt; }
+      return false;
+    }
+    s_in = 1.0 / bt;
+    if (i >= 1 && a.sub) csub = bt * a.s[i - 1];
+    if (lead) {
+      a.s[i] = s_in;
+      if (i >= 1) a.beta[i - 1] = bt;
+    }
+  } else if (a.sub && i >= 1) {
+    csub = a.beta[i - 1] * a.s[i - 1];
+  }
+  return true;
+}
+
+// One site of the product in floating point.  T = double: FP64.  T = float: the
+// mixed-precision product -- the off-diagonal part (differences and vector
+// potential) on FP32 copies of the vector, the diagonal (m c^2 + V - e0 and
+// -m c^2 + V - e0) on the FP64 vector itself, so that the -2 m c^2 of the lower
+// components adds no u32 * 2 m c^2 rounding to the product; the Lanczos
+// combination s_i y - c q^_{i-1} in FP64.
+template <int R, bool DIRI, bool HAS_V, class T>
+__device__ __forceinline__ v4 apply_site(const ApplyArgs& a, int x, int y, double s_in, double csub) {
   const int nx = a.nx, ny = a.ny;
   T C[4], xp[4], xm[4], yp[4], ym[4], dxv[4], dyv[4];
   double C64[4];
@@ -242,8 +249,245 @@ __global__ void __launch_bounds__(256) eig_apply(const ApplyArgs a) {
   } else {
     r.x = s_in * o[0]; r.y = s_in * o[1]; r.z = s_in * o[2]; r.w = s_in * o[3];
   }
-  if (valid) a.out[idx] = r;
+  return r;
+}
+
+// The mixed-precision product, one thread per site
+template <int R, bool DIRI, bool HAS_V>
+__global__ void __launch_bounds__(256) eig_apply32(const ApplyArgs a) {
+  double s_in, csub;
+  if (!apply_scalars(a, s_in, csub)) return;
+  // threads beyond the grid's edge repeat its last site and store nothing
+  const int xt = blockIdx.x * 32 + (threadIdx.x & 31), yt = blockIdx.y * 8 + (threadIdx.x >> 5);
+  const bool valid = xt < a.nx && yt < a.ny;
+  const int x = min(xt, a.nx - 1), y = min(yt, a.ny - 1);
+  const v4 r = apply_site<R, DIRI, HAS_V, float>(a, x, y, s_in, csub);
+  if (valid) a.out[(size_t)y * a.nx + x] = r;
   if (a.vmax) block_max(valid ? mag4(r) : 0u, a.vmax);
+}
+
+// The FP64 product in fixed point (dirac_fixed.cuh), a tile of 32 x 16 sites per
+// CTA, four rows per thread (32 x 4 and one row on small grids), LANCZOS: with the
+// scale and q^_{i-1} of an iteration; as in the FP64 Lanczos pass (dirac_pass64.cuh):
+// exponents of the tile's upper and lower components and of q^_{i-1}, the tile
+// and its halo as 58-bit (order 4: 55-bit) numbers in shared memory, each row of
+// the operator one sum of products, then times s_i.  Of the FP64 pipe only the
+// four conversions of the result are left; with some 40 multiply-adds a site it
+// bounded the product (2048^2 with V: 342 us, 0.9 TB/s).  Tiles with numbers
+// that are not finite, or none above 2^-894, take the floating-point form.
+constexpr int AP_WARPS = 4, AP_THREADS = 32 * AP_WARPS, AP_SLOTS = 16;
+
+template <int R, bool DIRI, bool HAS_V, int AP_RPT, bool LANCZOS>
+__global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const ApplyArgs a) {
+  constexpr int AP_TH = AP_WARPS * AP_RPT;
+  constexpr int W = TILE_W + 2 * R, F = R == 1 ? 58 : 55;
+  constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * AP_TH, HPT = (NH + AP_THREADS - 1) / AP_THREADS;
+  __shared__ __align__(16) longlong2 sq[2][(AP_TH + 2 * R) * W];
+  __shared__ int2 kt[AP_SLOTS];
+  __shared__ unsigned emax[4];
+  double s_in = 1.0, csub = 0.0;
+  if (LANCZOS && !apply_scalars(a, s_in, csub)) return;
+  if (threadIdx.x < 4) emax[threadIdx.x] = 0u;
+  __syncthreads();
+  const int nx = a.nx, ny = a.ny;
+  const int tx = threadIdx.x & 31, tg = threadIdx.x >> 5, lane = tx;
+  const int x0 = blockIdx.x * TILE_W, y0 = blockIdx.y * AP_TH, r0 = tg * AP_RPT;
+  const bool full = x0 + TILE_W <= nx && y0 + AP_TH <= ny;
+  const int rows_in = x0 + tx < nx ? ny - (y0 + r0) : 0;              // row k is in the grid if k < rows_in
+  const size_t idx0 = (size_t)(y0 + r0) * nx + (x0 + tx);             // used where in the grid
+  const bool has_sub = LANCZOS && csub != 0.0;
+  double q[AP_RPT][4], p[AP_RPT][4], hq[HPT][4];
+  int hat[HPT];
+#pragma unroll
+  for (int k = 0; k < AP_RPT; ++k) {
+    // sites beyond the grid's edge are halo of the sites inside
+    if (full) {
+      const v4 v = a.in[idx0 + (size_t)k * nx];
+      q[k][0] = v.x; q[k][1] = v.y; q[k][2] = v.z; q[k][3] = v.w;
+    } else {
+      load_site<DIRI>(a.in, x0 + tx, y0 + r0 + k, nx, ny, q[k]);
+    }
+    p[k][0] = p[k][1] = p[k][2] = p[k][3] = 0.0;
+    if (has_sub && k < rows_in) {
+      const v4 v = a.sub[idx0 + (size_t)k * nx];
+      p[k][0] = v.x; p[k][1] = v.y; p[k][2] = v.z; p[k][3] = v.w;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < HPT; ++u) {
+    const int h = threadIdx.x + u * AP_THREADS;
+    hat[u] = -1;
+    hq[u][0] = hq[u][1] = hq[u][2] = hq[u][3] = 0.0;
+    if (h < NH) {
+      int hrow, hcol;
+      if (h < NH_ROW) {                 // rows above / below
+        const int r = h / TILE_W;
+        hrow = (r < R) ? r : AP_TH + r;
+        hcol = (h % TILE_W) + R;
+      } else {                          // columns left / right
+        const int h2 = h - NH_ROW;
+        hrow = h2 / (2 * R) + R;
+        const int c = h2 % (2 * R);
+        hcol = (c < R) ? c : TILE_W + c;
+      }
+      hat[u] = hrow * W + hcol;
+      load_site<DIRI>(a.in, x0 + hcol - R, y0 + hrow - R, nx, ny, hq[u]);
+    }
+  }
+  unsigned m0 = 0u, m1 = 0u, m2 = 0u, m3 = 0u;
+#pragma unroll
+  for (int u = 0; u < HPT; ++u) {
+    m0 = max(m0, max(mag(hq[u][0]), mag(hq[u][1])));
+    m1 = max(m1, max(mag(hq[u][2]), mag(hq[u][3])));
+  }
+#pragma unroll
+  for (int k = 0; k < AP_RPT; ++k) {
+    m0 = max(m0, max(mag(q[k][0]), mag(q[k][1])));
+    m1 = max(m1, max(mag(q[k][2]), mag(q[k][3])));
+    m2 = max(m2, max(mag(p[k][0]), mag(p[k][1])));
+    m3 = max(m3, max(mag(p[k][2]), mag(p[k][3])));
+  }
+  m0 = __reduce_max_sync(0xffffffffu, m0);
+  m1 = __reduce_max_sync(0xffffffffu, m1);
+  m2 = __reduce_max_sync(0xffffffffu, m2);
+  m3 = __reduce_max_sync(0xffffffffu, m3);
+  if (lane < 4) atomicMax(&emax[lane], lane == 0 ? m0 : lane == 1 ? m1 : lane == 2 ? m2 : m3);
+  __syncthreads();
+  // a tile of zeros is exact in fixed point; a largest number that is not finite
+  // or below the clamp is not
+  bool plain = false;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) plain = plain || (emax[c] >> 21) == 0x7ffu || (emax[c] != 0u && (emax[c] >> 21) < 128u);
+  if (plain) {
+    unsigned m = 0u;
+    for (int k = 0; k < AP_RPT; ++k) {
+      if (k >= rows_in) break;
+      const v4 o = apply_site<R, DIRI, HAS_V, double>(a, x0 + tx, y0 + r0 + k, s_in, csub);
+      a.out[idx0 + (size_t)k * nx] = o;
+      m = max(m, mag4(o));
+    }
+    __syncwarp();
+    if (a.vmax) block_max(m, a.vmax);
+    return;
+  }
+  int be[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) be[c] = max((int)(emax[c] >> 21), 128);
+  const int at0 = (r0 + R) * W + tx + R;
+#pragma unroll
+  for (int k = 0; k < AP_RPT; ++k) {
+    sq[0][at0 + k * W] = make_longlong2(fx::to_fixed<F>(q[k][0], be[0]), fx::to_fixed<F>(q[k][1], be[0]));
+    sq[1][at0 + k * W] = make_longlong2(fx::to_fixed<F>(q[k][2], be[1]), fx::to_fixed<F>(q[k][3], be[1]));
+  }
+#pragma unroll
+  for (int u = 0; u < HPT; ++u) {
+    if (hat[u] >= 0) {
+      sq[0][hat[u]] = make_longlong2(fx::to_fixed<F>(hq[u][0], be[0]), fx::to_fixed<F>(hq[u][1], be[0]));
+      sq[1][hat[u]] = make_longlong2(fx::to_fixed<F>(hq[u][2], be[1]), fx::to_fixed<F>(hq[u][3], be[1]));
+    }
+  }
+  if (tg == 0) {
+    // coefficients as 60-bit fractions of the row's largest term: slots 0
+    // diagonal, 1 kx, 2 ky, 3 c A_x, 4 c A_y, 5 of q^_{i-1} (before the scaling by
+    // s_i), 6 V (its exponent alone), 7 the scale, of the upper and the lower row
+    const int j = lane & 7, ch = (lane >> 3) & 1;
+    double c = 0.0;
+    if (j == 0) c = ch ? a.ad : a.au;
+    if (j == 1) c = a.kx;
+    if (j == 2) c = a.ky;
+    if (j == 3) c = a.cax;
+    if (j == 4) c = a.cay;
+    if (j == 5) c = -csub / s_in;
+    const int xe = j == 6 ? (HAS_V ? a.vbe : 0) : fx::exp_field(c);
+    const int be_x = (j == 0 || j == 6) ? be[ch] : (j == 5 ? be[2 + ch] : be[1 - ch]);
+    int sc = xe ? xe + be_x : 0;
+    sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 1));
+    sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 2));
+    sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 4));
+    if (lane < AP_SLOTS) {
+      const fx::Limbs l = fx::split(fx::to_fixed<60>(c, max(sc - be_x, 63)));
+      kt[lane] = j == 7 ? make_int2(sc, 0) : make_int2(l.hi, l.lo);
+    }
+  }
+  __syncthreads();
+  const int es = fx::exp_field(s_in);
+  const fx::Limbs ks = fx::split(fx::to_fixed<60>(s_in, es));
+  const bool scaled = LANCZOS && s_in != 1.0;
+  unsigned m = 0u;
+  long long pot[AP_RPT];      // V as 60-bit fractions of the largest |V|
+#pragma unroll
+  for (int k = 0; k < AP_RPT; ++k)
+    pot[k] = HAS_V && k < rows_in ? fx::to_fixed<60>(a.V[idx0 + (size_t)k * nx], max(a.vbe, 63)) : 0;
+  auto half = [&](auto half_c) {
+    constexpr int HALF = decltype(half_c)::value;
+    const longlong2* const own = sq[HALF] + at0;
+    const longlong2* const oth = sq[1 - HALF] + at0;
+    const int2* const kc = kt + 8 * HALF;
+    auto coef = [&](int j) { const int2 v = kc[j]; return fx::Limbs{v.x, v.y}; };
+    const int sc = kc[7].x;
+    const int texp = sc - 2044 - F + (scaled ? es - 1022 : 0);
+    const bool normal = texp >= -1022 && texp <= 960;      // no result leaves the normal range
+    const int vsh = min(max(sc - be[HALF] - max(a.vbe, 63), 0), 63);   // V's scale within the row's
+    longlong2 col[AP_RPT + 2 * R];
+#pragma unroll
+    for (int j = 0; j < AP_RPT + 2 * R; ++j) col[j] = oth[(j - R) * W];
+#pragma unroll
+    for (int k = 0; k < AP_RPT; ++k) {
+      const longlong2* const row = oth + k * W;
+      const longlong2 xl = row[-1], xr = row[1], cv = own[k * W];
+      long long hxr = xl.x - xr.x, hxi = xr.y - xl.y;          // -D_x re, D_x im
+      long long hyr = col[k + R + 1].x - col[k + R - 1].x, hyi = col[k + R + 1].y - col[k + R - 1].y;
+      if constexpr (R == 2) {
+        const longlong2 xl2 = row[-2], xr2 = row[2];
+        hxr = 8 * hxr - (xl2.x - xr2.x);
+        hxi = 8 * hxi - (xr2.y - xl2.y);
+        hyr = 8 * hyr - (col[k + 2 * R].x - col[k].x);
+        hyi = 8 * hyi - (col[k + 2 * R].y - col[k].y);
+      }
+      fx::Acc s0, s1;
+      s0.mac(fx::split(hxi), coef(1));
+      s1.mac(fx::split(hxr), coef(1));
+      s0.mac(fx::split(HALF ? hyr : -hyr), coef(2));
+      s1.mac(fx::split(HALF ? hyi : -hyi), coef(2));
+      const fx::Limbs c0 = fx::split(cv.x), c1 = fx::split(cv.y);
+      s0.mac(c0, coef(0));
+      s1.mac(c1, coef(0));
+      if (a.cax != 0.0) {
+        s0.mac(fx::split(col[k + R].x), coef(3));
+        s1.mac(fx::split(col[k + R].y), coef(3));
+      }
+      if (a.cay != 0.0) {
+        s0.mac(fx::split(HALF ? -col[k + R].y : col[k + R].y), coef(4));
+        s1.mac(fx::split(HALF ? col[k + R].x : -col[k + R].x), coef(4));
+      }
+      if (has_sub) {
+        s0.mac(fx::split(fx::to_fixed<F>(p[k][2 * HALF], be[2 + HALF])), coef(5));
+        s1.mac(fx::split(fx::to_fixed<F>(p[k][2 * HALF + 1], be[2 + HALF])), coef(5));
+      }
+      if constexpr (HAS_V) {
+        const fx::Limbs kv = fx::split(pot[k] >> vsh);
+        s0.mac(c0, kv);
+        s1.mac(c1, kv);
+      }
+      long long v0 = s0.template value<28>(), v1 = s1.template value<28>();
+      if (scaled) {
+        fx::Acc t0, t1;
+        t0.mac(fx::split(v0), ks);
+        t1.mac(fx::split(v1), ks);
+        v0 = t0.template value<28>();
+        v1 = t1.template value<28>();
+      }
+      if (k < rows_in) {
+        const double2 o = normal ? make_double2(fx::to_double(v0, texp), fx::to_double(v1, texp))
+                                 : make_double2(fx::scale2((double)v0, texp), fx::scale2((double)v1, texp));
+        reinterpret_cast<double2*>(a.out + idx0 + (size_t)k * nx)[HALF] = o;
+        m = max(m, max(mag(o.x), mag(o.y)));
+      }
+    }
+  };
+  half(std::integral_constant<int, 0>{});
+  half(std::integral_constant<int, 1>{});
+  if (a.vmax) block_max(m, a.vmax);
 }
 
 // ---------------------------------------------------------------------------
@@ -260,6 +504,7 @@ __global__ void __launch_bounds__(256) eig_apply(const ApplyArgs a) {
 // every third vector meanwhile, at FP64_SHARE's cost ratio.
 // ---------------------------------------------------------------------------
 constexpr int FP64_SHARE = 3;   // one vector in so many goes to the FP64 pipe
+__device__ __forceinline__ bool fp64_vector(int jj, int nw) { return (jj / nw + jj % nw) % FP64_SHARE == FP64_SHARE - 1; }
 
 struct DotArgs {
   const v4* basis;
@@ -272,6 +517,10 @@ struct DotArgs {
   const EigDev* ed;
 };
 
+// A warp takes four rows of 32 numbers at a time: four pieces of one vector's
+// chunk, or (SHORT: chunks of 32 sites, small grids) one piece of each of four
+// vectors, so that as many loads are in flight.
+template <bool SHORT>
 __global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
   extern __shared__ __align__(32) unsigned char smem[];
   if (a.ed->breakdown | a.ed->error) return;
@@ -285,14 +534,33 @@ __global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
   const int zbe = max_field(a.vmax[3 * (a.j1 + 1) + a.stage]);
   const long long nchunks = (a.n + a.cs - 1) / a.cs;
   const v4* const z = a.basis + (size_t)(a.j1 + 1) * a.n;
+  // limb products of one number of q^ with its z, and the sums of a batch
+  auto products = [&](const v4& v, int t, int be, fx::Acc& ar, fx::Acc& ai, fx::Acc& am) {
+    const fx::Limbs x = fx::split(fx::to_fixed<58>(v.x, be)), y = fx::split(fx::to_fixed<58>(v.y, be));
+    const fx::Limbs z = fx::split(fx::to_fixed<58>(v.z, be)), w = fx::split(fx::to_fixed<58>(v.w, be));
+    const int4 s0 = zu[t], s1 = zd[t];
+    const fx::Limbs zx{s0.x, s0.y}, zy{s0.z, s0.w}, zz{s1.x, s1.y}, zw{s1.z, s1.w};
+    ar.mac(x, zx);
+    ar.mac(y, zy);
+    ar.mac(z, zz);
+    ar.mac(w, zw);
+    ai.mac(x, zy);
+    ai.mac(z, zw);
+    am.mac(y, zx);
+    am.mac(w, zz);
+  };
+  auto add_sums = [&](int jj, long long re, long long im) {
+    const fx::WarpSum sr = fx::warp_sum(re), si = fx::warp_sum(im);
+    if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += fx::to_double(lane == 0 ? sr : si);
+  };
+  v4 none;
+  none.x = none.y = none.z = none.w = 0.0;
   for (long long ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
     const long long base = ch * a.cs;
     const int len = (int)min((long long)a.cs, a.n - base);
     __syncthreads();
     for (int t = threadIdx.x; t < a.cs; t += blockDim.x) {
-      v4 v;
-      v.x = v.y = v.z = v.w = 0.0;
-      if (t < len) v = z[base + t];
+      const v4 v = t < len ? z[base + t] : none;
       const fx::Limbs x = fx::split(fx::to_fixed<58>(v.x, zbe)), y = fx::split(fx::to_fixed<58>(v.y, zbe));
       const fx::Limbs u = fx::split(fx::to_fixed<58>(v.z, zbe)), w = fx::split(fx::to_fixed<58>(v.w, zbe));
       zu[t] = make_int4(x.hi, x.lo, y.hi, y.lo);
@@ -300,71 +568,74 @@ __global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
       zf[t] = v;
     }
     __syncthreads();
-    for (int jj = warp; jj < count; jj += nw) {
-      const v4* __restrict__ q = a.basis + (size_t)(a.j0 + jj) * a.n + base;
-      if ((jj / nw + warp) % FP64_SHARE == FP64_SHARE - 1) {
-        double re = 0.0, im = 0.0;
+    if constexpr (SHORT) {
+      for (int j0 = 4 * warp; j0 < count; j0 += 4 * nw) {
+        const v4* __restrict__ q = a.basis + (size_t)(a.j0 + j0) * a.n + base;
+        v4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = lane < len && j0 + u < count ? q[(size_t)u * a.n + lane] : none;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int jj = j0 + u;
+          if (jj < count) {
+            const int be = jj + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + jj) + 2]);
+            fx::Acc ar, ai, am;
+            products(v[u], lane, be, ar, ai, am);
+            add_sums(jj, ar.template value<28>(), ai.template value<28>() - am.template value<28>());
+          }
+        }
+      }
+    } else {
+      for (int jj = warp; jj < count; jj += nw) {
+        const v4* __restrict__ q = a.basis + (size_t)(a.j0 + jj) * a.n + base;
+        if (fp64_vector(jj, nw)) {
+          double re = 0.0, im = 0.0;
+          for (int t0 = 0; t0 < len; t0 += 128) {
+            v4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int t = t0 + 32 * u + lane;
+              v[u] = t < len ? q[t] : none;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const v4 zz = zf[min(t0 + 32 * u + lane, a.cs - 1)];
+              re = fma(v[u].x, zz.x, fma(v[u].y, zz.y, fma(v[u].z, zz.z, fma(v[u].w, zz.w, re))));
+              im = fma(v[u].x, zz.y, fma(-v[u].y, zz.x, fma(v[u].z, zz.w, fma(-v[u].w, zz.z, im))));
+            }
+          }
+          // both sums over the warp with one addition per level: even lanes re, odd lanes im
+          double part = (lane & 1 ? im : re) + __shfl_xor_sync(0xffffffffu, lane & 1 ? re : im, 1);
+#pragma unroll
+          for (int o = 16; o > 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+          if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += part;
+          continue;
+        }
+        const int be = jj + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + jj) + 2]);
+        long long re = 0, im = 0;   // at most 32 products below 2^56 in units of 2^60
         for (int t0 = 0; t0 < len; t0 += 128) {
           v4 v[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             const int t = t0 + 32 * u + lane;
-            v[u].x = v[u].y = v[u].z = v[u].w = 0.0;
-            if (t < len) v[u] = q[t];
+            v[u] = t < len ? q[t] : none;
           }
+          fx::Acc ar, ai, am;       // at most 16 products each: cross terms below 2^62
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const v4 zz = zf[min(t0 + 32 * u + lane, a.cs - 1)];
-            re = fma(v[u].x, zz.x, fma(v[u].y, zz.y, fma(v[u].z, zz.z, fma(v[u].w, zz.w, re))));
-            im = fma(v[u].x, zz.y, fma(-v[u].y, zz.x, fma(v[u].z, zz.w, fma(-v[u].w, zz.z, im))));
-          }
+          for (int u = 0; u < 4; ++u)
+            products(v[u], min(t0 + 32 * u + lane, a.cs - 1), be, ar, ai, am);   // (zero beyond the end)
+          re += ar.template value<28>();
+          im += ai.template value<28>() - am.template value<28>();
         }
-        // both sums over the warp with one addition per level: even lanes re, odd lanes im
-        double part = (lane & 1 ? im : re) + __shfl_xor_sync(0xffffffffu, lane & 1 ? re : im, 1);
-#pragma unroll
-        for (int o = 16; o > 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += part;
-        continue;
+        add_sums(jj, re, im);
       }
-      const int be = jj + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + jj) + 2]);
-      long long re = 0, im = 0;   // 64 products below 2^56 in units of 2^60
-      for (int t0 = 0; t0 < len; t0 += 128) {
-        v4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int t = t0 + 32 * u + lane;
-          v[u].x = v[u].y = v[u].z = v[u].w = 0.0;
-          if (t < len) v[u] = q[t];
-        }
-        fx::Acc ar, ai, am;       // at most 16 products each: cross terms below 2^62
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int t = t0 + 32 * u + lane;
-          const fx::Limbs x = fx::split(fx::to_fixed<58>(v[u].x, be)), y = fx::split(fx::to_fixed<58>(v[u].y, be));
-          const fx::Limbs z = fx::split(fx::to_fixed<58>(v[u].z, be)), w = fx::split(fx::to_fixed<58>(v[u].w, be));
-          const int4 s0 = zu[min(t, a.cs - 1)], s1 = zd[min(t, a.cs - 1)];   // (zero times it beyond the end)
-          const fx::Limbs zx{s0.x, s0.y}, zy{s0.z, s0.w}, zz{s1.x, s1.y}, zw{s1.z, s1.w};
-          ar.mac(x, zx);
-          ar.mac(y, zy);
-          ar.mac(z, zz);
-          ar.mac(w, zw);
-          ai.mac(x, zy);
-          ai.mac(z, zw);
-          am.mac(y, zx);
-          am.mac(w, zz);
-        }
-        re += ar.template value<28>();
-        im += ai.template value<28>() - am.template value<28>();
-      }
-      const fx::WarpSum sr = fx::warp_sum(re), si = fx::warp_sum(im);
-      if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += fx::to_double(lane == 0 ? sr : si);
     }
   }
   __syncthreads();
   for (int t = threadIdx.x; t < count; t += blockDim.x) {
     // units: (2^(be - 1022 - 58)) (2^(zbe - 1022 - 58)) 2^60
     const int be = t + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + t) + 2]);
-    const int e = (t / nw + t % nw) % FP64_SHARE == FP64_SHARE - 1 ? 0 : be + zbe - 2100;
+    const int e = !SHORT && fp64_vector(t, nw) ? 0 : be + zbe - 2100;
     a.part[(size_t)t * gridDim.x + blockIdx.x] = make_double2(fx::scale2(acc[t].x, e), fx::scale2(acc[t].y, e));
   }
 }
@@ -502,17 +773,31 @@ __device__ void block_partial(double v, double* out) {
   }
 }
 
-__global__ void __launch_bounds__(256) eig_update(const UpdArgs a) {
+// GROUPS: warps of a CTA that share the vectors of one set of sites.  1: each
+// thread has its own sites and walks all vectors.  8 (small grids, where that walk
+// is one chain of loads): 32 sites per CTA, vector quads dealt to eight warps,
+// whose parts are added in a fixed order.
+template <int GROUPS>
+__global__ void __launch_bounds__(256, 4) eig_update(const UpdArgs a) {
   if (a.ed->breakdown | a.ed->error) return;
+  constexpr int SITES = 256 / GROUPS;
+  __shared__ v4 part[GROUPS > 1 ? GROUPS : 1][GROUPS > 1 ? SITES : 1];
+  __shared__ float4 fpart[GROUPS > 1 ? GROUPS : 1][GROUPS > 1 ? SITES : 1];
   const int count = a.j1 - a.j0 + 1;
   const int zbe = max_field(*a.zmax);
+  const int site = GROUPS > 1 ? (int)threadIdx.x % SITES : (int)threadIdx.x;
+  const int grp = GROUPS > 1 ? (int)threadIdx.x / SITES : 0;
   double nrm = 0.0;
   unsigned m = 0u;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < a.n; x += stride) {
-    v4 zv = a.z[x];
+  const long long stride = (long long)gridDim.x * SITES;
+  for (long long x0 = (long long)blockIdx.x * SITES; x0 < a.n; x0 += stride) {
+    const long long x = x0 + site;
+    const bool in = x < a.n;
+    v4 zv;
+    zv.x = zv.y = zv.z = zv.w = 0.0;
+    if (grp == 0) zv = a.z[in ? x : 0];
     float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
-    const v4* __restrict__ q = a.basis + (size_t)a.j0 * a.n + x;
+    const v4* __restrict__ q = a.basis + (size_t)a.j0 * a.n + (in ? x : 0);
     auto one = [&](int jj, const v4& v, const int4& rc) {
       if (rc.w) {
         const double2 c = __ldg(a.coef + jj);
@@ -526,8 +811,8 @@ __global__ void __launch_bounds__(256) eig_update(const UpdArgs a) {
         f3 = fmaf(cr, qw, fmaf(ci, qz, f3));
       }
     };
-    int jj = 0;
-    for (; jj + 4 <= count; jj += 4) {
+    int jj = 4 * grp;
+    for (; jj + 4 <= count; jj += 4 * GROUPS) {
       const v4 q0 = q[(size_t)jj * a.n], q1 = q[(size_t)(jj + 1) * a.n];
       const v4 q2 = q[(size_t)(jj + 2) * a.n], q3 = q[(size_t)(jj + 3) * a.n];
       const int4 r0 = __ldg(a.rec + jj), r1 = __ldg(a.rec + jj + 1), r2 = __ldg(a.rec + jj + 2), r3 = __ldg(a.rec + jj + 3);
@@ -536,15 +821,34 @@ __global__ void __launch_bounds__(256) eig_update(const UpdArgs a) {
       one(jj + 2, q2, r2);
       one(jj + 3, q3, r3);
     }
-    for (; jj < count; ++jj) one(jj, q[(size_t)jj * a.n], __ldg(a.rec + jj));
-    // the FP32 sums in units of 2^(zbe - 1022)
-    zv.x -= fx::scale2((double)f0, zbe - 1022);
-    zv.y -= fx::scale2((double)f1, zbe - 1022);
-    zv.z -= fx::scale2((double)f2, zbe - 1022);
-    zv.w -= fx::scale2((double)f3, zbe - 1022);
-    a.z[x] = zv;
-    m = max(m, mag4(zv));
-    if (a.last) nrm = fma(zv.x, zv.x, fma(zv.y, zv.y, fma(zv.z, zv.z, fma(zv.w, zv.w, nrm))));
+    for (; jj < count; ++jj) one(jj, q[(size_t)jj * a.n], __ldg(a.rec + jj));   // the last quad's owner
+    if constexpr (GROUPS > 1) {
+      part[grp][site] = zv;
+      fpart[grp][site] = make_float4(f0, f1, f2, f3);
+      __syncthreads();
+      if (grp == 0) {
+#pragma unroll
+        for (int g = 1; g < GROUPS; ++g) {
+          const v4 p = part[g][site];
+          const float4 f = fpart[g][site];
+          if (p.x != 0.0 || p.y != 0.0 || p.z != 0.0 || p.w != 0.0) {
+            zv.x += p.x; zv.y += p.y; zv.z += p.z; zv.w += p.w;
+          }
+          f0 += f.x; f1 += f.y; f2 += f.z; f3 += f.w;
+        }
+      }
+      __syncthreads();
+    }
+    if (in && grp == 0) {
+      // the FP32 sums in units of 2^(zbe - 1022)
+      zv.x -= fx::scale2((double)f0, zbe - 1022);
+      zv.y -= fx::scale2((double)f1, zbe - 1022);
+      zv.z -= fx::scale2((double)f2, zbe - 1022);
+      zv.w -= fx::scale2((double)f3, zbe - 1022);
+      a.z[x] = zv;
+      m = max(m, mag4(zv));
+      if (a.last) nrm = fma(zv.x, zv.x, fma(zv.y, zv.y, fma(zv.z, zv.z, fma(zv.w, zv.w, nrm))));
+    }
   }
   block_max(m, a.zmax_out);
   if (a.last) block_partial(nrm, a.norm_part + blockIdx.x);
@@ -595,18 +899,22 @@ struct RitzArgs {
 // recurrence p_j = (a_j - x) p_{j-1} - b_{j-1}^2 p_{j-2}.  The pair is rescaled
 // by a power of two every 8 terms; an exact zero takes the sign opposite to
 // its predecessor (it counts as an eigenvalue at or below x of T_j).
+//
+// Signs, zeros and magnitudes are taken from the bits: an FP64 comparison costs as
+// much as a multiplication (76 cycles of a sub-partition).
 __device__ int sturm_count(const double* __restrict__ as, const double* __restrict__ b2s, int k, double x) {
   double p1 = 1.0, p2 = 0.0;
   int cnt = 0;
   for (int j = 0; j < k; ++j) {
     const double t = (j > 0) ? b2s[j - 1] * p2 : 0.0;
     double p = fma(as[j] - x, p1, -t);
-    if (p == 0.0) p = (p1 > 0.0 ? -1.0 : 1.0) * fabs(p1) * 0x1p-60;
-    cnt += (p < 0.0) != (p1 < 0.0);
+    if (((__double2hiint(p) & 0x7fffffff) | __double2loint(p)) == 0)
+      p = (__double2hiint(p1) < 0 ? 1.0 : -1.0) * fabs(p1) * 0x1p-60;
+    cnt += (int)((unsigned)(__double2hiint(p) ^ __double2hiint(p1)) >> 31);
     p2 = p1;
     p1 = p;
     if ((j & 7) == 7) {
-      const int e = ilogb(fmax(fabs(p1), fabs(p2)));
+      const int e = max(fx::exp_field(p1), fx::exp_field(p2)) - 1023;
       if (e > 400 || e < -400) {
         const double f = ldexp(1.0, -e);
         p1 *= f;
@@ -700,50 +1008,60 @@ __global__ void __launch_bounds__(256) eig_ritz_prep(const RitzArgs a) {
 }
 
 // LU of the scaled T - theta with partial pivoting (row interchanges kept in
-// piv): d diagonal of U, u1/u2 its first/second superdiagonal, l the
-// multipliers.  One thread.
+// piv): rd reciprocals of U's diagonal (one division a row: 434 cycles), u1/u2 its
+// first/second superdiagonal, l the multipliers.  One thread; the row being
+// eliminated stays in registers.
 __device__ void tridiag_lu(const double* __restrict__ as, const double* __restrict__ bs, int k, double theta,
-                           double* d, double* u1, double* u2, double* l, int* piv) {
+                           double* rd, double* u1, double* u2, double* l, int* piv) {
   const double tiny = DBL_EPSILON;   // T is scaled to norm <= 1
-  for (int j = 0; j < k; ++j) {
-    d[j] = as[j] - theta;
-    u1[j] = j < k - 1 ? bs[j] : 0.0;
-    u2[j] = 0.0;
-  }
+  double d = as[0] - theta, u = k > 1 ? bs[0] : 0.0;
   for (int j = 0; j < k - 1; ++j) {
     const double low = bs[j];                 // entry (j+1, j)
-    if (fabs(d[j]) >= fabs(low)) {
-      if (d[j] == 0.0) d[j] = tiny;
-      const double m = low / d[j];
+    const double dn = as[j + 1] - theta, un = j + 1 < k - 1 ? bs[j + 1] : 0.0;
+    if (fabs(d) >= fabs(low)) {
+      const double r = 1.0 / (d == 0.0 ? tiny : d);
+      const double m = low * r;
+      rd[j] = r;
+      u1[j] = u;
+      u2[j] = 0.0;
       l[j] = m;
-      d[j + 1] -= m * u1[j];
       piv[j] = 0;
+      d = fma(-m, u, dn);
+      u = un;
     } else {                                  // rows j and j+1 change places
-      const double m = d[j] / low;
-      const double dn = d[j + 1], un = (j + 1 < k - 1) ? u1[j + 1] : 0.0;
-      const double uj = u1[j];
-      d[j] = low;
+      const double r = 1.0 / low;
+      const double m = d * r;
+      rd[j] = r;
       u1[j] = dn;
       u2[j] = un;
-      d[j + 1] = uj - m * dn;
-      if (j + 1 < k - 1) u1[j + 1] = -m * un;
       l[j] = m;
       piv[j] = 1;
+      d = fma(-m, dn, u);
+      u = -m * un;
     }
   }
-  if (d[k - 1] == 0.0) d[k - 1] = tiny;
+  rd[k - 1] = 1.0 / (d == 0.0 ? tiny : d);
+  u1[k - 1] = u2[k - 1] = 0.0;
 }
 
 // x <- (T - theta)^{-1} x with the factors of tridiag_lu; one thread
-__device__ void tridiag_solve(int k, const double* d, const double* u1, const double* u2, const double* l,
+__device__ void tridiag_solve(int k, const double* rd, const double* u1, const double* u2, const double* l,
                               const int* piv, double* x) {
+  double c = x[0];
   for (int j = 0; j < k - 1; ++j) {
-    if (piv[j]) { const double t = x[j]; x[j] = x[j + 1]; x[j + 1] = t; }
-    x[j + 1] -= l[j] * x[j];
+    double n = x[j + 1];
+    if (piv[j]) { const double t = c; c = n; n = t; }
+    x[j] = c;
+    c = fma(-l[j], c, n);
   }
-  x[k - 1] /= d[k - 1];
-  if (k >= 2) x[k - 2] = (x[k - 2] - u1[k - 2] * x[k - 1]) / d[k - 2];
-  for (int j = k - 3; j >= 0; --j) x[j] = (x[j] - u1[j] * x[j + 1] - u2[j] * x[j + 2]) / d[j];
+  double x1 = c * rd[k - 1], x2 = 0.0;      // x[j + 1], x[j + 2]
+  x[k - 1] = x1;
+  for (int j = k - 2; j >= 0; --j) {
+    const double t = fma(-u2[j], x2, fma(-u1[j], x1, x[j])) * rd[j];
+    x[j] = t;
+    x2 = x1;
+    x1 = t;
+  }
 }
 
 // x /= ||x|| by one warp (x in global memory; the warp is synchronised on return)
@@ -763,29 +1081,37 @@ __device__ void warp_normalise(double* x, int k) {
 }
 
 // Ritz values: multisection for the r-th smallest eigenvalue (0-based) of the
-// scaled T, one warp each, 32 Sturm counts per round
-__global__ void __launch_bounds__(128) eig_ritz_values(const RitzArgs a) {
+// scaled T, one block of four warps each, 128 Sturm counts per round (8 rounds to
+// the last digit, where 32 points took 11)
+constexpr int RV_THREADS = 128;
+
+__global__ void __launch_bounds__(RV_THREADS) eig_ritz_values(const RitzArgs a) {
+  __shared__ int firsts[RV_THREADS / 32];
   const RitzOut* o = a.out;
   if (o->error || o->k == 0) return;
-  const int lane = threadIdx.x & 31;
-  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int w = (int)blockIdx.x;
   if (w >= o->n_exam) return;
   const int k = o->k;
   const int r = o->n_lo + w;
   double lo = o->g_lo, hi = o->g_hi;
+  auto point = [&](double l, double width, int i) { return l + width * (double)(i + 1) * (1.0 / (RV_THREADS + 1)); };
   for (int round = 0; round < 80; ++round) {
     const double width = hi - lo;
     if (width <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + 2.0 * DBL_EPSILON) break;
-    const double xq = lo + width * (double)(lane + 1) * (1.0 / 33.0);
-    const int c = sturm_count(a.as, a.b2s, k, xq);
+    const int c = sturm_count(a.as, a.b2s, k, point(lo, width, (int)threadIdx.x));
     const unsigned above = __ballot_sync(0xffffffffu, c > r);   // points past the eigenvalue
-    const int f = above ? __ffs(above) - 1 : 32;
-    const double nlo = __shfl_sync(0xffffffffu, xq, f > 0 ? f - 1 : 0);
-    const double nhi = __shfl_sync(0xffffffffu, xq, f < 32 ? f : 31);
-    if (f > 0) lo = nlo;
-    if (f < 32) hi = nhi;
+    if ((threadIdx.x & 31) == 0) firsts[threadIdx.x >> 5] = above ? __ffs(above) - 1 : 32;
+    __syncthreads();
+    int f = RV_THREADS;                                         // the first of them
+#pragma unroll
+    for (int q = RV_THREADS / 32 - 1; q >= 0; --q)
+      if (firsts[q] < 32) f = 32 * q + firsts[q];
+    __syncthreads();
+    const double l0 = lo;
+    if (f > 0) lo = point(l0, width, f - 1);
+    if (f < RV_THREADS) hi = point(l0, width, f);
   }
-  if (lane == 0) {
+  if (threadIdx.x == 0) {
     const double th = 0.5 * (lo + hi);
     a.th_s[w] = th;
     a.out->theta[w] = ldexp(th, o->exp2);
@@ -923,6 +1249,13 @@ struct DevMem {
     if (e_ != cudaSuccess) return fail(DIRAC_ECUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
   } while (0)
 
+int n_sms() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
+  return std::max(1, n);
+}
+
 ApplyArgs apply_args(const CtxView& v, double e0) {
   ApplyArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -936,28 +1269,47 @@ ApplyArgs apply_args(const CtxView& v, double e0) {
   a.au = mc2 - e0;
   a.ad = -mc2 - e0;
   a.V = v.V;
+  const double vm = std::max(std::fabs(v.vmin), std::fabs(v.vmax));
+  a.vbe = v.V && vm > 0.0 ? std::max(0, std::ilogb(vm) + 1023) : 0;
   return a;
 }
 
-template <int R, bool D, class T>
-cudaError_t launch_apply_rd(const ApplyArgs& a, cudaStream_t s) {
-  const dim3 grid((a.nx + 31) / 32, (a.ny + 7) / 8);
-  if (a.V) eig_apply<R, D, true, T><<<grid, 256, 0, s>>>(a);
-  else eig_apply<R, D, false, T><<<grid, 256, 0, s>>>(a);
+template <int R, bool D>
+cudaError_t launch_apply_rd(const ApplyArgs& a, cudaStream_t s, bool f32) {
+  if (f32) {
+    const dim3 grid((a.nx + 31) / 32, (a.ny + 7) / 8);
+    if (a.V) eig_apply32<R, D, true><<<grid, 256, 0, s>>>(a);
+    else eig_apply32<R, D, false><<<grid, 256, 0, s>>>(a);
+  } else {
+    // four rows a thread, or one on grids of less than two tall tiles per SM,
+    // where the time of one tile counts
+    const int tiles_x = (a.nx + TILE_W - 1) / TILE_W;
+    const bool tall = (long long)tiles_x * ((a.ny + 4 * AP_WARPS - 1) / (4 * AP_WARPS)) >= 2LL * n_sms();
+    const int th = tall ? 4 * AP_WARPS : AP_WARPS;
+    const dim3 grid(tiles_x, (a.ny + th - 1) / th);
+    auto go = [&](auto rpt, auto lanczos) {
+      constexpr int P = decltype(rpt)::value;
+      constexpr bool L = decltype(lanczos)::value;
+      if (a.V) eig_apply64<R, D, true, P, L><<<grid, AP_THREADS, 0, s>>>(a);
+      else eig_apply64<R, D, false, P, L><<<grid, AP_THREADS, 0, s>>>(a);
+    };
+    using std::integral_constant;
+    if (tall) {
+      if (a.ed) go(integral_constant<int, 4>{}, std::true_type{});
+      else go(integral_constant<int, 4>{}, std::false_type{});
+    } else {
+      if (a.ed) go(integral_constant<int, 1>{}, std::true_type{});
+      else go(integral_constant<int, 1>{}, std::false_type{});
+    }
+  }
   return cudaGetLastError();
-}
-
-template <class T>
-cudaError_t launch_apply_t(const CtxView& v, const ApplyArgs& a) {
-  if (v.order == 2) return v.boundary == DIRAC_DIRICHLET ? launch_apply_rd<1, true, T>(a, v.stream)
-                                                         : launch_apply_rd<1, false, T>(a, v.stream);
-  return v.boundary == DIRAC_DIRICHLET ? launch_apply_rd<2, true, T>(a, v.stream)
-                                       : launch_apply_rd<2, false, T>(a, v.stream);
 }
 
 // f32: the mixed-precision product (the Lanczos steps of a DIRAC_MIXED context)
 cudaError_t launch_apply(const CtxView& v, const ApplyArgs& a, bool f32 = false) {
-  return f32 ? launch_apply_t<float>(v, a) : launch_apply_t<double>(v, a);
+  const bool d = v.boundary == DIRAC_DIRICHLET;
+  if (v.order == 2) return d ? launch_apply_rd<1, true>(a, v.stream, f32) : launch_apply_rd<1, false>(a, v.stream, f32);
+  return d ? launch_apply_rd<2, true>(a, v.stream, f32) : launch_apply_rd<2, false>(a, v.stream, f32);
 }
 
 // Device time per kernel kind from CUDA events recorded between consecutive
@@ -1004,13 +1356,6 @@ struct KindTimer {
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
   }
 };
-
-int n_sms() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
-  return std::max(1, n);
-}
 
 }  // namespace eig
 }  // namespace dirac
@@ -1069,9 +1414,13 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
   int cs = (int)std::min<long long>(CH_MAX, std::max<long long>(32, (n + 4LL * sm - 1) / (4LL * sm)));
   cs = (cs + 31) / 32 * 32;
   const int n_dot = (int)std::min<long long>(4LL * sm, (n + cs - 1) / cs);
-  const int n_upd = (int)std::min<long long>(4LL * sm, std::max<long long>(1, (n + 255) / 256));
+  // update: one thread per site where that fills the GPU (a CTA per SM), else eight
+  const int upd_groups = n < 256LL * sm ? 8 : 1;
+  const int upd_sites = 256 / upd_groups;
+  const int n_upd = (int)std::min<long long>(4LL * sm, std::max<long long>(1, (n + upd_sites - 1) / upd_sites));
   const size_t dot_smem_max = (size_t)cs * 2 * sizeof(v4) + sizeof(double2) * (size_t)(kmax + 2);
-  EIG_TRY(cudaFuncSetAttribute(eig_dot, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dot_smem_max));
+  EIG_TRY(cudaFuncSetAttribute(eig_dot<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dot_smem_max));
+  EIG_TRY(cudaFuncSetAttribute(eig_dot<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dot_smem_max));
 
   // device memory: basis slots 0..max_iter, then (folded) one product buffer
   // and the n_want Ritz vectors before sorting
@@ -1210,7 +1559,8 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
     for (int p = 0; p < passes; ++p) {
       DotArgs da{basis, n, j0, i, cs, dpart, vmax, p, ed};
       const size_t smem = (size_t)cs * 2 * sizeof(v4) + sizeof(double2) * (size_t)(count + 1);
-      eig_dot<<<n_dot, 256, smem, s>>>(da);
+      if (cs == 32) eig_dot<true><<<n_dot, 256, smem, s>>>(da);
+      else eig_dot<false><<<n_dot, 256, smem, s>>>(da);
       EIG_TRY(cudaGetLastError());
       EIG_TRY(tm.mark(K_DOT));
       FinishArgs fa{dpart, n_dot, j0, i, i, p, p == passes - 1, reorth ? 1 : 0, sarr, coef, alpha, beta, ed, ashift,
@@ -1221,7 +1571,8 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
       const bool last = p == passes - 1;
       UpdArgs ua{z, basis, n, j0, i, coef, rec, last ? 1 : 0, npart, vmax + 3 * (i + 1) + p,
                  vmax + 3 * (i + 1) + (last ? 2 : 1), ed};
-      eig_update<<<n_upd, 256, 0, s>>>(ua);
+      if (upd_groups == 8) eig_update<8><<<n_upd, 256, 0, s>>>(ua);
+      else eig_update<1><<<n_upd, 256, 0, s>>>(ua);
       EIG_TRY(cudaGetLastError());
       EIG_TRY(tm.mark(K_UPDATE));
     }
@@ -1231,7 +1582,7 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
     ra.k = it;
     eig_ritz_prep<<<1, 256, 0, s>>>(ra);
     EIG_TRY(cudaGetLastError());
-    eig_ritz_values<<<(RITZ_CAP + 3) / 4, 128, 0, s>>>(ra);
+    eig_ritz_values<<<RITZ_CAP, RV_THREADS, 0, s>>>(ra);
     EIG_TRY(cudaGetLastError());
     eig_ritz_tvecs<<<(RITZ_CAP + 3) / 4, 128, 0, s>>>(ra);
     EIG_TRY(cudaGetLastError());

@@ -105,3 +105,85 @@ def test_non_finite_state_is_reported(bad):
     p.step(psi, 1e-4, 5)
     with pytest.raises(DiracError):
         p.sync()
+
+
+def hnorm(g, order, A, V):
+    """Bound of ||H|| of the discretised operator (m c^2 included)."""
+    c, mc2 = 137.036, 137.036 ** 2
+    f = 1.0 if order == 2 else 1.372
+    p = [f / h + abs(a) for h, a in zip((g.dx, g.dy), A)]
+    return np.sqrt(mc2 ** 2 + c * c * (p[0] ** 2 + p[1] ** 2)) + (0.0 if V is None else np.max(np.abs(V)))
+
+
+# short tiles (rows of 4) below two 32 x 16 tiles per SM, tall tiles above
+@pytest.mark.parametrize("nx,ny,order,boundary,hasv,A", [
+    (1, 1, 2, "periodic", False, (0.0, 0.0)), (33, 5, 4, "periodic", True, (3.0, -2.0)),
+    (31, 18, 2, "dirichlet", True, (0.0, 4.0)), (64, 16, 4, "dirichlet", False, (1.0, 0.0)),
+    (513, 420, 2, "periodic", True, (2.0, 1.0)), (705, 333, 4, "dirichlet", False, (0.0, -1.0))])
+def test_hamiltonian_product_matches_oracle(nx, ny, order, boundary, hasv, A):
+    import torch
+    g = wl.Grid(nx, ny, 0.1, 0.13)
+    psi = wl.random_spinor(g, nx + ny)
+    V = wl.random_potential(g, 4, scale=200.0) if hasv else None
+    p = prop_of(g, 1, order, boundary, V, A=A)
+    out = p.apply(torch.from_numpy(psi).cuda()).cpu().numpy()
+    op = ham.Operator(nx, ny, 0.1, 0.13, order=order, V=V, A=A,
+                      boundary=ham.DIRICHLET if boundary == "dirichlet" else ham.PERIODIC)
+    # a row has seven terms, each rounded a few times on either side
+    assert ham.norm(out - ham.apply(op, psi)) <= 16 * U * hnorm(g, order, A, V) * ham.norm(psi)
+
+
+@pytest.mark.parametrize("order", [2, 4])
+def test_hamiltonian_product_keeps_nan_inf_and_tiny_numbers_local(order):
+    """Tiles that fixed point cannot hold take the floating-point form."""
+    import torch
+    g = wl.Grid(96, 70, 0.1, 0.1)
+    psi = wl.random_spinor(g, 3)
+    p = prop_of(g, 1, order, "periodic")
+    clean = p.apply(torch.from_numpy(psi).cuda()).cpu().numpy()
+    psi[20, 40, 0] = np.nan
+    psi[60, 5, 1] = np.inf
+    out = p.apply(torch.from_numpy(psi).cuda()).cpu().numpy()
+    w = order // 2
+    near = np.zeros((70, 96), dtype=bool)
+    for y, x in ((20, 40), (60, 5)):
+        for k in range(-w, w + 1):
+            near[(y + k) % 70, x] = near[y, (x + k) % 96] = True
+    assert np.all(np.isfinite(out[~near])) and not np.any(np.all(np.isfinite(out[near]), axis=-1))
+    assert np.max(np.abs(out[~near] - clean[~near])) <= 16 * U * hnorm(g, order, (0, 0), None) * np.max(np.abs(clean)) / 1e3
+    tiny = wl.random_spinor(g, 3) * 1e-280
+    out = p.apply(torch.from_numpy(tiny).cuda()).cpu().numpy()
+    assert np.max(np.abs(out * 1e280 - clean)) <= 64 * U * hnorm(g, order, (0, 0), None) * 6
+
+
+@pytest.mark.parametrize("nx,ny", [(33, 20), (256, 192), (251, 173)])
+def test_gram_schmidt_reproduces_the_whole_of_t(nx, ny):
+    """All Ritz values of 30 iterations (no convergence asked for): every T entry
+    counts.  Chunks of 32 sites and eight warps per site on the small grid, full
+    chunks and one thread per site on the others."""
+    import torch
+    g = wl.Grid(nx, ny, 0.1, 0.1)
+    V = wl.smoothed_coulomb(g, 20.0, 0.5)
+    start = wl.random_spinor(g, 12)
+    start[:, : nx // 2] *= 1e-3
+    op = ham.Operator(nx, ny, 0.1, 0.1, V=V, shift=137.036 ** 2)
+    ref = lz.lanczos_eigs(op, start, n_want=30, max_iter=30, tol=1e9, window=(-1e9, 1e9), check_every=30)
+    p = prop_of(g, 1, 2, "periodic")
+    p.set_fields(torch.from_numpy(V).cuda(), shift=137.036 ** 2)
+    res = p.eigs(torch.from_numpy(start).cuda(), n_want=30, max_iter=30, tol=1e9, window=(-1e9, 1e9), check_every=30,
+                 vectors=True)
+    assert res.values.size == ref.values.size == 30
+    assert np.max(np.abs(res.values - ref.values)) <= 1e-11 * hnorm(g, 2, (0, 0), V)
+    v = res.vectors.cpu().numpy().reshape(30, -1)
+    assert np.max(np.abs(v.conj() @ v.T - np.eye(30))) <= 1e-12
+
+
+@pytest.mark.parametrize("scale", [1e-140, 1e140])
+def test_eigen_mode_start_vector_scale(scale):
+    import torch
+    g = wl.Grid(40, 33, 0.1, 0.1)
+    start = torch.from_numpy(wl.random_spinor(g, 2)).cuda()
+    p = prop_of(g, 1, 2, "dirichlet")
+    kw = dict(n_want=10, max_iter=20, tol=1e9, window=(-1e9, 1e9), check_every=20)
+    a, b = p.eigs(start, **kw), p.eigs(start * scale, **kw)
+    assert np.max(np.abs(a.values - b.values)) <= 1e-11 * hnorm(g, 2, (0, 0), None)
