@@ -219,7 +219,9 @@ __global__ void __launch_bounds__(QMAX * 32) adj_mmat(const MArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// per-site contraction: with w_j = sum_l M_jl q^_l (each component),
+// per-site contraction: with w_j = sum_l M_jl q^_l (each component, in fixed
+// point, dirac_fixed.cuh: a site's vectors share an exponent, a row of M another;
+// in FP64 these 128 multiply-adds a lane took 0.81 of the FP64 pipe),
 //   dV(x) += Im sum_j conj(q^'_j) . w_j,   A_x: Im sum_j conj(q^'_j) . sigma_x w_j,
 //   A_y: Im sum_j conj(q^'_j) . sigma_y w_j (summed over sites).
 // JW lanes per site (lane j holds the adjoint basis index j).
@@ -238,16 +240,36 @@ struct CArgs {
 };
 
 template <int JW>
-__global__ void __launch_bounds__(256) adj_contract(const CArgs a) {
-  __shared__ double2 Ms[KMAX][KMAX];
+__global__ void __launch_bounds__(256, 3) adj_contract(const CArgs a) {
+  // row j of M as 60-bit fractions of its largest number: re, im, -im
+  __shared__ int4 Mri[JW][JW + 1];
+  __shared__ int2 Mmi[JW][JW + 1];
+  __shared__ int Mbe[JW];
+  // the forward vectors of each warp's sites: limbs of (u.re, u.im), (d.re, d.im)
+  __shared__ int4 qs[8][32][2];
   const int kf = a.fwd->k_used, kb = a.bwd->k_used;
-  for (int t = threadIdx.x; t < KMAX * KMAX; t += blockDim.x) Ms[t / KMAX][t % KMAX] = a.M[t];
+  for (int j = threadIdx.x; j < JW; j += blockDim.x) {
+    int be = 0;
+    for (int l = 0; l < kf; ++l)
+      be = max(be, max(fx::exp_field(a.M[j * KMAX + l].x), fx::exp_field(a.M[j * KMAX + l].y)));
+    Mbe[j] = max(be, 128);
+  }
   __syncthreads();
-  const int lane = threadIdx.x & 31;
+  for (int t = threadIdx.x; t < JW * JW; t += blockDim.x) {
+    const int j = t / JW, l = t % JW;
+    const double2 m = j < kb && l < kf ? a.M[j * KMAX + l] : make_double2(0.0, 0.0);
+    const long long im = fx::to_fixed<60>(m.y, Mbe[j]);
+    const fx::Limbs x = fx::split(fx::to_fixed<60>(m.x, Mbe[j])), y = fx::split(im), z = fx::split(-im);
+    Mri[j][l] = make_int4(x.hi, x.lo, y.hi, y.lo);
+    Mmi[j][l] = make_int2(z.hi, z.lo);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int grp = lane / JW, j = lane % JW;   // site slot in the warp, adjoint index
   constexpr int SPW = 32 / JW;                // sites per warp
   const long long warp_g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+  const int mbe = Mbe[j];
   double accx = 0.0, accy = 0.0;
   for (long long base = warp_g * SPW; base < a.n; base += nwarps * SPW) {
     const long long x = base + grp;
@@ -258,18 +280,50 @@ __global__ void __launch_bounds__(256) adj_contract(const CArgs a) {
     pj = ql;
     if (valid && j < kf) ql = (j == 0) ? a.q1[x] : a.qf[(size_t)(j - 1) * a.n + x];
     if (valid && j < kb) pj = (j == 0) ? a.p1[x] : a.pb[(size_t)(j - 1) * a.n + x];
-    double ur = 0.0, ui = 0.0, dr = 0.0, di = 0.0;   // w_j (upper, lower)
-    for (int l = 0; l < kf; ++l) {
-      const int src = grp * JW + l;
-      const double qx = __shfl_sync(0xffffffffu, ql.x, src), qy = __shfl_sync(0xffffffffu, ql.y, src);
-      const double qz = __shfl_sync(0xffffffffu, ql.z, src), qw = __shfl_sync(0xffffffffu, ql.w, src);
-      const double2 m = Ms[j < kb ? j : 0][l];
-      ur = fma(m.x, qx, fma(-m.y, qy, ur));
-      ui = fma(m.x, qy, fma(m.y, qx, ui));
-      dr = fma(m.x, qz, fma(-m.y, qw, dr));
-      di = fma(m.x, qw, fma(m.y, qz, di));
+    // the site's largest number
+    const unsigned mx = max((unsigned)__double2hiint(ql.x) << 1, (unsigned)__double2hiint(ql.y) << 1);
+    const unsigned mz = max((unsigned)__double2hiint(ql.z) << 1, (unsigned)__double2hiint(ql.w) << 1);
+    unsigned m = max(mx, mz);
+#pragma unroll
+    for (int o = JW / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const int be = max((int)(m >> 21), 128);
+    const fx::Limbs l0 = fx::split(fx::to_fixed<60>(ql.x, be)), l1 = fx::split(fx::to_fixed<60>(ql.y, be));
+    const fx::Limbs l2 = fx::split(fx::to_fixed<60>(ql.z, be)), l3 = fx::split(fx::to_fixed<60>(ql.w, be));
+    __syncwarp();
+    qs[warp][lane][0] = make_int4(l0.hi, l0.lo, l1.hi, l1.lo);
+    qs[warp][lane][1] = make_int4(l2.hi, l2.lo, l3.hi, l3.lo);
+    __syncwarp();
+    // w_j = sum_l M_jl q_l (upper, lower), two vectors' products at a time: the
+    // factors are below 2^60, so x stays below 2^62; w, at most 64 products, below
+    // 2^63 in units of 2^63
+    long long w[4] = {0, 0, 0, 0};
+#pragma unroll 4
+    for (int lb = 0; lb < kf; lb += 2) {
+      fx::Acc s[4];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int l = lb + u;               // (zero from kf on)
+        const int4 qu = qs[warp][grp * JW + l][0], qd = qs[warp][grp * JW + l][1];
+        const int4 mm = Mri[j][l];
+        const int2 mn = Mmi[j][l];
+        const fx::Limbs mr{mm.x, mm.y}, mi{mm.z, mm.w}, mj{mn.x, mn.y};
+        const fx::Limbs ar{qu.x, qu.y}, ai{qu.z, qu.w}, br{qd.x, qd.y}, bi{qd.z, qd.w};
+        s[0].mac(ar, mr);
+        s[0].mac(ai, mj);
+        s[1].mac(ai, mr);
+        s[1].mac(ar, mi);
+        s[2].mac(br, mr);
+        s[2].mac(bi, mj);
+        s[3].mac(bi, mr);
+        s[3].mac(br, mi);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) w[c] += s[c].template value<31>();
     }
-    if (!(valid && j < kb)) { ur = ui = dr = di = 0.0; }
+    // units: 2^63 (2^(be - 1022 - 60)) (2^(mbe - 1022 - 60))
+    const int e = be + mbe - 2101;
+    const double ur = fx::scale2((double)w[0], e), ui = fx::scale2((double)w[1], e);
+    const double dr = fx::scale2((double)w[2], e), di = fx::scale2((double)w[3], e);
     // Im conj(p) . w for the identity, sigma_x (swap) and sigma_y (u' = -i d, d' = i u)
     const double dv = (pj.x * ui - pj.y * ur) + (pj.z * di - pj.w * dr);
     const double dax = (pj.x * di - pj.y * dr) + (pj.z * ui - pj.w * ur);
@@ -581,9 +635,8 @@ dirac_status dirac_adjoint_gradient(dirac_ctx* ctx, const void* psi0_dev, int ns
     for (int k = cnt - 1; k >= 0; --k) {
       const int step = n0 + k;
       const double* a = A_xy_host + 2 * step;
-      // Krylov space of psi_n (the step's result in `work` is not used)
-      ADJ_TRY(cudaMemcpyAsync(work, seg + (size_t)k * n, vb, cudaMemcpyDeviceToDevice, s));
-      ADJ_CHECK(dirac_lanczos_steps(ctx, work, 1, dt, m, 0.0, a, nullptr));
+      // Krylov space of psi_n (not the step)
+      ADJ_CHECK(krylov_space(ctx, seg + (size_t)k * n, work, dt, m, a));
       // Krylov space of lambda_{n+1}, and lambda_n = exp(+i H_n dt) lambda_{n+1}
       ADJ_TRY(cudaMemcpyAsync(lam1, lam, vb, cudaMemcpyDeviceToDevice, s));
       ADJ_CHECK(dirac_lanczos_steps(back.c, lam, 1, -dt, m, 0.0, a, nullptr));

@@ -280,6 +280,7 @@ struct Engine {
   int step_mode = DIRAC_STEP_AUTO;
   int barrier_extra = 0;           // 1 only inside dirac_debug_barrier_timeout
   bool muladd64 = false;           // FP64 kernels in multiply-adds (set by the adjoint for its call)
+  bool keep_psi = false;           // with it, one-launch steps leave psi as it is (dirac_krylov_space)
   int* d_blk_prob = nullptr;
   int* d_step = nullptr;
   // per-call tables: [Problem x nprob][ChebParams x nprob][FieldStep x nfield]
@@ -685,6 +686,7 @@ dirac_status Engine::run(vec4* const* psi, int nsteps, double dt, int m, double 
     if (hp[b].kx != hp[b].ky) lp.iso = 0;
   lp.diri = boundary == DIRAC_DIRICHLET ? 1 : 0;
   lp.tol = tol;
+  lp.keep_psi = keep_psi ? 1 : 0;
   lp.step = d_step;
   lp.redo_budget = redo_budget(precision, m);
   lp.kappa_redo = kappa_redo(precision);
@@ -891,6 +893,20 @@ dirac_status ctx_view(dirac_ctx* ctx, CtxView* v) {
 }
 
 void ctx_muladd64(dirac_ctx* ctx, bool on) { ctx->e.muladd64 = on; }
+
+dirac_status krylov_space(dirac_ctx* ctx, const void* psi_dev, void* work_dev, double dt, int m, const double* A_xy_host) {
+  Engine& e = ctx->e;
+  vec4* psi = static_cast<vec4*>(const_cast<void*>(psi_dev));
+  const bool in_place = e.muladd64 && e.use_step_kernel(1);
+  if (!in_place) {   // the per-pass recombination would overwrite the state
+    CUDA_TRY(cudaMemcpyAsync(work_dev, psi_dev, sizeof(vec4) * (size_t)e.P[0].n, cudaMemcpyDeviceToDevice, e.stream));
+    psi = static_cast<vec4*>(work_dev);
+  }
+  e.keep_psi = in_place;
+  const dirac_status s = e.run(&psi, 1, dt, m, 0.0, A_xy_host);
+  e.keep_psi = false;
+  return s;
+}
 
 dirac_status operator_interval(dirac_ctx* ctx, double ax_max, double ay_max, double* c0, double* half) {
   if (!ctx) return fail(DIRAC_EINVAL, "null context");

@@ -147,6 +147,11 @@ cudaError_t launch_recombine64(const RecombParams& rp, int grid, cudaStream_t s)
 cudaError_t launch_pass_muladd(int order, bool diri, bool hasv, const LaunchParams& p, const LaunchShape& ls,
                                cudaStream_t s);
 
+// The Krylov space of psi for one step (basis and scalars in the context), without
+// the step itself where the multiply-add one-launch kernel runs; `work_dev`: a
+// field that the other forms use as the state.
+dirac_status krylov_space(dirac_ctx* ctx, const void* psi_dev, void* work_dev, double dt, int m, const double* A_xy_host);
+
 // FP64 kernels of this context in multiply-adds from now on (or not)
 void ctx_muladd64(dirac_ctx* ctx, bool on);
 

@@ -177,6 +177,7 @@ struct LaunchParams {
   int has_ay;               // 0: A_y = 0 in every step and problem (host: picks the kernel)
   int iso;                  // kx = ky in every problem (fixed-point FP64 path; host: picks the kernel)
   int diri;                 // Dirichlet boundaries (kernels that take the boundary at run time)
+  int keep_psi;             // multiply-add one-launch step: Krylov space only, psi is left as it is
   double mcc, dt, tol;      // dt = |dt|
   const int* step;          // step counter of the running call (index into fields)
 };
@@ -1203,7 +1204,7 @@ lanczos_step(const __grid_constant__ LaunchParams lp, const __grid_constant__ Co
     __syncthreads();
   }
   const int err = sst.error;
-  if (!err) {
+  if (!err && !lp.keep_psi) {
     // psi <- sum_j C_j q^_j on this CTA's tiles (no CTA reads psi any more)
     if (threadIdx.x <= KMAX) {
       cr_s[threadIdx.x] = sst.coef_re[threadIdx.x];
