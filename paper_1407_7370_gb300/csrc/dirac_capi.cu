@@ -280,7 +280,7 @@ struct Engine {
   int step_mode = DIRAC_STEP_AUTO;
   int barrier_extra = 0;           // 1 only inside dirac_debug_barrier_timeout
   bool muladd64 = false;           // FP64 kernels in multiply-adds (set by the adjoint for its call)
-  bool keep_psi = false;           // with it, one-launch steps leave psi as it is (dirac_krylov_space)
+  bool keep_psi = false;           // with it, one-launch steps leave psi as it is (krylov_space)
   int* d_blk_prob = nullptr;
   int* d_step = nullptr;
   // per-call tables: [Problem x nprob][ChebParams x nprob][FieldStep x nfield]
@@ -364,7 +364,7 @@ int tiles_of(int nx, int ny, int th) { return ((nx + TILE_W - 1) / TILE_W) * ((n
 // asked for by dirac_batch_set_launch_shape (32: the tall tiles, 16: the short
 // ones), 0 for none: short tiles while the tall ones are fewer than two per SM,
 // where a pass takes the time of one tile (m = 20, ms per step, short / tall:
-// 256^2 0.31 / 0.37, 384^2 0.45 / 0.45, 512^2 0.60 / 0.55, 1024^2 1.58 / 1.43).
+// 256^2 0.31 / 0.37, 384^2 0.45 / 0.45, 512^2 0.60 / 0.57, 1024^2 1.58 / 1.42).
 int fx_tile_height(int set, const std::vector<HostProblem>& P, int n_sm) {
   if (set) return set == 32 ? 16 : 8;
   long long t = 0;

@@ -273,8 +273,9 @@ __global__ void __launch_bounds__(256) eig_apply32(const ApplyArgs a) {
 // and its halo as 58-bit (order 4: 55-bit) numbers in shared memory, each row of
 // the operator one sum of products, then times s_i.  Of the FP64 pipe only the
 // four conversions of the result are left; with some 40 multiply-adds a site it
-// bounded the product (2048^2 with V: 342 us, 0.9 TB/s).  Tiles with numbers
-// that are not finite, or none above 2^-894, take the floating-point form.
+// bounded the product (2048^2 with V: 342 us, 0.9 TB/s; now 115 us, 2.6 TB/s,
+// bound by latency and instruction issue).  Tiles with numbers that are not
+// finite, or none above 2^-894, take the floating-point form.
 constexpr int AP_WARPS = 4, AP_THREADS = 32 * AP_WARPS, AP_SLOTS = 16;
 
 template <int R, bool DIRI, bool HAS_V, int AP_RPT, bool LANCZOS>
@@ -501,7 +502,10 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
 // the memory bandwidth delivers the vector; conversion and limb products take
 // 270.  Sums are exact to 2^-56 of the largest product per four sites, then
 // integers over the chunk and FP64 from chunk to chunk.  The FP64 pipe takes
-// every third vector meanwhile, at FP64_SHARE's cost ratio.
+// every third vector meanwhile, at FP64_SHARE's cost ratio (512 to 270).
+// 100 iterations on 1024^2 with two orthogonalisations: 80 ms without that
+// share, 73 with it; the reads take 50 at the copy bandwidth.  In FP64 alone
+// the whole run took 327 ms, now 145.
 // ---------------------------------------------------------------------------
 constexpr int FP64_SHARE = 3;   // one vector in so many goes to the FP64 pipe
 __device__ __forceinline__ bool fp64_vector(int jj, int nw) { return (jj / nw + jj % nw) % FP64_SHARE == FP64_SHARE - 1; }
@@ -674,7 +678,7 @@ struct FinishArgs {
   EigDev* ed;
   double ashift;        // shift of A for the breakdown scale (s direct, 0 folded)
   const unsigned* vmax;
-  int4* rec;            // update record of q^_j: see eig_update
+  int4* rec;            // update record of q^_j (eig_update)
 };
 
 // A coefficient of the update below this part of ||z|| (by |h_j|) is applied in
@@ -727,7 +731,8 @@ __global__ void __launch_bounds__(256) eig_dot_finish(const FinishArgs a) {
 // z -= sum_j coef_j q^_j; with `last`, per-CTA partials of ||z||^2.  Vectors with
 // small coefficients (SMALL_COEF) are accumulated in FP32, as fractions of their
 // own largest number and of z's; the rest in FP64.  Eight FP64 multiply-adds per
-// site and vector took 512 cycles of a sub-partition against the 190 of the read.
+// site and vector took 512 cycles of a sub-partition against the 190 of the read
+// (100 iterations on 1024^2: now 57 ms, the reads 50).
 // Record of vector j: coefficient (re, im) as FP32 in units of z's largest number
 // over q^_j's, q^_j's exponent field, and 1 for FP64.
 // ---------------------------------------------------------------------------

@@ -109,7 +109,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
 
 struct LaunchShape {
   int n_sm;          // SMs of the device
-  int th;            // tile height (32 or 16; fixed-point FP64: 32 or 8)
+  int th;            // tile height (32 or 16; fixed-point FP64: 16 or 8)
   int cta_cap;       // 0: as many CTAs per SM as fit; else at most this many
 };
 

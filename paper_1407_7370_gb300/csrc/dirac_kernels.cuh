@@ -532,11 +532,13 @@ __device__ __forceinline__ double pos_max(double a, double b) {
 // The scalar update of one problem after pass i (as finish_pass, by one warp,
 // the totals in every lane), arranged for latency: a chain of FP64 operations
 // at 64 to 76 cycles each is what every CTA waits for between two passes.  The
+// problem's energy shift comes as an argument (the one-launch step keeps it in
+// shared memory: its fences empty L1, and the read was a round trip to L2).  The
 // two square roots run in two lanes at once, and the products that the state and
 // the next pass need are formed one per lane by the same three multiplications.
 template <bool FX>
 __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* pr, DevState* st, int i, double P, double Y,
-                                   double X) {
+                                         double X, double shift) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const bool ok = fx::exp_field(P) != 0x7ff && fx::exp_field(Y) != 0x7ff && fx::exp_field(X) != 0x7ff && X > 0.0;
@@ -560,7 +562,6 @@ __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* 
   const double psi_norm_old = st->psi_norm, cum_old = st->cum_err, kappa_old = st->kappa_max;
   const int yexp = FX ? (int)st->pc_cur.yexp : 0, yexp_prev = FX ? (int)st->pc_prev.yexp : 0;
   const PassCoef pc_now = st->pc_cur;
-  const double shift = pr->shift;
   __syncwarp();
 
   const double unscale = pow2(-yexp);
@@ -1059,7 +1060,8 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
     if constexpr (F32) {
       // One of P, Y, X per warp: an FP64 addition occupies a sub-partition for 76
       // cycles.  The CTA that completes the problem: each thread its slots, then
-      // quantity j by warp j.  (1024^2: 20.0 -> 18.6 us a pass with finish_fast)
+      // quantity j by warp j.  With finish_fast: 512^2 m = 16, copies included,
+      // 637 -> 626 us a step; 48 problems of 64^2 to 256^2 3.53 -> 3.49 ms.
       static_assert(COOP == false && SUB == 1 && NW >= 4, "FP32 pass");
       if (warp < 3) {
         double v = lane < NW ? red[lane][warp] : 0.0;
@@ -1110,7 +1112,7 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
         __syncthreads();
         if (warp == 0) {
           if (lane == 0) pr->st->counter = 0u;
-          finish_fast<false>(lp, pr, pr->st, i, red[0][0], red[0][1], red[0][2]);
+          finish_fast<false>(lp, pr, pr->st, i, red[0][0], red[0][1], red[0][2], pr->shift);
         }
       }
     } else {

@@ -12,11 +12,11 @@ namespace dirac {
 // Tiles of 32 x TH sites.  A tile worker has fx_warps warps with fx_rows rows a
 // thread; a CTA (one per SM) holds fx_workers of them, so that one worker's loads
 // and barriers overlap the others' arithmetic.  TH = 16: four workers of four
-// warps, four rows a thread (128 registers): 2048^2, m = 20 in 4.65 ms against
-// 4.83 with two workers of eight warps on 32-row tiles and 5.05 with three of
-// eight warps and two rows a thread (80 registers).  TH = 8: three workers of
-// eight warps, one row a thread, for grids of few tiles, where the time of one
-// tile counts (64^2, m = 10: 123 against 167 us).
+// warps, four rows a thread (128 registers): 2048^2, m = 20 in 4.6 ms against 4.83
+// with two workers of eight warps on 32-row tiles and 5.05 with three of eight
+// warps and two rows a thread (80 registers).  TH = 8: three workers of eight
+// warps, one row a thread, for grids of few tiles, where the time of one tile
+// counts (64^2, m = 10: 111 us a step; the tall tiles took 167).
 template <int TH>
 __host__ __device__ constexpr int fx_warps() { return TH == 16 ? 4 : 8; }
 template <int TH>
@@ -186,7 +186,7 @@ __device__ __forceinline__ void pass_sums64(const LaunchParams& lp, const Proble
       __syncthreads();
       if (warp == 0) {
         if (lane == 0) pr->st->counter = 0u;
-        finish_fast<true>(lp, pr, pr->st, i, tot[0], tot[1], tot[2]);
+        finish_fast<true>(lp, pr, pr->st, i, tot[0], tot[1], tot[2], pr->shift);
       }
       __syncthreads();
     }
@@ -210,9 +210,18 @@ __device__ __forceinline__ void pass_sums64(const LaunchParams& lp, const Proble
 // Per tile: load and form (all loads of a thread in flight at once), exponents
 // -> barrier -> fixed point into shared memory, coefficients at the tile's
 // scale -> barrier -> the upper, then the lower components.
+//
+// The FP64 multiply-adds of this pass (40 a site) kept the FP64 pipe, 64 cycles
+// a warp instruction, busy for 0.8 of the time.  Now the pipe is a third busy
+// and the integer pipes 0.40 and 0.46; what bounds the pass is latency, four
+// warps a sub-partition being what 128 registers allow (stall cycles an
+// instruction: fixed latencies 1.9, loads 1.3, shared memory 1.2).  A step of
+// m = 20 with V, A constant: 1024^2 2.50 -> 1.42 ms; 4096^2, m = 10: 17.3 ->
+// 8.4 ms; 64^2, m = 10: 194 -> 111 us.  A pass of 2048^2: 206 us, 2.6 TB/s.
 template <int R, int TH, bool DIRI, bool HAS_V, bool ISO, bool COOP>
 __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevState* coop_st,
-                                            unsigned long long* coop_slots, int step, unsigned epoch) {
+                                            unsigned long long* coop_slots, int step, unsigned epoch,
+                                            double* coop_shift) {
   constexpr int RPT = fx_rows<TH>();
   constexpr int NTS = 32 * fx_warps<TH>();  // threads of a worker
   constexpr int SUB = fx_workers<TH>();
@@ -270,6 +279,7 @@ __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevSta
         if ((j & 7) == 3) c = fs->cAx;
         if ((j & 7) == 4) c = fs->cAy;
         sg.coef[j] = c;
+        if (COOP && TH == 8 && j == 6) *coop_shift = pr->shift;
         if (j == 0) {
           sg.psi = pr->psi;
           sg.basis = static_cast<vec4*>(pr->basis);
@@ -620,7 +630,7 @@ __global__ void __launch_bounds__(fx_threads<TH>(), 1) lanczos_pass64(const __gr
   // programmatic dependent launch: nothing the previous kernel wrote is read
   // before this point
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  pass_body64<R, TH, DIRI, HAS_V, ISO, false>(lp, nullptr, nullptr, *lp.step, 0u);
+  pass_body64<R, TH, DIRI, HAS_V, ISO, false>(lp, nullptr, nullptr, *lp.step, 0u, nullptr);
   // the next kernel may be scheduled now (it waits for our completion)
   asm volatile("griddepcontrol.launch_dependents;");
 }
@@ -629,10 +639,11 @@ __global__ void __launch_bounds__(fx_threads<TH>(), 1) lanczos_pass64(const __gr
 // psi <- sum_j C_j q^_j (Eq. 17), q^_1 = psi, q^_j = basis[j-2] for j >= 2.  In
 // FP64 the 16 multiply-adds per site and vector took 1024 cycles of a
 // sub-partition against the 190 that reading the vector takes; in limbs they
-// take about as long as the read.  Each site has its own scale, that of its
+// take somewhat longer than the read (m = 20, us, in brackets the time of the
+// reads at the copy bandwidth: 256^2 21 (7), 512^2 56 (26), 1024^2 173 (104),
+// 2048^2 649 (415); the FP64 multiply-adds alone would take 530 us at 1024^2).  Each site has its own scale, that of its
 // largest |C_j q^_j| so far (the sums are shifted when a batch of D vectors
-// raises it), so the relative error of every site is about 2^-54 of its
-// largest term.
+// raises it), so the error of every site is about 2^-54 of its largest term.
 // ---------------------------------------------------------------------------
 struct FxCoef {
   fx::Limbs re, im, mim;   // C_j and -Im C_j as 59-bit fractions of 2^(be - 1022)
@@ -745,12 +756,15 @@ lanczos_step64(const __grid_constant__ LaunchParams lp, const __grid_constant__ 
   constexpr int NT = fx_threads<TH>();
   __shared__ DevState sst;
   __shared__ FxCoef fc_s[KMAX + 2];
-  __shared__ double tot[3];
+  __shared__ double tot[3], shift_s;
   __shared__ int failed;
   const Problem* pr = lp.probs;
   DevState* gst = lp.states;
   const int warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) failed = 0;
+  if (threadIdx.x == 0) {
+    failed = 0;
+    if constexpr (TH == 16) shift_s = pr->shift;
+  }
   {
     const unsigned* src = reinterpret_cast<const unsigned*>(gst);
     unsigned* dst = reinterpret_cast<unsigned*>(&sst);
@@ -764,7 +778,7 @@ lanczos_step64(const __grid_constant__ LaunchParams lp, const __grid_constant__ 
     const int i = max(1, sst.cur_pass);
     ++iter;
     unsigned long long* slots = ca.packets + (iter & 1) * 6 * (size_t)ca.cap;
-    pass_body64<R, TH, DIRI, HAS_V, ISO, true>(lp, &sst, slots, step, (unsigned)iter);
+    pass_body64<R, TH, DIRI, HAS_V, ISO, true>(lp, &sst, slots, step, (unsigned)iter, &shift_s);
     // the grid totals, in the same order in every CTA
     collect_partials(slots, ca.bar_count, tot, (unsigned)iter, ca.bar, &failed);
     __syncthreads();
@@ -772,7 +786,7 @@ lanczos_step64(const __grid_constant__ LaunchParams lp, const __grid_constant__ 
       if (threadIdx.x == 0) { gst->error = ERR_BARRIER; gst->stopped = 1; }
       return;   // psi untouched; the host reports the timeout
     }
-    if (warp == 0) finish_fast<true>(lp, pr, &sst, i, tot[0], tot[1], tot[2]);
+    if (warp == 0) finish_fast<true>(lp, pr, &sst, i, tot[0], tot[1], tot[2], shift_s);
     __syncthreads();
   }
   const int err = sst.error;
