@@ -187,3 +187,27 @@ def test_eigen_mode_start_vector_scale(scale):
     kw = dict(n_want=10, max_iter=20, tol=1e9, window=(-1e9, 1e9), check_every=20)
     a, b = p.eigs(start, **kw), p.eigs(start * scale, **kw)
     assert np.max(np.abs(a.values - b.values)) <= 1e-11 * hnorm(g, 2, (0, 0), None)
+
+
+@pytest.mark.parametrize("mode", ["one_launch", "passes"])
+@pytest.mark.parametrize("m", [16, 17])
+def test_gradient_in_both_launch_forms(mode, m):
+    """The backward sweep's Krylov spaces without recombination (one launch) and
+    from a copy of the state (per pass); m up to 16 and above take different
+    contraction widths.  Tolerances of the gradient's parity with the oracle (the
+    Krylov error is below 1e-18)."""
+    import torch
+    from oracle import adjoint as adj
+    C = 137.036
+    g = wl.Grid(6, 5, 0.4, 0.4)
+    V = wl.soft_core(g, 2.0) + 0.3 * wl.random_potential(g, 3, scale=1.0)
+    op = ham.Operator(6, 5, 0.4, 0.4, V=V, shift=C * C)
+    psi0 = wl.positive_energy_packet(g, p0=(2.0, 1.0), sigma_x=0.8)
+    A = np.random.default_rng(3).uniform(-1.0, 1.0, (4, 2))
+    p = prop_of(g, m, 2, "periodic", mode=mode)
+    p.set_fields(torch.from_numpy(V).cuda(), shift=C * C)
+    res = p.adjoint_gradient(torch.from_numpy(psi0).cuda(), 4, 2e-5, m, A, observable="px", checkpoint_every=3)
+    ref = adj.gradient(op, psi0, 2e-5, A, "px", None)
+    dV = res.dV.cpu().numpy().reshape(-1)
+    assert np.max(np.abs(dV - ref.dV)) <= 1e-9 * np.max(np.abs(ref.dV))
+    assert np.max(np.abs(res.dA - ref.dA)) <= 1e-9 * np.max(np.abs(ref.dA))
