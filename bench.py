@@ -39,7 +39,7 @@ CFG = wl.LASER_PACKET_1024
 SITE_BYTES = 32            # complex128 spinor
 PASS_BYTES_PER_SITE = 3 * SITE_BYTES   # read q_i, read q_{i-1}, write q_{i+1} (V = 0)
 PASS_BYTES_PER_SITE_MIXED = 3 * 16      # the same accesses in complex64
-PASS_FLOPS_PER_SITE = 80   # FP64 flops of one Lanczos iteration per site: stencil 44, -beta q 8, two dot products 16, normalisation 12
+PASS_FLOPS_PER_SITE = 80   # flops of one Lanczos iteration per site: stencil 44, -beta q 8, two dot products 16, normalisation 12
 RECOMB_FLOPS_PER_VECTOR = 16   # psi += C_j q_j: a complex multiply-add on both spinor components
 
 
@@ -52,11 +52,12 @@ def STEP_BYTES_PER_SITE_MIXED(m):    # complex64 basis; psi read and written in 
 
 
 # DRAM traffic per launch from the last ncu capture of each kernel on the
-# configured grid, valid only for the kernel sources it was taken with (sha1
-# of dirac_kernels.cuh and dirac_step32.cu).
-TRAFFIC = {"lanczos_step<double>": ("9b89fde1270a", 1.638854e9 + 1.302428e9),
-           "lanczos_pass<float>": ("9b89fde1270a", 33.635584e6 + 0.662016e6),
-           "lanczos_step_m32": ("9b89fde1270a", 316.990208e6 + 487.315200e6)}
+# configured grid, valid only for the kernel sources it was taken with
+# (kernel_sha).
+TRAFFIC_SOURCES = ("dirac_kernels.cuh", "dirac_step32.cu", "dirac_pass64.cuh", "dirac_fixed.cuh")
+TRAFFIC = {"lanczos_step64": ("c644ac97325d", 1.607975e9 + 1.366588e9),
+           "lanczos_pass<float>": ("c644ac97325d", 33.650176e6 + 0.514560e6),
+           "lanczos_step_m32": ("c644ac97325d", 317.762816e6 + 487.556352e6)}
 
 
 def rounded(x, digits=6):
@@ -74,7 +75,7 @@ def rounded(x, digits=6):
 def kernel_sha() -> str:
     import hashlib
     h = hashlib.sha1()
-    for name in ("dirac_kernels.cuh", "dirac_step32.cu"):
+    for name in TRAFFIC_SOURCES:
         h.update(open(os.path.join(ROOT, "paper_1407_7370_gb300", "csrc", name), "rb").read())
     return h.hexdigest()[:12]
 
@@ -107,15 +108,19 @@ def measured_alu_peaks():
         return None
 
 
-def alu_roofline(achieved, alu, kernel, extra=None):
-    """Roofline of an FP64-bound kernel against the measured FP64 peak (the
-    derived one beside it)."""
+def fp64_roofline(gbs, hbm_peak, flops, alu, kernel, extra=None):
+    """Roofline of a kernel with FP64 results.  Its products are taken in fixed
+    point on the integer pipes, which the FP64 peak does not bound, so the roof
+    is the copy bandwidth against the algorithmic bytes; beside it the method's
+    flops as a rate and over the FP64 peak (above 1: more than the FP64 pipe
+    could do)."""
     peak = alu["fp64"] if alu else FP64_PEAK_DERIVED
-    r = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+    r = {"bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
          "kernel": kernel,
-         "peak_source": ("measured by dirac_measure_peak (FP64 FMA chains on every SM)" if alu
-                         else "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"),
-         "peak_derived": FP64_PEAK_DERIVED, "frac_of_derived": achieved / FP64_PEAK_DERIVED}
+         "flops": {"achieved": flops, "fp64_peak": peak, "unit": "TFLOP/s", "over_fp64_peak": flops / peak,
+                   "peak_source": ("measured by dirac_measure_peak (FP64 FMA chains on every SM)" if alu
+                                   else "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"),
+                   "peak_derived": FP64_PEAK_DERIVED}}
     if extra:
         r.update(extra)
     return r
@@ -483,7 +488,7 @@ def measure_batch(args, torch, world, dist, gi, pk):
             b = STEP_BYTES_PER_SITE_MIXED(m) if prec == "mixed" else STEP_BYTES_PER_SITE(m)
             gbs = b * sites / (step_ms / 1e3 / step_n) / 1e9
             hbm_alg = {"achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
-                       "kernel": "lanczos_step_m32" if prec == "mixed" else "lanczos_step<double>",
+                       "kernel": "lanczos_step_m32" if prec == "mixed" else "lanczos_step64",
                        "kernel_avg_us": 1e3 * step_ms / step_n, "bytes_per_site_per_step": b}
         else:
             sb = 16 if prec == "mixed" else 32
@@ -613,9 +618,10 @@ def measure_eigen(torch, gi, pk, side=None, iters=None, alu=None):
     return {"workload": c["name"], "per_z": per_z, "z_of_timing": c["z_main"], "iterations": k, "seconds": t,
             "value": n * k / t, "unit": "site-matvecs/s (Lanczos iterations x sites / s)",
             "ms_per_iteration": 1e3 * t / k, "gpu_launches": res.launches, "kernel_ms": res.ms, "clocks": clk,
-            "roofline": alu_roofline(achieved, alu, "eig_dot + eig_update (Gram-Schmidt, twice)",
-                                     {"traffic": None, "share": gs_ms / max(1e-9, sum(res.ms.values())),
-                                      "flops_per_site_vector": GS_FLOPS_PER_SITE_VECTOR}),
+            "roofline": fp64_roofline(gbytes / (gs_ms / 1e3) / 1e9, hbm_peak, achieved, alu,
+                                      "eig_dot + eig_update (Gram-Schmidt, twice)",
+                                      {"traffic": None, "share": gs_ms / max(1e-9, sum(res.ms.values())),
+                                       "flops_per_site_vector": GS_FLOPS_PER_SITE_VECTOR}),
             "hbm": {"achieved": gbytes / (gs_ms / 1e3) / 1e9, "peak": hbm_peak, "unit": "GB/s",
                     "frac": gbytes / (gs_ms / 1e3) / 1e9 / hbm_peak,
                     "bytes_per_site_vector": GS_BYTES_PER_SITE_VECTOR},
@@ -630,6 +636,7 @@ ADJ_CFG = dict(
          "Coulomb Z=1, a=0.5",
     side=1024, dx=0.05, m=16, dt=2e-4, steps=2000, ncoef=64, block=4, ckpt=50)
 CONTRACT_FLOPS_PER_SITE = 16 * 16 * 16   # 8 FMA per (j, l) pair of the two 16-vector bases
+CONTRACT_BYTES_PER_SITE = 2 * 16 * SITE_BYTES   # both bases read once
 
 
 PAPER_CFG = dict(
@@ -726,11 +733,12 @@ def measure_adjoint(torch, gi, pk, steps=None, alu=None):
            "ms_forward": res.info["ms_forward"], "ms_backward": res.info["ms_backward"],
            "quadrature_nodes": res.info["quadrature_nodes"], "gpu_launches": res.info["launches"],
            "loss": res.loss, "clocks": clk,
-           "roofline": alu_roofline(flops, alu, "adj_contract<16> (per-site bilinear form)",
-                                    {"traffic": None, "kernel_avg_us": per_launch * 1e6,
-                                     "flops_per_site": CONTRACT_FLOPS_PER_SITE,
-                                     "share_of_backward": prof.info["ms_contract"] /
-                                     max(1e-9, prof.info["ms_backward"])})}
+           "roofline": fp64_roofline(CONTRACT_BYTES_PER_SITE * n / per_launch / 1e9, pk.get("hbm_gbs", 6800.0),
+                                     flops, alu, "adj_contract<16> (per-site bilinear form)",
+                                     {"traffic": None, "kernel_avg_us": per_launch * 1e6,
+                                      "flops_per_site": CONTRACT_FLOPS_PER_SITE,
+                                      "share_of_backward": prof.info["ms_contract"] /
+                                      max(1e-9, prof.info["ms_backward"])})}
     prop.close()
     del Vs, psi0
     torch.cuda.empty_cache()
@@ -838,22 +846,22 @@ def _run_ours(args, crop_future):
                               "clocks": r["clocks"]}), flush=True)
         return 0
     bytes_step = g.n_sites * SITE_BYTES
-    # FP64 path: bound by the FP64 pipe
+    # FP64 path
     f = runs["fp64"]
     fk = kernel_stats(f)
     if fk["one_launch"]:
-        f_kernel = "lanczos_step<double>"
+        f_kernel = "lanczos_step64"
         f_flops_site = (PASS_FLOPS_PER_SITE + RECOMB_FLOPS_PER_VECTOR) * m   # one launch = one step
         f_bytes_site = STEP_BYTES_PER_SITE(m)
     else:
-        f_kernel = "lanczos_pass<double>"
+        f_kernel = "lanczos_pass64"
         f_flops_site, f_bytes_site = PASS_FLOPS_PER_SITE, PASS_BYTES_PER_SITE
     flops = f_flops_site * g.n_sites / fk["launch_s"] / 1e12
-    roofline = alu_roofline(flops, alu, f_kernel,
-                            {"traffic": traffic_for(f_kernel, g), "kernel_avg_us": fk["launch_s"] * 1e6,
-                             "kernel_share": fk["share"], "flops_per_site_per_launch": f_flops_site,
-                             "fp32_peak_measured": alu["fp32"] if alu else None})
     f_gbs = f_bytes_site * g.n_sites / fk["launch_s"] / 1e9
+    roofline = fp64_roofline(f_gbs, hbm_peak, flops, alu, f_kernel,
+                             {"traffic": traffic_for(f_kernel, g), "kernel_avg_us": fk["launch_s"] * 1e6,
+                              "kernel_share": fk["share"], "flops_per_site_per_launch": f_flops_site,
+                              "fp32_peak_measured": alu["fp32"] if alu else None})
     if roofline["traffic"] is not None:   # the ncu DRAM bytes of a launch over its live duration
         roofline["dram_gbs"] = roofline["traffic"] / fk["launch_s"] / 1e9
         roofline["dram_frac_of_hbm"] = roofline["dram_gbs"] / hbm_peak

@@ -230,10 +230,12 @@ dirac_status dirac_batch_set_fields(dirac_batch* batch, int problem, const doubl
 
 /*
  * Launch shape of the Lanczos passes: tile height 32 or 16 sites and a cap
- * on resident CTAs per SM (0: no cap).  Without a call the tile height is
- * chosen per run (FP64: from the tile count per SM; mixed: 16).  Used by the
- * autotuner; results do not depend on it beyond the order of floating-point
- * sums.
+ * on resident CTAs per SM (0: no cap).  The FP64 path takes 32 as its tall
+ * tiles (16 rows) and 16 as its short ones (8 rows).  Without a call the
+ * tile height is chosen per run (FP64: from the tile count per SM; mixed:
+ * 16).  Used by the autotuner; results do not depend on it beyond the order
+ * of floating-point sums and, FP64, the exponent that the numbers of a tile
+ * share (2^-58 of its largest).
  */
 dirac_status dirac_batch_set_launch_shape(dirac_batch* batch, int tile_height, int ctas_per_sm);
 

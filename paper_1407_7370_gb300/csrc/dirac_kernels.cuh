@@ -1060,8 +1060,8 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
     if constexpr (F32) {
       // One of P, Y, X per warp: an FP64 addition occupies a sub-partition for 76
       // cycles.  The CTA that completes the problem: each thread its slots, then
-      // quantity j by warp j.  With finish_fast: 512^2 m = 16, copies included,
-      // 637 -> 626 us a step; 48 problems of 64^2 to 256^2 3.53 -> 3.49 ms.
+      // quantity j by warp j.  With finish_fast, two steps of m = 16:
+      // 512^2 from host buffers 637 -> 626 us, 48 problems of 128^2 to 512^2 3.53 -> 3.49 ms.
       static_assert(COOP == false && SUB == 1 && NW >= 4, "FP32 pass");
       if (warp < 3) {
         double v = lane < NW ? red[lane][warp] : 0.0;
