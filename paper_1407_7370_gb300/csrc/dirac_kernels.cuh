@@ -668,6 +668,10 @@ __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* 
   const double vk = __shfl_sync(full, sqrt(vr * vr + vi * vi), i - 1);
   if (!stop) stop = (beta_hat * lp.dt * vk <= lp.tol);               // adaptive Krylov dimension (Sec. 4, Eq. 18)
   if (!stop) return;
+  // several lanes have stored coefficients of a next pass that the tolerance now
+  // calls off: before lane 0 stores those of the next step over them (shuffles
+  // order no memory)
+  __syncwarp();
   // C_j = nu_1 / nu_j * v_j applied to q^_j; Eq. 18 estimate from v_k
   if (lane < i) {
     const double f = nu1 * inv_nu_j;
