@@ -128,7 +128,6 @@ struct ApplyArgs {
   int iter;
   int prologue;         // 1: s_i and beta_{i-1} from norm_part, breakdown test, scale by s_i
   unsigned* vmax;       // largest number of `out` (or null)
-  int vbe;              // exponent field of max |V| (0: V = 0)
 };
 
 template <bool DIRI, class T>
@@ -275,8 +274,12 @@ __global__ void __launch_bounds__(256) eig_apply32(const ApplyArgs a) {
 // four conversions of the result are left; with some 40 multiply-adds a site it
 // bounded the product (2048^2 with V: 342 us, 0.9 TB/s; now 115 us, 2.6 TB/s,
 // bound by latency and instruction issue).  Tiles with numbers that are not
-// finite, or none above 2^-894, take the floating-point form.
+// finite, or none above 2^-894, take the floating-point form.  So do tiles whose
+// V is so uneven that the row of its smallest |V| would have to be computed at a
+// scale more than AP_V_LOSS bits above its own terms (a wall, a spike): there the
+// shared scale costs the digits that FP64 keeps at the sites of small V.
 constexpr int AP_WARPS = 4, AP_THREADS = 32 * AP_WARPS, AP_SLOTS = 16;
+constexpr int AP_V_LOSS = 3;   // of the 5 bits more than FP64's 53 that the numbers of a tile have
 
 template <int R, bool DIRI, bool HAS_V, int AP_RPT, bool LANCZOS>
 __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const ApplyArgs a) {
@@ -285,10 +288,10 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
   constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * AP_TH, HPT = (NH + AP_THREADS - 1) / AP_THREADS;
   __shared__ __align__(16) longlong2 sq[2][(AP_TH + 2 * R) * W];
   __shared__ int2 kt[AP_SLOTS];
-  __shared__ unsigned emax[4];
+  __shared__ unsigned emax[6];   // largest of u, d, q^_{i-1}'s u and d, |V|, and the complement of the smallest |V|
   double s_in = 1.0, csub = 0.0;
   if (LANCZOS && !apply_scalars(a, s_in, csub)) return;
-  if (threadIdx.x < 4) emax[threadIdx.x] = 0u;
+  if (threadIdx.x < 6) emax[threadIdx.x] = 0u;
   __syncthreads();
   const int nx = a.nx, ny = a.ny;
   const int tx = threadIdx.x & 31, tg = threadIdx.x >> 5, lane = tx;
@@ -297,10 +300,11 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
   const int rows_in = x0 + tx < nx ? ny - (y0 + r0) : 0;              // row k is in the grid if k < rows_in
   const size_t idx0 = (size_t)(y0 + r0) * nx + (x0 + tx);             // used where in the grid
   const bool has_sub = LANCZOS && csub != 0.0;
-  double q[AP_RPT][4], p[AP_RPT][4], hq[HPT][4];
+  double q[AP_RPT][4], p[AP_RPT][4], hq[HPT][4], V[AP_RPT];
   int hat[HPT];
 #pragma unroll
   for (int k = 0; k < AP_RPT; ++k) {
+    V[k] = HAS_V && k < rows_in ? a.V[idx0 + (size_t)k * nx] : 0.0;
     // sites beyond the grid's edge are halo of the sites inside
     if (full) {
       const v4 v = a.in[idx0 + (size_t)k * nx];
@@ -353,12 +357,38 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
   m2 = __reduce_max_sync(0xffffffffu, m2);
   m3 = __reduce_max_sync(0xffffffffu, m3);
   if (lane < 4) atomicMax(&emax[lane], lane == 0 ? m0 : lane == 1 ? m1 : lane == 2 ? m2 : m3);
+  if constexpr (HAS_V) {
+    unsigned vhi = 0u, vlo = 0u;
+#pragma unroll
+    for (int k = 0; k < AP_RPT; ++k) {
+      vhi = max(vhi, mag(V[k]));                       // (zero outside the grid)
+      if (k < rows_in) vlo = max(vlo, ~mag(V[k]));
+    }
+    vhi = __reduce_max_sync(0xffffffffu, vhi);
+    vlo = __reduce_max_sync(0xffffffffu, vlo);
+    if (lane < 2) atomicMax(&emax[4 + lane], lane == 0 ? vhi : vlo);
+  }
   __syncthreads();
   // a tile of zeros is exact in fixed point; a largest number that is not finite
   // or below the clamp is not
   bool plain = false;
 #pragma unroll
   for (int c = 0; c < 4; ++c) plain = plain || (emax[c] >> 21) == 0x7ffu || (emax[c] != 0u && (emax[c] >> 21) < 128u);
+  int be[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) be[c] = max((int)(emax[c] >> 21), 128);
+  const int vbe = HAS_V ? (int)(emax[4] >> 21) : 0;   // exponent field of the tile's largest |V| (0: V = 0)
+  if constexpr (HAS_V) {
+    // the scale that V asks for against that of the other terms with the smallest |V|
+    const int vmin = (int)(~emax[5] >> 21), ek = max(fx::exp_field(a.kx), fx::exp_field(a.ky));
+    const int eo = max(ek, max(fx::exp_field(a.cax), fx::exp_field(a.cay)));
+    const int es = has_sub ? fx::exp_field(csub) - fx::exp_field(s_in) + 1023 : -4096;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int others = max(max(vmin, fx::exp_field(h ? a.ad : a.au)) + be[h], max(eo + be[1 - h], es + be[2 + h]));
+      plain = plain || (vbe && vbe + be[h] > others + AP_V_LOSS);
+    }
+  }
   if (plain) {
     unsigned m = 0u;
     for (int k = 0; k < AP_RPT; ++k) {
@@ -371,9 +401,6 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
     if (a.vmax) block_max(m, a.vmax);
     return;
   }
-  int be[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) be[c] = max((int)(emax[c] >> 21), 128);
   const int at0 = (r0 + R) * W + tx + R;
 #pragma unroll
   for (int k = 0; k < AP_RPT; ++k) {
@@ -399,7 +426,7 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
     if (j == 3) c = a.cax;
     if (j == 4) c = a.cay;
     if (j == 5) c = -csub / s_in;
-    const int xe = j == 6 ? (HAS_V ? a.vbe : 0) : fx::exp_field(c);
+    const int xe = j == 6 ? vbe : fx::exp_field(c);
     const int be_x = (j == 0 || j == 6) ? be[ch] : (j == 5 ? be[2 + ch] : be[1 - ch]);
     int sc = xe ? xe + be_x : 0;
     sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, 1));
@@ -415,10 +442,9 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
   const fx::Limbs ks = fx::split(fx::to_fixed<60>(s_in, es));
   const bool scaled = LANCZOS && s_in != 1.0;
   unsigned m = 0u;
-  long long pot[AP_RPT];      // V as 60-bit fractions of the largest |V|
+  long long pot[AP_RPT];      // V as 60-bit fractions of the tile's largest |V|
 #pragma unroll
-  for (int k = 0; k < AP_RPT; ++k)
-    pot[k] = HAS_V && k < rows_in ? fx::to_fixed<60>(a.V[idx0 + (size_t)k * nx], max(a.vbe, 63)) : 0;
+  for (int k = 0; k < AP_RPT; ++k) pot[k] = HAS_V ? fx::to_fixed<60>(V[k], max(vbe, 63)) : 0;
   auto half = [&](auto half_c) {
     constexpr int HALF = decltype(half_c)::value;
     const longlong2* const own = sq[HALF] + at0;
@@ -428,7 +454,7 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
     const int sc = kc[7].x;
     const int texp = sc - 2044 - F + (scaled ? es - 1022 : 0);
     const bool normal = texp >= -1022 && texp <= 960;      // no result leaves the normal range
-    const int vsh = min(max(sc - be[HALF] - max(a.vbe, 63), 0), 63);   // V's scale within the row's
+    const int vsh = min(max(sc - be[HALF] - max(vbe, 63), 0), 63);   // V's scale within the row's
     longlong2 col[AP_RPT + 2 * R];
 #pragma unroll
     for (int j = 0; j < AP_RPT + 2 * R; ++j) col[j] = oth[(j - R) * W];
@@ -1274,8 +1300,6 @@ ApplyArgs apply_args(const CtxView& v, double e0) {
   a.au = mc2 - e0;
   a.ad = -mc2 - e0;
   a.V = v.V;
-  const double vm = std::max(std::fabs(v.vmin), std::fabs(v.vmax));
-  a.vbe = v.V && vm > 0.0 ? std::max(0, std::ilogb(vm) + 1023) : 0;
   return a;
 }
 

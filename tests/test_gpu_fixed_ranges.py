@@ -1,5 +1,6 @@
-"""Call sequences, states and potentials at the ends of what the fixed-point FP64
-kernels take."""
+"""States, potentials and call sequences at the ends of what the fixed-point FP64
+kernels take: wide ranges of values inside a tile or a vector, norms that change
+between calls, adaptive steps, and fields that are refused."""
 import numpy as np
 import pytest
 
@@ -27,6 +28,17 @@ def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
+def bnd(boundary):
+    return ham.DIRICHLET if boundary == "dirichlet" else ham.PERIODIC
+
+
+def hnorm(g, order, A=(0.0, 0.0)):
+    """Bound of ||H|| without V."""
+    f = 1.0 if order == 2 else 1.372
+    p = [f / h + abs(a) for h, a in zip((g.dx, g.dy), A)]
+    return np.sqrt(MC2 ** 2 + C * C * (p[0] ** 2 + p[1] ** 2))
+
+
 # --- adaptive steps ---------------------------------------------------------
 
 @pytest.mark.parametrize("mode", ["one_launch", "passes"])
@@ -49,3 +61,54 @@ def test_adaptive_step_leaves_one_diagonal_for_both_rows(mode, tol):
         au0, ad0 = np.frombuffer(p.export_state()[:40], dtype=np.float64)[3:5]
         assert abs(au0 - ad0 - 2 * MC2) <= 4 * U * 2 * MC2
     assert lz.rel_l2(psi.cpu().numpy(), ref) <= 1e-14 * 3
+
+
+# --- potentials with a wide range -------------------------------------------
+
+@pytest.mark.parametrize("wall", [1e8, 1e12, 1e30])
+@pytest.mark.parametrize("nx,ny,order,boundary", [(75, 41, 2, "periodic"), (97, 50, 4, "dirichlet"),
+                                                  (513, 420, 4, "periodic"), (705, 333, 2, "dirichlet")])
+def test_hamiltonian_product_beside_a_wall(nx, ny, order, boundary, wall):
+    """Sites where V = 0 keep the accuracy that they have without the wall, in the
+    tiles that hold a part of it too; sites of the wall that of the wall's size."""
+    g = wl.Grid(nx, ny, 0.1, 0.13)
+    psi = wl.random_spinor(g, nx)
+    V = np.zeros((ny, nx))
+    V[:, nx - 21:] = wall
+    V[ny // 2, 10] = -wall
+    op = ham.Operator(nx, ny, 0.1, 0.13, order=order, V=V, A=(3.0, -2.0), boundary=bnd(boundary))
+    ref = ham.apply(op, psi)
+    out = make(g, 1, order, boundary, V, A=(3.0, -2.0)).apply(dev(psi)).cpu().numpy()
+    free = V == 0.0
+    assert ham.norm((out - ref)[free]) <= 16 * U * hnorm(g, order, (3.0, -2.0)) * ham.norm(psi)
+    assert ham.norm((out - ref)[~free]) <= 16 * U * wall * ham.norm(psi)
+
+
+@pytest.mark.parametrize("nx,ny,order", [(75, 41, 2), (513, 420, 4)])
+def test_hamiltonian_product_with_potential_over_many_decades(nx, ny, order):
+    g = wl.Grid(nx, ny, 0.1, 0.13)
+    rng = np.random.default_rng(5)
+    psi = wl.random_spinor(g, 3)
+    V = 10.0 ** rng.uniform(-6.0, 14.0, size=(ny, nx)) * rng.choice([-1.0, 1.0], size=(ny, nx))
+    op = ham.Operator(nx, ny, 0.1, 0.13, order=order, V=V)
+    out = make(g, 1, order, V=V).apply(dev(psi)).cpu().numpy()
+    err = np.max(np.abs(out - ham.apply(op, psi)), axis=-1)
+    assert np.max(err / (hnorm(g, order) + np.abs(V))) <= 16 * U * np.max(np.abs(psi))
+
+
+@pytest.mark.parametrize("order", [2, 4])
+def test_eigen_mode_does_not_see_a_wall_out_of_reach(order):
+    """Ten products of half width 1 (2) reach 10 (20) sites; the wall is further
+    away but in the same tiles."""
+    g = wl.Grid(97, 83, 0.1, 0.1)
+    start = np.zeros((83, 97, 2), complex)
+    start[36:46, 40:50] = wl.random_spinor(wl.Grid(10, 10, 0.1, 0.1), 4)
+    V = np.zeros((83, 97))
+    V[:, :18] = V[:, 72:] = 1e14
+    kw = dict(n_want=10, max_iter=10, tol=1e9, window=(-1e9, 1e9), check_every=10)
+    free = make(g, 1, order, shift=MC2).eigs(dev(start), **kw)
+    wall = make(g, 1, order, V=V, shift=MC2).eigs(dev(start), **kw)
+    assert free.values.size == wall.values.size == 10
+    assert np.max(np.abs(free.values - wall.values)) <= 1e-11 * hnorm(g, order)
+
+
