@@ -529,21 +529,22 @@ __device__ __forceinline__ double pos_max(double a, double b) {
   return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
 }
 
-// The scalar update of one problem after pass i (as finish_pass, by one warp,
-// the totals in every lane), arranged for latency: a chain of FP64 operations
-// at 64 to 76 cycles each is what every CTA waits for between two passes.  The
+// The scalar update of one problem after pass i of the fixed-point path (as
+// finish_pass<true>, by one warp, the totals in every lane), arranged for latency: a
+// chain of FP64 operations at 64 to 76 cycles each is what every CTA waits for
+// between two passes (the mixed pass keeps finish_pass: with this one and a sum per
+// warp, two steps of m = 20 at 1024^2 went from 981 to 988 us).  The
 // problem's energy shift comes as an argument (the one-launch step keeps it in
 // shared memory: its fences empty L1, and the read was a round trip to L2).  The
 // two square roots run in two lanes at once, and the products that the state and
 // the next pass need are formed one per lane by the same three multiplications.
-template <bool FX>
-__device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* pr, DevState* st, int i, double P, double Y,
+static __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* pr, DevState* st, int i, double P, double Y,
                                          double X, double shift) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const bool ok = fx::exp_field(P) != 0x7ff && fx::exp_field(Y) != 0x7ff && fx::exp_field(X) != 0x7ff && X > 0.0;
   if (lp.probe || !ok) {
-    finish_pass<FX>(lp, pr, st, i, P, Y, X);
+    finish_pass<true>(lp, pr, st, i, P, Y, X);
     return;
   }
   // everything the update reads, before lane 0 changes it
@@ -556,12 +557,10 @@ __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* 
   const double alpha_next = have_next ? st->alpha[i + 1] : (i >= 2 ? st->alpha[i - 1] : 0.0);
   const double beta_next = have_next ? st->beta[i + 1] : 0.0;
   const double scale_old = i == 1 ? 0.0 : st->scale;
-  // beta_{i-1} is nu_i times: FX 1 / nu_{i-1} (and the scales), else the estimate of pass i - 1
-  const double bfac = i >= 2 ? (FX ? st->inv_nu[i - 1] : st->beta[i - 1]) : 0.0;
+  const double bfac = i >= 2 ? st->inv_nu[i - 1] : 0.0;   // beta_{i-1} = nu_i / nu_{i-1}, and the scales
   const double nu1_old = st->nu[1], alpha1_old = st->alpha[1], beta1_old = st->beta[1];
   const double psi_norm_old = st->psi_norm, cum_old = st->cum_err, kappa_old = st->kappa_max;
-  const int yexp = FX ? (int)st->pc_cur.yexp : 0, yexp_prev = FX ? (int)st->pc_prev.yexp : 0;
-  const PassCoef pc_now = st->pc_cur;
+  const int yexp = (int)st->pc_cur.yexp, yexp_prev = (int)st->pc_prev.yexp;
   __syncwarp();
 
   const double unscale = pow2(-yexp);
@@ -573,17 +572,16 @@ __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* 
   const double y2 = y * y, xy = X * y;
   // lane 0: nu_i; 1: beta_i (estimate); 2: beta_{i-1} from the measured norm;
   // 3: kappa = Y / s2; 4: kappa_redo s2; 5: alpha_i - sigma_i; 8: s2; of the next
-  // pass's coefficients 6: gd, 7: the coupling, 9: g (FX: 1)
+  // pass's coefficients 6: gd, 7: the coupling
   double f0 = D, f1 = y2, f2 = 1.0, f3 = 1.0;
   if (lane == 0) { f0 = xy; f1 = 1.0; }
   if (lane == 1) { f2 = z; f3 = unscale; }
-  if (lane == 2) { f0 = xy; f1 = bfac; f2 = FX ? pow2(-yexp_prev) : 1.0; }
+  if (lane == 2) { f0 = xy; f1 = bfac; f2 = pow2(-yexp_prev); }
   if (lane == 3) { f0 = Y; f1 = X; f2 = z; f3 = z; }
   if (lane == 4) { f2 = lp.kappa_redo; }
   if (lane == 5) { f0 = P; f2 = unscale; }
-  if (lane == 6) { f0 = P; if (!FX) { f2 = z; f3 = xy; } }
-  if (lane == 7) { f2 = y2; f3 = unscale; if (!FX) { f1 = z; f3 = y; } }
-  if (lane == 9) { f0 = z; f1 = FX ? 0.0 : xy; }
+  if (lane == 6) { f0 = P; }
+  if (lane == 7) { f2 = y2; f3 = unscale; }
   const double prod = (f0 * f1) * (f2 * f3);
   // lane 0: the next diagonal mc^2 - s - sigma', 1: -mc^2 - s - sigma', 5: alpha_i
   const double alpha5 = prod + sigma;
@@ -597,13 +595,7 @@ __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* 
   const double sig = redo ? alpha : (have_next || i >= 2 ? alpha_next : alpha);
   const double diag = ((lane == 1 ? -lp.mcc : lp.mcc) - shift) - sig;
   if (redo) {
-    if constexpr (FX) {
-      if (lane < 2) (lane ? st->pc_cur.ad0 : st->pc_cur.au0) = diag;
-    } else if (lane < 2) {
-      const float hi = (float)diag, lo = (float)(diag - (double)hi);
-      if (lane == 0) { st->pc_cur.au0 = diag; st->pc_cur.au_hi = hi; st->pc_cur.au_lo = lo; }
-      else { st->pc_cur.ad0 = diag; st->pc_cur.ad_hi = hi; st->pc_cur.ad_lo = lo; }
-    }
+    if (lane < 2) (lane ? st->pc_cur.ad0 : st->pc_cur.au0) = diag;
     if (lane == 0) {
       st->redo_left = redo_left - 1;
       st->sigma[i] = alpha;
@@ -616,26 +608,11 @@ __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* 
   int stop = (i >= lp.m) || brk;
   const double nu1 = i == 1 ? nu : nu1_old;
   const double psi_norm = i == 1 ? nu : psi_norm_old;
-  if constexpr (FX) {
-    if (!stop) {
-      if (lane == 0) st->pc_prev.yexp = (float)yexp;
-      if (lane < 2) (lane ? st->pc_cur.ad0 : st->pc_cur.au0) = diag;
-      if (lane == 6) st->pc_cur.gd = prod;
-      if (lane == 7) st->pc_cur.e = prod;
-    }
-  } else {
-    // the coefficients and their FP32 copies (the diagonals with the remainder),
-    // one per lane: 0, 1 diagonals, 6 gd, 7 coupling, 9 g
-    const double c = lane < 2 ? diag : prod;
-    const float hi = (float)c, lo = (float)(c - (double)hi);
-    if (!stop) {
-      if (lane == 10) st->pc_prev = pc_now;
-      if (lane == 0) { st->pc_cur.au0 = c; st->pc_cur.au_hi = hi; st->pc_cur.au_lo = lo; }
-      if (lane == 1) { st->pc_cur.ad0 = c; st->pc_cur.ad_hi = hi; st->pc_cur.ad_lo = lo; }
-      if (lane == 6) { st->pc_cur.gd = c; st->pc_cur.gdf = hi; }
-      if (lane == 7) { st->pc_cur.e = c; st->pc_cur.ef = hi; }
-      if (lane == 9) { st->pc_cur.g = c; st->pc_cur.gf = hi; }
-    }
+  if (!stop) {
+    if (lane == 0) st->pc_prev.yexp = (float)yexp;
+    if (lane < 2) (lane ? st->pc_cur.ad0 : st->pc_cur.au0) = diag;
+    if (lane == 6) st->pc_cur.gd = prod;
+    if (lane == 7) st->pc_cur.e = prod;
   }
   if (lane == 0) {
     st->nu[i] = nu;
@@ -648,12 +625,10 @@ __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* 
     if (pos) st->kappa_max = pos_max(kappa_old, kappa);
     if (!stop) {
       st->sigma[i + 1] = sig;
-      if constexpr (FX) {
-        st->pc_cur.g = 1.0;
-        // norm of the next vector: sqrt(s2), by its exponent
-        const int e_nu = pos ? (fx::exp_field(s2) - 1023) >> 1 : 0;
-        st->pc_cur.yexp = (float)max(-1000, min(1000, -(log2_floor(beta_next > 0.0 ? beta_next : beta_hat) + e_nu)));
-      }
+      st->pc_cur.g = 1.0;
+      // norm of the next vector: sqrt(s2), by its exponent
+      const int e_nu = pos ? (fx::exp_field(s2) - 1023) >> 1 : 0;
+      st->pc_cur.yexp = (float)max(-1000, min(1000, -(log2_floor(beta_next > 0.0 ? beta_next : beta_hat) + e_nu)));
       st->cur_pass = i + 1;
     }
   }
@@ -688,8 +663,7 @@ __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Problem* 
     const double s1 = (i == 1) ? alpha : alpha1_old;   // next step's first shift
     const double b1 = (i == 1) ? beta_hat : (i == 2 ? bprev : beta1_old);
     st->sigma[1] = s1;
-    st->pc_cur = make_coef(1.0, 0.0, 0.0, lp.mcc - shift - s1, -lp.mcc - shift - s1,
-                           FX ? next_yexp(b1, nu1) : 0.f);
+    st->pc_cur = make_coef(1.0, 0.0, 0.0, lp.mcc - shift - s1, -lp.mcc - shift - s1, next_yexp(b1, nu1));
     st->sigma_valid = 1;
     st->stopped = 1;
   }
@@ -1061,127 +1035,67 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
     accX = warp_sum(accX);
     if (lane == 0) { red[warp][0] = (double)accP; red[warp][1] = (double)accY; red[warp][2] = (double)accX; }
     __syncthreads();
-    if constexpr (F32) {
-      // One of P, Y, X per warp: an FP64 addition occupies a sub-partition for 76
-      // cycles.  The CTA that completes the problem: each thread its slots, then
-      // quantity j by warp j.  With finish_fast, two steps of m = 16:
-      // 512^2 from host buffers 637 -> 626 us, 48 problems of 128^2 to 512^2 3.53 -> 3.49 ms.
-      static_assert(COOP == false && SUB == 1 && NW >= 4, "FP32 pass");
-      if (warp < 3) {
-        double v = lane < NW ? red[lane][warp] : 0.0;
+    if (warp == 0) {
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+      if (lane < NW) { s0 = red[lane][0]; s1 = red[lane][1]; s2 = red[lane][2]; }
 #pragma unroll
-        for (int o = NW / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) pr->partials[3 * (blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr)) + warp] = v;
+      for (int o = (NW > 16 ? 16 : 8); o > 0; o >>= 1) {   // NW <= 32 warps
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
       }
+      if (lane == 0) {
+        if constexpr (COOP) {
+          coop_slots[3 * blockIdx.x + 0] = s0;
+          coop_slots[3 * blockIdx.x + 1] = s1;
+          coop_slots[3 * blockIdx.x + 2] = s2;
+          last_flag = 0;
+        } else {
+          const int slot = blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr);
+          pr->partials[3 * slot + 0] = s0;
+          pr->partials[3 * slot + 1] = s1;
+          pr->partials[3 * slot + 2] = s2;
+          // release our partial / acquire everybody else's
+          cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
+          last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
+                       (unsigned)pr->ntiles);
+        }
+      }
+    }
+    __syncthreads();
+    if (!COOP && last_flag) {
+      // the problem is complete: the whole CTA sums its slots in a fixed
+      // order (thread-strided, the warp tree, then the warps in turn), the
+      // loads of SB slots per thread in flight at once, so that a pass of
+      // eight CTAs per SM waits for two L2 round trips here, not five
+      const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
+      const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
+      constexpr int SB = 5;
+      double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+      for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
+        double v[SB][3];
+#pragma unroll
+        for (int k = 0; k < SB; ++k) {
+          const int s = s0 + k * NT;
+          const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
+          v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
+          v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
+          v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < SB; ++k) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
+      }
+      t0 = warp_sum(t0);
+      t1 = warp_sum(t1);
+      t2 = warp_sum(t2);
+      if (lane == 0) { red[warp][0] = t0; red[warp][1] = t1; red[warp][2] = t2; }
       __syncthreads();
-      if (threadIdx.x == 0) {
-        // release our partial / acquire everybody else's
-        cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
-        last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
-                     (unsigned)pr->ntiles);
-      }
-      __syncthreads();
-      if (last_flag) {
-        __shared__ double all[3][NT];
-        const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
-        const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
-        constexpr int SB = 5;
-        double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-        for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
-          double v[SB][3];
-#pragma unroll
-          for (int k = 0; k < SB; ++k) {
-            const int s = s0 + k * NT;
-            const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
-            v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
-            v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
-            v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
-          }
-#pragma unroll
-          for (int k = 0; k < SB; ++k) {
-            if (s0 - (int)threadIdx.x + k * NT < nslots) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
-          }
-        }
-        all[0][threadIdx.x] = t0;
-        all[1][threadIdx.x] = t1;
-        all[2][threadIdx.x] = t2;
-        __syncthreads();
-        if (warp < 3) {
-          double v = 0.0;
-#pragma unroll
-          for (int w = 0; w < NW; ++w) v += all[warp][32 * w + lane];
-          v = warp_sum(v);
-          if (lane == 0) red[0][warp] = v;
-        }
-        __syncthreads();
-        if (warp == 0) {
-          if (lane == 0) pr->st->counter = 0u;
-          finish_fast<false>(lp, pr, pr->st, i, red[0][0], red[0][1], red[0][2], pr->shift);
-        }
-      }
-    } else {
       if (warp == 0) {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        if (lane < NW) { s0 = red[lane][0]; s1 = red[lane][1]; s2 = red[lane][2]; }
+        t0 = red[0][0]; t1 = red[0][1]; t2 = red[0][2];
 #pragma unroll
-        for (int o = (NW > 16 ? 16 : 8); o > 0; o >>= 1) {   // NW <= 32 warps
-          s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-          s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        }
-        if (lane == 0) {
-          if constexpr (COOP) {
-            coop_slots[3 * blockIdx.x + 0] = s0;
-            coop_slots[3 * blockIdx.x + 1] = s1;
-            coop_slots[3 * blockIdx.x + 2] = s2;
-            last_flag = 0;
-          } else {
-            const int slot = blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr);
-            pr->partials[3 * slot + 0] = s0;
-            pr->partials[3 * slot + 1] = s1;
-            pr->partials[3 * slot + 2] = s2;
-            // release our partial / acquire everybody else's
-            cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
-            last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
-                         (unsigned)pr->ntiles);
-          }
-        }
-      }
-      __syncthreads();
-      if (!COOP && last_flag) {
-        // the problem is complete: the whole CTA sums its slots in a fixed
-        // order (thread-strided, the warp tree, then the warps in turn), the
-        // loads of SB slots per thread in flight at once, so that a pass of
-        // eight CTAs per SM waits for two L2 round trips here, not five
-        const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
-        const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
-        constexpr int SB = 5;
-        double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-        for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
-          double v[SB][3];
-#pragma unroll
-          for (int k = 0; k < SB; ++k) {
-            const int s = s0 + k * NT;
-            const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
-            v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
-            v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
-            v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
-          }
-#pragma unroll
-          for (int k = 0; k < SB; ++k) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
-        }
-        t0 = warp_sum(t0);
-        t1 = warp_sum(t1);
-        t2 = warp_sum(t2);
-        if (lane == 0) { red[warp][0] = t0; red[warp][1] = t1; red[warp][2] = t2; }
-        __syncthreads();
-        if (warp == 0) {
-          t0 = red[0][0]; t1 = red[0][1]; t2 = red[0][2];
-#pragma unroll
-          for (int w = 1; w < NW; ++w) { t0 += red[w][0]; t1 += red[w][1]; t2 += red[w][2]; }
-          if (lane == 0) pr->st->counter = 0u;
-          finish_pass<false>(lp, pr, pr->st, i, t0, t1, t2);
-        }
+        for (int w = 1; w < NW; ++w) { t0 += red[w][0]; t1 += red[w][1]; t2 += red[w][2]; }
+        if (lane == 0) pr->st->counter = 0u;
+        finish_pass<false>(lp, pr, pr->st, i, t0, t1, t2);
       }
     }
     __syncthreads();

@@ -186,7 +186,7 @@ __device__ __forceinline__ void pass_sums64(const LaunchParams& lp, const Proble
       __syncthreads();
       if (warp == 0) {
         if (lane == 0) pr->st->counter = 0u;
-        finish_fast<true>(lp, pr, pr->st, i, tot[0], tot[1], tot[2], pr->shift);
+        finish_fast(lp, pr, pr->st, i, tot[0], tot[1], tot[2], pr->shift);
       }
       __syncthreads();
     }
@@ -786,7 +786,7 @@ lanczos_step64(const __grid_constant__ LaunchParams lp, const __grid_constant__ 
       if (threadIdx.x == 0) { gst->error = ERR_BARRIER; gst->stopped = 1; }
       return;   // psi untouched; the host reports the timeout
     }
-    if (warp == 0) finish_fast<true>(lp, pr, &sst, i, tot[0], tot[1], tot[2], shift_s);
+    if (warp == 0) finish_fast(lp, pr, &sst, i, tot[0], tot[1], tot[2], shift_s);
     __syncthreads();
   }
   const int err = sst.error;

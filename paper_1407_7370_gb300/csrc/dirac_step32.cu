@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(NT, 2) lanczos_step_m32(const __grid_constant_
               t1 = warp_sum(t1);
               t2 = warp_sum(t2);
               if (lane == 0) pr->st->counter = 0u;
-              finish_fast<false>(lp, pr, pr->st, i, t0, t1, t2, pr->shift);
+              finish_pass<false>(lp, pr, pr->st, i, t0, t1, t2);
             }
           }
         }
@@ -667,7 +667,7 @@ __global__ void __launch_bounds__(NT, 2) lanczos_step_m32(const __grid_constant_
         t0 = warp_sum(t0);
         t1 = warp_sum(t1);
         t2 = warp_sum(t2);
-        finish_fast<false>(lp, lp.probs, &sst, i_single, t0, t1, t2, lp.probs->shift);
+        finish_pass<false>(lp, lp.probs, &sst, i_single, t0, t1, t2);
       }
       __syncthreads();
     }
