@@ -376,6 +376,19 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
     }
     return;
   }
+  // FX: the scale of y^_1 was chosen for the norm of the state before (for 1 after a
+  // multiply-add step).  Where this state's is so far from it that y^ or its sums may
+  // have left the range of FP64, run pass 1 again at this state's scale.
+  if (FX && i == 1 && isfinite(X) && X > 0.0 && st->redo_left > 0) {
+    const double nu = X * rsqrt(X), b1 = st->k_used > 0 ? st->beta[1] : 0.0;
+    const float yexp = next_yexp(b1, nu);
+    const bool far = fabsf(yexp - st->pc_cur.yexp) > 200.f;
+    __syncwarp();
+    if (far) {
+      if (lane == 0) { st->pc_cur.yexp = yexp; st->redo_left -= 1; }
+      return;
+    }
+  }
   if (!ok) {
     if (lane == 0) { st->error = ERR_NONFINITE; st->stopped = 1; }
     return;
@@ -411,7 +424,7 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
   const double y = rsqrt(X);            // 1 / nu_i
   const double nu = X * y;
   const double rX = y * y;
-  const double dd = P * rX;             // alpha_i - sigma_i
+  const double dd = FX ? (P * y) * y : P * rX;   // alpha_i - sigma_i (FX: 1 / X may overflow)
   const double alpha = FX ? fma(dd, unscale, sigma) : sigma + dd;
   const double s2 = fma(-P, dd, Y);     // nu_i^2 beta_i^2 (estimate)
   const double rs = s2 > 0.0 ? rsqrt(s2) : 0.0;
@@ -461,7 +474,7 @@ __device__ inline void finish_pass(const LaunchParams& lp, const Problem* pr, De
       st->sigma[i + 1] = sig;
       st->pc_prev = pc_now;
       if constexpr (FX)
-        st->pc_cur = make_coef(1.0, dd, s2 * rX * unscale, lp.mcc - shift - sig, -lp.mcc - shift - sig,
+        st->pc_cur = make_coef(1.0, dd, (s2 * y * unscale) * y, lp.mcc - shift - sig, -lp.mcc - shift - sig,
                                next_yexp(beta_next_prev > 0.0 ? beta_next_prev : beta_hat, sq));
       else
         st->pc_cur = make_coef(rs, rs * dd, sq * rX, lp.mcc - shift - sig, -lp.mcc - shift - sig);
@@ -542,7 +555,12 @@ static __device__ __noinline__ void finish_fast(const LaunchParams& lp, const Pr
                                          double X, double shift) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const bool ok = fx::exp_field(P) != 0x7ff && fx::exp_field(Y) != 0x7ff && fx::exp_field(X) != 0x7ff && X > 0.0;
+  // X within 2^+-1000, Y and X Y within 2^+-900: then X Y and its differences down to
+  // 2^-106 of it, their roots and the products below are normal numbers.  The rest (a
+  // probe, sums that are not finite, states of extreme norm or scaled for another
+  // one) takes finish_pass.
+  const int ex = fx::exp_field(X) - 1023, ey = fx::exp_field(Y) - 1023;
+  const bool ok = fx::exp_field(P) != 0x7ff && abs(ex) <= 1000 && abs(ey) <= 900 && abs(ex + ey) <= 900;
   if (lp.probe || !ok) {
     finish_pass<true>(lp, pr, st, i, P, Y, X);
     return;

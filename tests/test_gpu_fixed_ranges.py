@@ -112,3 +112,69 @@ def test_eigen_mode_does_not_see_a_wall_out_of_reach(order):
     assert np.max(np.abs(free.values - wall.values)) <= 1e-11 * hnorm(g, order)
 
 
+# --- norms at the ends of the range, and norms that change ------------------
+
+def run_steps(p, psi0, k, n=2, m=8):
+    psi = dev(psi0 * 2.0 ** k)
+    info = p.steps(psi, n, 1e-4, m, info=True)
+    return psi.cpu().numpy() * 2.0 ** -k, info
+
+
+@pytest.mark.parametrize("mode", ["one_launch", "passes"])
+@pytest.mark.parametrize("order", [2, 4])
+def test_norm_may_change_between_calls(mode, order):
+    """The scalars that a context carries from step to step are those of the state
+    before; the next state may have any norm whose square is a normal number."""
+    g = wl.Grid(75, 41, 0.1, 0.1)
+    psi0 = wl.random_spinor(g, 5)
+    V = wl.random_potential(g, 2, scale=30.0)
+    ref, ri = run_steps(make(g, 8, order, V=V, mode=mode), psi0, 0)
+    p = make(g, 8, order, V=V, mode=mode)
+    for k in (0, 260, -260, 480, -480, 0, -300):
+        out, info = run_steps(p, psi0, k)
+        assert lz.rel_l2(out, ref) <= 1e-14 * 2, k
+        assert info.k_used == 8 and not info.breakdown
+        assert np.allclose(info.alpha, ri.alpha, rtol=1e-12, atol=1e-12 * hnorm(g, order))
+        assert np.allclose(info.beta, ri.beta, rtol=1e-9, atol=0)
+
+
+@pytest.mark.parametrize("mode", ["one_launch", "passes"])
+def test_state_whose_squared_norm_is_subnormal(mode):
+    """2^-517 |psi0| ~ 2^-512: the sum of squares keeps 2^-1074 of about 2^-1024, so
+    norms are good to 2^-50 and what they scale likewise."""
+    g = wl.Grid(33, 20, 0.1, 0.1)
+    psi0 = wl.random_spinor(g, 5)
+    psi0 *= 2.0 ** 5 / ham.norm(psi0)
+    ref, _ = run_steps(make(g, 8, mode=mode), psi0, 0)
+    out, info = run_steps(make(g, 8, mode=mode), psi0, -517)
+    assert info.k_used == 8 and not info.breakdown
+    assert lz.rel_l2(out, ref) <= 16 * 2.0 ** -50
+
+
+@pytest.mark.parametrize("k", [260, -260])
+def test_step_of_another_norm_after_a_gradient(k):
+    """The gradient's multiply-add passes leave no scale of y^."""
+    g = wl.Grid(12, 10, 0.4, 0.4)
+    V = wl.soft_core(g, 2.0)
+    psi0 = wl.positive_energy_packet(g, p0=(2.0, 1.0), sigma_x=0.8)
+    ref, _ = run_steps(make(g, 8, V=V, shift=MC2), psi0, 0)
+    p = make(g, 8, V=V, shift=MC2)
+    p.adjoint_gradient(dev(psi0), 2, 2e-5, 8, np.zeros((2, 2)), observable="px", checkpoint_every=2)
+    out, _ = run_steps(p, psi0, k)
+    assert lz.rel_l2(out, ref) <= 1e-14 * 2
+
+
+@pytest.mark.parametrize("mode", ["one_launch", "passes"])
+def test_all_zero_state_stays_zero(mode):
+    import torch
+    g = wl.Grid(70, 40, 0.1, 0.1)
+    p = make(g, 6, mode=mode)
+    psi = torch.zeros((40, 70, 2), dtype=torch.complex128, device="cuda")
+    info = p.steps(psi, 2, 1e-4, 6, info=True)
+    assert not np.any(psi.cpu().numpy()) and info.k_used == 1 and info.norm == 0.0
+    psi0 = wl.random_spinor(g, 1)
+    ref, _ = lz.propagate(ham.Operator(70, 40, 0.1, 0.1), psi0.copy(), 1e-4, 6, 2)
+    out, _ = run_steps(p, psi0, 0, m=6)
+    assert lz.rel_l2(out, ref) <= 1e-14 * 2
+
+
