@@ -106,7 +106,8 @@ dirac_status dirac_set_stream(dirac_ctx* ctx, void* cuda_stream);
  * Eq. 16; dirac_pulse_sin2_mean computes it for a sin^2 pulse).
  * energy_shift s: the recurrence runs on H - s and the step multiplies by
  * exp(-i s dt) -- exact in exact arithmetic; reported alpha are of H - s.
- * Errors: DIRAC_EINVAL (non-finite scalars), DIRAC_ECUDA.
+ * Errors: DIRAC_EINVAL (non-finite scalars or entries of V; the fields stay as
+ * they were), DIRAC_ECUDA.
  */
 dirac_status dirac_set_fields(dirac_ctx* ctx, const double* V_dev, double A_x, double A_y,
                               double energy_shift);

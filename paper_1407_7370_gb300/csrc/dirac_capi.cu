@@ -510,6 +510,16 @@ dirac_status Engine::set_fields(int b, const double* V_dev, double ax, double ay
     return fail(DIRAC_EINVAL, "non-finite field scalar");
   HostProblem& q = P[b];
   if (V_dev) {
+    // checked before anything of the problem changes: a refused V leaves the fields
+    // as they were
+    double* mm = d_partials;   // two doubles of scratch (rewritten by every pass)
+    minmax_kernel<<<1, 256, 0, stream>>>(V_dev, q.n, mm);
+    ++launches;
+    CUDA_TRY(cudaGetLastError());
+    double h[2];
+    CUDA_TRY(cudaMemcpyAsync(h, mm, sizeof(h), cudaMemcpyDeviceToHost, stream));
+    CUDA_TRY(cudaStreamSynchronize(stream));
+    if (!std::isfinite(h[0]) || !std::isfinite(h[1])) return fail(DIRAC_EINVAL, "V has non-finite entries");
     const bool f32 = precision != DIRAC_FP64;
     if (!q.V) CUDA_TRY(cudaMalloc(&q.V, (f32 ? sizeof(float) : sizeof(double)) * q.n));
     if (f32) {
@@ -522,14 +532,8 @@ dirac_status Engine::set_fields(int b, const double* V_dev, double ax, double ay
       q.V64 = static_cast<double*>(q.V);
     }
     CUDA_TRY(cudaMemcpyAsync(q.V64, V_dev, sizeof(double) * q.n, cudaMemcpyDeviceToDevice, stream));
-    double* mm = d_partials;   // two doubles of scratch (rewritten by every pass)
-    minmax_kernel<<<1, 256, 0, stream>>>(V_dev, q.n, mm);
-    ++launches;
-    CUDA_TRY(cudaGetLastError());
-    double h[2];
-    CUDA_TRY(cudaMemcpyAsync(h, mm, sizeof(h), cudaMemcpyDeviceToHost, stream));
+    // the caller may free or change V on any stream once this returns
     CUDA_TRY(cudaStreamSynchronize(stream));
-    if (!std::isfinite(h[0]) || !std::isfinite(h[1])) return fail(DIRAC_EINVAL, "V has non-finite entries");
     q.vmin = h[0];
     q.vmax = h[1];
     q.has_v = true;

@@ -178,3 +178,28 @@ def test_all_zero_state_stays_zero(mode):
     assert lz.rel_l2(out, ref) <= 1e-14 * 2
 
 
+# --- fields that are refused ------------------------------------------------
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_refused_potential_leaves_the_fields_as_they_were(precision, bad):
+    from paper_1407_7370_gb300._native import DiracError
+    g = wl.Grid(70, 40, 0.1, 0.1)
+    psi0 = wl.positive_energy_packet(g, p0=(3.0, 1.0), sigma_x=0.5)
+    V = wl.random_potential(g, 2, scale=30.0)
+    outs = []
+    for refuse in (False, True):
+        p = make(g, 8, V=V, shift=MC2, precision=precision)
+        psi = dev(psi0)
+        p.step(psi, 1e-4, 8)
+        if refuse:
+            W = V * 1e6
+            W[3, 5] = bad
+            with pytest.raises(DiracError):
+                p.set_fields(dev(W), shift=MC2)
+        p.step(psi, 1e-4, 8)
+        p.sync()
+        outs.append(psi.cpu().numpy())
+    assert np.array_equal(outs[0], outs[1])
+
+
