@@ -545,8 +545,8 @@ __device__ __forceinline__ double pos_max(double a, double b) {
 // The scalar update of one problem after pass i of the fixed-point path (as
 // finish_pass<true>, by one warp, the totals in every lane), arranged for latency: a
 // chain of FP64 operations at 64 to 76 cycles each is what every CTA waits for
-// between two passes (the mixed pass keeps finish_pass: with this one and a sum per
-// warp, two steps of m = 20 at 1024^2 went from 981 to 988 us).  The
+// between two passes (the mixed pass keeps finish_pass: with this one, two steps of
+// m = 20 at 1024^2 took 992 us instead of 970).  The
 // problem's energy shift comes as an argument (the one-launch step keeps it in
 // shared memory: its fences empty L1, and the read was a round trip to L2).  The
 // two square roots run in two lanes at once, and the products that the state and
@@ -1053,67 +1053,130 @@ __device__ __forceinline__ void pass_body(const LaunchParams& lp, const DevState
     accX = warp_sum(accX);
     if (lane == 0) { red[warp][0] = (double)accP; red[warp][1] = (double)accY; red[warp][2] = (double)accX; }
     __syncthreads();
-    if (warp == 0) {
-      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-      if (lane < NW) { s0 = red[lane][0]; s1 = red[lane][1]; s2 = red[lane][2]; }
+    if constexpr (F32) {
+      // One of P, Y, X per warp: an FP64 addition occupies a sub-partition for 76
+      // cycles.  The CTA that completes the problem: each thread its slots, then
+      // quantity j by warp j, in the tile buffer (3 KB more of shared memory per CTA
+      // cost as much as this gains).  Against three sums by one warp, two steps:
+      // 1024^2, m = 20 987 -> 970 us, 512^2, m = 16 from host buffers 645 -> 615 us,
+      // 48 problems of 128^2 to 512^2 3.54 -> 3.49 ms.
+      static_assert(COOP == false && SUB == 1 && NW >= 4, "FP32 pass");
+      if (warp < 3) {
+        double v = lane < NW ? red[lane][warp] : 0.0;
 #pragma unroll
-      for (int o = (NW > 16 ? 16 : 8); o > 0; o >>= 1) {   // NW <= 32 warps
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        for (int o = NW / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) pr->partials[3 * (blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr)) + warp] = v;
       }
-      if (lane == 0) {
-        if constexpr (COOP) {
-          coop_slots[3 * blockIdx.x + 0] = s0;
-          coop_slots[3 * blockIdx.x + 1] = s1;
-          coop_slots[3 * blockIdx.x + 2] = s2;
-          last_flag = 0;
-        } else {
-          const int slot = blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr);
-          pr->partials[3 * slot + 0] = s0;
-          pr->partials[3 * slot + 1] = s1;
-          pr->partials[3 * slot + 2] = s2;
-          // release our partial / acquire everybody else's
-          cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
-          last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
-                       (unsigned)pr->ntiles);
-        }
-      }
-    }
-    __syncthreads();
-    if (!COOP && last_flag) {
-      // the problem is complete: the whole CTA sums its slots in a fixed
-      // order (thread-strided, the warp tree, then the warps in turn), the
-      // loads of SB slots per thread in flight at once, so that a pass of
-      // eight CTAs per SM waits for two L2 round trips here, not five
-      const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
-      const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
-      constexpr int SB = 5;
-      double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-      for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
-        double v[SB][3];
-#pragma unroll
-        for (int k = 0; k < SB; ++k) {
-          const int s = s0 + k * NT;
-          const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
-          v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
-          v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
-          v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
-        }
-#pragma unroll
-        for (int k = 0; k < SB; ++k) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
-      }
-      t0 = warp_sum(t0);
-      t1 = warp_sum(t1);
-      t2 = warp_sum(t2);
-      if (lane == 0) { red[warp][0] = t0; red[warp][1] = t1; red[warp][2] = t2; }
       __syncthreads();
-      if (warp == 0) {
-        t0 = red[0][0]; t1 = red[0][1]; t2 = red[0][2];
+      if (threadIdx.x == 0) {
+        // release our partial / acquire everybody else's
+        cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
+        last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
+                     (unsigned)pr->ntiles);
+      }
+      __syncthreads();
+      if (last_flag) {
+        static_assert(sizeof(tile_s) >= 3 * NT * sizeof(double), "partials of the threads");
+        double(*const all)[NT] = reinterpret_cast<double(*)[NT]>(&tile_s[0][0][0]);
+        const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
+        const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
+        constexpr int SB = 5;
+        double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+        for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
+          double v[SB][3];
 #pragma unroll
-        for (int w = 1; w < NW; ++w) { t0 += red[w][0]; t1 += red[w][1]; t2 += red[w][2]; }
-        if (lane == 0) pr->st->counter = 0u;
-        finish_pass<false>(lp, pr, pr->st, i, t0, t1, t2);
+          for (int k = 0; k < SB; ++k) {
+            const int s = s0 + k * NT;
+            const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
+            v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
+            v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
+            v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
+          }
+#pragma unroll
+          for (int k = 0; k < SB; ++k) {
+            if (s0 - (int)threadIdx.x + k * NT < nslots) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
+          }
+        }
+        all[0][threadIdx.x] = t0;
+        all[1][threadIdx.x] = t1;
+        all[2][threadIdx.x] = t2;
+        __syncthreads();
+        if (warp < 3) {
+          double v = 0.0;
+#pragma unroll
+          for (int w = 0; w < NW; ++w) v += all[warp][32 * w + lane];
+          v = warp_sum(v);
+          if (lane == 0) red[0][warp] = v;
+        }
+        __syncthreads();
+        if (warp == 0) {
+          if (lane == 0) pr->st->counter = 0u;
+          finish_pass<false>(lp, pr, pr->st, i, red[0][0], red[0][1], red[0][2]);
+        }
+      }
+    } else {
+      if (warp == 0) {
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+        if (lane < NW) { s0 = red[lane][0]; s1 = red[lane][1]; s2 = red[lane][2]; }
+#pragma unroll
+        for (int o = (NW > 16 ? 16 : 8); o > 0; o >>= 1) {   // NW <= 32 warps
+          s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+          s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+        if (lane == 0) {
+          if constexpr (COOP) {
+            coop_slots[3 * blockIdx.x + 0] = s0;
+            coop_slots[3 * blockIdx.x + 1] = s1;
+            coop_slots[3 * blockIdx.x + 2] = s2;
+            last_flag = 0;
+          } else {
+            const int slot = blockIdx.x - cta_of_tile(pr->tile_begin, cq, cr);
+            pr->partials[3 * slot + 0] = s0;
+            pr->partials[3 * slot + 1] = s1;
+            pr->partials[3 * slot + 2] = s2;
+            // release our partial / acquire everybody else's
+            cuda::atomic_ref<unsigned, cuda::thread_scope_device> ticket(pr->st->counter);
+            last_flag = (ticket.fetch_add((unsigned)seg_tiles, cuda::memory_order_acq_rel) + seg_tiles ==
+                         (unsigned)pr->ntiles);
+          }
+        }
+      }
+      __syncthreads();
+      if (!COOP && last_flag) {
+        // the problem is complete: the whole CTA sums its slots in a fixed
+        // order (thread-strided, the warp tree, then the warps in turn), the
+        // loads of SB slots per thread in flight at once, so that a pass of
+        // eight CTAs per SM waits for two L2 round trips here, not five
+        const int cta_lo = cta_of_tile(pr->tile_begin, cq, cr);
+        const int nslots = cta_of_tile(pr->tile_begin + pr->ntiles - 1, cq, cr) - cta_lo + 1;
+        constexpr int SB = 5;
+        double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+        for (int s0 = threadIdx.x; s0 < nslots; s0 += SB * NT) {
+          double v[SB][3];
+#pragma unroll
+          for (int k = 0; k < SB; ++k) {
+            const int s = s0 + k * NT;
+            const double* ps = pr->partials + 3 * (s < nslots ? s : 0);
+            v[k][0] = s < nslots ? __ldcg(ps + 0) : 0.0;
+            v[k][1] = s < nslots ? __ldcg(ps + 1) : 0.0;
+            v[k][2] = s < nslots ? __ldcg(ps + 2) : 0.0;
+          }
+#pragma unroll
+          for (int k = 0; k < SB; ++k) { t0 += v[k][0]; t1 += v[k][1]; t2 += v[k][2]; }
+        }
+        t0 = warp_sum(t0);
+        t1 = warp_sum(t1);
+        t2 = warp_sum(t2);
+        if (lane == 0) { red[warp][0] = t0; red[warp][1] = t1; red[warp][2] = t2; }
+        __syncthreads();
+        if (warp == 0) {
+          t0 = red[0][0]; t1 = red[0][1]; t2 = red[0][2];
+#pragma unroll
+          for (int w = 1; w < NW; ++w) { t0 += red[w][0]; t1 += red[w][1]; t2 += red[w][2]; }
+          if (lane == 0) pr->st->counter = 0u;
+          finish_pass<false>(lp, pr, pr->st, i, t0, t1, t2);
+        }
       }
     }
     __syncthreads();
