@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(256) eig_apply32(const ApplyArgs a) {
 // CTA, four rows per thread (32 x 4 and one row on small grids), LANCZOS: with the
 // scale and q^_{i-1} of an iteration; as in the FP64 Lanczos pass (dirac_pass64.cuh):
 // exponents of the tile's upper and lower components and of q^_{i-1}, the tile
-// and its halo as 58-bit (order 4: 55-bit) numbers in shared memory, each row of
+// and its halo as 59-bit numbers in shared memory, each row of
 // the operator one sum of products, then times s_i.  Of the FP64 pipe only the
 // four conversions of the result are left; with some 40 multiply-adds a site it
 // bounded the product (2048^2 with V: 342 us, 0.9 TB/s; now 115 us, 2.6 TB/s,
@@ -279,12 +279,12 @@ __global__ void __launch_bounds__(256) eig_apply32(const ApplyArgs a) {
 // scale more than AP_V_LOSS bits above its own terms (a wall, a spike): there the
 // shared scale costs the digits that FP64 keeps at the sites of small V.
 constexpr int AP_WARPS = 4, AP_THREADS = 32 * AP_WARPS, AP_SLOTS = 16;
-constexpr int AP_V_LOSS = 3;   // of the 5 bits more than FP64's 53 that the numbers of a tile have
+constexpr int AP_V_LOSS = 3;   // of the 6 bits more than FP64's 53 that the numbers of a tile have
 
 template <int R, bool DIRI, bool HAS_V, int AP_RPT, bool LANCZOS>
 __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const ApplyArgs a) {
   constexpr int AP_TH = AP_WARPS * AP_RPT;
-  constexpr int W = TILE_W + 2 * R, F = R == 1 ? 58 : 55;
+  constexpr int W = TILE_W + 2 * R, F = fx::ROW_BITS;
   constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * AP_TH, HPT = (NH + AP_THREADS - 1) / AP_THREADS;
   __shared__ __align__(16) longlong2 sq[2][(AP_TH + 2 * R) * W];
   __shared__ int2 kt[AP_SLOTS];
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
   const int vbe = HAS_V ? (int)(emax[4] >> 21) : 0;   // exponent field of the tile's largest |V| (0: V = 0)
   if constexpr (HAS_V) {
     // the scale that V asks for against that of the other terms with the smallest |V|
-    const int vmin = (int)(~emax[5] >> 21), ek = max(fx::exp_field(a.kx), fx::exp_field(a.ky));
+    const int vmin = (int)(~emax[5] >> 21), ek = max(fx::exp_field(a.kx), fx::exp_field(a.ky)) + (R == 1 ? 0 : 3);
     const int eo = max(ek, max(fx::exp_field(a.cax), fx::exp_field(a.cay)));
     const int es = has_sub ? fx::exp_field(csub) - fx::exp_field(s_in) + 1023 : -4096;
 #pragma unroll
@@ -421,8 +421,8 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
     const int j = lane & 7, ch = (lane >> 3) & 1;
     double c = 0.0;
     if (j == 0) c = ch ? a.ad : a.au;
-    if (j == 1) c = a.kx;
-    if (j == 2) c = a.ky;
+    if (j == 1) c = R == 1 ? a.kx : 8.0 * a.kx;   // of the inner difference
+    if (j == 2) c = R == 1 ? a.ky : 8.0 * a.ky;
     if (j == 3) c = a.cax;
     if (j == 4) c = a.cay;
     if (j == 5) c = -csub / s_in;
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
     const int2* const kc = kt + 8 * HALF;
     auto coef = [&](int j) { const int2 v = kc[j]; return fx::Limbs{v.x, v.y}; };
     const int sc = kc[7].x;
-    const int texp = sc - 2044 - F + (scaled ? es - 1022 : 0);
+    const int texp = sc - 2044 - F + (fx::ROW_SHIFT - 28) + (scaled ? es - 1022 : 0);
     const bool normal = texp >= -1022 && texp <= 960;      // no result leaves the normal range
     const int vsh = min(max(sc - be[HALF] - max(vbe, 63), 0), 63);   // V's scale within the row's
     longlong2 col[AP_RPT + 2 * R];
@@ -466,10 +466,10 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
       long long hyr = col[k + R + 1].x - col[k + R - 1].x, hyi = col[k + R + 1].y - col[k + R - 1].y;
       if constexpr (R == 2) {
         const longlong2 xl2 = row[-2], xr2 = row[2];
-        hxr = 8 * hxr - (xl2.x - xr2.x);
-        hxi = 8 * hxi - (xr2.y - xl2.y);
-        hyr = 8 * hyr - (col[k + 2 * R].x - col[k].x);
-        hyi = 8 * hyi - (col[k + 2 * R].y - col[k].y);
+        hxr -= fx::eighth(xl2.x - xr2.x);
+        hxi -= fx::eighth(xr2.y - xl2.y);
+        hyr -= fx::eighth(col[k + 2 * R].x - col[k].x);
+        hyi -= fx::eighth(col[k + 2 * R].y - col[k].y);
       }
       fx::Acc s0, s1;
       s0.mac(fx::split(hxi), coef(1));
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
         s0.mac(c0, kv);
         s1.mac(c1, kv);
       }
-      long long v0 = s0.template value<28>(), v1 = s1.template value<28>();
+      long long v0 = s0.template value<fx::ROW_SHIFT>(), v1 = s1.template value<fx::ROW_SHIFT>();
       if (scaled) {
         fx::Acc t0, t1;
         t0.mac(fx::split(v0), ks);

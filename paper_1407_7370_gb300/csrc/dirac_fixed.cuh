@@ -4,12 +4,13 @@
 // 76 cycles (measured: DFMA 64, DADD and DMUL 76, every conversion from or to
 // FP64 64), while a 32 x 32 + 64 bit integer multiply-add (IMAD.WIDE), a
 // 64-bit add or a 32-bit shift takes 2.  A product of two 60-bit numbers in
-// two 30-bit limbs is three IMAD.WIDE, accumulated exactly over a whole row of
-// the operator and rounded once at its end; converting a double by shifting
-// its mantissa is about a dozen integer instructions.  So sums of products
-// whose operands share a scale are several times cheaper here than on the
-// FP64 pipe, at 5 to 9 bits more than FP64's 53 relative to the largest
-// operand of the group that shares the scale.
+// two 32-bit limbs is three IMAD.WIDE (four with the product of the lower
+// limbs), accumulated without rounding and rounded once at the end of the sum;
+// converting a double by shifting its mantissa is about a dozen integer
+// instructions.  So sums of products whose operands share a scale are several
+// times cheaper here than on the FP64 pipe, at 5 to 7 bits more than FP64's 53
+// relative to the largest operand of the group that shares the scale (and that
+// many fewer for an operand so much smaller than the largest).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -49,10 +50,19 @@ __device__ __forceinline__ Limbs split(long long v) {
   l.hi = (int)(v >> 32) + (int)((unsigned)v >> 31);
   return l;
 }
-__device__ __forceinline__ Limbs neg(const Limbs& a) { return split(-(((long long)a.hi << 32) + a.lo)); }
 
-// Sum of products a b, a and b in limbs, without their lo x lo: h in units of
-// 2^64, x of 2^32 (both wrap like unsigned numbers).
+// Rows of the operator: numbers of ROW_BITS bits times coefficients of 60, summed in
+// Acc and rounded to units of 2^(32 + ROW_SHIFT).  A difference of the stencil (of
+// both directions, in order 4 with an eighth of the outer one: 4.5 numbers) and five
+// more products stay below 2^63 in Acc's cross terms and below 2^62 in the result.
+// The products' lo x lo that Acc drops are each up to 2^-57 of a number times a
+// coefficient, both the largest: with 58 bits (and 55 in order 4, the outer
+// difference not divided) the root mean square error of a row was 2^-57.2 (2^-54.2)
+// of the sum of its terms on an even tile, now 2^-58.1 (2^-57.4); FP64's is 2^-56.8.
+constexpr int ROW_BITS = 59, ROW_SHIFT = 29;
+
+// Sum of products a b, a and b in limbs, without their lo x lo (2^62 each at most,
+// of either sign): h in units of 2^64, x of 2^32 (both wrap like unsigned numbers).
 struct Acc {
   unsigned long long h = 0, x = 0;
   __device__ __forceinline__ void mac(const Limbs& a, const Limbs& b) {
@@ -66,6 +76,8 @@ struct Acc {
     return (long long)((h << (32 - S)) + (unsigned long long)((long long)(x + (1ULL << (S - 1))) >> S));
   }
 };
+
+__device__ __forceinline__ long long eighth(long long v) { return (v + 4) >> 3; }   // rounded
 
 // Sum of squares: x holds half of the cross terms; lo x lo, never negative, is
 // kept too (to 2^-29 of itself): without it the sum had a bias

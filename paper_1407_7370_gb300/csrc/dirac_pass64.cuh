@@ -204,8 +204,11 @@ __device__ __forceinline__ void pass_sums64(const LaunchParams& lp, const Proble
 // sums are fixed point: a tile (with its halo) shares one exponent for the
 // upper and one for the lower components of q^_i, another pair for q^_{i-1},
 // taken from their largest numbers; every row of the operator is one sum of
-// products, rounded once to 2^-60 of its largest term.  y^ enters the sums as
-// 60 bits of the warp's largest number, each tile's sums are exact integers.
+// products, good to 2^-58 of the row's scale (ROW_BITS, dirac_fixed.cuh): a site's y^
+// has the accuracy that FP64 gives it as long as its numbers are within about 2^-4
+// of the largest of its tile, and 2^-58 of that largest below.  y^ enters the sums
+// as 60 bits of the warp's largest number; each tile's sums are integers, the
+// squares with their lowest partial products, P without them.
 //
 // Per tile: load and form (all loads of a thread in flight at once), exponents
 // -> barrier -> fixed point into shared memory, coefficients at the tile's
@@ -227,9 +230,7 @@ __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevSta
   constexpr int SUB = fx_workers<TH>();
   constexpr int NW = SUB * fx_warps<TH>();  // warps
   constexpr int W = TILE_W + 2 * R;
-  // bits of q^ and q^_{i-1}: the differences (2 x 2 terms; order 4: 36) and
-  // the row sums then stay below 2^62
-  constexpr int F = R == 1 ? 58 : 55;
+  constexpr int F = fx::ROW_BITS;           // bits of q^ and q^_{i-1}
   constexpr int NH_ROW = 2 * R * TILE_W, NH = NH_ROW + 2 * R * TH;
   constexpr int HPT = (NH + NTS - 1) / NTS; // halo sites per thread
   static_assert(2 * RPT <= 8, "bounds of the per-tile sums");
@@ -274,8 +275,8 @@ __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevSta
       if (!COOP || epoch == 1u) {   // what the passes of a step share
         const FieldStep* const fs = lp.fields + step * lp.fstride + b;
         double c = 0.0;
-        if ((j & 7) == 1) c = pr->kx;
-        if ((j & 7) == 2) c = pr->ky;
+        if ((j & 7) == 1) c = R == 1 ? pr->kx : 8.0 * pr->kx;   // of the inner difference
+        if ((j & 7) == 2) c = R == 1 ? pr->ky : 8.0 * pr->ky;
         if ((j & 7) == 3) c = fs->cAx;
         if ((j & 7) == 4) c = fs->cAy;
         sg.coef[j] = c;
@@ -490,7 +491,7 @@ __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevSta
         const int sc = kc[7].x;
         const int be_own = max((int)(sm.emax[par][HALF] >> 21), 128);
         bad = bad || be_own == 0x7ff || (sm.emax[par][2 + HALF] >> 21) == 0x7ffu;
-        const int texp = sc - 2044 - F + sg.yexp;       // unit of y as stored
+        const int texp = sc - 2044 - F + (fx::ROW_SHIFT - 28) + sg.yexp;       // unit of y as stored
         // columns of the other half: rows r0 - R .. r0 + RPT + R - 1
         longlong2 col[RPT + 2 * R];
 #pragma unroll
@@ -510,10 +511,10 @@ __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevSta
             long long hyr = col[k + R + 1].x - col[k + R - 1].x, hyi = col[k + R + 1].y - col[k + R - 1].y;
             if constexpr (R == 2) {
               const longlong2 xl2 = row[-2], xr2 = row[2];
-              hxr = 8 * hxr - (xl2.x - xr2.x);
-              hxi = 8 * hxi - (xr2.y - xl2.y);
-              hyr = 8 * hyr - (col[k + 2 * R].x - col[k].x);
-              hyi = 8 * hyi - (col[k + 2 * R].y - col[k].y);
+              hxr -= fx::eighth(xl2.x - xr2.x);
+              hxi -= fx::eighth(xr2.y - xl2.y);
+              hyr -= fx::eighth(col[k + 2 * R].x - col[k].x);
+              hyi -= fx::eighth(col[k + 2 * R].y - col[k].y);
             }
             const fx::Limbs kx = coef(1);
             if constexpr (ISO) {
@@ -557,8 +558,8 @@ __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevSta
               }
             }
           }
-          v[k][0] = s0.template value<28>();
-          v[k][1] = s1.template value<28>();
+          v[k][0] = s0.template value<fx::ROW_SHIFT>();
+          v[k][1] = s1.template value<fx::ROW_SHIFT>();
           if (!full && k >= rows_in) v[k][0] = v[k][1] = 0;
           vor |= (unsigned)((v[k][0] ^ (v[k][0] >> 63)) >> 32) | (unsigned)((v[k][1] ^ (v[k][1] >> 63)) >> 32);
           vec4* const y_out = sg.y_out;
@@ -578,7 +579,7 @@ __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevSta
         for (int k = 0; k < RPT; ++k) {
           longlong2 cv = own[k * W];
           if (!full && k >= rows_in) cv.x = cv.y = 0;
-          const fx::Limbs c0 = fx::split(cv.x << (58 - F)), c1 = fx::split(cv.y << (58 - F));
+          const fx::Limbs c0 = fx::split(cv.x), c1 = fx::split(cv.y);
           const fx::Limbs w0 = fx::split((v[k][0] << sl) >> 2), w1 = fx::split((v[k][1] << sl) >> 2);
           aP.mac(c0, w0);
           aP.mac(c1, w1);
@@ -587,9 +588,9 @@ __device__ __forceinline__ void pass_body64(const LaunchParams& lp, const DevSta
           aX.sqr(c0);
           aX.sqr(c1);
         }
-        // |q^| < 2^58 and |w| < 2^60: eight terms of q^ w stay below 2^61 in
-        // units of 2^60, of w^2 below 2^63, of q^2 below 2^59
-        const int qe = be_own - 1022 - 58, ye = texp + 2 - sl;
+        // |q^| < 2^59 and |w| < 2^60: eight terms of q^ w stay below 2^62 in
+        // units of 2^60, of w^2 below 2^63, of q^2 below 2^61
+        const int qe = be_own - 1022 - F, ye = texp + 2 - sl;
         const fx::WarpSum wp = fx::warp_sum(aP.template value<28>());
         const fx::WarpSum wy = fx::warp_sum(aY.value()), wx = fx::warp_sum(aX.value());
         const int j = lane - 6 * pend_tiles - 3 * HALF;

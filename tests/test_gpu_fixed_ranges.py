@@ -203,3 +203,35 @@ def test_refused_potential_leaves_the_fields_as_they_were(precision, bad):
     assert np.array_equal(outs[0], outs[1])
 
 
+# --- accuracy of the products and sums --------------------------------------
+
+def product_longdouble(psi, g, order, A):
+    """(H - m c^2) psi with periodic boundaries in extended precision."""
+    f = psi.astype(np.clongdouble)
+    c = np.longdouble(C)
+    r = lambda o, ax: np.roll(f, -o, axis=ax)
+
+    def d(ax, h):
+        if order == 2:
+            return (r(1, ax) - r(-1, ax)) * (c / (2 * np.longdouble(h)))
+        return (8 * (r(1, ax) - r(-1, ax)) - (r(2, ax) - r(-2, ax))) * (c / (12 * np.longdouble(h)))
+    px, py = -1j * d(1, g.dx) + c * np.longdouble(A[0]) * f, -1j * d(0, g.dy) + c * np.longdouble(A[1]) * f
+    mc2 = c * c
+    up = px[..., 1] - 1j * py[..., 1]
+    lo = -2 * mc2 * f[..., 1] + px[..., 0] + 1j * py[..., 0]
+    return np.stack((up, lo), axis=-1)
+
+
+@pytest.mark.parametrize("nx,ny", [(96, 64), (544, 400)])
+@pytest.mark.parametrize("order", [2, 4])
+def test_product_is_as_accurate_as_in_fp64(nx, ny, order):
+    """On a state without a wide range the root mean square error of H psi against
+    extended precision is no larger than that of the oracle's FP64 arithmetic."""
+    g = wl.Grid(nx, ny, 0.1, 0.13)
+    A = (7.0, -5.0)
+    psi = wl.random_spinor(g, 9)
+    exact = product_longdouble(psi, g, order, A)
+    op = ham.Operator(nx, ny, 0.1, 0.13, order=order, A=A, shift=MC2)
+    out = make(g, 1, order, A=A, shift=MC2).apply(dev(psi)).cpu().numpy()
+    rms = lambda a: float(np.sqrt(np.mean(np.abs(a - exact) ** 2)))
+    assert rms(out) <= rms(ham.apply(op, psi))
