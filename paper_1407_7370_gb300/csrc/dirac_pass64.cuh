@@ -642,9 +642,12 @@ __global__ void __launch_bounds__(fx_threads<TH>(), 1) lanczos_pass64(const __gr
 // sub-partition against the 190 that reading the vector takes; in limbs they
 // take somewhat longer than the read (m = 20, us, in brackets the time of the
 // reads at the copy bandwidth: 256^2 21 (7), 512^2 56 (26), 1024^2 173 (104),
-// 2048^2 649 (415); the FP64 multiply-adds alone would take 530 us at 1024^2).  Each site has its own scale, that of its
-// largest |C_j q^_j| so far (the sums are shifted when a batch of D vectors
-// raises it), so the error of every site is about 2^-54 of its largest term.
+// 2048^2 649 (415); the FP64 multiply-adds alone would take 530 us at 1024^2).  The upper and the lower component
+// of each site have a scale of their own, that of the largest |C_j q^_j| so far
+// (the sums are shifted when a batch of D vectors raises it).  A product drops up to
+// 2^-56 of that largest term, an eighth of what each of FP64's 2 k multiply-adds may.
+// (One scale for both components left the lower one of a slow packet 2^-48 of itself;
+// the second costs 0.4 % of a step at 1024^2.)
 // ---------------------------------------------------------------------------
 struct FxCoef {
   fx::Limbs re, im, mim;   // C_j and -Im C_j as 59-bit fractions of 2^(be - 1022)
@@ -667,7 +670,7 @@ __device__ __forceinline__ void recombine_site_fx(vec4* psi, const vec4* basis, 
   // units of 2^62
   static_assert(D % 4 == 0 && 2 * KMAX <= 64, "bounds of the sums");
   long long sum[4] = {0, 0, 0, 0};
-  int be = 1100;   // exponent sum of the largest term (terms below 2^-938 count as zero)
+  int beu = 1100, bed = 1100;   // exponent sums of the largest terms (those below 2^-938 count as zero)
   for (int j0 = 1; j0 <= k; j0 += D) {
     vec4 v[D];
 #pragma unroll
@@ -675,18 +678,20 @@ __device__ __forceinline__ void recombine_site_fx(vec4* psi, const vec4* basis, 
       const int j = j0 + u;
       if (j <= k) v[u] = j == 1 ? psi[s] : basis[(size_t)(j - 2) * n + s];
     }
-    int nb = be;
+    int nu = beu, nd = bed;
 #pragma unroll
     for (int u = 0; u < D; ++u) {
       if (j0 + u <= k) {
         const unsigned a = max((unsigned)__double2hiint(v[u].x) << 1, (unsigned)__double2hiint(v[u].y) << 1);
         const unsigned b = max((unsigned)__double2hiint(v[u].z) << 1, (unsigned)__double2hiint(v[u].w) << 1);
-        nb = max(nb, (int)(max(a, b) >> 21) + coef[j0 + u].be);
+        nu = max(nu, (int)(a >> 21) + coef[j0 + u].be);
+        nd = max(nd, (int)(b >> 21) + coef[j0 + u].be);
       }
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) sum[c] = fx::shr_round(sum[c], nb - be);
-    be = nb;
+    for (int c = 0; c < 4; ++c) sum[c] = fx::shr_round(sum[c], c < 2 ? nu - beu : nd - bed);
+    beu = nu;
+    bed = nd;
 #pragma unroll
     for (int g = 0; g < D; g += 4) {
       fx::Acc acc[4];
@@ -694,9 +699,9 @@ __device__ __forceinline__ void recombine_site_fx(vec4* psi, const vec4* basis, 
       for (int u = g; u < g + 4; ++u) {
         if (j0 + u <= k) {
           const FxCoef cf = coef[j0 + u];
-          const int bq = max(be - cf.be, 63);
-          const fx::Limbs x = fx::split(fx::to_fixed<59>(v[u].x, bq)), y = fx::split(fx::to_fixed<59>(v[u].y, bq));
-          const fx::Limbs z = fx::split(fx::to_fixed<59>(v[u].z, bq)), w = fx::split(fx::to_fixed<59>(v[u].w, bq));
+          const int bu = max(beu - cf.be, 63), bd = max(bed - cf.be, 63);
+          const fx::Limbs x = fx::split(fx::to_fixed<59>(v[u].x, bu)), y = fx::split(fx::to_fixed<59>(v[u].y, bu));
+          const fx::Limbs z = fx::split(fx::to_fixed<59>(v[u].z, bd)), w = fx::split(fx::to_fixed<59>(v[u].w, bd));
           acc[0].mac(x, cf.re);
           acc[0].mac(y, cf.mim);
           acc[1].mac(y, cf.re);
@@ -711,12 +716,12 @@ __device__ __forceinline__ void recombine_site_fx(vec4* psi, const vec4* basis, 
       for (int c = 0; c < 4; ++c) sum[c] += acc[c].template value<30>();
     }
   }
-  const int e = be - 2044 - 56;   // 2^62 of the products' 2^-118
+  const int eu = beu - 2044 - 56, ed = bed - 2044 - 56;   // 2^62 of the products' 2^-118
   vec4 o;
-  o.x = fx::to_double(sum[0], e);
-  o.y = fx::to_double(sum[1], e);
-  o.z = fx::to_double(sum[2], e);
-  o.w = fx::to_double(sum[3], e);
+  o.x = fx::to_double(sum[0], eu);
+  o.y = fx::to_double(sum[1], eu);
+  o.z = fx::to_double(sum[2], ed);
+  o.w = fx::to_double(sum[3], ed);
   psi[s] = o;
 }
 

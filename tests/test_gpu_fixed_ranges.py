@@ -235,3 +235,25 @@ def test_product_is_as_accurate_as_in_fp64(nx, ny, order):
     out = make(g, 1, order, A=A, shift=MC2).apply(dev(psi)).cpu().numpy()
     rms = lambda a: float(np.sqrt(np.mean(np.abs(a - exact) ** 2)))
     assert rms(out) <= rms(ham.apply(op, psi))
+
+
+@pytest.mark.parametrize("mode", ["one_launch", "passes"])
+def test_small_component_of_a_slow_packet(mode):
+    """The lower components (2^-20 of the upper ones, and fed by them) keep their own
+    accuracy through the recombination: one short step against the Taylor series."""
+    g = wl.Grid(75, 41, 0.1, 0.1)
+    psi0 = wl.random_spinor(g, 5)
+    psi0[..., 1] *= 2.0 ** -20
+    dt = 1e-9
+    op = ham.Operator(g.nx, g.ny, g.dx, g.dy)
+    ref, term = psi0.copy(), psi0.copy()
+    for k in range(1, 8):   # (dt ||H||)^8 / 8! < 1e-38
+        term = ham.apply(op, term) * (-1j * dt / k)
+        ref = ref + term
+    psi = dev(psi0)
+    p = make(g, 7, mode=mode)
+    p.step(psi, dt, 7)
+    p.sync()
+    out = psi.cpu().numpy()
+    assert lz.rel_l2(out[..., 0], ref[..., 0]) <= 1e-14
+    assert lz.rel_l2(out[..., 1], ref[..., 1]) <= 1e-14
