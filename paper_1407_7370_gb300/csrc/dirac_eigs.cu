@@ -522,16 +522,22 @@ __global__ void __launch_bounds__(AP_THREADS, LANCZOS ? 4 : 5) eig_apply64(const
 // per-CTA partials, the z chunk staged in shared memory, one warp per vector at
 // a time.
 //
-// The products are 58-bit fixed point (dirac_fixed.cuh), each vector relative to
-// its own largest number: in FP64 the eight multiply-adds per site and vector
-// occupied a sub-partition for 512 cycles, against the 190 in which its share of
-// the memory bandwidth delivers the vector; conversion and limb products take
-// 270.  Sums are exact to 2^-56 of the largest product per four sites, then
-// integers over the chunk and FP64 from chunk to chunk.  The FP64 pipe takes
-// every third vector meanwhile, at FP64_SHARE's cost ratio (512 to 270).
-// 100 iterations on 1024^2 with two orthogonalisations: 80 ms without that
-// share, 73 with it; the reads take 50 at the copy bandwidth.  In FP64 alone
-// the whole run took 327 ms, now 145.
+// The products are 58-bit fixed point (dirac_fixed.cuh): in FP64 the eight
+// multiply-adds per site and vector occupied a sub-partition for 512 cycles,
+// against the 190 in which its share of the memory bandwidth delivers the vector;
+// conversion and limb products take about 290.  z has an exponent per site, a
+// vector one per 128 sites (its chunk's largest so far), so that a flat floor under
+// a peak keeps its share of the sum: a product is off by 2^-58 of the largest
+// numbers of its 128 or 256 sites for its truncation and, with either sign, up to
+// 2^-54 for the lower limbs' product; over a chunk that is about 2^-53 of its part
+// of the norms, the rounding of one FP64 operation.  Chunks are added in FP64.  (With
+// one exponent per vector a floor of 2^-29 under a peak, 2^-37 of the squared norm,
+// was lost: three vectors were orthogonal to 5e-12; the exponents cost 2.5 % of the
+// run, keeping the lower limbs' products instead 7 %.)  The FP64 pipe takes every
+// third vector meanwhile, at FP64_SHARE's cost ratio (512 to 290): without that
+// share a run was 5 % longer.  100 iterations on 1024^2 with two orthogonalisations:
+// 327 ms in FP64 alone, now 149; the reads of both kernels take 100 at the copy
+// bandwidth.
 // ---------------------------------------------------------------------------
 constexpr int FP64_SHARE = 3;   // one vector in so many goes to the FP64 pipe
 __device__ __forceinline__ bool fp64_vector(int jj, int nw) { return (jj / nw + jj % nw) % FP64_SHARE == FP64_SHARE - 1; }
@@ -542,8 +548,6 @@ struct DotArgs {
   int j0, j1;           // z is slot j1 + 1
   int cs;               // sites per chunk (multiple of 32, <= CH_MAX)
   double2* part;        // [j - j0][CTA], the last row ||z||^2
-  const unsigned* vmax; // largest numbers: [3 slot + stage]
-  int stage;            // of z: 0 after the product, 1 after the first update
   const EigDev* ed;
 };
 
@@ -553,19 +557,22 @@ struct DotArgs {
 template <bool SHORT>
 __global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
   extern __shared__ __align__(32) unsigned char smem[];
+  __shared__ unsigned zmax[8];
   if (a.ed->breakdown | a.ed->error) return;
   int4* const zu = reinterpret_cast<int4*>(smem);       // limbs of (x, y), then of (z, w)
   int4* const zd = zu + a.cs;
   v4* const zf = reinterpret_cast<v4*>(zd + a.cs);
-  double2* acc = reinterpret_cast<double2*>(zf + a.cs);
+  int* const zk = reinterpret_cast<int*>(zf + a.cs);     // exponent of the chunk's z less that of the site
+  double2* acc = reinterpret_cast<double2*>(zk + a.cs);
   const int count = a.j1 - a.j0 + 2;
   for (int t = threadIdx.x; t < count; t += blockDim.x) acc[t] = make_double2(0.0, 0.0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int zbe = max_field(a.vmax[3 * (a.j1 + 1) + a.stage]);
+  int zbe = 0;                                // exponent field of the largest number of z's chunk
   const long long nchunks = (a.n + a.cs - 1) / a.cs;
   const v4* const z = a.basis + (size_t)(a.j1 + 1) * a.n;
   // limb products of one number of q^ with its z, and the sums of a batch
-  auto products = [&](const v4& v, int t, int be, fx::Acc& ar, fx::Acc& ai, fx::Acc& am) {
+  auto products = [&](const v4& v, int t, int chunk_be, fx::Acc& ar, fx::Acc& ai, fx::Acc& am) {
+    const int be = chunk_be + zk[t];
     const fx::Limbs x = fx::split(fx::to_fixed<58>(v.x, be)), y = fx::split(fx::to_fixed<58>(v.y, be));
     const fx::Limbs z = fx::split(fx::to_fixed<58>(v.z, be)), w = fx::split(fx::to_fixed<58>(v.w, be));
     const int4 s0 = zu[t], s1 = zd[t];
@@ -579,23 +586,31 @@ __global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
     am.mac(y, zx);
     am.mac(w, zz);
   };
-  auto add_sums = [&](int jj, long long re, long long im) {
+  // units: (2^(be - 1022 - 58)) (2^(zbe - 1022 - 58)) 2^60
+  auto add_sums = [&](int jj, int be, long long re, long long im) {
     const fx::WarpSum sr = fx::warp_sum(re), si = fx::warp_sum(im);
-    if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += fx::to_double(lane == 0 ? sr : si);
+    if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += fx::scale2(fx::to_double(lane == 0 ? sr : si), be + zbe - 2100);
   };
   v4 none;
   none.x = none.y = none.z = none.w = 0.0;
   for (long long ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
     const long long base = ch * a.cs;
     const int len = (int)min((long long)a.cs, a.n - base);
+    const int t = threadIdx.x;                // cs <= CH_MAX threads
+    const v4 v = t < len ? z[base + t] : none;
+    const unsigned m = __reduce_max_sync(0xffffffffu, mag4(v));
+    __syncthreads();                          // the chunk before has been read
+    if (lane == 0) zmax[warp] = m;
     __syncthreads();
-    for (int t = threadIdx.x; t < a.cs; t += blockDim.x) {
-      const v4 v = t < len ? z[base + t] : none;
-      const fx::Limbs x = fx::split(fx::to_fixed<58>(v.x, zbe)), y = fx::split(fx::to_fixed<58>(v.y, zbe));
-      const fx::Limbs u = fx::split(fx::to_fixed<58>(v.z, zbe)), w = fx::split(fx::to_fixed<58>(v.w, zbe));
+    zbe = max_field(__reduce_max_sync(0xffffffffu, lane < nw ? zmax[lane] : 0u));
+    if (t < a.cs) {
+      const int sbe = max_field(mag4(v));
+      const fx::Limbs x = fx::split(fx::to_fixed<58>(v.x, sbe)), y = fx::split(fx::to_fixed<58>(v.y, sbe));
+      const fx::Limbs u = fx::split(fx::to_fixed<58>(v.z, sbe)), w = fx::split(fx::to_fixed<58>(v.w, sbe));
       zu[t] = make_int4(x.hi, x.lo, y.hi, y.lo);
       zd[t] = make_int4(u.hi, u.lo, w.hi, w.lo);
       zf[t] = v;
+      zk[t] = zbe - sbe;
     }
     __syncthreads();
     if constexpr (SHORT) {
@@ -608,10 +623,10 @@ __global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
         for (int u = 0; u < 4; ++u) {
           const int jj = j0 + u;
           if (jj < count) {
-            const int be = jj + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + jj) + 2]);
+            const int be = max_field(__reduce_max_sync(0xffffffffu, mag4(v[u])));
             fx::Acc ar, ai, am;
             products(v[u], lane, be, ar, ai, am);
-            add_sums(jj, ar.template value<28>(), ai.template value<28>() - am.template value<28>());
+            add_sums(jj, be, ar.template value<28>(), ai.template value<28>() - am.template value<28>());
           }
         }
       }
@@ -641,7 +656,7 @@ __global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
           if (lane < 2) reinterpret_cast<double*>(acc + jj)[lane] += part;
           continue;
         }
-        const int be = jj + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + jj) + 2]);
+        int be = 0;
         long long re = 0, im = 0;   // at most 32 products below 2^56 in units of 2^60
         for (int t0 = 0; t0 < len; t0 += 128) {
           v4 v[4];
@@ -650,24 +665,25 @@ __global__ void __launch_bounds__(256, 4) eig_dot(const DotArgs a) {
             const int t = t0 + 32 * u + lane;
             v[u] = t < len ? q[t] : none;
           }
-          fx::Acc ar, ai, am;       // at most 16 products each: cross terms below 2^62
+          const int nb = max_field(__reduce_max_sync(0xffffffffu, max(max(mag4(v[0]), mag4(v[1])), max(mag4(v[2]), mag4(v[3])))));
+          if (nb > be) {
+            re = fx::shr_round(re, nb - be);
+            im = fx::shr_round(im, nb - be);
+            be = nb;
+          }
+          fx::Acc ar, ai, am;   // at most 16 products each: cross terms below 2^62
 #pragma unroll
           for (int u = 0; u < 4; ++u)
             products(v[u], min(t0 + 32 * u + lane, a.cs - 1), be, ar, ai, am);   // (zero beyond the end)
           re += ar.template value<28>();
           im += ai.template value<28>() - am.template value<28>();
         }
-        add_sums(jj, re, im);
+        add_sums(jj, be, re, im);
       }
     }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < count; t += blockDim.x) {
-    // units: (2^(be - 1022 - 58)) (2^(zbe - 1022 - 58)) 2^60
-    const int be = t + 1 == count ? zbe : max_field(a.vmax[3 * (a.j0 + t) + 2]);
-    const int e = !SHORT && fp64_vector(t, nw) ? 0 : be + zbe - 2100;
-    a.part[(size_t)t * gridDim.x + blockIdx.x] = make_double2(fx::scale2(acc[t].x, e), fx::scale2(acc[t].y, e));
-  }
+  for (int t = threadIdx.x; t < count; t += blockDim.x) a.part[(size_t)t * gridDim.x + blockIdx.x] = acc[t];
 }
 
 // <q, z> of one vector in FP64: per-CTA partials (the folded mode's Rayleigh quotients)
@@ -1447,7 +1463,8 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
   const int upd_groups = n < 256LL * sm ? 8 : 1;
   const int upd_sites = 256 / upd_groups;
   const int n_upd = (int)std::min<long long>(4LL * sm, std::max<long long>(1, (n + upd_sites - 1) / upd_sites));
-  const size_t dot_smem_max = (size_t)cs * 2 * sizeof(v4) + sizeof(double2) * (size_t)(kmax + 2);
+  const size_t z_smem = (size_t)cs * (2 * sizeof(v4) + sizeof(int));   // a chunk of z: limbs, numbers, exponents
+  const size_t dot_smem_max = z_smem + sizeof(double2) * (size_t)(kmax + 2);
   EIG_TRY(cudaFuncSetAttribute(eig_dot<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dot_smem_max));
   EIG_TRY(cudaFuncSetAttribute(eig_dot<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dot_smem_max));
 
@@ -1586,8 +1603,8 @@ dirac_status dirac_lanczos_eigs(dirac_ctx* ctx, const void* start_dev, int n_wan
     const int j0 = reorth ? 0 : i;
     const int count = i - j0 + 1;
     for (int p = 0; p < passes; ++p) {
-      DotArgs da{basis, n, j0, i, cs, dpart, vmax, p, ed};
-      const size_t smem = (size_t)cs * 2 * sizeof(v4) + sizeof(double2) * (size_t)(count + 1);
+      DotArgs da{basis, n, j0, i, cs, dpart, ed};
+      const size_t smem = z_smem + sizeof(double2) * (size_t)(count + 1);
       if (cs == 32) eig_dot<true><<<n_dot, 256, smem, s>>>(da);
       else eig_dot<false><<<n_dot, 256, smem, s>>>(da);
       EIG_TRY(cudaGetLastError());

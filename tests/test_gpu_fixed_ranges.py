@@ -257,3 +257,24 @@ def test_small_component_of_a_slow_packet(mode):
     out = psi.cpu().numpy()
     assert lz.rel_l2(out[..., 0], ref[..., 0]) <= 1e-14
     assert lz.rel_l2(out[..., 1], ref[..., 1]) <= 1e-14
+
+
+def ritz_gram(p, start, k):
+    """|Y^H Y - 1| of all Ritz vectors Y of k iterations, and their values."""
+    import torch
+    res = p.eigs(dev(start), n_want=k, max_iter=k, tol=1e9, window=(-1e9, 1e9), check_every=k, vectors=True)
+    assert res.values.size == k
+    v = res.vectors.reshape(k, -1)
+    return (v.conj() @ v.T - torch.eye(k, device=v.device)).abs().cpu().numpy(), res.values
+
+
+def test_gram_schmidt_of_a_peak_on_a_flat_floor():
+    """The floor (2^-29 of the peak, a million sites) carries 2^-37 of the squared
+    norm: products of small numbers count.  Three vectors: nine inner products, each
+    good to a few 2^-53 of the norms, and T's eigenvectors, whose values are far
+    apart, as good."""
+    g = wl.Grid(1024, 1024, 0.1, 0.1)
+    start = wl.random_spinor(g, 12) * 2.0 ** -29
+    start[500, 500] = (1.0, 0.5j)
+    gram, _ = ritz_gram(make(g, 1, shift=MC2), start, 3)
+    assert np.max(gram) <= 256 * U
