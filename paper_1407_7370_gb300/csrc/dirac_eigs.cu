@@ -724,10 +724,15 @@ struct FinishArgs {
 };
 
 // A coefficient of the update below this part of ||z|| (by |h_j|) is applied in
-// FP32: its products' rounding, 2^-24 of it, summed over at most 8192 vectors,
-// stays below 2^-53 ||z||.  After the first orthogonalisation, and for all but
-// the last one or two vectors before it, the coefficients are far smaller.
-constexpr double SMALL_COEF = 0x1p-36;
+// FP32, in sums of at most FP32_RUN vectors that are then added in FP64.  Such a
+// sum's terms are at most 2^-38 ||z|| each, so that its 256 roundings come to at most
+// 256 2^-24 64 2^-38 ||z||, 2^-55 ||z|| a vector (the truncation of the numbers, 2^-23
+// of a term, is far less): an eighth of what the two roundings of the FP64
+// multiply-adds may come to, however many vectors there are.  After the first
+// orthogonalisation, and for all but the last one or two vectors before it, the
+// coefficients are far smaller.  (Runs of 32 vectors made the kernel 5 % slower.)
+constexpr double SMALL_COEF = 0x1p-38;
+constexpr int FP32_RUN = 128;
 
 __global__ void __launch_bounds__(256) eig_dot_finish(const FinishArgs a) {
   if (a.ed->breakdown | a.ed->error) return;
@@ -774,7 +779,7 @@ __global__ void __launch_bounds__(256) eig_dot_finish(const FinishArgs a) {
 // small coefficients (SMALL_COEF) are accumulated in FP32, as fractions of their
 // own largest number and of z's; the rest in FP64.  Eight FP64 multiply-adds per
 // site and vector took 512 cycles of a sub-partition against the 190 of the read
-// (100 iterations on 1024^2: now 57 ms, the reads 50).
+// (100 iterations on 1024^2: now 58 ms, the reads 50).
 // Record of vector j: coefficient (re, im) as FP32 in units of z's largest number
 // over q^_j's, q^_j's exponent field, and 1 for FP64.
 // ---------------------------------------------------------------------------
@@ -844,6 +849,15 @@ __global__ void __launch_bounds__(256, 4) eig_update(const UpdArgs a) {
     zv.x = zv.y = zv.z = zv.w = 0.0;
     if (grp == 0) zv = a.z[in ? x : 0];
     float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
+    // the FP32 sums, in units of 2^(zbe - 1022), into z
+    auto flush = [&]() {
+      const double unit = __hiloint2double(zbe << 20, 0);
+      zv.x = fma((double)(-2.f * f0), unit, zv.x);
+      zv.y = fma((double)(-2.f * f1), unit, zv.y);
+      zv.z = fma((double)(-2.f * f2), unit, zv.z);
+      zv.w = fma((double)(-2.f * f3), unit, zv.w);
+      f0 = f1 = f2 = f3 = 0.f;
+    };
     const v4* __restrict__ q = a.basis + (size_t)a.j0 * a.n + (in ? x : 0);
     auto one = [&](int jj, const v4& v, const int4& rc) {
       if (rc.w) {
@@ -858,7 +872,7 @@ __global__ void __launch_bounds__(256, 4) eig_update(const UpdArgs a) {
         f3 = fmaf(cr, qw, fmaf(ci, qz, f3));
       }
     };
-    int jj = 4 * grp;
+    int jj = 4 * grp, run = 0;
     for (; jj + 4 <= count; jj += 4 * GROUPS) {
       const v4 q0 = q[(size_t)jj * a.n], q1 = q[(size_t)(jj + 1) * a.n];
       const v4 q2 = q[(size_t)(jj + 2) * a.n], q3 = q[(size_t)(jj + 3) * a.n];
@@ -867,6 +881,11 @@ __global__ void __launch_bounds__(256, 4) eig_update(const UpdArgs a) {
       one(jj + 1, q1, r1);
       one(jj + 2, q2, r2);
       one(jj + 3, q3, r3);
+      run += 4;
+      if (run == FP32_RUN - 4) {     // (up to three more come after the last four)
+        flush();
+        run = 0;
+      }
     }
     for (; jj < count; ++jj) one(jj, q[(size_t)jj * a.n], __ldg(a.rec + jj));   // the last quad's owner
     if constexpr (GROUPS > 1) {
@@ -881,17 +900,13 @@ __global__ void __launch_bounds__(256, 4) eig_update(const UpdArgs a) {
           if (p.x != 0.0 || p.y != 0.0 || p.z != 0.0 || p.w != 0.0) {
             zv.x += p.x; zv.y += p.y; zv.z += p.z; zv.w += p.w;
           }
-          f0 += f.x; f1 += f.y; f2 += f.z; f3 += f.w;
+          f0 += f.x; f1 += f.y; f2 += f.z; f3 += f.w;   // (seven more roundings)
         }
       }
       __syncthreads();
     }
     if (in && grp == 0) {
-      // the FP32 sums in units of 2^(zbe - 1022)
-      zv.x -= fx::scale2((double)f0, zbe - 1022);
-      zv.y -= fx::scale2((double)f1, zbe - 1022);
-      zv.z -= fx::scale2((double)f2, zbe - 1022);
-      zv.w -= fx::scale2((double)f3, zbe - 1022);
+      flush();
       a.z[x] = zv;
       m = max(m, mag4(zv));
       if (a.last) nrm = fma(zv.x, zv.x, fma(zv.y, zv.y, fma(zv.z, zv.z, fma(zv.w, zv.w, nrm))));

@@ -278,3 +278,18 @@ def test_gram_schmidt_of_a_peak_on_a_flat_floor():
     start[500, 500] = (1.0, 0.5j)
     gram, _ = ritz_gram(make(g, 1, shift=MC2), start, 3)
     assert np.max(gram) <= 256 * U
+
+
+@pytest.mark.parametrize("nx,ny,k", [(61, 47, 250), (251, 173, 140)])
+def test_values_of_many_iterations(nx, ny, k):
+    """T of k iterations, with every coefficient of the update counting: the small ones
+    are applied in FP32, 128 vectors at a time (by eight warps a site on the small
+    grid)."""
+    g = wl.Grid(nx, ny, 0.1, 0.1)
+    V = wl.smoothed_coulomb(g, 20.0, 0.5)
+    start = wl.random_spinor(g, 12)
+    kw = dict(n_want=k, max_iter=k, tol=1e9, window=(-1e9, 1e9), check_every=k)
+    res = make(g, 1, V=V, shift=MC2).eigs(dev(start), **kw)
+    ref = lz.lanczos_eigs(ham.Operator(nx, ny, 0.1, 0.1, V=V, shift=MC2), start, **kw)
+    assert res.values.size == ref.values.size == k
+    assert np.max(np.abs(res.values - ref.values)) <= 1e-11 * (hnorm(g, 2) + np.max(np.abs(V)))
