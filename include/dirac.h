@@ -259,8 +259,8 @@ dirac_status dirac_batch_sync(dirac_batch* batch, dirac_step_info* info);
  * states psi_dev (the states themselves and the scalar blocks are left
  * unchanged), keeps the fastest, and, when the environment variable
  * DIRAC_AUTOTUNE_CACHE names a file, records the choice there by a
- * signature of the problem set (precision, stencil, boundary, sizes, m,
- * GPU) and reuses it on later calls.  A_xy_host: as for dirac_batch_steps
+ * signature of the problem set (precision, stencil, boundary, sites and
+ * tiles, m, the kernels' generation, GPU) and reuses it on later calls.  A_xy_host: as for dirac_batch_steps
  * (for `steps` steps) or NULL.  Allocates scratch (the states' size).
  */
 typedef struct {

@@ -1294,17 +1294,24 @@ dirac_status dirac_batch_autotune(dirac_batch* bt, void* const* psi_dev, double 
   if (steps < 1) return fail(DIRAC_EINVAL, "steps must be >= 1");
   Engine& e = bt->e;
   const int np = e.nprob();
-  long long sites = 0;
-  for (const HostProblem& q : e.P) sites += q.n;
-  char sig[256];
+  long long sites = 0, tiles = 0;
+  for (const HostProblem& q : e.P) {
+    sites += q.n;
+    tiles += tiles_of(q.nx, q.ny, 16);
+  }
+  // Which kernels the tile heights select: 32 and 16 stand for 16 and 8 rows of the
+  // fixed-point FP64 kernels, for themselves on the mixed path (and stood for
+  // themselves on the FP64 path of before, whose lines had no `kern`)
+  const char* kern = e.precision == DIRAC_FP64 ? "fixed" : "f32";
+  char sig[512];
   {
     int dev = 0;
     cudaDeviceProp prop;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
     for (char* c = prop.name; *c; ++c) if (*c == ' ') *c = '_';
-    snprintf(sig, sizeof(sig), "prec=%d,order=%d,bnd=%d,nprob=%d,sites=%lld,m=%d,sm=%d,gpu=%s", e.precision,
-             e.order, e.boundary, np, sites, m, e.shape.n_sm, prop.name);
+    snprintf(sig, sizeof(sig), "prec=%d,order=%d,bnd=%d,nprob=%d,sites=%lld,tiles=%lld,m=%d,kern=%s,sm=%d,gpu=%s",
+             e.precision, e.order, e.boundary, np, sites, tiles, m, kern, e.shape.n_sm, prop.name);
   }
   const char* cache = std::getenv("DIRAC_AUTOTUNE_CACHE");
   if (cache && cache[0]) {

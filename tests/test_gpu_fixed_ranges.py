@@ -293,3 +293,28 @@ def test_values_of_many_iterations(nx, ny, k):
     ref = lz.lanczos_eigs(ham.Operator(nx, ny, 0.1, 0.1, V=V, shift=MC2), start, **kw)
     assert res.values.size == ref.values.size == k
     assert np.max(np.abs(res.values - ref.values)) <= 1e-11 * (hnorm(g, 2) + np.max(np.abs(V)))
+
+
+# --- the autotuner's cache --------------------------------------------------
+
+def test_autotune_cache_of_other_kernels_is_not_taken(tmp_path, monkeypatch):
+    """A line without the kernels' tag (tile heights that meant others) is not
+    taken; a batch of the same sites in other shapes has a line of its own."""
+    from paper_1407_7370_gb300 import BatchPropagator
+    f = tmp_path / "tune.txt"
+    monkeypatch.setenv("DIRAC_AUTOTUNE_CACHE", str(f))
+
+    def tune(grids):
+        bp = BatchPropagator(grids, m_max=4)
+        psis = []
+        for k, (nx, ny, dx, dy) in enumerate(grids):
+            bp.set_fields(k)
+            psis.append(dev(wl.random_spinor(wl.Grid(nx, ny, dx, dy), k)))
+        return bp.autotune(psis, 1e-4, 4, steps=1)
+    grids = [(64, 48, 0.1, 0.1), (96, 32, 0.1, 0.1)]
+    assert not tune(grids)["from_cache"] and tune(grids)["from_cache"]
+    key, rest = f.read_text().split(" ", 1)
+    old = [s for s in key.split(",") if s.split("=")[0] in ("prec", "order", "bnd", "nprob", "sites", "m", "sm", "gpu")]
+    f.write_text(",".join(old) + " " + rest)
+    assert not tune(grids)["from_cache"]
+    assert not tune([(3072, 1, 0.1, 0.1), (1, 3072, 0.1, 0.1)])["from_cache"]
