@@ -21,8 +21,8 @@
 // Every sum is taken in a fixed order (per-CTA partials, then one warp), so
 // results are bitwise reproducible.  No kernel waits on another CTA.
 //
-// The Ritz values come from a Sturm-sequence multisection on T_k (one warp
-// per eigenvalue, 32 points per round), their vectors from inverse iteration
+// The Ritz values come from a Sturm-sequence multisection on T_k (four warps
+// per eigenvalue, 128 points per round), their vectors from inverse iteration
 // with a partially pivoted LU of T_k - theta (two solves, orthogonalised
 // within clusters of close values); T_k is scaled by a power of two so that
 // the characteristic-polynomial recurrence stays in range.
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(256) eig_apply32(const ApplyArgs a) {
 // and its halo as 59-bit numbers in shared memory, each row of
 // the operator one sum of products, then times s_i.  Of the FP64 pipe only the
 // four conversions of the result are left; with some 40 multiply-adds a site it
-// bounded the product (2048^2 with V: 342 us, 0.9 TB/s; now 115 us, 2.6 TB/s,
+// bounded the product (2048^2 with V: 342 us, 0.9 TB/s; now 110 us, 2.7 TB/s,
 // bound by latency and instruction issue).  Tiles with numbers that are not
 // finite, or none above 2^-894, take the floating-point form.  So do tiles whose
 // V is so uneven that the row of its smallest |V| would have to be computed at a

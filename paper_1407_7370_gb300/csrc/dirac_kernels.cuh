@@ -322,7 +322,8 @@ __device__ inline void cheb_expm_e1(const ChebParams& cp, int k, double alpha_j,
 // FX (the FP64 path): the pass stores 2^yexp y^ with yexp an integer chosen
 // before it, and g = 1 on that vector: forming q^ then takes one multiply-add
 // per number instead of two, and no scale can overflow.  P and Y come in for
-// the scaled vector.
+// the scaled vector.  This form serves the probe, states at the ends of the range and
+// sums that are not finite; the other passes take finish_fast.
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 // floor(log2 x) of a positive normal number; 0 for zero
 __device__ __forceinline__ int log2_floor(double x) { return x > 0.0 ? fx::exp_field(x) - 1023 : 0; }
