@@ -55,9 +55,9 @@ def STEP_BYTES_PER_SITE_MIXED(m):    # complex64 basis; psi read and written in 
 # configured grid, valid only for the kernel sources it was taken with
 # (kernel_sha).
 TRAFFIC_SOURCES = ("dirac_kernels.cuh", "dirac_step32.cu", "dirac_pass64.cuh", "dirac_fixed.cuh")
-TRAFFIC = {"lanczos_step64": ("c644ac97325d", 1.607975e9 + 1.366588e9),
-           "lanczos_pass<float>": ("c644ac97325d", 33.650176e6 + 0.514560e6),
-           "lanczos_step_m32": ("c644ac97325d", 317.762816e6 + 487.556352e6)}
+TRAFFIC = {"lanczos_step64": ("662118b2716e", 1.609525e9 + 1.366620e9),
+           "lanczos_pass<float>": ("662118b2716e", 33.638400e6 + 0.492800e6),
+           "lanczos_step_m32": ("662118b2716e", 316.996608e6 + 487.166720e6)}
 
 
 def rounded(x, digits=6):
