@@ -207,21 +207,30 @@ __global__ void split_float_kernel(const double* in, float* hi, float* lo, long 
   }
 }
 
-__global__ void minmax_kernel(const double* v, long long n, double* out) {
-  __shared__ double smin[256], smax[256];
+// min and max of v by one block (-inf, inf if an entry is not finite), eight loads of
+// a thread in flight: V may be read here for the first time
+constexpr int MINMAX_THREADS = 1024;
+__global__ void __launch_bounds__(MINMAX_THREADS) minmax_kernel(const double* v, long long n, double* out) {
+  __shared__ double smin[MINMAX_THREADS], smax[MINMAX_THREADS];
+  constexpr int U = 8;
   double lo = 1e308, hi = -1e308;
   bool bad = false;
-  for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-    const double x = v[i];
-    lo = fmin(lo, x);
-    hi = fmax(hi, x);
-    if (!isfinite(x)) bad = true;
+  for (long long i = threadIdx.x; i < n; i += U * MINMAX_THREADS) {
+    double x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u] = v[min(i + u * MINMAX_THREADS, n - 1)];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      lo = fmin(lo, x[u]);
+      hi = fmax(hi, x[u]);
+      if (!isfinite(x[u])) bad = true;
+    }
   }
   if (bad) { lo = -INFINITY; hi = INFINITY; }
   smin[threadIdx.x] = lo;
   smax[threadIdx.x] = hi;
   __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
+  for (int s = MINMAX_THREADS / 2; s > 0; s >>= 1) {
     if (threadIdx.x < s) {
       smin[threadIdx.x] = fmin(smin[threadIdx.x], smin[threadIdx.x + s]);
       smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + s]);
@@ -510,24 +519,24 @@ dirac_status Engine::set_fields(int b, const double* V_dev, double ax, double ay
     return fail(DIRAC_EINVAL, "non-finite field scalar");
   HostProblem& q = P[b];
   if (V_dev) {
-    // checked before anything of the problem changes: a refused V leaves the fields
+    // checked before anything that a step reads changes: a refused V leaves the fields
     // as they were
+    const bool f32 = precision != DIRAC_FP64;
+    if (!q.V) CUDA_TRY(cudaMalloc(&q.V, (f32 ? sizeof(float) : sizeof(double)) * q.n));
+    if (f32 && !q.Vlo) CUDA_TRY(cudaMalloc(&q.Vlo, sizeof(float) * q.n));
+    if (f32 && !q.V64) CUDA_TRY(cudaMalloc(&q.V64, sizeof(double) * q.n));
     double* mm = d_partials;   // two doubles of scratch (rewritten by every pass)
-    minmax_kernel<<<1, 256, 0, stream>>>(V_dev, q.n, mm);
+    minmax_kernel<<<1, MINMAX_THREADS, 0, stream>>>(V_dev, q.n, mm);
     ++launches;
     CUDA_TRY(cudaGetLastError());
     double h[2];
     CUDA_TRY(cudaMemcpyAsync(h, mm, sizeof(h), cudaMemcpyDeviceToHost, stream));
     CUDA_TRY(cudaStreamSynchronize(stream));
     if (!std::isfinite(h[0]) || !std::isfinite(h[1])) return fail(DIRAC_EINVAL, "V has non-finite entries");
-    const bool f32 = precision != DIRAC_FP64;
-    if (!q.V) CUDA_TRY(cudaMalloc(&q.V, (f32 ? sizeof(float) : sizeof(double)) * q.n));
     if (f32) {
-      if (!q.Vlo) CUDA_TRY(cudaMalloc(&q.Vlo, sizeof(float) * q.n));
       split_float_kernel<<<256, 256, 0, stream>>>(V_dev, static_cast<float*>(q.V), q.Vlo, q.n);
       ++launches;
       CUDA_TRY(cudaGetLastError());
-      if (!q.V64) CUDA_TRY(cudaMalloc(&q.V64, sizeof(double) * q.n));
     } else {
       q.V64 = static_cast<double*>(q.V);
     }
@@ -1559,7 +1568,7 @@ extern "C" dirac_status dirac_lanczos_step_noalloc(const dirac_problem* pb, void
   // spectral interval of H - s (needs the range of V: read back two doubles)
   double vmin = 0.0, vmax = 0.0;
   if (pb->V_dev) {
-    minmax_kernel<<<1, 256, 0, stream>>>(pb->V_dev, n, partials);
+    minmax_kernel<<<1, MINMAX_THREADS, 0, stream>>>(pb->V_dev, n, partials);
     CUDA_TRY(cudaGetLastError());
     double h[2];
     CUDA_TRY(cudaMemcpyAsync(h, partials, sizeof(h), cudaMemcpyDeviceToHost, stream));
